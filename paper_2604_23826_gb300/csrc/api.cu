@@ -79,7 +79,8 @@ struct stats_ctx {
   long long* d_fn = nullptr;
   double* d_slots = nullptr;            // FP64 scratch: block slots + ticket
   int slot_grid = 0;
-  double* d_core_slots = nullptr;       // CUDA-core comparators (wide FP64, FP32) scratch
+  void* d_core_slots = nullptr;         // CUDA-core passes (wide FP64, FP32) scratch: block slots
+  size_t core_bytes = 0;
   unsigned int* d_core_ticket = nullptr;
   int core_grid = 0;
   float* d_fshift = nullptr;            // BF16X3/X4: pivot as float
@@ -328,6 +329,17 @@ stats_status ensure_slots(stats_ctx* c, int grid) {
   CK(c, cudaMalloc(&c->d_slots, n * sizeof(double)));
   CK(c, cudaMemset(c->d_slots, 0, n * sizeof(double)));
   c->slot_grid = grid;
+  return STATS_OK;
+}
+
+// Scratch of the CUDA-core passes (block slots), grown as a call needs it.
+stats_status ensure_core_slots(stats_ctx* c, size_t bytes) {
+  if (c->core_bytes >= bytes) return STATS_OK;
+  if (c->d_core_slots) CK(c, cudaFree(c->d_core_slots));
+  c->d_core_slots = nullptr;
+  c->core_bytes = 0;
+  CK(c, cudaMalloc(&c->d_core_slots, bytes));
+  c->core_bytes = bytes;
   return STATS_OK;
 }
 
@@ -946,8 +958,36 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
     S.acc_S_lo = c->d_fS_lo;
     S.acc_n = c->d_fn;
     CK(c, launch_split(S, T, split_x4(c, nrows), g, st));
-  } else if (c->mode == STATS_FP32 || c->p > 12) {
-    // tiled CUDA-core pass: FP32-core, or FP64 for tables wider than the row kernel
+  } else if (c->mode == STATS_FP32) {
+    Core32Params C{};
+    C.p = c->p;
+    for (int j = 0; j < c->p; ++j) {
+      C.cols[j] = dcols[j];
+      C.dtype[j] = c->dtypes[j];
+      if (c->dtypes[j] == F32 && aligned16(dcols[j]))
+        C.quick[j >> 5] |= 1u << (j & 31);
+      else
+        C.any_slow = 1;
+    }
+    if (!c->shift_set) {
+      CK(c, launch_set_shift(dcols, c->dtypes.data(), c->p, nrows, c->d_shift, st));
+      c->shift_set = true;
+    }
+    C.shift = c->d_shift;
+    core32_plan(c->p, nrows, c->sms, c->grid, C);
+    const stats_status s = ensure_core_slots(c, core32_slot_bytes(C));
+    if (s != STATS_OK) return s;
+    C.flush_rows = c->flush_rows > 0 ? c->flush_rows : 64;
+    C.nrows = nrows;
+    C.slots = reinterpret_cast<float*>(c->d_core_slots);
+    C.acc_s = c->d_fs;
+    C.acc_s_lo = c->d_fs_lo;
+    C.acc_S = c->d_fS;
+    C.acc_S_lo = c->d_fS_lo;
+    C.acc_n = c->d_fn;
+    CK(c, launch_core32(C, st));
+  } else if (c->p > 12) {
+    // tiled CUDA-core pass: FP64 tables wider than the row kernel
     CoreParams C{};
     for (int j = 0; j < c->p; ++j) {
       C.cols[j] = dcols[j];
@@ -974,18 +1014,17 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
       CK(c, cudaMalloc(&c->d_core_slots, bytes));
       CK(c, cudaMemset(c->d_core_slots, 0, bytes));
       c->core_grid = g;
-      c->d_core_ticket = reinterpret_cast<unsigned int*>(c->d_core_slots + core_slot_doubles(g));
+      c->d_core_ticket = reinterpret_cast<unsigned int*>(static_cast<double*>(c->d_core_slots) + core_slot_doubles(g));
     }
-    C.flush_rows = c->flush_rows > 0 ? c->flush_rows : 64;
     C.nrows = nrows;
-    C.slots = c->d_core_slots;
+    C.slots = static_cast<double*>(c->d_core_slots);
     C.ticket = c->d_core_ticket;
     C.acc_s = c->d_fs;
     C.acc_s_lo = c->d_fs_lo;
     C.acc_S = c->d_fS;
     C.acc_S_lo = c->d_fS_lo;
     C.acc_n = c->d_fn;
-    CK(c, launch_core(C, c->mode == STATS_FP32, g, st));
+    CK(c, launch_core(C, g, st));
   } else {
     Fp64Params P{};
     for (int j = 0; j < c->p; ++j) {

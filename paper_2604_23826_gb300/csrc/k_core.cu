@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kThreads) core_kernel(const __grid_constant__ 
           if (diag_sub && tx == 0) sacc[i] += a[i];
         }
       }
-      if (flush_pairs && (since += rows) >= P.flush_rows) {
+      if (flush_pairs && (since += rows) >= 64) {
         since = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -182,19 +182,12 @@ __global__ void __launch_bounds__(kThreads) core_kernel(const __grid_constant__ 
 
 size_t core_slot_doubles(int grid) { return static_cast<size_t>(grid) * 4 * kCoreSlotDoubles; }
 
-cudaError_t launch_core(const CoreParams& P, bool fp32, int grid, cudaStream_t stream) {
-  const size_t smem = 2 * kT * kLd * (fp32 ? sizeof(float) : sizeof(double));
-  if (fp32) {
-    cudaError_t e = cudaFuncSetAttribute(core_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    core_kernel<float><<<grid, kThreads, smem, stream>>>(P);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(core_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    core_kernel<double><<<grid, kThreads, smem, stream>>>(P);
-  }
+cudaError_t launch_core(const CoreParams& P, int grid, cudaStream_t stream) {
+  const size_t smem = 2 * kT * kLd * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(core_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  core_kernel<double><<<grid, kThreads, smem, stream>>>(P);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,318 @@
+// k_core32.cu -- the FP32-core pass (STATS_FP32): n, X^T 1 and X^T X of x - c with FP32 FMA on the
+// CUDA cores, flushed into FP32 (hi, lo) pairs at least every 64 rows (arxiv 2604.23826, "Data
+// Representation and Sufficient Statistics" with the shift of "Numerical Considerations").
+//
+// Bound: FP32 FMA for more than about fifty columns (p (p + 1) / 2 per row at 128 per clock and
+// SM), HBM below.  So the layout spends shared-memory reads and issue slots on as little else as
+// possible:
+//   - the output's upper triangle is cut into 8 x 4 register micro-tiles, one per thread: three
+//     128-bit shared loads feed 32 FMAs (the row's 8 left values are the same for most of a warp, a
+//     broadcast; the 4 right values of consecutive lanes are consecutive, conflict-free).  Only
+//     tiles on or above the diagonal exist, so 100 columns cost 5408 FMAs a row for 5050 entries;
+//   - when there are fewer tiles than threads, the rows of a stage are dealt to several slices of
+//     threads; when there are more, groups of blocks take a part of the tiles each.  core32_plan
+//     picks the number of groups by the instructions a row costs;
+//   - columns are copied as they lie (cp.async, 16 bytes, two stages ahead), then one pass turns a
+//     stage into rows of x - c (lanes = columns: conflict-free both ways) and adds the column sums.
+// Columns of other types, or not 16-byte aligned, are converted (x - c in FP64) into the same
+// stage by plain loads.
+// 1e6 rows x 100 columns: 8.78 ms as 64 x 64 tiles of scalar shared loads with an FP64 subtraction
+// per element, about 0.13 ms now (its FMAs alone take 0.125 ms at 80 TFLOP/s).
+// Each block writes one slot of (hi, lo) pairs; a second kernel adds the slots of an entry in row
+// order, in three-term FP32 expansions and then FP64 pairs (a fixed order: a given grid
+// reproduces its bits).
+#include <algorithm>
+
+#include "core.cuh"
+
+namespace ss {
+
+namespace {
+
+using namespace core;
+
+constexpr int kMI = 8, kMJ = 4, kE = kMI * kMJ;
+constexpr int kNT = 512;
+constexpr int kStageFloats = 16384;  // columns (padded) x rows of a stage, at most
+constexpr int kTreeBytes = (kNT / 2) * kE * 8;  // the slices' pairs on their way to one slot
+
+__host__ __device__ inline int width_of(int p) { return (p + kMI - 1) / kMI * kMI; }
+__host__ __device__ inline size_t raw_bytes(int W, int R) { return static_cast<size_t>(W) * (R + 4) * 4; }
+__host__ __device__ inline size_t row_bytes(int W, int R) { return static_cast<size_t>(R) * (W + 4) * 4; }
+
+__global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ Core32Params P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int p = P.p, W = width_of(p), R = 1 << P.log_rows, S = W + 4, K = R + 4;
+  float* raw = reinterpret_cast<float*>(smem);                         // [2][W][K], as the columns lie
+  float* X = reinterpret_cast<float*>(smem + 2 * raw_bytes(W, R));      // [R][S], rows of x - c
+  const int tid = threadIdx.x;
+  const int g = blockIdx.x % P.groups, range = blockIdx.x / P.groups;
+  const int64_t nst = (P.nrows + R - 1) >> P.log_rows;
+  const int64_t st0 = nst * range / P.ranges, st1 = nst * (range + 1) / P.ranges;
+
+  // compute: slice tid / tg takes rows slice, slice + slices, ... of a stage for tile tid % tg
+  const int tg = P.tiles_per_group, slice = tid / tg, tl = tid % tg;
+  const int tile = g * tg + tl;
+  const bool active = slice < P.slices && tile < P.ntiles;
+  int bi = 0, bj = 0;
+  if (active) tile_of<kMI, kMJ>(tile, p, bi, bj);
+  float acc[kMI][kMJ], hi[kMI][kMJ], lo[kMI][kMJ];
+#pragma unroll
+  for (int i = 0; i < kMI; ++i)
+#pragma unroll
+    for (int j = 0; j < kMJ; ++j) acc[i][j] = hi[i][j] = lo[i][j] = 0.f;
+  int since = 0;
+  auto flush = [&] {
+    since = 0;
+#pragma unroll
+    for (int i = 0; i < kMI; ++i)
+#pragma unroll
+      for (int j = 0; j < kMJ; ++j) {
+        pair_add(hi[i][j], lo[i][j], acc[i][j]);
+        acc[i][j] = 0.f;
+      }
+  };
+
+  // conversion: this thread's column and its share of the stage's row quads
+  const int cc = tid % W, cq = tid / W, ncq = kNT / W;
+  const bool quick = cc < p && (P.quick[cc >> 5] >> (cc & 31) & 1u);
+  const float shift = quick ? static_cast<float>(P.shift[cc]) : 0.f;
+  float shi = 0.f, slo = 0.f;
+
+  auto issue = [&](int64_t st) {
+    float* dst = raw + (st & 1) * (raw_bytes(W, R) / 4);
+    const int64_t r0 = st << P.log_rows;
+    const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - r0));
+    const int lq = P.log_rows - 2;  // quads of a column: 2^lq
+    for (int i = tid; i < (p << lq); i += kNT) {
+      const int c = i >> lq, k = (i & ((1 << lq) - 1)) * 4;
+      if (!(P.quick[c >> 5] >> (c & 31) & 1u)) continue;
+      const int have = min(4, max(0, rows - k));
+      const float* src = static_cast<const float*>(P.cols[c]) + r0 + (have ? k : 0);
+      cp_async16(smem_u32(dst + c * K + k), src, 4 * have);
+    }
+    if (P.any_slow)
+      for (int i = tid; i < (p << P.log_rows); i += kNT) {
+        const int c = i >> P.log_rows, k = i & (R - 1);
+        if (P.quick[c >> 5] >> (c & 31) & 1u) continue;
+        if (k < rows) {
+          float v;
+          if (P.dtype[c] == F32)
+            v = static_cast<const float*>(P.cols[c])[r0 + k] - static_cast<float>(P.shift[c]);
+          else
+            v = static_cast<float>(load_as_double(P.cols[c], P.dtype[c], r0 + k) - P.shift[c]);
+          dst[c * K + k] = v;
+        }
+      }
+  };
+
+  if (st0 < st1) issue(st0);
+  cp_async_commit();
+  if (st0 + 1 < st1) issue(st0 + 1);
+  cp_async_commit();
+  for (int64_t st = st0; st < st1; ++st) {
+    cp_async_wait<1>();
+    __syncthreads();  // the stage has landed; the last stage's rows have been read
+    const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - (st << P.log_rows)));
+    if (cq < ncq) {
+      const float* src = raw + (st & 1) * (raw_bytes(W, R) / 4) + cc * K;
+      float s = 0.f;
+      for (int k = 4 * cq; k < R; k += 4 * ncq) {
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (cc < p) {
+          const float4 x = *reinterpret_cast<const float4*>(src + k);
+          v[0] = k < rows ? x.x - shift : 0.f;
+          v[1] = k + 1 < rows ? x.y - shift : 0.f;
+          v[2] = k + 2 < rows ? x.z - shift : 0.f;
+          v[3] = k + 3 < rows ? x.w - shift : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) X[(k + i) * S + cc] = v[i];
+        s += (v[0] + v[1]) + (v[2] + v[3]);
+      }
+      pair_add(shi, slo, s);
+    }
+    __syncthreads();
+    if (st + 2 < st1) issue(st + 2);
+    cp_async_commit();
+    if (active) {
+      const float* xa = X + kMI * bi;
+      const float* xb = X + kMJ * bj;
+      for (int k = slice; k < rows;) {
+        if (since == P.flush_rows) flush();
+        const int m = min((rows - k + P.slices - 1) / P.slices, P.flush_rows - since);
+        since += m;
+        for (int i = 0; i < m; ++i, k += P.slices) {
+          const float4 a0 = *reinterpret_cast<const float4*>(xa + k * S);
+          const float4 a1 = *reinterpret_cast<const float4*>(xa + k * S + 4);
+          const float4 b4 = *reinterpret_cast<const float4*>(xb + k * S);
+          const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+          const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+          for (int u = 0; u < kMI; ++u)
+#pragma unroll
+            for (int v = 0; v < kMJ; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+        }
+      }
+    }
+  }
+  cp_async_wait<0>();
+  flush();
+  // the slices' pairs, added in a fixed tree through shared memory
+  float2* buf = reinterpret_cast<float2*>(smem);
+  for (int n = P.slices; n > 1;) {
+    const int h = (n + 1) / 2;
+    __syncthreads();
+    if (slice >= h && slice < n) {
+#pragma unroll
+      for (int e = 0; e < kE; ++e)
+        buf[e * (kNT / 2) + (slice - h) * tg + tl] = make_float2(hi[e / kMJ][e % kMJ], lo[e / kMJ][e % kMJ]);
+    }
+    __syncthreads();
+    if (slice < n - h) {
+#pragma unroll
+      for (int e = 0; e < kE; ++e) {
+        const float2 v = buf[e * (kNT / 2) + slice * tg + tl];
+        pair_add(hi[e / kMJ][e % kMJ], lo[e / kMJ][e % kMJ], v.x);
+        lo[e / kMJ][e % kMJ] += v.y;
+      }
+    }
+    n = h;
+  }
+  float2* slot = reinterpret_cast<float2*>(P.slots) + static_cast<size_t>(blockIdx.x) * core32_slot_pairs(p, tg);
+  if (slice == 0) {
+#pragma unroll
+    for (int e = 0; e < kE; ++e)
+      slot[static_cast<size_t>(e) * tg + tl] = make_float2(hi[e / kMJ][e % kMJ], lo[e / kMJ][e % kMJ]);
+  }
+  __syncthreads();
+  if (cq < ncq) buf[cq * W + cc] = make_float2(shi, slo);
+  __syncthreads();
+  if (tid < W) {
+    float h = 0.f, l = 0.f;
+    for (int i = 0; i < ncq; ++i) {
+      const float2 v = buf[i * W + tid];
+      pair_add(h, l, v.x);
+      l += v.y;
+    }
+    slot[static_cast<size_t>(kE) * tg + tid] = make_float2(h, l);
+  }
+}
+
+// Adds the ranges' slots of 32 entries per block (kSeg consecutive runs of ranges at once) into
+// the accumulators.  Within a run a three-term FP32 expansion keeps every rounding of the pairs'
+// additions (72 bits; FP64 adds would cost 64 cycles a warp each); the runs are added in order in
+// FP64 pairs.
+constexpr int kSeg = 8;
+__device__ __forceinline__ float two_sum32(float& s, float v) {
+  const float t = s + v, bp = t - s, e = (s - (t - bp)) + (v - bp);
+  s = t;
+  return e;
+}
+
+__global__ void __launch_bounds__(32 * kSeg) core32_merge_kernel(const __grid_constant__ Core32Params P) {
+  __shared__ double sh[kSeg][32], sl[kSeg][32];
+  const int p = P.p, tg = P.tiles_per_group, lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int nS = P.ntiles * kE;
+  const int x = blockIdx.x * 32 + lane;  // entry: tiles' values, then the column sums
+  const size_t sp = core32_slot_pairs(p, tg);
+  int j = -1, k = -1;
+  size_t off = 0;
+  if (x < nS) {
+    const int e = x / P.ntiles, t = x % P.ntiles, g = t / tg;
+    int bi, bj;
+    tile_of<kMI, kMJ>(t, p, bi, bj);
+    j = kMI * bi + e / kMJ;
+    k = kMJ * bj + e % kMJ;
+    if (j > k || k >= p) j = -1;
+    off = static_cast<size_t>(g) * sp + static_cast<size_t>(e) * tg + (t - g * tg);
+  } else if (x < nS + p) {
+    j = k = x - nS;
+    off = static_cast<size_t>(kE) * tg + j;
+  }
+  float h = 0.f, l = 0.f, ll = 0.f;
+  if (j >= 0) {
+    const float2* src = reinterpret_cast<const float2*>(P.slots) + off;
+    const size_t step = static_cast<size_t>(P.groups) * sp;
+    const int r0 = P.ranges * seg / kSeg, r1 = P.ranges * (seg + 1) / kSeg;
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) {
+      const float2 v = __ldcg(src + r * step);
+      const float e1 = two_sum32(h, v.x);
+      const float e2 = two_sum32(l, e1);
+      ll += e2 + two_sum32(l, v.y);
+    }
+  }
+  double dh = h, dl = 0.0;
+  pair_add(dh, dl, static_cast<double>(l));
+  dl += ll;
+  sh[seg][lane] = dh;
+  sl[seg][lane] = dl;
+  __syncthreads();
+  if (seg == 0 && j >= 0) {
+    for (int s = 1; s < kSeg; ++s) {
+      pair_add(dh, dl, sh[s][lane]);
+      dl += sl[s][lane];
+    }
+    const int idx = x < nS ? j * p - j * (j - 1) / 2 + (k - j) : j;
+    double* ah = (x < nS ? P.acc_S : P.acc_s) + idx;
+    double* al = (x < nS ? P.acc_S_lo : P.acc_s_lo) + idx;
+    double vh = *ah, vl = *al;
+    pair_add(vh, vl, dh);
+    *ah = vh;
+    *al = vl + dl;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.acc_n += P.nrows;
+}
+
+size_t smem_bytes(int W, int R) {
+  return std::max<size_t>(2 * raw_bytes(W, R) + row_bytes(W, R), kTreeBytes);
+}
+
+}  // namespace
+
+// The cut of p columns and nrows rows for `sms` SMs (or `blocks` blocks, when positive).
+void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P) {
+  const int W = width_of(p), M = tile_count(p, kMI, kMJ);
+  P.ntiles = M;
+  // groups of blocks over the tiles: the fewest warp instructions a row costs the SMs together,
+  // ~35 per warp of tiles (32 FMAs and 3 loads; warps run four at a time) and ~14 per 128
+  // converted values in every group
+  double best = 0;
+  for (int G = (M + kNT - 1) / kNT; G <= 4 * ((M + kNT - 1) / kNT); ++G) {
+    const int tg = (M + G - 1) / G, ks = kNT / tg;
+    if (tg * (G - 1) >= M) continue;
+    const int quads = ((tg * ks + 31) / 32 + 3) / 4;
+    const double cost = G * (quads * 4 * 35.0 / ks + W * 14.0 / 128);
+    if (best == 0 || cost < best) {
+      best = cost;
+      P.groups = G;
+      P.tiles_per_group = tg;
+      P.slices = ks;
+    }
+  }
+  // rows of a stage: as many as shared memory takes, fewer while that would leave SMs without one
+  int lr = 6;
+  const int want = std::max(1, (blocks > 0 ? blocks : sms) / P.groups);
+  while (lr < 11 && (W << (lr + 1)) <= kStageFloats && (nrows >> (lr + 1)) >= 2 * int64_t(want)) ++lr;
+  P.log_rows = lr;
+  const int64_t nst = (nrows + (int64_t(1) << lr) - 1) >> lr;
+  P.ranges = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, nst)));
+}
+
+size_t core32_slot_bytes(const Core32Params& P) {
+  return static_cast<size_t>(P.groups) * P.ranges * core32_slot_pairs(P.p, P.tiles_per_group) * sizeof(float2);
+}
+
+cudaError_t launch_core32(const Core32Params& P, cudaStream_t stream) {
+  const size_t smem = smem_bytes(width_of(P.p), 1 << P.log_rows);
+  cudaError_t e = cudaFuncSetAttribute(core32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  core32_kernel<<<P.groups * P.ranges, kNT, smem, stream>>>(P);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  core32_merge_kernel<<<(P.ntiles * kE + P.p + 31) / 32, 32 * kSeg, 0, stream>>>(P);
+  return cudaGetLastError();
+}
+
+}  // namespace ss

@@ -275,8 +275,34 @@ cudaError_t launch_narrow(const NarrowParams& P, bool x4, int grid, cudaStream_t
 cudaError_t launch_narrow_shift(const NarrowTab* tabs, const int* which, int count, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// CUDA-core comparators for any width: FP64 (raw / shifted) and FP32-core.
+// CUDA-core passes for any width: FP32-core (k_core32.cu), FP64 raw or shifted (k_core.cu).
 // ---------------------------------------------------------------------------
+struct Core32Params {
+  const void* cols[256];
+  int32_t dtype[256];
+  uint32_t quick[8];    // bit c: column c is FP32 and 16-byte aligned (copied asynchronously)
+  int32_t any_slow;     // some column is not
+  const double* shift;  // p pivots
+  int32_t p;
+  int32_t flush_rows;   // rows of a thread between flushes into (hi, lo) pairs
+  int64_t nrows;
+  // the cut (core32_plan): micro-tiles, groups of blocks over them, row slices of a block,
+  // 2^log_rows rows a stage, row ranges; groups * ranges blocks
+  int32_t ntiles, groups, tiles_per_group, slices, log_rows, ranges;
+  float* slots;         // scratch: core32_slot_bytes
+  double* acc_s;        // ctx accumulators, double-double
+  double* acc_s_lo;
+  double* acc_S;
+  double* acc_S_lo;
+  long long* acc_n;
+};
+// (hi, lo) pairs of a block's slot: its tiles' entries, then the padded columns' sums
+__host__ __device__ inline size_t core32_slot_pairs(int p, int tiles_per_group) {
+  return static_cast<size_t>(tiles_per_group) * 32 + (p + 7) / 8 * 8;
+}
+void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P);
+size_t core32_slot_bytes(const Core32Params& P);
+cudaError_t launch_core32(const Core32Params& P, cudaStream_t stream);
 constexpr int kCoreSlotDoubles = 2 * (32 * 32 + 32);
 struct CoreParams {
   const void* cols[256];
@@ -286,7 +312,6 @@ struct CoreParams {
   int32_t nblk;         // ceil(p / 64)
   int32_t ntiles;
   int32_t ksplit;
-  int32_t flush_rows;   // FP32 only: rows between flushes into (hi, lo) pairs
   int64_t nrows;
   double* slots;        // scratch: core_slot_doubles(grid)
   unsigned int* ticket;
@@ -297,7 +322,7 @@ struct CoreParams {
   long long* acc_n;
 };
 size_t core_slot_doubles(int grid);
-cudaError_t launch_core(const CoreParams& P, bool fp32, int grid, cudaStream_t stream);
+cudaError_t launch_core(const CoreParams& P, int grid, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------
 // Finalize (one block): recombination, exact centering, cov / corr, Jacobi.
