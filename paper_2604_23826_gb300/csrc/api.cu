@@ -81,8 +81,6 @@ struct stats_ctx {
   int slot_grid = 0;
   void* d_core_slots = nullptr;         // CUDA-core passes (wide FP64, FP32) scratch: block slots
   size_t core_bytes = 0;
-  unsigned int* d_core_ticket = nullptr;
-  int core_grid = 0;
   float* d_fshift = nullptr;            // BF16X3/X4: pivot as float
   float* d_wide_slots = nullptr;        // BF16X3/X4, p > 64 on tcgen05: per-CTA slots
   int wide_grid_alloc = 0;
@@ -987,13 +985,12 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
     C.acc_n = c->d_fn;
     CK(c, launch_core32(C, st));
   } else if (c->p > 12) {
-    // tiled CUDA-core pass: FP64 tables wider than the row kernel
-    CoreParams C{};
+    Core64Params C{};
+    C.p = c->p;
     for (int j = 0; j < c->p; ++j) {
       C.cols[j] = dcols[j];
       C.dtype[j] = c->dtypes[j];
     }
-    C.p = c->p;
     if (c->mode != STATS_FP64) {
       if (!c->shift_set) {
         CK(c, launch_set_shift(dcols, c->dtypes.data(), c->p, nrows, c->d_shift, st));
@@ -1001,30 +998,17 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
       }
       C.shift = c->d_shift;
     }
-    C.nblk = (c->p + 63) / 64;
-    C.ntiles = C.nblk * (C.nblk + 1) / 2;
-    const int64_t max_split = std::max<int64_t>(1, nrows / 4096);
-    C.ksplit = static_cast<int>(std::min<int64_t>(max_split, (4 * c->sms + C.ntiles - 1) / C.ntiles));
-    if (c->grid > 0) C.ksplit = std::max(1, c->grid / C.ntiles);
-    const int g = C.ntiles * C.ksplit;
-    if (!c->d_core_slots || c->core_grid < g) {
-      if (c->d_core_slots) CK(c, cudaFree(c->d_core_slots));
-      c->d_core_slots = nullptr;
-      const size_t bytes = core_slot_doubles(g) * sizeof(double) + 256;
-      CK(c, cudaMalloc(&c->d_core_slots, bytes));
-      CK(c, cudaMemset(c->d_core_slots, 0, bytes));
-      c->core_grid = g;
-      c->d_core_ticket = reinterpret_cast<unsigned int*>(static_cast<double*>(c->d_core_slots) + core_slot_doubles(g));
-    }
+    CK(c, core64_plan(c->p, nrows, C.shift != nullptr, c->sms, c->grid, C));
+    const stats_status s = ensure_core_slots(c, core64_slot_bytes(C));
+    if (s != STATS_OK) return s;
     C.nrows = nrows;
     C.slots = static_cast<double*>(c->d_core_slots);
-    C.ticket = c->d_core_ticket;
     C.acc_s = c->d_fs;
     C.acc_s_lo = c->d_fs_lo;
     C.acc_S = c->d_fS;
     C.acc_S_lo = c->d_fS_lo;
     C.acc_n = c->d_fn;
-    CK(c, launch_core(C, g, st));
+    CK(c, launch_core64(C, st));
   } else {
     Fp64Params P{};
     for (int j = 0; j < c->p; ++j) {

@@ -203,6 +203,17 @@ __device__ __forceinline__ uint64_t fixed_rn(double x, int sh) {
   return q;
 }
 
+// Exact FP32 -> FP64 on the integer pipe (the FP64 unit, conversions included, runs 2 operations
+// per clock and SM).
+__device__ __forceinline__ double f32_to_f64(float v) {
+  const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xFFu;
+  if (e - 1u < 254u)
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)),
+                            static_cast<int>(u << 29));
+  if ((u << 1) == 0) return __hiloint2double(static_cast<int>(u), 0);
+  return static_cast<double>(v);  // subnormal, infinite or NaN
+}
+
 // Biased binary exponent field of a double (0 for zero / subnormal).
 __device__ __forceinline__ int dbl_exp_field(double x) {
   return static_cast<int>((static_cast<uint64_t>(__double_as_longlong(x)) >> 52) & 0x7FF);

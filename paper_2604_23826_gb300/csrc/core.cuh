@@ -47,15 +47,6 @@ __device__ __forceinline__ double i32_to_f64(int32_t v) {
   const uint32_t hi = (static_cast<uint32_t>(v) & 0x80000000u) + (static_cast<uint32_t>(1023 + 30 - lz) << 20) + (n >> 11);
   return v == 0 ? 0.0 : __hiloint2double(static_cast<int>(hi), static_cast<int>(n << 21));
 }
-__device__ __forceinline__ double f32_to_f64(float v) {
-  const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xFFu;
-  if (e - 1u < 254u)
-    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)),
-                            static_cast<int>(u << 29));
-  if ((u << 1) == 0) return __hiloint2double(static_cast<int>(u), 0);
-  return static_cast<double>(v);  // subnormal, infinite or NaN
-}
-
 __device__ __forceinline__ double load_as_double(const void* col, int dt, int64_t r) {
   switch (dt) {
     case I16: return i32_to_f64(static_cast<const int16_t*>(col)[r]);

@@ -1,0 +1,275 @@
+// k_core64.cu -- the plain FP64 CUDA-core pass for tables of more than 12 columns (STATS_FP64 with
+// raw moments, STATS_FP64_SHIFTED on x - c), arxiv 2604.23826, "Data Representation and Sufficient
+// Statistics" with the shift of "Numerical Considerations".
+//
+// Bound: the FP64 unit, 2 operations per clock and SM on GB300 (64 cycles a warp instruction,
+// conversions and additions alike), so p (p + 1) / 2 FMAs plus 2 p additions a row set the time and
+// everything else only has to stay off that unit and keep it fed:
+//   - the output's upper triangle is cut into register micro-tiles of 4 x 4 or 2 x 2 entries, one
+//     per thread, so little is multiplied that nobody reads (48 columns: 1248 of 1176);
+//   - the rows of a stage are dealt to slices of a block's threads, so a few tiles fill all lanes;
+//     core64_plan picks micro-tile, block size, slices and groups by the FP64 cycles a row costs;
+//   - values are read as they lie (lanes = rows), turned into FP64 by integer instructions, shifted
+//     and stored as rows of an odd stride (conflict-free); several blocks per SM overlap the
+//     loads of one with the FMAs of another.
+// 250,001 rows x 48 columns: 6.60 ms as 64 x 64 tiles on 61 blocks, 0.67 ms now (FMAs, shift and
+// sums of those rows alone: 0.50 ms), plus 12 us to add the slots.
+// Each block writes one slot; a second kernel adds an entry's slots in row order into the ctx's
+// double-double accumulators (a fixed order: a given grid reproduces its bits).
+#include <algorithm>
+
+#include "core.cuh"
+
+namespace ss {
+
+namespace {
+
+using namespace core;
+
+constexpr int kMaxThreads = 512;
+constexpr int kBatch = 8;  // loads a lane has in flight
+
+__host__ __device__ inline int row_stride(int p, int MI) { return ((p + MI - 1) / MI * MI) | 1; }
+
+// the bits of value r of a column; to_f64 turns them into the value
+__device__ __forceinline__ uint64_t load_bits(const void* col, int dt, int64_t r) {
+  if (dt == F64 || dt == I64) return static_cast<const uint64_t*>(col)[r];
+  if (dt == I16) return static_cast<uint32_t>(static_cast<const int16_t*>(col)[r]);
+  return static_cast<const uint32_t*>(col)[r];
+}
+__device__ __forceinline__ double to_f64(uint64_t b, int dt) {
+  if (dt == F64) return __longlong_as_double(static_cast<long long>(b));
+  if (dt == F32) return f32_to_f64(__uint_as_float(static_cast<uint32_t>(b)));
+  if (dt == I64) return static_cast<double>(static_cast<long long>(b));
+  return i32_to_f64(static_cast<int32_t>(b));
+}
+
+template <int MI>
+__global__ void __launch_bounds__(kMaxThreads) core64_kernel(const __grid_constant__ Core64Params P) {
+  constexpr int kE = MI * MI;
+  extern __shared__ __align__(16) uint8_t smem[];
+  double* X = reinterpret_cast<double*>(smem);  // [R][S], rows of x - c
+  const int p = P.p, R = 1 << P.log_rows, S = row_stride(p, MI);
+  const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
+  const int g = blockIdx.x % P.groups, range = blockIdx.x / P.groups;
+  const int64_t nst = (P.nrows + R - 1) >> P.log_rows;
+  const int64_t st0 = nst * range / P.ranges, st1 = nst * (range + 1) / P.ranges;
+
+  const int tg = P.tiles_per_group, slice = tid / tg, tl = tid % tg;
+  const int tile = g * tg + tl;
+  const bool active = slice < P.slices && tile < P.ntiles;
+  int bi = 0, bj = 0;
+  if (active) tile_of<MI, MI>(tile, p, bi, bj);
+  double acc[MI][MI];
+#pragma unroll
+  for (int i = 0; i < MI; ++i)
+#pragma unroll
+    for (int j = 0; j < MI; ++j) acc[i][j] = 0.0;
+  const int cc = tid % p, cq = tid / p, ncq = NT / p;  // column sums: this thread's column and rows
+  double s = 0.0;
+  // the columns that pad the last micro-tile are zero
+  for (int i = tid; i < R * (S - p); i += NT) X[(i / (S - p)) * S + p + i % (S - p)] = 0.0;
+
+  for (int64_t st = st0; st < st1; ++st) {
+    const int64_t r0 = st << P.log_rows;
+    const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - r0));
+    const int lc = P.log_rows - 5, nitems = p << lc;  // items: 32 rows of a column
+    __syncthreads();  // the last stage's rows have been read
+    for (int i0 = warp; i0 < nitems; i0 += kBatch * nwarps) {
+      uint64_t v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int it = i0 + u * nwarps, c = it >> lc, k = ((it & ((1 << lc) - 1)) << 5) + lane;
+        v[u] = 0;
+        if (it < nitems && k < rows) v[u] = load_bits(P.cols[c], P.dtype[c], r0 + k);
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int it = i0 + u * nwarps, c = it >> lc, k = ((it & ((1 << lc) - 1)) << 5) + lane;
+        if (it < nitems) {
+          double x = to_f64(v[u], P.dtype[c]);
+          if (P.shift) x -= P.shift[c];
+          X[k * S + c] = x;
+        }
+      }
+    }
+    __syncthreads();
+    if (g == 0 && cq < ncq)
+      for (int k = cq; k < rows; k += ncq) s += X[k * S + cc];
+    if (active) {
+      const double* xa = X + MI * bi;
+      const double* xb = X + MI * bj;
+#pragma unroll 2
+      for (int k = slice; k < rows; k += P.slices) {
+        double a[MI], b[MI];
+#pragma unroll
+        for (int i = 0; i < MI; ++i) a[i] = xa[k * S + i];
+#pragma unroll
+        for (int j = 0; j < MI; ++j) b[j] = xb[k * S + j];
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+          for (int j = 0; j < MI; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      }
+    }
+  }
+  // the slices' partial sums, added in a fixed tree through shared memory
+  double* buf = X;
+  for (int n = P.slices; n > 1;) {
+    const int h = (n + 1) / 2;
+    __syncthreads();
+    if (slice >= h && slice < n) {
+#pragma unroll
+      for (int e = 0; e < kE; ++e) buf[e * (NT / 2) + (slice - h) * tg + tl] = acc[e / MI][e % MI];
+    }
+    __syncthreads();
+    if (slice < n - h) {
+#pragma unroll
+      for (int e = 0; e < kE; ++e) acc[e / MI][e % MI] += buf[e * (NT / 2) + slice * tg + tl];
+    }
+    n = h;
+  }
+  double* slot = P.slots + static_cast<size_t>(blockIdx.x) * core64_slot_doubles(p, tg, MI);
+  if (slice == 0) {
+#pragma unroll
+    for (int e = 0; e < kE; ++e) slot[static_cast<size_t>(e) * tg + tl] = acc[e / MI][e % MI];
+  }
+  __syncthreads();
+  if (cq < ncq) buf[cq * p + cc] = s;
+  __syncthreads();
+  if (g == 0 && tid < p) {
+    double t = 0.0;
+    for (int i = 0; i < ncq; ++i) t += buf[i * p + tid];
+    slot[static_cast<size_t>(kE) * tg + tid] = t;
+  }
+}
+
+// Adds the ranges' slots of 32 entries per block, kSeg consecutive runs of ranges at once, in
+// double-double; the runs in order, then into the accumulators.
+constexpr int kSeg = 16;
+
+template <int MI>
+__global__ void __launch_bounds__(32 * kSeg) core64_merge_kernel(const __grid_constant__ Core64Params P) {
+  __shared__ double sh[kSeg][32], sl[kSeg][32];
+  constexpr int kE = MI * MI;
+  const int p = P.p, tg = P.tiles_per_group, lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int nS = P.ntiles * kE;
+  const int x = blockIdx.x * 32 + lane;
+  const size_t sd = core64_slot_doubles(p, tg, MI);
+  int j = -1, k = -1;
+  size_t off = 0;
+  if (x < nS) {
+    const int e = x / P.ntiles, t = x % P.ntiles, g = t / tg;
+    int bi, bj;
+    tile_of<MI, MI>(t, p, bi, bj);
+    j = MI * bi + e / MI;
+    k = MI * bj + e % MI;
+    if (j > k || k >= p) j = -1;
+    off = static_cast<size_t>(g) * sd + static_cast<size_t>(e) * tg + (t - g * tg);
+  } else if (x < nS + p) {
+    j = k = x - nS;
+    off = static_cast<size_t>(kE) * tg + j;
+  }
+  double h = 0.0, l = 0.0;
+  if (j >= 0) {
+    const double* src = P.slots + off;
+    const size_t step = static_cast<size_t>(P.groups) * sd;
+    const int r0 = P.ranges * seg / kSeg, r1 = P.ranges * (seg + 1) / kSeg;
+#pragma unroll 4
+    for (int r = r0; r < r1; ++r) pair_add(h, l, __ldcg(src + r * step));
+  }
+  sh[seg][lane] = h;
+  sl[seg][lane] = l;
+  __syncthreads();
+  if (seg == 0 && j >= 0) {
+    for (int i = 1; i < kSeg; ++i) {
+      pair_add(h, l, sh[i][lane]);
+      l += sl[i][lane];
+    }
+    const int idx = x < nS ? j * p - j * (j - 1) / 2 + (k - j) : j;
+    double* ah = (x < nS ? P.acc_S : P.acc_s) + idx;
+    double* al = (x < nS ? P.acc_S_lo : P.acc_s_lo) + idx;
+    double vh = *ah, vl = *al;
+    pair_add(vh, vl, h);
+    *ah = vh;
+    *al = vl + l;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.acc_n += P.nrows;
+}
+
+size_t smem_bytes(const Core64Params& P) {
+  return std::max<size_t>((size_t(1) << P.log_rows) * row_stride(P.p, P.micro) * sizeof(double),
+                          static_cast<size_t>(P.micro) * P.micro * (P.threads / 2) * sizeof(double));
+}
+
+const void* kernel_of(int micro) {
+  return micro == 4 ? reinterpret_cast<const void*>(core64_kernel<4>) : reinterpret_cast<const void*>(core64_kernel<2>);
+}
+
+}  // namespace
+
+// The cut of p columns and nrows rows for `sms` SMs (or `blocks` blocks, when positive).
+cudaError_t core64_plan(int p, int64_t nrows, bool shifted, int sms, int blocks, Core64Params& P) {
+  double best = 0;
+  for (int micro : {4, 2}) {
+    const int M = core::tile_count(p, micro, micro);
+    for (int nt = 128; nt <= kMaxThreads; nt += 128) {
+      if (nt < p) continue;  // the column sums take a thread per column
+      const int G0 = (M + nt - 1) / nt;
+      for (int G = G0; G <= G0 + 8; ++G) {
+        const int tg = (M + G - 1) / G, ks = nt / tg;
+        if (tg * (G - 1) >= M) continue;
+        // FP64 warp instructions a row costs one of the SM's four schedulers: the tiles' FMAs, the
+        // shift in every group, the column sums in one
+        const double fmas = ((tg * ks + 31) / 32 + 3) / 4 * double(micro * micro) / ks;
+        const double cost = G * (fmas + (shifted ? p / 128.0 : 0.0)) + double(nt) / (nt / p * p) * p / 128.0;
+        if (best == 0 || cost < best) {
+          best = cost;
+          P.micro = micro;
+          P.threads = nt;
+          P.ntiles = M;
+          P.groups = G;
+          P.tiles_per_group = tg;
+          P.slices = ks;
+        }
+      }
+    }
+  }
+  // rows of a stage: about 32 KB, fewer while that would leave SMs without one
+  int lr = 5;
+  while (lr < 9 && (row_stride(p, P.micro) << (lr + 1)) <= 4096 &&
+         (nrows >> (lr + 1)) >= 4 * int64_t(std::max(1, sms / P.groups)))
+    ++lr;
+  P.log_rows = lr;
+  const size_t smem = smem_bytes(P);
+  cudaError_t e = cudaFuncSetAttribute(kernel_of(P.micro), cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  int per = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of(P.micro), P.threads, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t nst = (nrows + (int64_t(1) << lr) - 1) >> lr;
+  const int64_t want = blocks > 0 ? blocks : int64_t(sms) * std::max(1, std::min(per, 4));
+  P.ranges = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want / P.groups, nst)));
+  return cudaSuccess;
+}
+
+size_t core64_slot_bytes(const Core64Params& P) {
+  return static_cast<size_t>(P.groups) * P.ranges * core64_slot_doubles(P.p, P.tiles_per_group, P.micro) * sizeof(double);
+}
+
+cudaError_t launch_core64(const Core64Params& P, cudaStream_t stream) {
+  const size_t smem = smem_bytes(P);
+  const int grid = P.groups * P.ranges, mgrid = (P.ntiles * P.micro * P.micro + P.p + 31) / 32;
+  cudaError_t e = cudaFuncSetAttribute(kernel_of(P.micro), cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  if (P.micro == 4) {
+    core64_kernel<4><<<grid, P.threads, smem, stream>>>(P);
+    core64_merge_kernel<4><<<mgrid, 32 * kSeg, 0, stream>>>(P);
+  } else {
+    core64_kernel<2><<<grid, P.threads, smem, stream>>>(P);
+    core64_merge_kernel<2><<<mgrid, 32 * kSeg, 0, stream>>>(P);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace ss

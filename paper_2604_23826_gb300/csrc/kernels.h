@@ -275,7 +275,7 @@ cudaError_t launch_narrow(const NarrowParams& P, bool x4, int grid, cudaStream_t
 cudaError_t launch_narrow_shift(const NarrowTab* tabs, const int* which, int count, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// CUDA-core passes for any width: FP32-core (k_core32.cu), FP64 raw or shifted (k_core.cu).
+// CUDA-core passes for any width: FP32-core (k_core32.cu), FP64 raw or shifted (k_core64.cu).
 // ---------------------------------------------------------------------------
 struct Core32Params {
   const void* cols[256];
@@ -303,26 +303,29 @@ __host__ __device__ inline size_t core32_slot_pairs(int p, int tiles_per_group) 
 void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P);
 size_t core32_slot_bytes(const Core32Params& P);
 cudaError_t launch_core32(const Core32Params& P, cudaStream_t stream);
-constexpr int kCoreSlotDoubles = 2 * (32 * 32 + 32);
-struct CoreParams {
+struct Core64Params {
   const void* cols[256];
   int32_t dtype[256];
   const double* shift;  // p pivots or nullptr (raw moments)
   int32_t p;
-  int32_t nblk;         // ceil(p / 64)
-  int32_t ntiles;
-  int32_t ksplit;
   int64_t nrows;
-  double* slots;        // scratch: core_slot_doubles(grid)
-  unsigned int* ticket;
-  double* acc_s;
+  // the cut (core64_plan): order of the micro-tiles, their number, threads of a block, groups of
+  // blocks over the tiles, row slices of a block, 2^log_rows rows a stage, row ranges
+  int32_t micro, ntiles, threads, groups, tiles_per_group, slices, log_rows, ranges;
+  double* slots;        // scratch: core64_slot_bytes
+  double* acc_s;        // ctx accumulators, double-double
   double* acc_s_lo;
   double* acc_S;
   double* acc_S_lo;
   long long* acc_n;
 };
-size_t core_slot_doubles(int grid);
-cudaError_t launch_core(const CoreParams& P, int grid, cudaStream_t stream);
+// doubles of a block's slot: its tiles' entries, then the column sums
+__host__ __device__ inline size_t core64_slot_doubles(int p, int tiles_per_group, int micro) {
+  return static_cast<size_t>(tiles_per_group) * micro * micro + p;
+}
+cudaError_t core64_plan(int p, int64_t nrows, bool shifted, int sms, int blocks, Core64Params& P);
+size_t core64_slot_bytes(const Core64Params& P);
+cudaError_t launch_core64(const Core64Params& P, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------
 // Finalize (one block): recombination, exact centering, cov / corr, Jacobi.

@@ -76,3 +76,20 @@ def test_fp32_core_alignment_calls_and_grids(p, offset, parts, grid):
 @pytest.mark.parametrize("offset", [0, 1])
 def test_fp32_core_column_types(offset):
     check([G.STATS_I16, G.STATS_F32, G.STATS_I32, G.STATS_F64, G.STATS_I64] * 3, 5_001, G.STATS_FP32, 3, offset)
+
+
+@pytest.mark.parametrize("n", [1, 33, 4_099, 40_003])
+@pytest.mark.parametrize("p", [13, 16, 31, 48, 65, 127, 128, 200, 256])
+@pytest.mark.parametrize("mode", [G.STATS_FP64, G.STATS_FP64_SHIFTED])
+def test_fp64_core_widths_and_rows(mode, p, n):
+    check([G.STATS_F64] * p, n, mode, 7 * p + n)
+
+
+@pytest.mark.parametrize("p,parts,grid", [(14, 3, 0), (50, 1, 5), (140, 2, 1)])
+def test_fp64_core_calls_and_grids(p, parts, grid):
+    check([G.STATS_F64] * p, 10_007, G.STATS_FP64_SHIFTED, p, 1, parts, grid)
+
+
+@pytest.mark.parametrize("mode", [G.STATS_FP64, G.STATS_FP64_SHIFTED])
+def test_fp64_core_column_types(mode):
+    check([G.STATS_I16, G.STATS_F32, G.STATS_I32, G.STATS_F64, G.STATS_I64] * 3, 5_001, mode, 4, 1)
