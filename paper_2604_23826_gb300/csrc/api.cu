@@ -249,27 +249,16 @@ stats_status exact_plan(int p, const int32_t* dtypes, bool bounded, const double
       slot += cp[j].k;
     }
     if (slot > kDigits) return STATS_EINVAL;
-    // per digit slot: source column (-1 the ones column, -2 padding), byte, signed top byte
-    int8_t col[kDigits], byt[kDigits], sg[kDigits];
-    for (int q = 0; q < kDigits; ++q) {
-      col[q] = -2;
-      byt[q] = 0;
-      sg[q] = 0;
-    }
-    col[0] = -1;
-    for (int j = 0; j < p; ++j)
-      for (int a = 0; a < cp[j].k; ++a) {
-        col[cp[j].off + a] = static_cast<int8_t>(j);
-        byt[cp[j].off + a] = static_cast<int8_t>(a);
-        sg[cp[j].off + a] = (cp[j].is_signed && a == cp[j].k - 1) ? 1 : 0;
-      }
-    for (int q = 0; q < kDigitPairs; ++q) {
-      xp.pc0[q] = col[2 * q];
-      xp.pb0[q] = byt[2 * q];
-      xp.ps0[q] = sg[2 * q];
-      xp.pc1[q] = col[2 * q + 1];
-      xp.pb1[q] = byt[2 * q + 1];
-      xp.ps1[q] = sg[2 * q + 1];
+    for (int q = 0; q < kDigitPairs; ++q) xp.bias[q] = 0x64006400u;
+    for (int j = 0; j < p; ++j) {
+      const int k = cp[j].k, bits = 8 * k;
+      xp.field_add[j] = cp[j].is_signed ? uint64_t(1) << (bits - 1) : 0;
+      // a 32-bit value in a full-width unsigned field: its sign bit would be a violation
+      xp.field_chk[j] = k == 8                            ? 0
+                        : dtypes[j] == I32 && k == 4 ? (cp[j].is_signed ? 0 : uint64_t(1) << 31)
+                                                          : ~((uint64_t(1) << bits) - 1);
+      const int top = cp[j].off + k - 1;
+      if (cp[j].is_signed) xp.bias[top / 2] += top % 2 ? 0x800000u : 0x80u;
     }
   }
   for (int j = 0; j < p; ++j) {

@@ -170,56 +170,83 @@ struct ConvT1 {
 };
 
 // ---- the generic converter: any plan of at most 32 digits over at most 16 columns ----
-template <class Src>
-__device__ __forceinline__ int64_t load_as_int(const ExactParams& P, const Src& src, int j) {
-  switch (P.dtype[j]) {
-    case I16: return src.i16(j);
-    case I32: return src.i32(j);
-    case I64: return src.i64(j);
-    case F32: return static_cast<int64_t>(fixed_rn<true>(static_cast<double>(src.f32(j)), P.real_shift[j]));
-    default: return static_cast<int64_t>(fixed_rn<true>(src.f64(j), P.real_shift[j]));
-  }
-}
-
+// A row's digits are its bytes: the value 1, then each column's field.  Each column is loaded
+// once, biased to an unsigned field (a signed field's top byte XOR 0x80 is the value plus
+// 2^(8k-1)) and appended to a 64-bit register; every eight bytes that fill it leave as four f16
+// pairs, whose bias takes a signed top byte's 128 off again.  The column loop is uniform across
+// the warp, so its branches cost one instruction each.  (Bound: instruction issue, as for Table 1.
+// Eight mixed columns, 36 B a row, 2e7 rows: extracting every digit from its column anew took
+// 2.50 ms, this way 0.71 ms.)
 struct ConvGeneric {
   template <int TILE>
   __device__ __forceinline__ static SmemSrc smem_src(const uint8_t* st, const ExactParams& P, int r) {
     return SmemSrc{st, &P, r};
   }
-  template <class Src>
-  __device__ __forceinline__ static uint32_t byte_of(const ExactParams& P, const Src& src, int c, int b, int sg) {
-    if (c == -1) return 1u;
-    if (c < 0) return 0u;
-    const uint64_t v = static_cast<uint64_t>(load_as_int(P, src, c));
-    return static_cast<uint32_t>((v >> (8 * b)) & 0xFF) ^ (sg ? 0x80u : 0u);
+  // q = round(x * 2^sh) as a field of 56 bits, biased when signed; range violations into bad
+  __device__ __forceinline__ static uint64_t real_field(const ExactParams& P, double x, int j, uint32_t& bad) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+    const int ef = static_cast<int>((hi >> 20) & 0x7FFu), sh = P.real_shift[j];
+    bad |= ef > P.real_emax[j];
+    if (!P.is_signed[j]) bad |= (hi >> 31) & (((hi << 1) | lo) != 0);  // negative, not -0
+    // the scaling is an exponent-field add, the rounding one conversion on the FP64 unit; a scaled
+    // value below the normal range rounds to 0, a subnormal input is scaled by integers
+    uint64_t q;
+    if (ef == 0)
+      q = ((hi << 1) | lo) ? fixed_rn<true>(x, sh) : 0;
+    else
+      q = ef + sh > 0 ? static_cast<uint64_t>(__double2ll_rn(__hiloint2double(
+                            static_cast<int>(hi + (static_cast<uint32_t>(sh) << 20)), static_cast<int>(lo))))
+                      : 0;
+    return q;
+  }
+  __device__ __forceinline__ static void emit(const ExactParams& P, uint64_t v, int e, uint32_t (&w)[16]) {
+    constexpr uint32_t M = 0x64646464u;  // bytes of the f16 exponent 0x64
+    const uint32_t lo = static_cast<uint32_t>(v), hi = static_cast<uint32_t>(v >> 32);
+    const uint32_t d0 = half2_sub(__byte_perm(lo, M, 0x4140), P.bias[4 * e]);
+    const uint32_t d1 = half2_sub(__byte_perm(lo, M, 0x4342), P.bias[4 * e + 1]);
+    const uint32_t d2 = half2_sub(__byte_perm(hi, M, 0x4140), P.bias[4 * e + 2]);
+    const uint32_t d3 = half2_sub(__byte_perm(hi, M, 0x4342), P.bias[4 * e + 3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q == e) {
+        w[4 * q] = d0;
+        w[4 * q + 1] = d1;
+        w[4 * q + 2] = d2;
+        w[4 * q + 3] = d3;
+      }
   }
   template <class Src>
   __device__ __forceinline__ static void row(const ExactParams& P, const Src& src, uint32_t (&w)[16],
                                              uint32_t& bad) {
-#pragma unroll
-    for (int j = 0; j < kMaxCols; ++j) {
-      if (j >= P.p) break;
+    uint64_t acc = 1;  // the ones column's digit
+    int nb = 8, e = 0;
+#pragma unroll 1
+    for (int j = 0; j < P.p; ++j) {
       const int dt = P.dtype[j];
-      if (dt == F32 || dt == F64) {
-        const double x = dt == F32 ? static_cast<double>(src.f32(j)) : src.f64(j);
-        const uint64_t ux = static_cast<uint64_t>(__double_as_longlong(x));
-        bad |= dbl_exp_field(x) > P.real_emax[j];
-        if (!P.is_signed[j]) bad |= (ux >> 63) & ((ux << 1) != 0);  // negative, not -0
+      uint64_t u;
+      if (dt == I16 || dt == I32) {
+        const uint32_t t = static_cast<uint32_t>(dt == I16 ? src.i16(j) : src.i32(j)) + static_cast<uint32_t>(P.field_add[j]);
+        bad |= (t & static_cast<uint32_t>(P.field_chk[j])) != 0;
+        u = t;
+      } else if (dt == I64) {
+        u = static_cast<uint64_t>(src.i64(j)) + P.field_add[j];
+        bad |= (u & P.field_chk[j]) != 0;
       } else {
-        const int64_t v = load_as_int(P, src, j);
-        const int k = P.kbytes[j];
-        if (k < 8) {
-          const uint64_t u = static_cast<uint64_t>(P.is_signed[j] ? v + (int64_t(1) << (8 * k - 1)) : v);
-          bad |= (u >> (8 * k)) != 0;
-        }
+        const double x = dt == F64 ? src.f64(j) : f32_to_f64(src.f32(j));
+        u = (real_field(P, x, j, bad) + P.field_add[j]) & ((uint64_t(1) << 56) - 1);
+      }
+      acc |= u << nb;
+      nb += 8 * P.kbytes[j];
+      if (nb >= 64) {
+        emit(P, acc, e++, w);
+        nb -= 64;
+        // the bytes of u that did not fit: u >> (kbits - nb), none when the field ended at 64
+        acc = nb ? u >> (8 * P.kbytes[j] - nb) : 0;
       }
     }
-#pragma unroll
-    for (int q = 0; q < kDigitPairs; ++q) {
-      const uint32_t lo = byte_of(P, src, P.pc0[q], P.pb0[q], P.ps0[q]);
-      const uint32_t hi = byte_of(P, src, P.pc1[q], P.pb1[q], P.ps1[q]);
-      const uint32_t bias = (P.ps0[q] ? 0x80u : 0u) | (P.ps1[q] ? 0x800000u : 0u);
-      w[q] = half2_sub(lo | (hi << 16) | kH1024, kH1024 | bias);
+    for (; e < 4; ++e) {
+      emit(P, acc, e, w);
+      acc = 0;
     }
   }
 };

@@ -37,11 +37,11 @@ struct ExactParams {
   int32_t real_emax[kMaxCols];   // real columns: largest allowed biased exponent field
   int32_t kbytes[kMaxCols];      // digit bytes of the column's field
   int32_t is_signed[kMaxCols];   // field is two's complement (top byte signed)
-  // Generic plan, per digit pair q: source column of the low / high digit
-  // (-1 = the ones column, -2 = zero padding), its byte index, and whether it is
-  // the signed top byte of its field.
-  int8_t pc0[kDigitPairs], pb0[kDigitPairs], ps0[kDigitPairs];
-  int8_t pc1[kDigitPairs], pb1[kDigitPairs], ps1[kDigitPairs];
+  // Generic plan: what turns an integer column into its unsigned field (2^(8k-1) when signed), the
+  // bits that must then be clear, and per digit pair the f16 pair to subtract from 1024 + byte
+  // (1024, and 128 more for a signed top byte)
+  uint64_t field_add[kMaxCols], field_chk[kMaxCols];
+  uint32_t bias[kDigitPairs];
   int32_t p;
   int32_t direct;       // 1: some column is not 16-byte aligned -- consumers read global memory directly
   int32_t shape;        // launch shape (0 .. kExactShapes - 1)
