@@ -1073,12 +1073,14 @@ stats_status run_finalize(stats_ctx* c, int want_pca, int pca_on, const double* 
   JacobiParams J{};
   if (grid > 0) {
     if (!c->d_jac) CK(c, cudaMalloc(&c->d_jac, jacobi_scratch_doubles(pa) * sizeof(double)));
-    const size_t m = (pa + 15) / 16 * 16;
+    const size_t m = jacobi_order(pa);
     J.a = c->d_jac;
     J.b = J.a + m * m;
     J.v = J.b + m * m;
     J.w = J.v + m * m;
-    double* basis = J.w + m * m;
+    J.g = J.w + m * m;
+    J.x = J.g + m * m;
+    double* basis = J.x + m * m;
     J.q = basis + static_cast<size_t>(pa) * pa;
     J.slots = J.q + (m / 16) * 256;
     J.bar = reinterpret_cast<unsigned int*>(J.slots + 1024);
@@ -1886,6 +1888,7 @@ stats_status stats_finalize_batched(stats_ctx* const* ctxs, int32_t count, int32
   }
   const bool want_pca = evals || evecs;
   std::vector<FinalParams> params(count);
+  std::vector<EigJob> jobs;  // decompositions by the batched eigen-solver, the widest first
   std::vector<size_t> off(count);
   size_t total = 0;
   for (int i = 0; i < count; ++i) {
@@ -1893,17 +1896,29 @@ stats_status stats_finalize_batched(stats_ctx* const* ctxs, int32_t count, int32
     total += static_cast<size_t>(ctxs[i]->lay.total);
   }
   stats_ctx* c0 = ctxs[0];
-  const size_t pbytes = round256(count * sizeof(FinalParams));
+  const size_t pbytes = round256(count * sizeof(FinalParams)), jbytes = round256(count * sizeof(EigJob));
   void* dbuf = nullptr;
-  CK(c0, cudaMalloc(&dbuf, pbytes + total * sizeof(double)));
-  double* dout = reinterpret_cast<double*>(static_cast<char*>(dbuf) + pbytes);
+  CK(c0, cudaMalloc(&dbuf, pbytes + jbytes + total * sizeof(double)));
+  EigJob* djobs = reinterpret_cast<EigJob*>(static_cast<char*>(dbuf) + pbytes);
+  double* dout = reinterpret_cast<double*>(static_cast<char*>(dbuf) + pbytes + jbytes);
   for (int i = 0; i < count; ++i) {
     build_final_params(ctxs[i], want_pca ? 1 : 0, pca_on, params[i]);
     params[i].out = dout + off[i];  // the work scratch stays per context
+    if (want_pca && batched_eigen_deferred(ctxs[i]->pa)) {
+      const FinalLayout& L = ctxs[i]->lay;
+      params[i].defer_m = -1;
+      jobs.push_back(EigJob{params[i].out + (pca_on ? L.corr : L.cov), params[i].out + L.evals, params[i].out + L.evecs,
+                            params[i].out + L.flags, ctxs[i]->pa, 0});
+    }
   }
+  std::stable_sort(jobs.begin(), jobs.end(), [](const EigJob& x, const EigJob& y) { return x.n > y.n; });
   std::vector<double> h(total);
   cudaError_t e = cudaMemcpy(dbuf, params.data(), count * sizeof(FinalParams), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = launch_finalize_batched(reinterpret_cast<const FinalParams*>(dbuf), count, nullptr);
+  if (e == cudaSuccess && !jobs.empty())
+    e = cudaMemcpy(djobs, jobs.data(), jobs.size() * sizeof(EigJob), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = launch_finalize_batched(reinterpret_cast<const FinalParams*>(dbuf), count, djobs, static_cast<int>(jobs.size()),
+                                nullptr);
   if (e == cudaSuccess) e = cudaMemcpy(h.data(), dout, total * sizeof(double), cudaMemcpyDeviceToHost);
   cudaFree(dbuf);
   if (e != cudaSuccess) return cuda_fail(c0, e);

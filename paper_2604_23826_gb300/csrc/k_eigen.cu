@@ -1,0 +1,734 @@
+// k_eigen.cu -- the eigen-solver spread over the GPU (arxiv 2604.23826, "Principal Component
+// Analysis Results"), for 24 or more analysis columns or with a seed: a cooperative grid, one
+// 256-thread block per SM at most, whose blocks meet at bounded grid-wide barriers.
+//
+//   1. (seed) accepted only if its columns are orthonormal to 1e-9; T = V^T A V.  Cold: T = A, V = I.
+//   2. FP32 Jacobi on T scaled to order one: up to 96 columns in one block's shared memory (a round
+//      is two block barriers), above that block-cyclic over the grid: pairs of 16-column blocks,
+//      a 32 x 32 problem each, swept once in shared memory, then every 32 x 32 block of T and V
+//      multiplied by the pairs' rotations: two grid barriers a block round.
+//   3. X = V Q, then the Ogita-Aishima refinement in FP64: W = A X, S = X^T W, G = X^T X, the
+//      correction E from S, G and X <- X + X E, until E is below 5e-9 (its square is left): two or
+//      three steps of four products, each spread over the grid in 16 x 16 tiles.
+//   4. If eigenvalues are too close for the refinement (or it fails), block-cyclic Jacobi in FP64,
+//      from the refined basis (or from the matrix as it came).
+// Bound: FP64, at 2 operations per clock and SM.  FP64 Jacobi alone spent it on chains of divisions
+// and square roots of one warp (256 columns, 11 sweeps: 14.7 ms); the products of step 3 are four
+// times 256^3 multiplications a step, 30 us each over 152 SMs, and step 2 has no FP64 at all.
+#include <math.h>
+
+#include "common.cuh"
+#include "eigen.cuh"
+#include "kernels.h"
+
+namespace ss {
+
+namespace {
+
+using namespace eig;
+
+constexpr int kJW = 8;         // FP64 block Jacobi: indices per block
+constexpr int kJP = 2 * kJW;   // order of a block pair's diagonal problem
+static_assert(kJP * kJP == kThreads, "one thread per entry of a block-pair tile");
+constexpr int kFW = 16, kFP = 2 * kFW;  // the same for the FP32 block Jacobi
+constexpr int kFLd = kFP + 1;
+constexpr unsigned long long kGridWaitNs = 2000000000ull;  // a grid-wide wait gives up after 2 s
+constexpr unsigned int kDead = 0x80000000u;
+
+__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* a) {
+  unsigned int v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+struct Grid {
+  unsigned int* bar;  // arrivals since the launch; bit 31: a wait has run out
+  unsigned int target;
+  unsigned long long wait_ns;
+  int* s_ok;
+
+  // Grid-wide barrier of a cooperative launch.  Thread 0 of each block publishes the block's writes
+  // (fence) and arrives on a count that only grows; the others' arrivals are polled for.  A wait that
+  // outlasts wait_ns marks the count; every block that sees the mark leaves (false).
+  __device__ bool sync() {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      target += gridDim.x;
+      __threadfence();
+      unsigned int v = atomicAdd(bar, 1u) + 1u;
+      if (v < target) {
+        const unsigned long long t0 = global_ns();
+        for (unsigned int n = 1;; ++n) {
+          v = ld_acquire_u32(bar);
+          if (v >= target) break;  // everyone is here, or the mark is set
+          if ((n & 63u) == 0 && global_ns() - t0 > wait_ns) {
+            v = atomicOr(bar, kDead) | kDead;
+            break;
+          }
+        }
+      }
+      __threadfence();
+      *s_ok = (v & kDead) == 0;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+  }
+};
+
+struct Shared {
+  Scratch32 s32;
+  double x[16][17], y[16][17], z[16][17], t[16][17];
+  double qa[kJP][kJP + 1], qb[kJP][kJP + 1];
+  double c[8], s[8];
+  double lambda[256];
+  double red[8];
+  unsigned long long key[256];
+  int order[256];
+  unsigned long long best[8];
+  int best_i[8];
+  double val;
+  int ok;
+};
+constexpr size_t kDynFloats32 = jacobi32_floats(k32Max);  // step 2 in one block
+constexpr size_t kDynFloatsF = jacobi32_floats(kFP) + 4 * kFP * kFLd;  // step 2 over the grid
+constexpr size_t kDynBytes = sizeof(float) * (kDynFloats32 > kDynFloatsF ? kDynFloats32 : kDynFloatsF);
+
+// Z(i, j) = sum_k X(i, k) Y(k, j) for 16 x 16 tiles shared out over the grid; X, Y: element
+// functions, put(i, j, value)
+template <class FX, class FY, class Put>
+__device__ void grid_product(int m, Shared& S, FX&& X, FY&& Y, Put&& put) {
+  const int nt = m / 16, r = threadIdx.x / 16, c = threadIdx.x % 16;
+  for (int t = blockIdx.x; t < nt * nt; t += gridDim.x) {
+    const int i0 = (t / nt) * 16, j0 = (t % nt) * 16;
+    double acc = 0.0;
+    double nx = X(i0 + r, c), ny = Y(r, j0 + c);
+    for (int k0 = 0; k0 < m; k0 += 16) {
+      S.x[r][c] = nx;
+      S.y[r][c] = ny;
+      __syncthreads();
+      if (k0 + 16 < m) {
+        nx = X(i0 + r, k0 + 16 + c);
+        ny = Y(k0 + 16 + r, j0 + c);
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) acc = fma(S.x[r][k], S.y[k][c], acc);
+      __syncthreads();
+    }
+    put(i0 + r, j0 + c, acc);
+  }
+}
+
+// S = X^T W and G = X^T X (both symmetric): the tiles on or above the diagonal of each, shared out
+// over the grid
+__device__ void grid_grams(int m, Shared& S, const double* X, const double* W, double* SO, double* GO) {
+  const int nt = m / 16, r = threadIdx.x / 16, c = threadIdx.x % 16, half = nt * (nt + 1) / 2;
+  for (int t = blockIdx.x; t < 2 * half; t += gridDim.x) {
+    int I = 0, J = t % half;
+    while (J >= nt - I) {
+      J -= nt - I;
+      ++I;
+    }
+    J += I;
+    const double* Y = t < half ? W : X;
+    double* O = t < half ? SO : GO;
+    double acc = 0.0;
+    double nx = __ldcg(X + static_cast<size_t>(r) * m + I * 16 + c), ny = __ldcg(Y + static_cast<size_t>(r) * m + J * 16 + c);
+    for (int k0 = 0; k0 < m; k0 += 16) {
+      S.x[r][c] = nx;
+      S.y[r][c] = ny;
+      __syncthreads();
+      if (k0 + 16 < m) {
+        nx = __ldcg(X + static_cast<size_t>(k0 + 16 + r) * m + I * 16 + c);
+        ny = __ldcg(Y + static_cast<size_t>(k0 + 16 + r) * m + J * 16 + c);
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) acc = fma(S.x[k][r], S.y[k][c], acc);
+      __syncthreads();
+    }
+    // both halves hold the same value
+    if (I == J) {
+      S.z[r][c] = acc;
+      __syncthreads();
+      acc = r <= c ? acc : S.z[c][r];
+      __stcg(O + static_cast<size_t>(I * 16 + r) * m + J * 16 + c, acc);
+      __syncthreads();
+    } else {
+      __stcg(O + static_cast<size_t>(I * 16 + r) * m + J * 16 + c, acc);
+      __stcg(O + static_cast<size_t>(J * 16 + c) * m + I * 16 + r, acc);
+    }
+  }
+}
+
+// the blocks' slots[0 .. grid) added (or their maximum taken) in a fixed order, in every thread
+__device__ double slots_total(const double* slots, Shared& S) {
+  double v = 0.0;
+  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += kThreads) v += __ldcg(slots + b);
+  return block_total(v, S.red);
+}
+__device__ double slots_max(const double* slots, Shared& S) {
+  double v = 0.0;
+  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += kThreads) v = fmax(v, __ldcg(slots + b));
+  return block_max(v, S.red);
+}
+
+// FP32 block-cyclic Jacobi over the grid (m a multiple of 32): A and its next copy B, V = I on entry.
+// Returns the sweeps, -1 after a wait that ran out.
+__device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float* dyn, float* A, float* B, float* V,
+                             float* Q) {
+  const int m = J.m, nb = m / kFW, np = nb / 2, tid = threadIdx.x;
+  float* sA = dyn + jacobi32_floats(kFP);
+  float* sQ = sA + kFP * kFLd;
+  float* sB = sQ + kFP * kFLd;
+  float* sT = sB + kFP * kFLd;
+  auto row_of = [](int bi, int bj, int l) { return l < kFW ? bi * kFW + l : bj * kFW + l - kFW; };
+  const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
+  double fro2 = 0.0, prev = 0.0;
+  int sweep = 0;
+  for (; sweep < 20; ++sweep) {
+    float o = 0.f, d = 0.f;
+    for (int i = gtid; i < m * m; i += nthreads) {
+      const float x = __ldcg(A + i);
+      if (i / m != i % m)
+        o = fmaf(x, x, o);
+      else
+        d = fmaf(x, x, d);
+    }
+    const double bo = block_total(static_cast<double>(o), S.red), bd = block_total(static_cast<double>(d), S.red);
+    if (tid == 0) {
+      __stcg(J.slots + blockIdx.x, bo);
+      __stcg(J.slots + 512 + blockIdx.x, bd);
+    }
+    if (!grid.sync()) return -1;
+    const double off = slots_total(J.slots, S);
+    if (sweep == 0) fro2 = off + slots_total(J.slots + 512, S);
+    if (!(off > 1e-14 * fro2) || (sweep > 0 && off <= 1e-9 * fro2 && off > 0.25 * prev)) break;
+    prev = off;
+    for (int br = 0; br < nb - 1; ++br) {
+      for (int P = blockIdx.x; P < np; P += gridDim.x) {
+        int bi, bj;
+        pair_of(br, P, nb, bi, bj);
+        float* pA = dyn;
+        float* pV = dyn + 2 * kFP * kFP;
+        for (int e = tid; e < kFP * kFP; e += kThreads) {
+          const int r = e / kFP, c = e % kFP;
+          pA[e] = __ldcg(A + static_cast<size_t>(row_of(bi, bj, r)) * m + row_of(bi, bj, c));
+          pV[e] = r == c ? 1.f : 0.f;
+        }
+        __syncthreads();
+        int copy;
+        jacobi32<kFP>(pA, pV, 1, S.s32, copy);
+        pA += copy * kFP * kFP;
+        pV += copy * kFP * kFP;
+        for (int e = tid; e < kFP * kFP; e += kThreads) {
+          const int r = e / kFP, c = e % kFP;
+          __stcg(B + static_cast<size_t>(row_of(bi, bj, r)) * m + row_of(bi, bj, c), pA[e]);
+          __stcg(Q + static_cast<size_t>(P) * kFP * kFP + e, pV[e]);
+        }
+        __syncthreads();
+      }
+      if (!grid.sync()) return -1;
+      // Q_P^T A[P rows][P' cols] Q_P' for P < P' (and its transpose), and V[strip][P' cols] Q_P'
+      const int nA = np * (np - 1) / 2, nItems = nA + (m / kFP) * np;
+      const int tr = (tid / 16) * 2, tc = (tid % 16) * 2;
+      for (int it = blockIdx.x; it < nItems; it += gridDim.x) {
+        const bool isA = it < nA;
+        int P1 = 0, P2, bi = 0, bj = 0, ci, cj;
+        if (isA) {
+          P2 = it;
+          while (P2 >= np - 1 - P1) {
+            P2 -= np - 1 - P1;
+            ++P1;
+          }
+          P2 += P1 + 1;
+          pair_of(br, P1, nb, bi, bj);
+        } else {
+          P1 = (it - nA) / np;  // strip
+          P2 = (it - nA) % np;
+        }
+        pair_of(br, P2, nb, ci, cj);
+        for (int e = tid; e < kFP * kFP; e += kThreads) {
+          const int r = e / kFP, c = e % kFP;
+          const int gr = isA ? row_of(bi, bj, r) : P1 * kFP + r;
+          sA[r * kFLd + c] = __ldcg((isA ? A : V) + static_cast<size_t>(gr) * m + row_of(ci, cj, c));
+          sB[r * kFLd + c] = __ldcg(Q + static_cast<size_t>(P2) * kFP * kFP + e);
+          if (isA) sQ[r * kFLd + c] = __ldcg(Q + static_cast<size_t>(P1) * kFP * kFP + e);
+        }
+        __syncthreads();
+        float* L = sA;
+        if (isA) {
+          float t00 = 0.f, t01 = 0.f, t10 = 0.f, t11 = 0.f;
+#pragma unroll 8
+          for (int k = 0; k < kFP; ++k) {
+            const float a0 = sQ[k * kFLd + tr], a1 = sQ[k * kFLd + tr + 1], b0 = sA[k * kFLd + tc], b1 = sA[k * kFLd + tc + 1];
+            t00 = fmaf(a0, b0, t00);
+            t01 = fmaf(a0, b1, t01);
+            t10 = fmaf(a1, b0, t10);
+            t11 = fmaf(a1, b1, t11);
+          }
+          sT[tr * kFLd + tc] = t00;
+          sT[tr * kFLd + tc + 1] = t01;
+          sT[(tr + 1) * kFLd + tc] = t10;
+          sT[(tr + 1) * kFLd + tc + 1] = t11;
+          __syncthreads();
+          L = sT;
+        }
+        float y[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll 8
+        for (int k = 0; k < kFP; ++k) {
+          const float a0 = L[tr * kFLd + k], a1 = L[(tr + 1) * kFLd + k], b0 = sB[k * kFLd + tc], b1 = sB[k * kFLd + tc + 1];
+          y[0][0] = fmaf(a0, b0, y[0][0]);
+          y[0][1] = fmaf(a0, b1, y[0][1]);
+          y[1][0] = fmaf(a1, b0, y[1][0]);
+          y[1][1] = fmaf(a1, b1, y[1][1]);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            const int gc = row_of(ci, cj, tc + v);
+            if (isA) {
+              const int gr = row_of(bi, bj, tr + u);
+              __stcg(B + static_cast<size_t>(gr) * m + gc, y[u][v]);
+              __stcg(B + static_cast<size_t>(gc) * m + gr, y[u][v]);
+            } else {
+              __stcg(V + static_cast<size_t>(P1 * kFP + tr + u) * m + gc, y[u][v]);
+            }
+          }
+        __syncthreads();
+      }
+      float* t = A;
+      A = B;
+      B = t;
+      if (!grid.sync()) return -1;
+    }
+  }
+  return sweep;
+}
+
+// FP64 block-cyclic Jacobi over the grid: diagonalises A (B: its next copy), rotating V's columns.
+// Returns the sweeps (A then points to the diagonal form), -1 after a wait that ran out.
+__device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V) {
+  const int tid = threadIdx.x, m = J.m, nb = m / kJW, np = nb / 2;
+  const int lr_ = tid / kJP, lc_ = tid % kJP;
+  const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
+  double fro2 = 0.0, prev = 0.0;
+  int sweep = 0;
+  for (; sweep < 60; ++sweep) {
+    double o = 0.0, d = 0.0;
+    for (int i = gtid; i < m * m; i += nthreads) {
+      const double x = __ldcg(A + i);
+      if (i / m != i % m)
+        o = fma(x, x, o);
+      else
+        d = fma(x, x, d);
+    }
+    const double bo = block_total(o, S.red), bd = block_total(d, S.red);
+    if (tid == 0) {
+      __stcg(J.slots + blockIdx.x, bo);
+      __stcg(J.slots + 512 + blockIdx.x, bd);
+    }
+    if (!grid.sync()) return -1;
+    const double off = slots_total(J.slots, S);
+    if (sweep == 0) fro2 = off + slots_total(J.slots + 512, S);
+    // converged: off-diagonal mass negligible, or (block updates leave rounding noise in every
+    // off-diagonal entry) no longer falling quadratically once below 1e-26 of ||A||^2
+    if (off == 0.0 || off <= 1e-34 * fro2 || (sweep > 0 && off <= 1e-26 * fro2 && off > 0.0625 * prev)) break;
+    prev = off;
+    for (int br = 0; br < nb - 1; ++br) {
+      // (1) every block pair's kJP x kJP diagonal problem: one cyclic Jacobi sweep in shared
+      //     memory, its rotations accumulated in Q (to J.q), its result written to B
+      for (int P = blockIdx.x; P < np; P += gridDim.x) {
+        int bi, bj;
+        pair_of(br, P, nb, bi, bj);
+        const int gr = lr_ < kJW ? bi * kJW + lr_ : bj * kJW + lr_ - kJW;
+        const int gc = lc_ < kJW ? bi * kJW + lc_ : bj * kJW + lc_ - kJW;
+        S.x[lr_][lc_] = __ldcg(A + static_cast<size_t>(gr) * m + gc);
+        S.y[lr_][lc_] = lr_ == lc_ ? 1.0 : 0.0;
+        __syncthreads();
+        for (int lr = 0; lr < kJP - 1; ++lr) {
+          if (tid < kJP / 2) {
+            int p, q;
+            pair_of(lr, tid, kJP, p, q);
+            double c = 1.0, sn = 0.0;
+            const double apq = S.x[p][q];
+            if (apq != 0.0) {
+              const double dd = S.x[q][q] - S.x[p][p];
+              const double t = (dd >= 0.0 ? 2.0 * apq : -2.0 * apq) / (fabs(dd) + sqrt(dd * dd + 4.0 * apq * apq));
+              c = rsqrt(t * t + 1.0);
+              sn = t * c;
+            }
+            S.c[tid] = c;
+            S.s[tid] = sn;
+          }
+          __syncthreads();
+          if (tid < (kJP / 2) * kJP) {  // rows p, q
+            const int i = tid / kJP, k = tid % kJP;
+            int p, q;
+            pair_of(lr, i, kJP, p, q);
+            const double c = S.c[i], sn = S.s[i];
+            if (sn != 0.0) {
+              const double apk = S.x[p][k], aqk = S.x[q][k];
+              S.x[p][k] = c * apk - sn * aqk;
+              S.x[q][k] = sn * apk + c * aqk;
+            }
+          }
+          __syncthreads();
+          {  // columns p, q of the problem (first half of the threads) and of Q (second half)
+            const int u = tid % ((kJP / 2) * kJP);
+            const int i = u / kJP, k = u % kJP;
+            int p, q;
+            pair_of(lr, i, kJP, p, q);
+            const double c = S.c[i], sn = S.s[i];
+            const bool onS = tid < (kJP / 2) * kJP;
+            double(*X)[kJP + 1] = onS ? S.x : S.y;
+            if (sn != 0.0) {
+              const double xkp = X[k][p], xkq = X[k][q];
+              // the rotated pair's off-diagonal entries are zero by construction
+              X[k][p] = (onS && k == q) ? 0.0 : c * xkp - sn * xkq;
+              X[k][q] = (onS && k == p) ? 0.0 : sn * xkp + c * xkq;
+            }
+          }
+          __syncthreads();
+        }
+        __stcg(J.q + static_cast<size_t>(P) * kJP * kJP + tid, S.y[lr_][lc_]);
+        __stcg(B + static_cast<size_t>(gr) * m + gc, S.x[lr_][lc_]);
+        __syncthreads();
+      }
+      if (!grid.sync()) return -1;
+      // (2) the other blocks of A, Q_P^T A[P rows][P' cols] Q_P' (into B), and V's columns,
+      //     V[rows][P' cols] Q_P' (in place: every entry belongs to one item)
+      const int nA = np * np, nItems = nA + (m / kJP) * np;
+      for (int it = blockIdx.x; it < nItems; it += gridDim.x) {
+        if (it < nA && it / np == it % np) continue;  // diagonal blocks came from step (1)
+        const bool isA = it < nA;
+        const int P2 = isA ? it % np : (it - nA) % np;
+        int ci, cj;
+        pair_of(br, P2, nb, ci, cj);
+        const int gc = lc_ < kJW ? ci * kJW + lc_ : cj * kJW + lc_ - kJW;
+        int gr;
+        if (isA) {
+          int bi, bj;
+          pair_of(br, it / np, nb, bi, bj);
+          gr = lr_ < kJW ? bi * kJW + lr_ : bj * kJW + lr_ - kJW;
+          S.x[lr_][lc_] = __ldcg(A + static_cast<size_t>(gr) * m + gc);
+          S.qa[lr_][lc_] = __ldcg(J.q + static_cast<size_t>(it / np) * kJP * kJP + tid);
+        } else {
+          gr = ((it - nA) / np) * kJP + lr_;
+          S.x[lr_][lc_] = __ldcg(V + static_cast<size_t>(gr) * m + gc);
+        }
+        S.qb[lr_][lc_] = __ldcg(J.q + static_cast<size_t>(P2) * kJP * kJP + tid);
+        __syncthreads();
+        if (isA) {
+          double t = 0.0;
+#pragma unroll
+          for (int k = 0; k < kJP; ++k) t = fma(S.qa[k][lr_], S.x[k][lc_], t);
+          S.t[lr_][lc_] = t;
+          __syncthreads();
+        }
+        double(*L)[kJP + 1] = isA ? S.t : S.x;
+        double y = 0.0;
+#pragma unroll
+        for (int k = 0; k < kJP; ++k) y = fma(L[lr_][k], S.qb[k][lc_], y);
+        __stcg((isA ? B : V) + static_cast<size_t>(gr) * m + gc, y);
+        __syncthreads();
+      }
+      double* t = A;
+      A = B;
+      B = t;
+      if (!grid.sync()) return -1;
+    }
+  }
+  return sweep;
+}
+
+}  // namespace
+
+// a, b, v, w, g, x: m x m; the FP64 rotations (a quarter of that is the FP32 ones'); the seed; slots
+size_t jacobi_scratch_doubles(int pa) {
+  const size_t m = jacobi_order(pa);
+  return 6 * m * m + static_cast<size_t>(pa) * pa + (m / kJP) * kJP * kJP + 1024 + 8;
+}
+
+int jacobi_grid_blocks(int pa, int sms) {
+  const int np = jacobi_order(pa) / kJP;
+  int g = 2 * np * np;
+  if (g > sms) g = sms;
+  if (g > 256) g = 256;  // two partial sums per block, at 0 and 512 of the 1024 slots
+  return g < 1 ? 1 : g;
+}
+
+__global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_constant__ JacobiParams J) {
+  extern __shared__ __align__(16) float dyn[];
+  __shared__ Shared S;
+  if (__ldcg(J.ctl) == 0) return;  // the finalize kernel found the eigenpairs undefined
+  const int tid = threadIdx.x, pa = J.pa, m = J.m;
+  const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
+  Grid grid{J.bar, 0u, J.wait_ns > 0 ? static_cast<unsigned long long>(J.wait_ns) : kGridWaitNs, &S.ok};
+  double* flags = J.out + J.flags_off;
+  double* A = J.a;
+  double* V = J.v;
+  const double* T = J.a;  // what step 2 diagonalises
+  bool seeded = false;
+  int sweeps = 0;
+  // a block told to be absent leaves before its first arrival: the other blocks' waits at that
+  // barrier run out after wait_ns and the call reports the timeout (the failure path of a stalled
+  // block, taken without a fault)
+  bool alive = static_cast<int>(blockIdx.x) != J.absent_block;
+  auto at = [m](int i, int j) { return static_cast<size_t>(i) * m + j; };
+
+  // ||A||_F^2, and the seed into V
+  if (alive) {
+    double f = 0.0;
+    for (int i = gtid; i < m * m; i += nthreads) {
+      const double x = __ldcg(A + i);
+      f = fma(x, x, f);
+      if (J.basis) {
+        const int r = i / m, c = i % m;
+        __stcg(V + i, r < pa && c < pa ? J.basis[static_cast<size_t>(c) * pa + r] : r == c ? 1.0 : 0.0);
+      }
+    }
+    f = block_total(f, S.red);
+    if (tid == 0) __stcg(J.slots + blockIdx.x, f);
+    alive = grid.sync();
+  }
+  const double fro2 = alive ? slots_total(J.slots, S) : 0.0;
+  if (alive && J.basis) {
+    // the seed is used only if its columns are orthonormal: max |V^T V - I| <= 1e-9
+    double dev = 0.0;
+    grid_product(
+        m, S, [&](int i, int k) { return __ldcg(V + at(k, i)); }, [&](int k, int j) { return __ldcg(V + at(k, j)); },
+        [&](int i, int j, double v) {
+          const double x = fabs(v - (i == j ? 1.0 : 0.0));
+          dev = fmax(dev, x == x ? x : 1.0);
+        });
+    dev = block_max(dev, S.red);
+    if (tid == 0) __stcg(J.slots + 512 + blockIdx.x, dev);
+    alive = grid.sync();
+    seeded = alive && slots_max(J.slots + 512, S) <= 1e-9;
+    if (seeded) {  // T = V^T A V
+      grid_product(
+          m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(V + at(k, j)); },
+          [&](int i, int j, double v) { __stcg(J.w + at(i, j), v); });
+      alive = grid.sync();
+      if (alive)
+        grid_product(
+            m, S, [&](int i, int k) { return __ldcg(V + at(k, i)); }, [&](int k, int j) { return __ldcg(J.w + at(k, j)); },
+            [&](int i, int j, double v) { __stcg(J.b + at(i, j), v); });
+      alive = alive && grid.sync();
+      T = J.b;
+    }
+  }
+
+  bool refined = false;  // lambda and X hold the result
+  bool warm = false;     // X is orthonormal, but some eigenvalues are too close for the refinement
+  double* X = J.x;
+  double* Xn = V;
+  // FP32 has to hold the matrix scaled to order one, FP64 the squares of its entries
+  if (alive && fro2 > 1e-280 && fro2 < 1e280) {
+    const int E = scale_exponent(fro2);
+    float* F = reinterpret_cast<float*>(J.g);  // two m x m FP32 matrices
+    float* Q32 = reinterpret_cast<float*>(J.x);  // V of step 2
+    auto t32 = [&](int r, int c) {
+      if (T == J.a) return scaled32(__ldcg(T + at(r, c)), E);
+      return scaled32(0.5 * (__ldcg(T + at(r, c)) + __ldcg(T + at(c, r))), E);
+    };
+    if (m <= k32Max) {
+      if (blockIdx.x == 0) {
+        float* sA = dyn;
+        float* sV = dyn + 2 * m * m;
+        for (int i = tid; i < m * m; i += kThreads) {
+          sA[i] = t32(i / m, i % m);
+          sV[i] = i / m == i % m ? 1.f : 0.f;
+        }
+        __syncthreads();
+        int n = 0, copy = 0;
+        switch (m) {
+          case 16: n = jacobi32<16>(sA, sV, 20, S.s32, copy); break;
+          case 32: n = jacobi32<32>(sA, sV, 20, S.s32, copy); break;
+          case 48: n = jacobi32<48>(sA, sV, 20, S.s32, copy); break;
+          case 64: n = jacobi32<64>(sA, sV, 20, S.s32, copy); break;
+          case 80: n = jacobi32<80>(sA, sV, 20, S.s32, copy); break;
+          default: n = jacobi32<96>(sA, sV, 20, S.s32, copy); break;
+        }
+        sV += copy * m * m;
+        for (int i = tid; i < m * m; i += kThreads) __stcg(Q32 + i, sV[i]);
+        if (tid == 0) __stcg(J.slots + 1023, static_cast<double>(n));
+      }
+      alive = grid.sync();
+      sweeps = alive ? static_cast<int>(__ldcg(J.slots + 1023)) : 0;
+    } else {
+      for (int i = gtid; i < m * m; i += nthreads) {
+        __stcg(F + i, t32(i / m, i % m));
+        __stcg(Q32 + i, i / m == i % m ? 1.f : 0.f);
+      }
+      alive = grid.sync();
+      if (alive) {
+        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32, reinterpret_cast<float*>(J.q));
+        alive = sweeps >= 0;
+      }
+    }
+    // X = V Q (into w first: Q lies where X goes)
+    if (alive) {
+      if (seeded)
+        grid_product(
+            m, S, [&](int i, int k) { return __ldcg(V + at(i, k)); },
+            [&](int k, int j) { return f32_to_f64(__ldcg(Q32 + at(k, j))); },
+            [&](int i, int j, double v) { __stcg(J.w + at(i, j), v); });
+      else
+        for (int i = gtid; i < m * m; i += nthreads) __stcg(J.w + i, f32_to_f64(__ldcg(Q32 + i)));
+      alive = grid.sync();
+    }
+    double* W = J.x;  // A X, then the corrections
+    X = J.w;
+    const double noise = 16.0 * 1.1102230246251565e-16 * sqrt(fro2);
+    for (int it = 0; alive && it < 5; ++it) {
+      grid_product(
+          m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(X + at(k, j)); },
+          [&](int i, int j, double v) { __stcg(W + at(i, j), v); });
+      if (!(alive = grid.sync())) break;
+      grid_grams(m, S, X, W, J.b, J.g);
+      if (!(alive = grid.sync())) break;
+      if (tid < m) S.lambda[tid] = __ldcg(J.b + at(tid, tid)) / __ldcg(J.g + at(tid, tid));
+      __syncthreads();
+      int bad = 0;
+      double mx = 0.0;
+      for (int i = gtid; i < m * m; i += nthreads) {
+        const int r = i / m, c = i % m;
+        const double e = correction(r, c, __ldcg(J.b + i), __ldcg(J.g + i), S.lambda[r], S.lambda[c], noise, bad);
+        mx = fmax(mx, fabs(e));
+        __stcg(W + i, e);
+      }
+      mx = block_max(mx, S.red);
+      const double fb = block_max(static_cast<double>(bad), S.red);
+      if (tid == 0) {
+        __stcg(J.slots + blockIdx.x, mx);
+        __stcg(J.slots + 512 + blockIdx.x, fb);
+      }
+      if (!(alive = grid.sync())) break;
+      mx = slots_max(J.slots, S);
+      const double anybad = slots_max(J.slots + 512, S);
+      if (anybad > 1.5 || mx > 0.5) break;  // not a refinement any more
+      grid_product(
+          m, S, [&](int i, int k) { return __ldcg(X + at(i, k)); }, [&](int k, int j) { return __ldcg(W + at(k, j)); },
+          [&](int i, int j, double v) { __stcg(Xn + at(i, j), __ldcg(X + at(i, j)) + v); });
+      if (!(alive = grid.sync())) break;
+      double* t = X;
+      X = Xn;
+      Xn = t;
+      if (mx <= kRefined) {
+        refined = anybad == 0.0;
+        warm = !refined;
+        break;
+      }
+    }
+  }
+  if (alive && !refined) {
+    if (warm) {  // A <- X^T A X, symmetrised, and on from there
+      double* W = J.x;
+      grid_product(
+          m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(X + at(k, j)); },
+          [&](int i, int j, double v) { __stcg(W + at(i, j), v); });
+      alive = grid.sync();
+      if (alive)
+        grid_product(
+            m, S, [&](int i, int k) { return __ldcg(X + at(k, i)); }, [&](int k, int j) { return __ldcg(W + at(k, j)); },
+            [&](int i, int j, double v) { __stcg(J.b + at(i, j), v); });
+      alive = alive && grid.sync();
+      if (alive)
+        for (int i = gtid; i < m * m; i += nthreads)
+          __stcg(A + i, 0.5 * (__ldcg(J.b + i) + __ldcg(J.b + at(i % m, i / m))));
+    } else {
+      X = V;
+      for (int i = gtid; alive && i < m * m; i += nthreads) __stcg(X + i, (i / m == i % m) ? 1.0 : 0.0);
+      seeded = false;
+    }
+    alive = alive && grid.sync();
+    if (alive) {
+      const int n = grid_jacobi64(J, grid, S, A, J.b, X);
+      alive = n >= 0;
+      sweeps += max(n, 0);
+      if (alive && tid < m) S.lambda[tid] = __ldcg(A + at(tid, tid));
+      __syncthreads();
+    }
+  }
+  if (!alive) {
+    if (tid == 0) flags[5] = 1.0;
+    return;
+  }
+  // descending order (ties by index), eigenvector signs: largest-magnitude component positive
+  if (tid < pa) {
+    S.key[tid] = order_key(S.lambda[tid]);
+    S.order[tid] = tid;
+  }
+  __syncthreads();
+  if (tid < pa) {
+    int rank = 0;
+    const unsigned long long k = S.key[tid];
+    for (int d = 0; d < pa; ++d) rank += (S.key[d] > k || (S.key[d] == k && d < tid)) ? 1 : 0;
+    S.order[rank] = tid;
+  }
+  __syncthreads();
+  double* evals = J.out + J.evals_off;
+  double* evecs = J.out + J.evecs_off;
+  for (int k = blockIdx.x; k < pa; k += gridDim.x) {
+    const int col = S.order[k];
+    double vi = 0.0;
+    unsigned long long best = 0;
+    int bi = kThreads;
+    if (tid < pa) {
+      vi = __ldcg(X + at(tid, col));
+      best = magnitude_key(vi);
+      bi = tid;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) {
+        best = ob;
+        bi = oi;
+      }
+    }
+    if ((tid & 31) == 0) {
+      S.best[tid >> 5] = best;
+      S.best_i[tid >> 5] = bi;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      unsigned long long bb = S.best[0];
+      int ii = S.best_i[0];
+      for (int w = 1; w < kThreads / 32; ++w)
+        if (S.best[w] > bb || (S.best[w] == bb && S.best_i[w] < ii)) {
+          bb = S.best[w];
+          ii = S.best_i[w];
+        }
+      S.val = __ldcg(X + at(ii, col)) < 0.0 ? -1.0 : 1.0;
+      evals[k] = S.lambda[col];
+    }
+    __syncthreads();
+    if (tid < pa) evecs[static_cast<size_t>(k) * pa + tid] = S.val * vi;
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    flags[2] = sweeps;
+    flags[3] = 1.0;
+    flags[6] = seeded ? 1.0 : 0.0;
+  }
+}
+
+cudaError_t launch_jacobi_grid(const JacobiParams& J, int grid, cudaStream_t stream) {
+  if (grid < 1 || J.m > 256 || J.m < 16) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(jacobi_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(kDynBytes));
+  if (e != cudaSuccess) return e;
+  void* args[] = {const_cast<JacobiParams*>(&J)};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(jacobi_grid_kernel), dim3(grid), dim3(kThreads), args,
+                                     kDynBytes, stream);
+}
+
+}  // namespace ss

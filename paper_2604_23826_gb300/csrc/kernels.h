@@ -353,8 +353,9 @@ struct FinalParams {
   double* out;                 // device result buffer (layout: final_layout())
   double* work;                // device scratch: 2 * pa * pa doubles
   // When set, the eigen-decomposition is left to jacobi_grid_kernel: the matrix goes to
-  // defer_A (defer_m x defer_m, zero-padded to an even order) and *defer_ctl = 1 when the
-  // eigenpairs are wanted and defined (0 otherwise).
+  // defer_A (defer_m x defer_m, zero-padded to the solver's order) and *defer_ctl = 1 when the
+  // eigenpairs are wanted and defined (0 otherwise).  defer_m < 0: it is left to the batched
+  // eigen-solver, flags[7] saying the same.
   double* defer_A;
   int32_t* defer_ctl;
   int32_t defer_m;
@@ -384,32 +385,41 @@ __host__ __device__ inline FinalLayout final_layout(int p, int pa) {
 //        [2] Jacobi sweeps, [3] eigenpairs computed (1) or not (0),
 //        [5] a grid-wide wait of jacobi_grid_kernel ran out (1), [6] its seed basis was used (1)
 cudaError_t launch_finalize(const FinalParams& P, cudaStream_t stream);
-// d_params: count FinalParams in device memory, one block each
-cudaError_t launch_finalize_batched(const FinalParams* d_params, int count, cudaStream_t stream);
+// An eigen-decomposition of a batch (n of batched_eigen_deferred), after its context's finalize block.
+struct EigJob {
+  const double* matrix;  // n x n, in the context's result buffer
+  double* evals;
+  double* evecs;
+  double* flags;
+  int32_t n, pad;
+};
+bool batched_eigen_deferred(int pa);
+// d_params: count FinalParams in device memory, one block each; d_jobs: the deferred decompositions
+cudaError_t launch_finalize_batched(const FinalParams* d_params, int count, const EigJob* d_jobs, int njobs,
+                                    cudaStream_t stream);
 
-// Block-cyclic Jacobi spread over a cooperative grid.  The indices are cut into blocks
-// of 8; in each block round (the round-robin ordering over blocks) every pair of blocks
-// solves its 16 x 16 diagonal problem with one cyclic Jacobi sweep (the one-block
-// solver's rotation formula) in shared memory, then all 16 x 16 blocks of A and V are
-// updated with the pairs' accumulated rotations: two grid-wide barriers per block round.
-// A is double buffered (a round reads a and writes b).
+// The eigen-solver spread over a cooperative grid (k_eigen.cu).
 struct JacobiParams {
   double* a;                // m x m, holds the matrix on entry (written by the finalize kernel)
-  double* b;                // m x m
-  double* v;                // m x m eigenvector accumulator
-  double* w;                // m x m, warm start product
+  double* b;                // five more m x m arrays of scratch
+  double* v;
+  double* w;
+  double* g;
+  double* x;
   double* q;                // (m / 16) x 16 x 16: the rotation of every block pair of a round
   const double* basis;      // pa x pa, row k = a previous eigenvector k, or nullptr (cold start)
-  double* slots;            // >= grid partial sums
-  unsigned int* bar;        // [0] arrivals, [1] generation, [2] error; zero before each launch
+  double* slots;            // 1024 partial sums
+  unsigned int* bar;        // arrivals and the mark of a wait that ran out; zero before each launch
   const int32_t* ctl;       // written by the finalize kernel: 1 = decompose
   double* out;              // finalize result buffer
   int64_t evals_off, evecs_off, flags_off;
-  int32_t pa, m;            // analysis columns; m = pa rounded up to a multiple of 16
+  int32_t pa, m;            // analysis columns; m = jacobi_order(pa)
   int64_t wait_ns;          // limit of one grid-wide wait (<= 0: 2 s)
   int32_t absent_block;     // testing: this block leaves before its first arrival (-1: none)
 };
-// Doubles of scratch jacobi_grid_kernel needs for pa analysis columns (the five arrays above).
+// Order of the padded matrix: a multiple of 16, of 32 above 96 (the FP32 rotations' block pairs).
+__host__ __device__ inline int jacobi_order(int pa) { return pa <= 96 ? (pa + 15) / 16 * 16 : (pa + 31) / 32 * 32; }
+// Doubles of scratch jacobi_grid_kernel needs for pa analysis columns.
 size_t jacobi_scratch_doubles(int pa);
 // Blocks of the cooperative grid for pa columns on a device of `sms` SMs (0: not possible).
 int jacobi_grid_blocks(int pa, int sms);
