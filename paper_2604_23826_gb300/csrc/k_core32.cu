@@ -3,21 +3,23 @@
 // Representation and Sufficient Statistics" with the shift of "Numerical Considerations").
 //
 // Bound: FP32 FMA for more than about fifty columns (p (p + 1) / 2 per row at 128 per clock and
-// SM), HBM below.  So the layout spends shared-memory reads and issue slots on as little else as
-// possible:
+// SM), HBM below.  So the layout spends issue slots, shared-memory reads and barriers on as little
+// else as possible:
 //   - the output's upper triangle is cut into 8 x 4 register micro-tiles, one per thread: three
-//     128-bit shared loads feed 32 FMAs (the row's 8 left values are the same for most of a warp, a
-//     broadcast; the 4 right values of consecutive lanes are consecutive, conflict-free).  Only
-//     tiles on or above the diagonal exist, so 100 columns cost 5408 FMAs a row for 5050 entries;
+//     128-bit shared loads and four register pairs feed 16 packed FMAs of two entries each (which
+//     take two cycles, so the other instructions issue beside them).  Only tiles on or above the
+//     diagonal exist, so 100 columns cost 5408 FMAs a row for 5050 entries.  Tiles of 8 x 8 with
+//     eight warps and 255 registers were slower (779 against 485 us, both with plain FMAs);
 //   - when there are fewer tiles than threads, the rows of a stage are dealt to several slices of
 //     threads; when there are more, groups of blocks take a part of the tiles each.  core32_plan
 //     picks the number of groups by the instructions a row costs;
 //   - columns are copied as they lie (cp.async, 16 bytes, two stages ahead), then one pass turns a
-//     stage into rows of x - c (lanes = columns: conflict-free both ways) and adds the column sums.
+//     stage into rows of x - c (lanes = columns: conflict-free both ways) and adds the column sums,
+//     while other warps still multiply the stage before: one barrier a stage.
 // Columns of other types, or not 16-byte aligned, are converted (x - c in FP64) into the same
 // stage by plain loads.
 // 1e6 rows x 100 columns: 8.78 ms as 64 x 64 tiles of scalar shared loads with an FP64 subtraction
-// per element, 0.485 ms now (its FMAs alone: 0.135 ms).
+// per element, 0.427 ms now (its FMAs alone: 0.135 ms).
 // Each block writes one slot of (hi, lo) pairs; a second kernel adds the slots of an entry in row
 // order, in three-term FP32 expansions and then FP64 pairs (a fixed order: a given grid
 // reproduces its bits).
@@ -33,18 +35,44 @@ using namespace core;
 
 constexpr int kMI = 8, kMJ = 4, kE = kMI * kMJ;
 constexpr int kNT = 512;
-constexpr int kStageFloats = 16384;  // columns (padded) x rows of a stage, at most
-constexpr int kTreeBytes = (kNT / 2) * kE * 8;  // the slices' pairs on their way to one slot
+constexpr size_t kSmemMax = 226 * 1024;
+constexpr size_t kTreeBytes = (kNT / 2) * kE * 8;  // the slices' pairs on their way to one slot
 
 __host__ __device__ inline int width_of(int p) { return (p + kMI - 1) / kMI * kMI; }
 __host__ __device__ inline size_t raw_bytes(int W, int R) { return static_cast<size_t>(W) * (R + 4) * 4; }
 __host__ __device__ inline size_t row_bytes(int W, int R) { return static_cast<size_t>(R) * (W + 4) * 4; }
 
+// two FP32 values in a 64-bit register: one instruction works on both, each rounded as by itself
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 twice(float v) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+  return d;
+}
+__device__ __forceinline__ float2 parts(f32x2 v) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
+  return d;
+}
+__device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ Core32Params P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int p = P.p, W = width_of(p), R = 1 << P.log_rows, S = W + 4, K = R + 4;
-  float* raw = reinterpret_cast<float*>(smem);                         // [2][W][K], as the columns lie
-  float* X = reinterpret_cast<float*>(smem + 2 * raw_bytes(W, R));      // [R][S], rows of x - c
+  float* raw = reinterpret_cast<float*>(smem);                     // [2][W][K], as the columns lie
+  float* X = reinterpret_cast<float*>(smem + 2 * raw_bytes(W, R));  // [2][R][S], rows of x - c
   const int tid = threadIdx.x;
   const int g = blockIdx.x % P.groups, range = blockIdx.x / P.groups;
   const int64_t nst = (P.nrows + R - 1) >> P.log_rows;
@@ -56,20 +84,22 @@ __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ 
   const bool active = slice < P.slices && tile < P.ntiles;
   int bi = 0, bj = 0;
   if (active) tile_of<kMI, kMJ>(tile, p, bi, bj);
-  float acc[kMI][kMJ], hi[kMI][kMJ], lo[kMI][kMJ];
+  f32x2 acc[kMI / 2][kMJ], hi[kMI / 2][kMJ], lo[kMI / 2][kMJ];  // rows 2 i, 2 i + 1 of the tile together
 #pragma unroll
-  for (int i = 0; i < kMI; ++i)
+  for (int i = 0; i < kMI / 2; ++i)
 #pragma unroll
-    for (int j = 0; j < kMJ; ++j) acc[i][j] = hi[i][j] = lo[i][j] = 0.f;
+    for (int j = 0; j < kMJ; ++j) acc[i][j] = hi[i][j] = lo[i][j] = 0;
   int since = 0;
   auto flush = [&] {
     since = 0;
 #pragma unroll
-    for (int i = 0; i < kMI; ++i)
+    for (int i = 0; i < kMI / 2; ++i)
 #pragma unroll
-      for (int j = 0; j < kMJ; ++j) {
-        pair_add(hi[i][j], lo[i][j], acc[i][j]);
-        acc[i][j] = 0.f;
+      for (int j = 0; j < kMJ; ++j) {  // pair_add
+        const f32x2 s = add2(hi[i][j], acc[i][j]), bp = sub2(s, hi[i][j]);
+        lo[i][j] = add2(lo[i][j], add2(sub2(hi[i][j], sub2(s, bp)), sub2(acc[i][j], bp)));
+        hi[i][j] = s;
+        acc[i][j] = 0;
       }
   };
 
@@ -105,59 +135,75 @@ __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ 
         }
       }
   };
+  auto convert = [&](int64_t st) {
+    if (cq >= ncq) return;
+    const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - (st << P.log_rows)));
+    const float* src = raw + (st & 1) * (raw_bytes(W, R) / 4) + cc * K;
+    float* dst = X + (st & 1) * (row_bytes(W, R) / 4) + cc;
+    float s = 0.f;
+#pragma unroll 2
+    for (int k = 4 * cq; k < R; k += 4 * ncq) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (cc < p) {
+        const float4 x = *reinterpret_cast<const float4*>(src + k);
+        v[0] = k < rows ? x.x - shift : 0.f;
+        v[1] = k + 1 < rows ? x.y - shift : 0.f;
+        v[2] = k + 2 < rows ? x.z - shift : 0.f;
+        v[3] = k + 3 < rows ? x.w - shift : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) dst[(k + i) * S] = v[i];
+      s += (v[0] + v[1]) + (v[2] + v[3]);
+    }
+    pair_add(shi, slo, s);
+  };
 
+  // One barrier a stage: while stage st is multiplied, st + 1 is turned into rows by whichever warps
+  // are done, and st + 2 is on its way.
   if (st0 < st1) issue(st0);
   cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
   if (st0 + 1 < st1) issue(st0 + 1);
   cp_async_commit();
+  if (st0 < st1) convert(st0);
   for (int64_t st = st0; st < st1; ++st) {
-    cp_async_wait<1>();
-    __syncthreads();  // the stage has landed; the last stage's rows have been read
-    const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - (st << P.log_rows)));
-    if (cq < ncq) {
-      const float* src = raw + (st & 1) * (raw_bytes(W, R) / 4) + cc * K;
-      float s = 0.f;
-      for (int k = 4 * cq; k < R; k += 4 * ncq) {
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (cc < p) {
-          const float4 x = *reinterpret_cast<const float4*>(src + k);
-          v[0] = k < rows ? x.x - shift : 0.f;
-          v[1] = k + 1 < rows ? x.y - shift : 0.f;
-          v[2] = k + 2 < rows ? x.z - shift : 0.f;
-          v[3] = k + 3 < rows ? x.w - shift : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) X[(k + i) * S + cc] = v[i];
-        s += (v[0] + v[1]) + (v[2] + v[3]);
-      }
-      pair_add(shi, slo, s);
-    }
-    __syncthreads();
+    cp_async_wait<0>();
+    __syncthreads();  // st is rows, st + 1 has landed, and st's columns and st - 1's rows are free
     if (st + 2 < st1) issue(st + 2);
     cp_async_commit();
     if (active) {
-      const float* xa = X + kMI * bi;
-      const float* xb = X + kMJ * bj;
-      for (int k = slice; k < rows;) {
+      const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - (st << P.log_rows)));
+      const float* x = X + (st & 1) * (row_bytes(W, R) / 4) + slice * S;
+      const float* xa = x + kMI * bi;
+      const float* xb = x + kMJ * bj;
+      const int step = P.slices * S;
+      for (int left = (rows - slice + P.slices - 1) / P.slices; left > 0;) {
         if (since == P.flush_rows) flush();
-        const int m = min((rows - k + P.slices - 1) / P.slices, P.flush_rows - since);
+        const int m = min(left, P.flush_rows - since);
         since += m;
-        for (int i = 0; i < m; ++i, k += P.slices) {
-          const float4 a0 = *reinterpret_cast<const float4*>(xa + k * S);
-          const float4 a1 = *reinterpret_cast<const float4*>(xa + k * S + 4);
-          const float4 b4 = *reinterpret_cast<const float4*>(xb + k * S);
-          const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-          const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+        left -= m;
+#pragma unroll 2
+        for (int i = 0; i < m; ++i, xa += step, xb += step) {
+          const ulonglong2 a01 = *reinterpret_cast<const ulonglong2*>(xa);
+          const ulonglong2 a23 = *reinterpret_cast<const ulonglong2*>(xa + 4);
+          const float4 b4 = *reinterpret_cast<const float4*>(xb);
+          const f32x2 a[4] = {a01.x, a01.y, a23.x, a23.y};
+          const f32x2 b[4] = {twice(b4.x), twice(b4.y), twice(b4.z), twice(b4.w)};
 #pragma unroll
-          for (int u = 0; u < kMI; ++u)
+          for (int u = 0; u < kMI / 2; ++u)
 #pragma unroll
-            for (int v = 0; v < kMJ; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+            for (int v = 0; v < kMJ; ++v) fma2(acc[u][v], a[u], b[v]);
         }
       }
     }
+    if (st + 1 < st1) convert(st + 1);
   }
-  cp_async_wait<0>();
   flush();
+  auto at = [](const f32x2(&v)[kMI / 2][kMJ], int e) {  // entry e = 4 row + column of the tile
+    const float2 w = parts(v[e / kMJ / 2][e % kMJ]);
+    return (e / kMJ) & 1 ? w.y : w.x;
+  };
   // the slices' pairs, added in a fixed tree through shared memory
   float2* buf = reinterpret_cast<float2*>(smem);
   for (int n = P.slices; n > 1;) {
@@ -166,16 +212,24 @@ __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ 
     if (slice >= h && slice < n) {
 #pragma unroll
       for (int e = 0; e < kE; ++e)
-        buf[e * (kNT / 2) + (slice - h) * tg + tl] = make_float2(hi[e / kMJ][e % kMJ], lo[e / kMJ][e % kMJ]);
+        buf[e * (kNT / 2) + (slice - h) * tg + tl] = make_float2(at(hi, e), at(lo, e));
     }
     __syncthreads();
     if (slice < n - h) {
 #pragma unroll
-      for (int e = 0; e < kE; ++e) {
-        const float2 v = buf[e * (kNT / 2) + slice * tg + tl];
-        pair_add(hi[e / kMJ][e % kMJ], lo[e / kMJ][e % kMJ], v.x);
-        lo[e / kMJ][e % kMJ] += v.y;
-      }
+      for (int i = 0; i < kMI / 2; ++i)
+#pragma unroll
+        for (int j = 0; j < kMJ; ++j) {
+          const float2 v = buf[(2 * i * kMJ + j) * (kNT / 2) + slice * tg + tl];
+          const float2 w = buf[((2 * i + 1) * kMJ + j) * (kNT / 2) + slice * tg + tl];
+          float2 h = parts(hi[i][j]), l = parts(lo[i][j]);
+          pair_add(h.x, l.x, v.x);
+          pair_add(h.y, l.y, w.x);
+          l.x += v.y;
+          l.y += w.y;
+          asm("mov.b64 %0, {%1, %2};" : "=l"(hi[i][j]) : "f"(h.x), "f"(h.y));
+          asm("mov.b64 %0, {%1, %2};" : "=l"(lo[i][j]) : "f"(l.x), "f"(l.y));
+        }
     }
     n = h;
   }
@@ -183,7 +237,7 @@ __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ 
   if (slice == 0) {
 #pragma unroll
     for (int e = 0; e < kE; ++e)
-      slot[static_cast<size_t>(e) * tg + tl] = make_float2(hi[e / kMJ][e % kMJ], lo[e / kMJ][e % kMJ]);
+      slot[static_cast<size_t>(e) * tg + tl] = make_float2(at(hi, e), at(lo, e));
   }
   __syncthreads();
   if (cq < ncq) buf[cq * W + cc] = make_float2(shi, slo);
@@ -266,7 +320,7 @@ __global__ void __launch_bounds__(32 * kSeg) core32_merge_kernel(const __grid_co
 }
 
 size_t smem_bytes(int W, int R) {
-  return std::max<size_t>(2 * raw_bytes(W, R) + row_bytes(W, R), kTreeBytes);
+  return std::max<size_t>(2 * raw_bytes(W, R) + 2 * row_bytes(W, R), kTreeBytes);
 }
 
 }  // namespace
@@ -276,14 +330,14 @@ void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P) {
   const int W = width_of(p), M = tile_count(p, kMI, kMJ);
   P.ntiles = M;
   // groups of blocks over the tiles: the fewest warp instructions a row costs the SMs together,
-  // ~35 per warp of tiles (32 FMAs and 3 loads; warps run four at a time) and ~14 per 128
+  // ~42 per warp of tiles (16 double FMAs of two cycles, 3 loads, 4 copies; warps run four at a time) and ~14 per 128
   // converted values in every group
   double best = 0;
   for (int G = (M + kNT - 1) / kNT; G <= 4 * ((M + kNT - 1) / kNT); ++G) {
     const int tg = (M + G - 1) / G, ks = kNT / tg;
     if (tg * (G - 1) >= M) continue;
     const int quads = ((tg * ks + 31) / 32 + 3) / 4;
-    const double cost = G * (quads * 4 * 35.0 / ks + W * 14.0 / 128);
+    const double cost = G * (quads * 4 * 42.0 / ks + W * 14.0 / 128);
     if (best == 0 || cost < best) {
       best = cost;
       P.groups = G;
@@ -292,9 +346,9 @@ void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P) {
     }
   }
   // rows of a stage: as many as shared memory takes, fewer while that would leave SMs without one
-  int lr = 6;
+  int lr = 5;
   const int want = std::max(1, (blocks > 0 ? blocks : sms) / P.groups);
-  while (lr < 11 && (W << (lr + 1)) <= kStageFloats && (nrows >> (lr + 1)) >= 2 * int64_t(want)) ++lr;
+  while (lr < 11 && smem_bytes(W, 1 << (lr + 1)) <= kSmemMax && (nrows >> (lr + 1)) >= 2 * int64_t(want)) ++lr;
   P.log_rows = lr;
   const int64_t nst = (nrows + (int64_t(1) << lr) - 1) >> lr;
   P.ranges = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, nst)));
