@@ -1,7 +1,7 @@
 // api.cu -- the C ABI of libsuffstats (declared in include/stats.h): context
 // management, the digit plan of the exact pass, launches, host-streamed double
 // buffering, merge, checkpoint.  Every step of the pass itself runs in the
-// kernels of k_exact.cu / k_fp64.cu / k_finalize.cu; this file only validates
+// kernels of k_*.cu; this file only validates
 // arguments, owns device memory and orders work on streams.
 #include <math.h>
 #include <string.h>
@@ -77,9 +77,7 @@ struct stats_ctx {
   double* d_fS_lo = nullptr;
   double* d_shift = nullptr;
   long long* d_fn = nullptr;
-  double* d_slots = nullptr;            // FP64 scratch: block slots + ticket
-  int slot_grid = 0;
-  void* d_core_slots = nullptr;         // CUDA-core passes (wide FP64, FP32) scratch: block slots
+  void* d_core_slots = nullptr;         // CUDA-core passes (FP64, FP32) scratch: block slots
   size_t core_bytes = 0;
   float* d_fshift = nullptr;            // BF16X3/X4: pivot as float
   float* d_wide_slots = nullptr;        // BF16X3/X4, p > 64 on tcgen05: per-CTA slots
@@ -298,25 +296,10 @@ stats_status device_status(stats_ctx* c) {
   return STATS_OK;
 }
 
+// blocks of an exact pass
 int default_grid(stats_ctx* c) {
   if (c->grid > 0) return c->grid;
-  if (c->mode == STATS_EXACT) {
-    int per = exact_max_active_blocks(c->conv, c->xp.shape, c->xp.stages, c->xp.stage_bytes);
-    if (per < 1) per = 1;
-    return c->sms * per;
-  }
-  return c->sms * 2;
-}
-
-stats_status ensure_slots(stats_ctx* c, int grid) {
-  if (c->d_slots && c->slot_grid >= grid) return STATS_OK;
-  if (c->d_slots) CK(c, cudaFree(c->d_slots));
-  c->d_slots = nullptr;
-  const size_t n = fp64_slot_doubles(grid);
-  CK(c, cudaMalloc(&c->d_slots, n * sizeof(double)));
-  CK(c, cudaMemset(c->d_slots, 0, n * sizeof(double)));
-  c->slot_grid = grid;
-  return STATS_OK;
+  return c->sms * std::max(1, exact_max_active_blocks(c->conv, c->xp.shape, c->xp.stages, c->xp.stage_bytes));
 }
 
 // Scratch of the CUDA-core passes (block slots), grown as a call needs it.
@@ -881,8 +864,8 @@ stats_status run_narrow_batch(const std::vector<NarrowJob>& jobs, bool x4, cudaS
 
 stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, cudaStream_t st) {
   if (nrows == 0) return STATS_OK;
-  const int grid = default_grid(c);
   if (c->mode == STATS_EXACT) {
+    const int grid = default_grid(c);
     ExactParams P = c->xp;
     if (c->exact_shape >= 0 && c->exact_shape != P.shape && !exact_layout(P, c->exact_shape)) return STATS_EINVAL;
     P.direct = 0;
@@ -973,7 +956,7 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
     C.acc_S_lo = c->d_fS_lo;
     C.acc_n = c->d_fn;
     CK(c, launch_core32(C, st));
-  } else if (c->p > 12) {
+  } else {
     Core64Params C{};
     C.p = c->p;
     for (int j = 0; j < c->p; ++j) {
@@ -998,30 +981,6 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
     C.acc_S_lo = c->d_fS_lo;
     C.acc_n = c->d_fn;
     CK(c, launch_core64(C, st));
-  } else {
-    Fp64Params P{};
-    for (int j = 0; j < c->p; ++j) {
-      P.cols[j] = dcols[j];
-      P.dtype[j] = c->dtypes[j];
-    }
-    P.p = c->p;
-    P.nrows = nrows;
-    if (c->mode == STATS_FP64_SHIFTED) {
-      if (!c->shift_set) {
-        CK(c, launch_set_shift(dcols, c->dtypes.data(), c->p, nrows, c->d_shift, st));
-        c->shift_set = true;
-      }
-      P.shift = c->d_shift;
-    }
-    stats_status s = ensure_slots(c, grid);
-    if (s != STATS_OK) return s;
-    P.slots = c->d_slots;
-    P.acc_s = c->d_fs;
-    P.acc_s_lo = c->d_fs_lo;
-    P.acc_S = c->d_fS;
-    P.acc_S_lo = c->d_fS_lo;
-    P.acc_n = c->d_fn;
-    CK(c, launch_fp64(P, grid, st));
   }
   c->rows_enqueued += nrows;
   c->last = st;
@@ -1113,7 +1072,6 @@ void free_ctx(stats_ctx* c) {
   cudaFree(c->d_g);
   cudaFree(c->d_call);
   cudaFree(c->d_fs);
-  cudaFree(c->d_slots);
   cudaFree(c->d_fshift);
   cudaFree(c->d_core_slots);
   cudaFree(c->d_split_slots);

@@ -47,14 +47,33 @@ __device__ __forceinline__ double i32_to_f64(int32_t v) {
   const uint32_t hi = (static_cast<uint32_t>(v) & 0x80000000u) + (static_cast<uint32_t>(1023 + 30 - lz) << 20) + (n >> 11);
   return v == 0 ? 0.0 : __hiloint2double(static_cast<int>(hi), static_cast<int>(n << 21));
 }
+__device__ __forceinline__ double i64_to_f64(int64_t v) {
+  const uint64_t m = v < 0 ? 0ull - static_cast<uint64_t>(v) : static_cast<uint64_t>(v);
+  const int lz = __clzll(static_cast<long long>(m));
+  if (lz < 11) return static_cast<double>(v);  // more than 53 bits: rounds
+  if (v == 0) return 0.0;
+  // n: the significand with its leading one at bit 52, which the exponent's field adds back
+  const uint64_t n = m << (lz - 11);
+  const uint64_t bits = (static_cast<uint64_t>(v) & (1ull << 63)) + (static_cast<uint64_t>(1023 + 62 - lz) << 52) + n;
+  return __longlong_as_double(static_cast<long long>(bits));
+}
+
+// the bits of value r of a column, sign-extended integers below 64 bits; bits_to_f64 turns them into
+// the value.  Two steps, so that a thread can have many loads in flight.
+__device__ __forceinline__ uint64_t load_bits(const void* col, int dt, int64_t r) {
+  if (dt == F64 || dt == I64) return static_cast<const uint64_t*>(col)[r];
+  if (dt == I16) return static_cast<uint32_t>(static_cast<const int16_t*>(col)[r]);
+  return static_cast<const uint32_t*>(col)[r];
+}
+__device__ __forceinline__ double bits_to_f64(uint64_t b, int dt) {
+  if (dt == F64) return __longlong_as_double(static_cast<long long>(b));
+  if (dt == F32) return f32_to_f64(__uint_as_float(static_cast<uint32_t>(b)));
+  if (dt == I64) return i64_to_f64(static_cast<int64_t>(b));
+  return i32_to_f64(static_cast<int32_t>(b));
+}
+
 __device__ __forceinline__ double load_as_double(const void* col, int dt, int64_t r) {
-  switch (dt) {
-    case I16: return i32_to_f64(static_cast<const int16_t*>(col)[r]);
-    case I32: return i32_to_f64(static_cast<const int32_t*>(col)[r]);
-    case I64: return static_cast<double>(static_cast<const int64_t*>(col)[r]);
-    case F32: return f32_to_f64(static_cast<const float*>(col)[r]);
-    default: return static_cast<const double*>(col)[r];
-  }
+  return bits_to_f64(load_bits(col, dt, r), dt);
 }
 
 // 16-byte asynchronous copy to shared memory of which only the first `bytes` are read, the rest

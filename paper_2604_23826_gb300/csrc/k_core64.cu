@@ -1,5 +1,5 @@
-// k_core64.cu -- the plain FP64 CUDA-core pass for tables of more than 12 columns (STATS_FP64 with
-// raw moments, STATS_FP64_SHIFTED on x - c), arxiv 2604.23826, "Data Representation and Sufficient
+// k_core64.cu -- the plain FP64 CUDA-core pass (STATS_FP64 with raw moments, as in the paper;
+// STATS_FP64_SHIFTED on x - c), arxiv 2604.23826, "Data Representation and Sufficient
 // Statistics" with the shift of "Numerical Considerations".
 //
 // Bound: the FP64 unit, 2 operations per clock and SM on GB300 (64 cycles a warp instruction,
@@ -13,7 +13,9 @@
 //     and stored as rows of an odd stride (conflict-free); several blocks per SM overlap the
 //     loads of one with the FMAs of another.
 // 250,001 rows x 48 columns: 6.60 ms as 64 x 64 tiles on 61 blocks, 0.67 ms now (FMAs, shift and
-// sums of those rows alone: 0.50 ms), plus 12 us to add the slots.
+// sums of those rows alone: 0.50 ms), plus 12 us to add the slots.  Up to 12 columns one thread kept a
+// row's 90 sums in registers (2e7 rows of Table 1: 5.08 ms); its eight warps an SM spent half their
+// time on loads and conversions.  This way: 3.85 ms (90 operations a row alone: 2.9 ms).
 // Each block writes one slot; a second kernel adds an entry's slots in row order into the ctx's
 // double-double accumulators (a fixed order: a given grid reproduces its bits).
 #include <algorithm>
@@ -27,21 +29,28 @@ namespace {
 using namespace core;
 
 constexpr int kMaxThreads = 512;
-constexpr int kBatch = 8;  // loads a lane has in flight
+constexpr int kBatch = 4;  // loads a lane has in flight
 
 __host__ __device__ inline int row_stride(int p, int MI) { return ((p + MI - 1) / MI * MI) | 1; }
 
-// the bits of value r of a column; to_f64 turns them into the value
-__device__ __forceinline__ uint64_t load_bits(const void* col, int dt, int64_t r) {
-  if (dt == F64 || dt == I64) return static_cast<const uint64_t*>(col)[r];
-  if (dt == I16) return static_cast<uint32_t>(static_cast<const int16_t*>(col)[r]);
-  return static_cast<const uint32_t*>(col)[r];
-}
-__device__ __forceinline__ double to_f64(uint64_t b, int dt) {
-  if (dt == F64) return __longlong_as_double(static_cast<long long>(b));
-  if (dt == F32) return f32_to_f64(__uint_as_float(static_cast<uint32_t>(b)));
-  if (dt == I64) return static_cast<double>(static_cast<long long>(b));
-  return i32_to_f64(static_cast<int32_t>(b));
+// 32 nchunks rows of a column from row r0 on (those below `rows`) as x - c into X; a lane has
+// kBatch loads in flight.  The type is the template's, so a value costs a load, about ten integer
+// instructions and a store.
+template <int DT>
+__device__ __forceinline__ void convert_rows(const void* col, int64_t r0, int rows, int nchunks, bool shifted, double c,
+                                             double* X, int S) {
+  const int lane = threadIdx.x & 31;
+  for (int k0 = lane; k0 < 32 * nchunks; k0 += 32 * kBatch) {
+    uint64_t v[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) v[u] = k0 + 32 * u < rows ? load_bits(col, DT, r0 + k0 + 32 * u) : 0;
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u)
+      if (k0 + 32 * u < rows) {
+        const double x = bits_to_f64(v[u], DT);
+        X[(k0 + 32 * u) * S] = shifted ? x - c : x;
+      }
+  }
 }
 
 template <int MI>
@@ -50,7 +59,7 @@ __global__ void __launch_bounds__(kMaxThreads) core64_kernel(const __grid_consta
   extern __shared__ __align__(16) uint8_t smem[];
   double* X = reinterpret_cast<double*>(smem);  // [R][S], rows of x - c
   const int p = P.p, R = 1 << P.log_rows, S = row_stride(p, MI);
-  const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
+  const int tid = threadIdx.x, NT = blockDim.x, warp = tid >> 5, nwarps = NT >> 5;
   const int g = blockIdx.x % P.groups, range = blockIdx.x / P.groups;
   const int64_t nst = (P.nrows + R - 1) >> P.log_rows;
   const int64_t st0 = nst * range / P.ranges, st1 = nst * (range + 1) / P.ranges;
@@ -73,24 +82,19 @@ __global__ void __launch_bounds__(kMaxThreads) core64_kernel(const __grid_consta
   for (int64_t st = st0; st < st1; ++st) {
     const int64_t r0 = st << P.log_rows;
     const int rows = static_cast<int>(min(static_cast<int64_t>(R), P.nrows - r0));
-    const int lc = P.log_rows - 5, nitems = p << lc;  // items: 32 rows of a column
+    const int ng = (R + 127) / 128, nitems = p * ng;  // items: 128 rows of a column, fewer in a shorter stage
     __syncthreads();  // the last stage's rows have been read
-    for (int i0 = warp; i0 < nitems; i0 += kBatch * nwarps) {
-      uint64_t v[kBatch];
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        const int it = i0 + u * nwarps, c = it >> lc, k = ((it & ((1 << lc) - 1)) << 5) + lane;
-        v[u] = 0;
-        if (it < nitems && k < rows) v[u] = load_bits(P.cols[c], P.dtype[c], r0 + k);
-      }
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        const int it = i0 + u * nwarps, c = it >> lc, k = ((it & ((1 << lc) - 1)) << 5) + lane;
-        if (it < nitems) {
-          double x = to_f64(v[u], P.dtype[c]);
-          if (P.shift) x -= P.shift[c];
-          X[k * S + c] = x;
-        }
+    for (int it = warp; it < nitems; it += nwarps) {
+      const int c = it / ng, k = (it - c * ng) * 128, nch = min(R - k, 128) / 32;
+      const void* col = P.cols[c];
+      const double sh = P.shift ? P.shift[c] : 0.0;
+      double* dst = X + k * S + c;
+      switch (P.dtype[c]) {
+        case I16: convert_rows<I16>(col, r0 + k, rows - k, nch, P.shift, sh, dst, S); break;
+        case I32: convert_rows<I32>(col, r0 + k, rows - k, nch, P.shift, sh, dst, S); break;
+        case I64: convert_rows<I64>(col, r0 + k, rows - k, nch, P.shift, sh, dst, S); break;
+        case F32: convert_rows<F32>(col, r0 + k, rows - k, nch, P.shift, sh, dst, S); break;
+        default: convert_rows<F64>(col, r0 + k, rows - k, nch, P.shift, sh, dst, S); break;
       }
     }
     __syncthreads();
@@ -219,10 +223,10 @@ cudaError_t core64_plan(int p, int64_t nrows, bool shifted, int sms, int blocks,
       for (int G = G0; G <= G0 + 8; ++G) {
         const int tg = (M + G - 1) / G, ks = nt / tg;
         if (tg * (G - 1) >= M) continue;
-        // FP64 warp instructions a row costs one of the SM's four schedulers: the tiles' FMAs, the
-        // shift in every group, the column sums in one
+        // FP64 warp instructions a row costs one of the SM's four schedulers: the tiles' FMAs, in every
+        // group the shift and (a quarter of one a value) loading and converting, the column sums in one
         const double fmas = ((tg * ks + 31) / 32 + 3) / 4 * double(micro * micro) / ks;
-        const double cost = G * (fmas + (shifted ? p / 128.0 : 0.0)) + double(nt) / (nt / p * p) * p / 128.0;
+        const double cost = G * (fmas + (shifted ? 1.25 : 0.25) * p / 128.0) + double(nt) / (nt / p * p) * p / 128.0;
         if (best == 0 || cost < best) {
           best = cost;
           P.micro = micro;

@@ -85,7 +85,7 @@ __device__ __forceinline__ void gen_row(const T1Lut& L, uint64_t seed, uint64_t 
 
 template <bool L16>
 __global__ void __launch_bounds__(256) gen_table1_kernel(uint64_t seed, uint64_t row0, int64_t nrows,
-                                                         Fp64Params cols) {
+                                                         TableColumns cols) {
   __shared__ T1Lut L;
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(&g_t1lut);
@@ -164,7 +164,7 @@ cudaError_t launch_gen_table1(uint64_t seed, uint64_t row0, int64_t nrows, int l
   if (nrows <= 0) return cudaSuccess;
   cudaError_t e = t1_upload_lut();
   if (e != cudaSuccess) return e;
-  Fp64Params P{};
+  TableColumns P{};
   for (int j = 0; j < 12; ++j) P.cols[j] = cols[j];
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);

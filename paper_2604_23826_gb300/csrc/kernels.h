@@ -82,23 +82,16 @@ cudaError_t launch_exact(const ExactParams& P, int conv, int max_grid, cudaStrea
 int exact_max_active_blocks(int conv, int shape, int stages, int stage_bytes);
 
 // ---------------------------------------------------------------------------
-// FP64 CUDA-core passes (raw or shifted), fixed-order merge of block slots.
+// A table's columns as small kernels take them: the Table 1 generator, and the pivot of the shifted
+// modes, the mean of the first rows (k_pivot.cu).
 // ---------------------------------------------------------------------------
-struct Fp64Params {
-  const void* cols[256];
+struct TableColumns {
+  void* cols[256];
   int32_t dtype[256];
   int32_t p;
   int64_t nrows;
-  const double* shift;  // p values or nullptr (raw moments)
-  double* slots;        // scratch: grid * (T(p) + p) doubles
-  double* acc_s;        // ctx: p doubles (column sums, shifted when shift != nullptr)
-  double* acc_S;        // ctx: T(p) doubles, packed upper
-  double* acc_s_lo;     // ctx: p low parts (double-double)
-  double* acc_S_lo;     // ctx: T(p) low parts
-  long long* acc_n;     // ctx: row count
+  double* shift;  // p pivots
 };
-cudaError_t launch_fp64(const Fp64Params& P, int grid, cudaStream_t stream);
-size_t fp64_slot_doubles(int grid);  // slots + ticket word, zeroed once at allocation
 cudaError_t launch_set_shift(const void* const* cols, const int32_t* dtypes, int p, int64_t rows, double* shift,
                              cudaStream_t stream);
 

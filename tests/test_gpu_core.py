@@ -79,7 +79,7 @@ def test_fp32_core_column_types(offset):
 
 
 @pytest.mark.parametrize("n", [1, 33, 4_099, 40_003])
-@pytest.mark.parametrize("p", [13, 16, 31, 48, 65, 127, 128, 200, 256])
+@pytest.mark.parametrize("p", [1, 2, 3, 8, 12, 13, 16, 31, 48, 65, 127, 128, 200, 256])
 @pytest.mark.parametrize("mode", [G.STATS_FP64, G.STATS_FP64_SHIFTED])
 def test_fp64_core_widths_and_rows(mode, p, n):
     check([G.STATS_F64] * p, n, mode, 7 * p + n)
@@ -92,4 +92,5 @@ def test_fp64_core_calls_and_grids(p, parts, grid):
 
 @pytest.mark.parametrize("mode", [G.STATS_FP64, G.STATS_FP64_SHIFTED])
 def test_fp64_core_column_types(mode):
-    check([G.STATS_I16, G.STATS_F32, G.STATS_I32, G.STATS_F64, G.STATS_I64] * 3, 5_001, mode, 4, 1)
+    for k in (1, 2, 3):
+        check([G.STATS_I16, G.STATS_F32, G.STATS_I32, G.STATS_F64, G.STATS_I64] * k, 5_001, mode, 4, 1)
