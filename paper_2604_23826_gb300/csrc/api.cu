@@ -1506,7 +1506,7 @@ stats_status stats_accumulate_csv(stats_ctx* ctx, const char* path, int64_t skip
     CK(ctx, cudaMemsetAsync(S.status, 0, sizeof(uint32_t), st));
     CK(ctx, cudaMemsetAsync(S.bad, 0xFF, sizeof(unsigned long long), st));
     CK(ctx, launch_csv_lines(d_text[b], nb, S, st));
-    CK(ctx, launch_csv_parse(d_text[b], S, k, row_cap, ctx->sms, st));
+    CK(ctx, launch_csv_parse(d_text[b], nb, S, k, row_cap, ctx->sms, st));
     CK(ctx, cudaMemcpyAsync(&out->total, S.total, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     CK(ctx, cudaMemcpyAsync(&out->status, S.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     CK(ctx, cudaMemcpyAsync(&out->bad, S.bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));

@@ -4,14 +4,19 @@
 // the GPUs; "Data Representation and Sufficient Statistics": text parsing dominated, so
 // the table was converted to binary).
 //
-// Device parse of a text buffer, three launches and one small one:
-//   csv_count_kernel   newlines per 4 KB tile (16 bytes per thread, byte compares);
+// Device parse of a text buffer, four launches:
+//   csv_count_kernel   newlines per 4 KB tile, a warp each (eight 16-byte loads a lane in flight,
+//                      four bytes compared at a time);
 //   csv_scan_kernel    one block: exclusive prefix of the tile counts, the line count
 //                      (plus one for a last line without '\n');
 //   csv_index_kernel   each tile again: the offsets of its newlines, in order;
 //   csv_parse_kernel   one thread per line: the first k fields, converted and stored in
 //                      column j at the line's row (adjacent lines -> adjacent rows, so
 //                      the stores of a warp are contiguous).
+// Bound: instruction issue in the parse.  Fields are taken eight characters at a time: one
+// comparison finds the digits' end, three multiplications give their value; a character loop takes
+// the rest (exponents, more than 19 digits) and every error.  1.5e6 lines of Table 1 (115 MB):
+// parse 353 us a character at a time, 184 now; counting, scanning and indexing 142 us, 68 now.
 // Number conversion is exact.  A real field is M * 10^E with M < 10^19 (the significant
 // digits as an integer, trailing zeros moved into E) and -38 <= E <= 19.  For E >= 0 the product M * 10^E is formed in
 // 128-bit integers; for E < 0 the quotient M * 2^s / 10^-E (a 64-bit quotient and a sticky
@@ -40,110 +45,141 @@ namespace ss {
 
 namespace {
 
-constexpr int kCsvThreads = 256;  // x 16 bytes = one tile
-static_assert(kCsvThreads * 16 == kCsvTile, "a tile is 16 bytes per thread");
+constexpr int kCsvThreads = 256;  // a warp per tile in the counting and indexing kernels
 
-__device__ __forceinline__ int nl_count16(const char* t, int64_t pos, int64_t n, bool aligned) {
-  if (aligned && pos + 16 <= n) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(t + pos));
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    int c = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) c += ((w[i] >> (8 * b)) & 0xFFu) == '\n';
-    return c;
-  }
-  int c = 0;
-  for (int64_t i = pos; i < pos + 16 && i < n; ++i) c += t[i] == '\n';
-  return c;
-}
+// One warp per tile: lane l holds bytes 16 l .. 16 l + 15 of each of its kChunks 512-byte chunks.
+constexpr int kChunks = kCsvTile / 512;
 
-__device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int& total) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int x = v;
+// newlines of a lane's 16 bytes of every chunk, a bit per byte; all loads in flight at once
+__device__ __forceinline__ void newline_masks(const char* __restrict__ t, int64_t n, int64_t tile, bool aligned,
+                                              uint32_t (&mask)[kChunks]) {
+  const int64_t p0 = tile * kCsvTile + (threadIdx.x & 31) * 16;
+  if (aligned && (tile + 1) * kCsvTile <= n) {
+    uint4 v[kChunks];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_warp[wid] = x;
-  __syncthreads();
-  if (wid == 0) {
-    int w = lane < static_cast<int>(blockDim.x >> 5) ? s_warp[lane] : 0;
+    for (int c = 0; c < kChunks; ++c) v[c] = __ldg(reinterpret_cast<const uint4*>(t + p0 + c * 512));
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
+    for (int c = 0; c < kChunks; ++c) {
+      const uint32_t w[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
+      mask[c] = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t hit = __vcmpeq4(w[i], 0x0A0A0A0Au) & 0x01010101u;  // a 1 in each newline's byte
+        mask[c] |= ((hit * 0x10204080u) >> 28) << (4 * i);                // gathered into four bits
+      }
     }
-    if (lane < static_cast<int>(blockDim.x >> 5)) s_warp[lane] = w;
+    return;
   }
-  __syncthreads();
-  total = s_warp[(blockDim.x >> 5) - 1];
-  const int before = (wid > 0 ? s_warp[wid - 1] : 0) + x - v;
-  __syncthreads();
-  return before;
+#pragma unroll
+  for (int c = 0; c < kChunks; ++c) {
+    mask[c] = 0;
+    for (int i = 0; i < 16; ++i) {
+      const int64_t p = p0 + c * 512 + i;
+      if (p < n && t[p] == '\n') mask[c] |= 1u << i;
+    }
+  }
 }
 
-__global__ void __launch_bounds__(kCsvThreads) csv_count_kernel(const char* __restrict__ t, int64_t n,
+__global__ void __launch_bounds__(kCsvThreads) csv_count_kernel(const char* __restrict__ t, int64_t n, int64_t ntiles,
                                                                uint32_t* __restrict__ counts) {
-  __shared__ int s_warp[32];
   const bool aligned = (reinterpret_cast<uintptr_t>(t) & 15u) == 0;
-  const int64_t pos = static_cast<int64_t>(blockIdx.x) * kCsvTile + threadIdx.x * 16;
-  int total = 0;
-  block_exclusive_scan(nl_count16(t, pos, n, aligned), s_warp, total);
-  if (threadIdx.x == 0) counts[blockIdx.x] = static_cast<uint32_t>(total);
+  const int64_t tile = blockIdx.x * static_cast<int64_t>(kCsvThreads / 32) + (threadIdx.x >> 5);
+  if (tile >= ntiles) return;
+  uint32_t mask[kChunks];
+  newline_masks(t, n, tile, aligned, mask);
+  int c = 0;
+#pragma unroll
+  for (int i = 0; i < kChunks; ++i) c += __popc(mask[i]);
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31) == 0) counts[tile] = static_cast<uint32_t>(c);
 }
 
-// one block of 1024 threads; offs[i] = newlines before tile i; *total = lines
+// one block of 1024 threads, 4096 tiles a step; offs[i] = newlines before tile i; *total = lines
 __global__ void __launch_bounds__(1024) csv_scan_kernel(const char* __restrict__ t, int64_t n,
                                                        const uint32_t* __restrict__ counts, int64_t ntiles,
                                                        int64_t* __restrict__ offs, int64_t* __restrict__ ends,
                                                        int64_t ends_cap, int64_t* __restrict__ total) {
-  __shared__ long long s_part[1024];
-  const int tid = threadIdx.x;
-  const int64_t per = (ntiles + 1023) / 1024;
-  const int64_t t0 = tid * per, t1 = min(ntiles, t0 + per);
-  long long sum = 0;
-  for (int64_t i = t0; i < t1; ++i) sum += counts[i];
-  s_part[tid] = sum;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {  // inclusive scan (Hillis-Steele)
-    const long long y = tid >= o ? s_part[tid - o] : 0;
+  __shared__ uint32_t s_warp[2][32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int64_t before = 0;
+  int buf = 0;
+  for (int64_t i0 = 0; i0 < ntiles; i0 += 4096, buf ^= 1) {
+    const int64_t i = i0 + 4 * tid;
+    uint4 c = make_uint4(0, 0, 0, 0);
+    if (i + 4 <= ntiles) {
+      c = *reinterpret_cast<const uint4*>(counts + i);
+    } else {
+      if (i < ntiles) c.x = counts[i];
+      if (i + 1 < ntiles) c.y = counts[i + 1];
+      if (i + 2 < ntiles) c.z = counts[i + 2];
+    }
+    const uint32_t own = c.x + c.y + c.z + c.w;  // 4096 tiles hold at most 2^24 newlines
+    uint32_t x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[buf][warp] = x;
     __syncthreads();
-    s_part[tid] += y;
-    __syncthreads();
-  }
-  long long run = s_part[tid] - sum;
-  for (int64_t i = t0; i < t1; ++i) {
-    offs[i] = run;
-    run += counts[i];
+    uint32_t w = s_warp[buf][lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    const uint32_t ahead = __shfl_sync(0xffffffffu, w, (warp + 31) & 31), all = __shfl_sync(0xffffffffu, w, 31);
+    int64_t run = before + (warp ? ahead : 0) + (x - own);
+    const uint32_t cs[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + u < ntiles) {
+        offs[i + u] = run;
+        run += cs[u];
+      }
+    before += all;
   }
   if (tid == 0) {
-    const long long nl = s_part[1023];
-    long long lines = nl;
+    int64_t lines = before;
     if (n > 0 && t[n - 1] != '\n') {  // a last line without its newline ends at the text's end
-      if (nl < ends_cap) ends[nl] = n;
+      if (lines < ends_cap) ends[lines] = n;
       ++lines;
     }
     *total = lines;
   }
 }
 
-__global__ void __launch_bounds__(kCsvThreads) csv_index_kernel(const char* __restrict__ t, int64_t n,
+__global__ void __launch_bounds__(kCsvThreads) csv_index_kernel(const char* __restrict__ t, int64_t n, int64_t ntiles,
                                                                const int64_t* __restrict__ offs,
                                                                int64_t* __restrict__ ends, int64_t ends_cap) {
-  __shared__ int s_warp[32];
   const bool aligned = (reinterpret_cast<uintptr_t>(t) & 15u) == 0;
-  const int64_t pos = static_cast<int64_t>(blockIdx.x) * kCsvTile + threadIdx.x * 16;
-  int total = 0;
-  const int before = block_exclusive_scan(nl_count16(t, pos, n, aligned), s_warp, total);
-  int64_t line = offs[blockIdx.x] + before;
-  for (int64_t i = pos; i < pos + 16 && i < n; ++i)
-    if (t[i] == '\n') {
-      if (line < ends_cap) ends[line] = i;
-      ++line;
+  const int lane = threadIdx.x & 31;
+  const int64_t tile = blockIdx.x * static_cast<int64_t>(kCsvThreads / 32) + (threadIdx.x >> 5);
+  if (tile >= ntiles) return;
+  uint32_t mask[kChunks];
+  newline_masks(t, n, tile, aligned, mask);
+  int64_t line = offs[tile];
+  // two chunks' counts (at most 512 each) to a scan
+#pragma unroll
+  for (int c = 0; c < kChunks; c += 2) {
+    const uint32_t own = static_cast<uint32_t>(__popc(mask[c])) | static_cast<uint32_t>(__popc(mask[c + 1])) << 16;
+    uint32_t x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
+    const uint32_t all = __shfl_sync(0xffffffffu, x, 31);
+    x -= own;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      int64_t at = line + (u ? (all & 0xFFFFu) + (x >> 16) : (x & 0xFFFFu));
+      const int64_t p = tile * kCsvTile + (c + u) * 512 + lane * 16;
+      for (uint32_t m = mask[c + u]; m; m &= m - 1, ++at)
+        if (at < ends_cap) ends[at] = p + __ffs(static_cast<int>(m)) - 1;
+    }
+    line += (all & 0xFFFFu) + (all >> 16);
+  }
 }
 
 // ------------------------------- exact decimal -> binary -------------------------------
@@ -428,11 +464,116 @@ __device__ int64_t parse_field(const char* t, int64_t p, int64_t e, int32_t dt, 
   return p;
 }
 
+// ------------------------------- eight characters at a time -------------------------------
+// The eight bytes at p (the first in the lowest byte).  Two aligned words where both lie inside the
+// text; next to its ends byte by byte, with zeros past it.
+__device__ __forceinline__ uint64_t load8(const char* t, int64_t p, int64_t n) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(t + p);
+  const int sh = static_cast<int>(a & 7u);
+  if (p >= sh && p - sh + 16 <= n) {
+    const uint64_t* w = reinterpret_cast<const uint64_t*>(a - sh);
+    const uint64_t lo = __ldg(w);
+    if (sh == 0) return lo;
+    return lo >> (8 * sh) | __ldg(w + 1) << (64 - 8 * sh);
+  }
+  uint64_t v = 0;
+  for (int i = 0; i < 8; ++i)
+    if (p + i < n) v |= static_cast<uint64_t>(static_cast<unsigned char>(t[p + i])) << (8 * i);
+  return v;
+}
+
+// how many of the eight characters, from the first on, are digits; d: the bytes XOR '0'
+__device__ __forceinline__ int leading_digits(uint64_t d) {
+  const uint64_t other = (((d & 0x7F7F7F7F7F7F7F7Full) + 0x7676767676767676ull) | d) & 0x8080808080808080ull;
+  return other ? (__ffsll(static_cast<long long>(other)) - 1) >> 3 : 8;
+}
+// value of the first nd (1..8) digits: moved to the high bytes, then digits, pairs and fours joined
+__device__ __forceinline__ uint32_t digits_value(uint64_t d, int nd) {
+  uint64_t v = d << (64 - 8 * nd);
+  v = (v * 2561u >> 8) & 0x00FF00FF00FF00FFull;
+  v = (v * 6553601u >> 16) & 0x0000FFFF0000FFFFull;
+  return static_cast<uint32_t>(v * 42949672960001ull >> 32);
+}
+
+// A run of digits from p on into v (at most 19 of them kept count of; more overflow v, and the
+// caller refuses them).  Returns their number.
+__device__ __forceinline__ int digit_run(const char* t, int64_t p, int64_t n, const CsvTables& T, uint64_t& v,
+                                         uint64_t& next) {
+  int total = 0;
+  for (;;) {
+    const uint64_t w = load8(t, p + total, n), d = w ^ 0x3030303030303030ull;
+    const int nd = leading_digits(d);
+    if (nd) v = v * T.p10[nd] + digits_value(d, nd);
+    total += nd;
+    if (nd < 8) {
+      next = w >> (8 * nd);  // the characters that follow the run, the first in the low byte
+      return total;
+    }
+    if (total > 2 * STATS_CSV_MAX_DIGITS) return total;
+  }
+}
+
+// parse_field for the forms nearly all fields have -- an integer of at most 19 digits; a real of
+// digits and a point whose significant digits are at most 19 -- with the same result.  Anything
+// else (an exponent, more digits, a stray character) goes to parse_field from its start, which also
+// gives the error.
+__device__ __forceinline__ int64_t parse_field_fast(const char* t, int64_t n, int64_t p, int64_t e, int32_t dt, void* dst,
+                                                    uint32_t& status, const CsvTables& T) {
+  const int64_t start = p;
+  const char c = p < e ? t[p] : ',';
+  const bool neg = c == '-';
+  if (neg || c == '+') ++p;
+  uint64_t v = 0, next = 0;
+  int nd = digit_run(t, p, n, T, v, next);
+  p += nd;
+  if (dt == STATS_I16 || dt == STATS_I32 || dt == STATS_I64) {
+    const bool ends = p == e || (p < e && (next & 0xFF) == ',');
+    const uint64_t lim = dt == STATS_I16 ? 32767u : dt == STATS_I32 ? 2147483647u : 9223372036854775807ull;
+    if (nd == 0 || nd > STATS_CSV_MAX_DIGITS || !ends || v > lim + (neg ? 1u : 0u))
+      return parse_field(t, start, e, dt, dst, status, T);
+    const int64_t x = static_cast<int64_t>(neg ? 0 - v : v);
+    if (dt == STATS_I16)
+      *static_cast<int16_t*>(dst) = static_cast<int16_t>(x);
+    else if (dt == STATS_I32)
+      *static_cast<int32_t*>(dst) = static_cast<int32_t>(x);
+    else
+      *static_cast<int64_t*>(dst) = x;
+    return p;
+  }
+  int E = 0, sig = v ? nd : 0;  // digits that v may hold, leading zeros of the integer part left out
+  bool plain = nd > 0 && nd <= STATS_CSV_MAX_DIGITS;
+  if (p < e && (next & 0xFF) == '.') {
+    ++p;
+    const int nf = digit_run(t, p, n, T, v, next);
+    p += nf;
+    E = -nf;
+    sig += nf;
+    nd += nf;
+  }
+  plain = plain && sig <= STATS_CSV_MAX_DIGITS && (p == e || (p < e && (next & 0xFF) == ','));
+  if (!plain) return parse_field(t, start, e, dt, dst, status, T);
+  const bool f64 = dt == STATS_F64;
+  uint64_t bits = neg ? (f64 ? (uint64_t(1) << 63) : (uint64_t(1) << 31)) : 0;
+  if (v) {
+    uint32_t st = 0;
+    bits = decimal_to_bits(v, E, f64 ? 53 : 24, neg, st, T);
+    if (st) {
+      status |= st;
+      return -1;
+    }
+  }
+  if (f64)
+    *static_cast<uint64_t*>(dst) = bits;
+  else
+    *static_cast<uint32_t*>(dst) = static_cast<uint32_t>(bits);
+  return p;
+}
+
 __device__ __forceinline__ int dtype_size(int32_t dt) {
   return dt == STATS_I16 ? 2 : (dt == STATS_I32 || dt == STATS_F32) ? 4 : 8;
 }
 
-__global__ void __launch_bounds__(256) csv_parse_kernel(const char* __restrict__ t, CsvScratch S, int k,
+__global__ void __launch_bounds__(256) csv_parse_kernel(const char* __restrict__ t, int64_t nbytes, CsvScratch S, int k,
                                                        int64_t row_cap, const __grid_constant__ CsvTables TP) {
   __shared__ CsvTables T;
   for (int i = threadIdx.x; i < static_cast<int>(sizeof(CsvTables) / 8); i += blockDim.x)
@@ -451,7 +592,7 @@ __global__ void __launch_bounds__(256) csv_parse_kernel(const char* __restrict__
       uint64_t scratch;
       void* dst = store ? static_cast<void*>(static_cast<char*>(S.cols[j]) + row * dtype_size(dt))
                         : static_cast<void*>(&scratch);
-      const int64_t f = parse_field(t, p, e, dt, dst, status, T);
+      const int64_t f = parse_field_fast(t, nbytes, p, e, dt, dst, status, T);
       if (f < 0) break;
       if (j + 1 < k) {
         if (f >= e) {  // fewer than k fields
@@ -503,19 +644,19 @@ cudaError_t launch_csv_lines(const char* d_text, int64_t nbytes, const CsvScratc
   const int64_t ntiles = (nbytes + kCsvTile - 1) / kCsvTile;
   if (ntiles == 0) return cudaMemsetAsync(s.total, 0, sizeof(int64_t), st);
   if (ntiles > 0x7fffffff) return cudaErrorInvalidValue;
-  csv_count_kernel<<<static_cast<unsigned>(ntiles), kCsvThreads, 0, st>>>(d_text, nbytes, s.counts);
+  const unsigned blocks = static_cast<unsigned>((ntiles + kCsvThreads / 32 - 1) / (kCsvThreads / 32));
+  csv_count_kernel<<<blocks, kCsvThreads, 0, st>>>(d_text, nbytes, ntiles, s.counts);
   csv_scan_kernel<<<1, 1024, 0, st>>>(d_text, nbytes, s.counts, ntiles, s.offs, s.ends, s.ends_cap, s.total);
-  csv_index_kernel<<<static_cast<unsigned>(ntiles), kCsvThreads, 0, st>>>(d_text, nbytes, s.offs, s.ends,
-                                                                        s.ends_cap);
+  csv_index_kernel<<<blocks, kCsvThreads, 0, st>>>(d_text, nbytes, ntiles, s.offs, s.ends, s.ends_cap);
   return cudaGetLastError();
 }
 
-cudaError_t launch_csv_parse(const char* d_text, const CsvScratch& s, int k, int64_t row_cap, int sms,
+cudaError_t launch_csv_parse(const char* d_text, int64_t nbytes, const CsvScratch& s, int k, int64_t row_cap, int sms,
                              cudaStream_t st) {
   const int64_t want = (s.ends_cap + 255) / 256;
   const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(sms) * 8)));
   static const CsvTables tables = make_csv_tables();
-  csv_parse_kernel<<<grid, 256, 0, st>>>(d_text, s, k, row_cap, tables);
+  csv_parse_kernel<<<grid, 256, 0, st>>>(d_text, nbytes, s, k, row_cap, tables);
   return cudaGetLastError();
 }
 
@@ -737,7 +878,7 @@ stats_status stats_csv_parse(const char* d_text, int64_t nbytes, int32_t k, cons
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e == cudaSuccess && out.total > max_rows) res = STATS_EINVAL;
   if (e == cudaSuccess && res == STATS_OK) {
-    e = launch_csv_parse(d_text, S, k, max_rows, sms, st);
+    e = launch_csv_parse(d_text, nbytes, S, k, max_rows, sms, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out.status, S.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out.bad, S.bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -443,7 +443,7 @@ void csv_scratch_carve(void* base, int64_t nbytes, int64_t ends_cap, int k, CsvS
 cudaError_t launch_csv_lines(const char* d_text, int64_t nbytes, const CsvScratch& s, cudaStream_t st);
 // Parses the first k fields of lines [0, min(*total, ends_cap)) into s.cols (rows below
 // row_cap are stored; every line is checked); status and bad must be reset before.
-cudaError_t launch_csv_parse(const char* d_text, const CsvScratch& s, int k, int64_t row_cap, int sms,
+cudaError_t launch_csv_parse(const char* d_text, int64_t nbytes, const CsvScratch& s, int k, int64_t row_cap, int sms,
                              cudaStream_t st);
 
 // ---------------------------------------------------------------------------
