@@ -33,6 +33,7 @@
 // the default.  All waits are bounded; an expired wait marks the call failed (the
 // accumulator is then left unchanged).
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -120,6 +121,7 @@ __device__ __forceinline__ uint64_t fixed_f2i(double x, int sh) {
 // The field checks below are exactly the ranges those digit fields can carry.
 template <bool L16>
 struct ConvT1 {
+  static constexpr bool kPair = false;
   template <int TILE>
   __device__ __forceinline__ static SmemT1Src<L16, TILE> smem_src(const uint8_t* st, const ExactParams&, int r) {
     return SmemT1Src<L16, TILE>{st, r};
@@ -174,80 +176,113 @@ struct ConvT1 {
 // once, biased to an unsigned field (a signed field's top byte XOR 0x80 is the value plus
 // 2^(8k-1)) and appended to a 64-bit register; every eight bytes that fill it leave as four f16
 // pairs, whose bias takes a signed top byte's 128 off again.  The column loop is uniform across
-// the warp, so its branches cost one instruction each.  (Bound: instruction issue, as for Table 1.
+// the warp, so its branches cost one instruction each, and two rows of a lane share it.  (Bound: instruction issue, as for Table 1.
 // Eight mixed columns, 36 B a row, 2e7 rows: extracting every digit from its column anew took
-// 2.50 ms, this way 0.71 ms.)
+// 2.50 ms, this way 0.56 ms; 0.71 with one row a lane.)
 struct ConvGeneric {
   template <int TILE>
   __device__ __forceinline__ static SmemSrc smem_src(const uint8_t* st, const ExactParams& P, int r) {
     return SmemSrc{st, &P, r};
   }
-  // q = round(x * 2^sh) as a field of 56 bits, biased when signed; range violations into bad
-  __device__ __forceinline__ static uint64_t real_field(const ExactParams& P, double x, int j, uint32_t& bad) {
+  static constexpr bool kPair = true;  // two rows per lane share the walk over the columns
+  // q = round(x * 2^sh); range violations into bad
+  __device__ __forceinline__ static uint64_t real_field(double x, int sh, int emax, bool is_signed, uint32_t& bad) {
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
-    const int ef = static_cast<int>((hi >> 20) & 0x7FFu), sh = P.real_shift[j];
-    bad |= ef > P.real_emax[j];
-    if (!P.is_signed[j]) bad |= (hi >> 31) & (((hi << 1) | lo) != 0);  // negative, not -0
+    const int ef = static_cast<int>((hi >> 20) & 0x7FFu);
+    bad |= ef > emax;
+    if (!is_signed) bad |= (hi >> 31) & (((hi << 1) | lo) != 0);  // negative, not -0
     // the scaling is an exponent-field add, the rounding one conversion on the FP64 unit; a scaled
     // value below the normal range rounds to 0, a subnormal input is scaled by integers
-    uint64_t q;
-    if (ef == 0)
-      q = ((hi << 1) | lo) ? fixed_rn<true>(x, sh) : 0;
-    else
-      q = ef + sh > 0 ? static_cast<uint64_t>(__double2ll_rn(__hiloint2double(
-                            static_cast<int>(hi + (static_cast<uint32_t>(sh) << 20)), static_cast<int>(lo))))
-                      : 0;
-    return q;
+    if (ef == 0) return ((hi << 1) | lo) ? fixed_rn<true>(x, sh) : 0;
+    return ef + sh > 0 ? static_cast<uint64_t>(__double2ll_rn(__hiloint2double(
+                             static_cast<int>(hi + (static_cast<uint32_t>(sh) << 20)), static_cast<int>(lo))))
+                       : 0;
   }
-  __device__ __forceinline__ static void emit(const ExactParams& P, uint64_t v, int e, uint32_t (&w)[16]) {
+  template <int N>
+  __device__ __forceinline__ static void emit(const ExactParams& P, const uint64_t (&v)[N], int e, uint32_t (&w)[N][16]) {
     constexpr uint32_t M = 0x64646464u;  // bytes of the f16 exponent 0x64
-    const uint32_t lo = static_cast<uint32_t>(v), hi = static_cast<uint32_t>(v >> 32);
-    const uint32_t d0 = half2_sub(__byte_perm(lo, M, 0x4140), P.bias[4 * e]);
-    const uint32_t d1 = half2_sub(__byte_perm(lo, M, 0x4342), P.bias[4 * e + 1]);
-    const uint32_t d2 = half2_sub(__byte_perm(hi, M, 0x4140), P.bias[4 * e + 2]);
-    const uint32_t d3 = half2_sub(__byte_perm(hi, M, 0x4342), P.bias[4 * e + 3]);
+    uint32_t d[N][4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (q == e) {
-        w[4 * q] = d0;
-        w[4 * q + 1] = d1;
-        w[4 * q + 2] = d2;
-        w[4 * q + 3] = d3;
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t b = P.bias[4 * e + q];
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const uint32_t x = static_cast<uint32_t>(q < 2 ? v[i] : v[i] >> 32);
+        d[i][q] = half2_sub(__byte_perm(x, M, q & 1 ? 0x4342 : 0x4140), b);
       }
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      if (f == e) {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) w[i][4 * f + q] = d[i][q];
+      }
+  }
+  // N rows of this lane at once
+  template <int N, class Src>
+  __device__ __forceinline__ static void rows(const ExactParams& P, const Src (&src)[N], uint32_t (&w)[N][16],
+                                              uint32_t (&bad)[N]) {
+    uint64_t acc[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = 1;  // the ones column's digit
+    int nb = 8, e = 0;
+#pragma unroll 1
+    for (int j = 0; j < P.p; ++j) {
+      const int dt = P.dtype[j], kb = 8 * P.kbytes[j];
+      uint64_t u[N];
+      if (dt == I16 || dt == I32) {
+        const uint32_t add = static_cast<uint32_t>(P.field_add[j]), chk = static_cast<uint32_t>(P.field_chk[j]);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const uint32_t t = static_cast<uint32_t>(dt == I16 ? src[i].i16(j) : src[i].i32(j)) + add;
+          bad[i] |= t & chk;
+          u[i] = t;
+        }
+      } else if (dt == I64) {
+        const uint64_t add = P.field_add[j], chk = P.field_chk[j];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          u[i] = static_cast<uint64_t>(src[i].i64(j)) + add;
+          bad[i] |= (u[i] & chk) != 0;
+        }
+      } else {
+        const int sh = P.real_shift[j], emax = P.real_emax[j];
+        const bool is_signed = P.is_signed[j];
+        const uint64_t add = P.field_add[j];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const double x = dt == F64 ? src[i].f64(j) : f32_to_f64(src[i].f32(j));
+          u[i] = (real_field(x, sh, emax, is_signed, bad[i]) + add) & ((uint64_t(1) << 56) - 1);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < N; ++i) acc[i] |= u[i] << nb;
+      nb += kb;
+      if (nb >= 64) {
+        emit<N>(P, acc, e++, w);
+        nb -= 64;
+        // the bytes of u that did not fit: u >> (kb - nb), none when the field ended at 64
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc[i] = nb ? u[i] >> (kb - nb) : 0;
+      }
+    }
+    for (; e < 4; ++e) {
+      emit<N>(P, acc, e, w);
+#pragma unroll
+      for (int i = 0; i < N; ++i) acc[i] = 0;
+    }
   }
   template <class Src>
   __device__ __forceinline__ static void row(const ExactParams& P, const Src& src, uint32_t (&w)[16],
                                              uint32_t& bad) {
-    uint64_t acc = 1;  // the ones column's digit
-    int nb = 8, e = 0;
-#pragma unroll 1
-    for (int j = 0; j < P.p; ++j) {
-      const int dt = P.dtype[j];
-      uint64_t u;
-      if (dt == I16 || dt == I32) {
-        const uint32_t t = static_cast<uint32_t>(dt == I16 ? src.i16(j) : src.i32(j)) + static_cast<uint32_t>(P.field_add[j]);
-        bad |= (t & static_cast<uint32_t>(P.field_chk[j])) != 0;
-        u = t;
-      } else if (dt == I64) {
-        u = static_cast<uint64_t>(src.i64(j)) + P.field_add[j];
-        bad |= (u & P.field_chk[j]) != 0;
-      } else {
-        const double x = dt == F64 ? src.f64(j) : f32_to_f64(src.f32(j));
-        u = (real_field(P, x, j, bad) + P.field_add[j]) & ((uint64_t(1) << 56) - 1);
-      }
-      acc |= u << nb;
-      nb += 8 * P.kbytes[j];
-      if (nb >= 64) {
-        emit(P, acc, e++, w);
-        nb -= 64;
-        // the bytes of u that did not fit: u >> (kbits - nb), none when the field ended at 64
-        acc = nb ? u >> (8 * P.kbytes[j] - nb) : 0;
-      }
-    }
-    for (; e < 4; ++e) {
-      emit(P, acc, e, w);
-      acc = 0;
-    }
+    const Src one[1] = {src};
+    uint32_t x[1][16], b[1] = {0};
+    rows<1>(P, one, x, b);
+    bad |= b[0];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) w[q] = x[0][q];
   }
 };
 
@@ -467,21 +502,8 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) exact_pass_kernel(const __gri
       }
       const int valid = static_cast<int>(min(static_cast<int64_t>(kTile), P.nmain - row0));
       const uint8_t* st = stage_base + s * P.stage_bytes;
-#pragma unroll 1
-      for (int h = 0; h < RPW / 32; ++h) {
-        const int r = warp * RPW + h * 32 + lane;
-        uint32_t w[16];
-        if (r < valid && P.direct) {
-          GlobalSrc src{&P, row0 + r};
-          Conv::row(P, src, w, bad);
-        } else if (r < valid) {
-          Conv::row(P, Conv::template smem_src<kTile>(st, P, r), w, bad);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 16; ++q) w[q] = 0u;
-        }
-        warp_mma_32rows(tile, lane, w, acc);
-        if (++sub == kFlushRows / 32) {
+      auto count = [&](int n) {  // n sub-steps of 32 rows done (n divides kFlushRows / 32)
+        if ((sub += n) == kFlushRows / 32) {
           sub = 0;
           if (i32_in_smem(W))
             flush_f32(acc, si, lane);
@@ -491,6 +513,51 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) exact_pass_kernel(const __gri
             flushes = 0;
             flush_i32(get_i32, cta_acc, lane);
           }
+        }
+      };
+      if constexpr (Conv::kPair && RPW == 64) {
+        // both rows of the lane; one past the end is read as the last row and left out
+        const int r0 = warp * RPW + lane, r1 = r0 + 32, c0 = min(r0, valid - 1), c1 = min(r1, valid - 1);
+        uint32_t w[2][16], b[2] = {0, 0};
+        if (P.direct) {
+          const GlobalSrc src[2] = {{&P, row0 + c0}, {&P, row0 + c1}};
+          Conv::template rows<2>(P, src, w, b);
+        } else {
+          const auto s0 = Conv::template smem_src<kTile>(st, P, c0), s1 = Conv::template smem_src<kTile>(st, P, c1);
+          const std::remove_const_t<decltype(s0)> src[2] = {s0, s1};
+          Conv::template rows<2>(P, src, w, b);
+        }
+        if (r0 >= valid) {
+#pragma unroll
+          for (int q = 0; q < 16; ++q) w[0][q] = 0u;
+        } else {
+          bad |= b[0] != 0;
+        }
+        if (r1 >= valid) {
+#pragma unroll
+          for (int q = 0; q < 16; ++q) w[1][q] = 0u;
+        } else {
+          bad |= b[1] != 0;
+        }
+        warp_mma_32rows(tile, lane, w[0], acc);
+        warp_mma_32rows(tile, lane, w[1], acc);
+        count(2);
+      } else {
+#pragma unroll 1
+        for (int h = 0; h < RPW / 32; ++h) {
+          const int r = warp * RPW + h * 32 + lane;
+          uint32_t w[16];
+          if (r < valid && P.direct) {
+            GlobalSrc src{&P, row0 + r};
+            Conv::row(P, src, w, bad);
+          } else if (r < valid) {
+            Conv::row(P, Conv::template smem_src<kTile>(st, P, r), w, bad);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) w[q] = 0u;
+          }
+          warp_mma_32rows(tile, lane, w, acc);
+          count(1);
         }
       }
       __syncwarp();
