@@ -32,6 +32,16 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
   return c;
 }
 
+// Pivot of an FP32 column: the mean of its first k rows (1 <= k), added in FP64 in a fixed tree over
+// the warp that calls it, rounded to FP32 (in every lane).
+__device__ __forceinline__ float pivot_mean(const float* col, int k) {
+  double sum = 0.0;
+  for (int i = threadIdx.x & 31; i < k; i += 32) sum += static_cast<double>(col[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return static_cast<float>(sum / k);
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier + bulk-copy (TMA, non-tensor) helpers.
 // ---------------------------------------------------------------------------

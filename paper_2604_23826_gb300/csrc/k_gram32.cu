@@ -552,52 +552,63 @@ __global__ void __launch_bounds__(G32<P>::THREADS, 1) gram32_kernel(const __grid
   }
 }
 
-// The tables' slots, in slot order, into their double-double accumulators: block
-// (t, part) takes every `parts`-th packed-upper entry and column sum of table t.
+// A table's slots into its context's accumulators.  Block (table, word): one word of the lanes'
+// accumulators (a quarter of a 16 x 8 tile, or eight columns' sums), so that a slot's 32 pairs are one
+// 256-byte read; eight warps take consecutive runs of the slots, added in order, then the runs in order
+// (a fixed grid reproduces its bits).  One thread per entry walking all slots took 93 us for 64 tables
+// of 32 columns.
 template <int P, bool X4>
-__global__ void __launch_bounds__(256) gram32_merge_kernel(const Gram32Table* __restrict__ tabs, int parts) {
+__global__ void __launch_bounds__(256) gram32_merge_kernel(const Gram32Table* __restrict__ tabs) {
   using C = G32<P>;
   constexpr int E = C::E, TILES = C::TILES, NJ = C::NJ;
-  const Gram32Table& T = tabs[blockIdx.x / parts];
-  const int part = blockIdx.x % parts;
-  const int p = T.p;
-  const int Tn = p * (p + 1) / 2;
-  const float2* slots = reinterpret_cast<const float2*>(T.slots);
-  for (int e = part * 256 + threadIdx.x; e < Tn + p; e += parts * 256) {
-    float h = 0.f, l = 0.f;
-    if (e < Tn) {
-      int j = 0, rm = e;
-      while (rm >= p - j) {
-        rm -= p - j;
-        ++j;
-      }
-      const int k2 = j + rm;
-      const int I = P >= 16 ? j / 16 : 0, J = k2 / 8;
-      int tix = 0;
-      for (int i = 0; i < I; ++i) tix += NJ - 2 * i;
-      tix += J - 2 * I;
-      const int lr = j - 16 * I, lc = k2 - 8 * J;
-      const int ln = (lr & 7) * 4 + (lc >> 1);
-      const int w = 4 * tix + 2 * (lr >> 3) + (lc & 1);
-      add_slots(slots, T.nslots, E * 32, w * 32 + ln, h, l);
-      if (!X4 && j == k2) {  // BF16x3: + the diagonal of L^T L
-        const int wq = 4 * TILES + C::NM + (j >> 3), gq = j & 7;
-        for (int tt = 0; tt < 4; ++tt) add_slots(slots, T.nslots, E * 32, wq * 32 + gq * 4 + tt, h, l);
-      }
-    } else {
-      const int c = e - Tn, m = c >> 3, gg = c & 7;
-      const int w = 4 * TILES + m;
-      for (int tt = 0; tt < 4; ++tt) add_slots(slots, T.nslots, E * 32, w * 32 + gg * 4 + tt, h, l);
+  __shared__ float2 part[8][32];
+  const Gram32Table& T = tabs[blockIdx.x];
+  const int w = blockIdx.y, lane = threadIdx.x & 31, seg = threadIdx.x >> 5, p = T.p;
+  const int v0 = T.nslots * seg / 8, n = T.nslots * (seg + 1) / 8 - v0;
+  const float2* slots = reinterpret_cast<const float2*>(T.slots) + static_cast<size_t>(v0) * E * 32;
+  int j = -1, k = -1;  // this lane's entry, or (j == k, sums) its column
+  const bool sums = w >= 4 * TILES;
+  if (!sums) {
+    int I = 0, J = w / 4;
+    while (J >= NJ - 2 * I) {
+      J -= NJ - 2 * I;
+      ++I;
     }
-    double* dh = e < Tn ? &T.acc_S[e] : &T.acc_s[e - Tn];
-    double* dl = e < Tn ? &T.acc_S_lo[e] : &T.acc_s_lo[e - Tn];
+    J += 2 * I;
+    j = 16 * I + (lane >> 2) + 8 * ((w & 3) >> 1);
+    k = 8 * J + 2 * (lane & 3) + (w & 1);
+    if (j > k || k >= p) j = -1;
+  } else {
+    j = k = 8 * (w - 4 * TILES) + (lane >> 2);  // four lanes' partial sums of a column
+    if (j >= p) j = -1;
+  }
+  float h = 0.f, l = 0.f;
+  if (j >= 0) {
+    add_slots(slots, n, E * 32, w * 32 + lane, h, l);
+    if (!X4 && !sums && j == k) {  // BF16x3: + the diagonal of L^T L
+      const int wq = 4 * TILES + C::NM + (j >> 3);
+      for (int tt = 0; tt < 4; ++tt) add_slots(slots, n, E * 32, wq * 32 + (j & 7) * 4 + tt, h, l);
+    }
+  }
+  part[seg][lane] = make_float2(h, l);
+  __syncthreads();
+  if (seg == 0 && j >= 0 && (!sums || (lane & 3) == 0)) {
+    h = l = 0.f;
+    for (int tt = 0; tt < (sums ? 4 : 1); ++tt)
+      for (int s = 0; s < 8; ++s) {
+        const float2 x = part[s][lane + tt];
+        two_sum(h, l, x.x);
+        two_sum(h, l, x.y);
+      }
+    const int idx = sums ? j : j * p - j * (j - 1) / 2 + (k - j);
+    double* dh = (sums ? T.acc_s : T.acc_S) + idx;
+    double* dl = (sums ? T.acc_s_lo : T.acc_S_lo) + idx;
     const double vv = static_cast<double>(h) + static_cast<double>(l);
-    const double sd = *dh + vv;
-    const double bp = sd - *dh;
-    *dl += (*dh - (sd - bp)) + (vv - bp);
+    const double hi = *dh, sd = hi + vv, bp = sd - hi;
+    *dl += (hi - (sd - bp)) + (vv - bp);
     *dh = sd;
   }
-  if (part == 0 && threadIdx.x == 0) *T.acc_n += T.nrows;
+  if (w == 0 && threadIdx.x == 0) *T.acc_n += T.nrows;
 }
 
 template <int P, bool X4>
@@ -608,23 +619,21 @@ cudaError_t launch_p(const Gram32Launch& L, int grid, cudaStream_t st) {
   gram32_kernel<P, X4><<<grid, G32<P>::THREADS, smem, st>>>(L);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // merge: entries of a table spread over `parts` blocks, at least ~2 blocks per SM in all
-  const int entries = P * (P + 1) / 2 + P;
-  const int parts = std::max(1, std::min((entries + 255) / 256, (2 * grid + L.ntables - 1) / L.ntables));
-  gram32_merge_kernel<P, X4><<<L.ntables * parts, 256, 0, st>>>(L.tabs, parts);
+  gram32_merge_kernel<P, X4><<<dim3(L.ntables, 4 * G32<P>::TILES + G32<P>::NM), 256, 0, st>>>(L.tabs);
   return cudaGetLastError();
 }
 
-// pivot c_j = the mean of the table's first kPivotRows rows (or all, if fewer), rounded to FP32
+// pivot c_j = the mean of the table's first kPivotRows rows (or all, if fewer), rounded to FP32: a warp
+// per column, its rows loaded at once (one thread loading them one by one took 8 us)
 __global__ void gram32_shift_kernel(const Gram32Table* __restrict__ tabs, const int* __restrict__ which) {
   const Gram32Table& T = tabs[which[blockIdx.x]];
   const int k = static_cast<int>(min(static_cast<int64_t>(kPivotRows), T.nrows));
-  for (int j = threadIdx.x; j < T.p; j += blockDim.x) {
-    double sum = 0.0;
-    for (int i = 0; i < k; ++i) sum += static_cast<double>(T.cols[j][i]);
-    const float v = static_cast<float>(sum / k);
-    const_cast<float*>(T.shift)[j] = v;
-    T.shift_d[j] = static_cast<double>(v);
+  for (int j = threadIdx.x >> 5; j < T.p; j += blockDim.x >> 5) {
+    const float v = pivot_mean(T.cols[j], k);
+    if ((threadIdx.x & 31) == 0) {
+      const_cast<float*>(T.shift)[j] = v;
+      T.shift_d[j] = static_cast<double>(v);
+    }
   }
 }
 
@@ -632,7 +641,7 @@ __global__ void gram32_shift_kernel(const Gram32Table* __restrict__ tabs, const 
 
 cudaError_t launch_gram32_shift(const Gram32Table* tabs, const int* which, int count, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
-  gram32_shift_kernel<<<count, 64, 0, st>>>(tabs, which);
+  gram32_shift_kernel<<<count, 1024, 0, st>>>(tabs, which);
   return cudaGetLastError();
 }
 

@@ -506,16 +506,17 @@ __global__ void __launch_bounds__(256) narrow_merge_kernel(const __grid_constant
   }
 }
 
-// pivot c_j = the mean of the table's first kPivotRows rows (or all, if fewer), rounded to FP32
+// pivot c_j = the mean of the table's first kPivotRows rows (or all, if fewer), rounded to FP32: a warp
+// per column
 __global__ void narrow_shift_kernel(const NarrowTab* __restrict__ tabs, const int* __restrict__ which) {
   const NarrowTab& T = tabs[which[blockIdx.x]];
   const int k = static_cast<int>(min(static_cast<int64_t>(kPivotRows), T.nrows));
-  for (int j = threadIdx.x; j < T.p; j += blockDim.x) {
-    double sum = 0.0;
-    for (int i = 0; i < k; ++i) sum += static_cast<double>(T.base[static_cast<int64_t>(j) * T.ld + i]);
-    const float v = static_cast<float>(sum / k);
-    T.shift[j] = v;
-    T.shift_d[j] = static_cast<double>(v);
+  for (int j = threadIdx.x >> 5; j < T.p; j += blockDim.x >> 5) {
+    const float v = pivot_mean(T.base + static_cast<int64_t>(j) * T.ld, k);
+    if ((threadIdx.x & 31) == 0) {
+      T.shift[j] = v;
+      T.shift_d[j] = static_cast<double>(v);
+    }
   }
 }
 
@@ -543,7 +544,7 @@ cudaError_t launch_narrow(const NarrowParams& P, bool x4, int grid, cudaStream_t
 
 cudaError_t launch_narrow_shift(const NarrowTab* tabs, const int* which, int count, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
-  narrow_shift_kernel<<<count, 64, 0, st>>>(tabs, which);
+  narrow_shift_kernel<<<count, 1024, 0, st>>>(tabs, which);
   return cudaGetLastError();
 }
 

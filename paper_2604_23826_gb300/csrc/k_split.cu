@@ -308,26 +308,26 @@ __global__ void __launch_bounds__(kThreads) split_batched_kernel(const SplitPara
 }
 
 // pivot c_j = the mean of the first min(rows, kPivotRows) rows of FP32 columns, rounded to FP32
-// (called once, rows >= 1)
-__device__ void split_pivot(const SplitParams& P, int64_t rows, double* shift_d) {
+// (called once, rows >= 1): a warp per column, from warp `first` on in steps of `step`
+__device__ void split_pivot(const SplitParams& P, int64_t rows, double* shift_d, int first, int step) {
   const int k = static_cast<int>(min(static_cast<int64_t>(kPivotRows), rows));
-  for (int j = threadIdx.x; j < P.p; j += blockDim.x) {
-    const float* col = P.col_ptrs ? P.col_ptrs[j] : P.cols[j];
-    double sum = 0.0;
-    for (int i = 0; i < k; ++i) sum += static_cast<double>(col[i]);
-    const float v = static_cast<float>(sum / k);
-    const_cast<float*>(P.shift)[j] = v;
-    shift_d[j] = static_cast<double>(v);
+  for (int j = first; j < P.p; j += step) {
+    const float v = pivot_mean(P.col_ptrs ? P.col_ptrs[j] : P.cols[j], k);
+    if ((threadIdx.x & 31) == 0) {
+      const_cast<float*>(P.shift)[j] = v;
+      shift_d[j] = static_cast<double>(v);
+    }
   }
 }
 
 __global__ void split_shift_kernel(const __grid_constant__ SplitParams P, int64_t rows, double* shift_d) {
-  split_pivot(P, rows, shift_d);
+  const int wpb = blockDim.x >> 5;
+  split_pivot(P, rows, shift_d, blockIdx.x * wpb + (threadIdx.x >> 5), gridDim.x * wpb);
 }
 
 __global__ void split_shift_batched_kernel(const SplitParams* __restrict__ tabs, const int* __restrict__ which) {
   const SplitParams& P = tabs[which[blockIdx.x]];
-  split_pivot(P, P.nrows, P.shift_d);
+  split_pivot(P, P.nrows, P.shift_d, threadIdx.x >> 5, blockDim.x >> 5);
 }
 
 }  // namespace
@@ -370,12 +370,12 @@ cudaError_t launch_split_batched(const SplitParams* tabs, const int2* units, int
 
 cudaError_t launch_split_shift_batched(const SplitParams* tabs, const int* which, int count, cudaStream_t stream) {
   if (count <= 0) return cudaSuccess;
-  split_shift_batched_kernel<<<count, 64, 0, stream>>>(tabs, which);
+  split_shift_batched_kernel<<<count, 1024, 0, stream>>>(tabs, which);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_shift(const SplitParams& P, int64_t rows, double* shift_d, cudaStream_t stream) {
-  split_shift_kernel<<<1, 256, 0, stream>>>(P, rows, shift_d);
+  split_shift_kernel<<<(P.p + 7) / 8, 256, 0, stream>>>(P, rows, shift_d);
   return cudaGetLastError();
 }
 
