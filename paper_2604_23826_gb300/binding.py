@@ -465,10 +465,11 @@ def stats_finalize_batched(ctxs: Sequence[Ctx], pca_on: int = 0) -> list:
     n = len(ctxs)
     outs = []
     for c in ctxs:
-        pa = stats_num_analysis_columns(c)
+        pa = L.stats_num_analysis_columns(c.handle)
         outs.append(Analysis(np.zeros(pa), np.zeros((pa, pa)), np.zeros((pa, pa)), np.zeros(pa), np.zeros((pa, pa))))
     handles = np.fromiter((c.handle.value for c in ctxs), dtype=np.uint64, count=n)
-    ptrs = [np.fromiter((getattr(a, f).ctypes.data for a in outs), dtype=np.uint64, count=n)
+    # (an array's ctypes attribute costs a few times its __array_interface__, and a batch asks 5 times a table)
+    ptrs = [np.fromiter((getattr(a, f).__array_interface__["data"][0] for a in outs), dtype=np.uint64, count=n)
             for f in ("mean", "cov", "corr", "evals", "evecs")]
     _check(L.stats_finalize_batched(handles.ctypes.data, n, pca_on, *[x.ctypes.data for x in ptrs]),
            "stats_finalize_batched")

@@ -10,6 +10,7 @@
 #include <sys/stat.h>
 
 #include <algorithm>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <thread>
@@ -287,13 +288,24 @@ stats_status check_sticky(const stats_ctx* c) {
   return c->sticky != STATS_OK ? STATS_ESTATE : STATS_OK;
 }
 
-stats_status device_status(stats_ctx* c) {
-  unsigned int bits = 0;
-  CK(c, cudaMemcpy(&bits, c->d_status, sizeof(bits), cudaMemcpyDeviceToHost));
+stats_status status_of_bits(unsigned int bits) {
   if (bits & DEV_ETIMEOUT) return STATS_ETIMEOUT;
   if (bits & DEV_ERANGE) return STATS_ERANGE;
   if (bits & DEV_EOVERFLOW) return STATS_EOVERFLOW;
   return STATS_OK;
+}
+
+stats_status device_status(stats_ctx* c) {
+  unsigned int bits = 0;
+  CK(c, cudaMemcpy(&bits, c->d_status, sizeof(bits), cudaMemcpyDeviceToHost));
+  return status_of_bits(bits);
+}
+
+// the status word a finalize kernel left in its flags
+stats_status recorded_status(const double* flags) {
+  uint64_t bits = 0;
+  memcpy(&bits, flags + 4, sizeof(bits));
+  return status_of_bits(static_cast<unsigned int>(bits));
 }
 
 // blocks of an exact pass
@@ -1013,6 +1025,7 @@ void build_final_params(const stats_ctx* c, int want_pca, int pca_on, FinalParam
                 : nullptr;
   F.out = c->d_out;
   F.work = c->d_work;
+  F.status = c->d_status;
 }
 
 // From this many analysis columns on, the eigen-solver runs over the whole GPU
@@ -1022,7 +1035,8 @@ constexpr int kGridJacobiMinColumns = 24;
 
 // Finalize on the ctx's stream.  With want_pca, the eigen-decomposition runs either in the
 // finalize kernel (small p_a) or in the grid-wide solver, seeded by `seed` (host, p_a x p_a,
-// rows = eigenvectors) when given.  Synchronises.
+// rows = eigenvectors) when given.  Synchronises, once: what earlier work recorded in the status word
+// and the row count come with the result (h_out), instead of a wait and a copy each before it.
 stats_status run_finalize(stats_ctx* c, int want_pca, int pca_on, const double* seed = nullptr) {
   FinalParams F;
   build_final_params(c, want_pca, pca_on, F);
@@ -1063,14 +1077,13 @@ stats_status run_finalize(stats_ctx* c, int want_pca, int pca_on, const double* 
   if (grid > 0) CK(c, launch_jacobi_grid(J, grid, st));
   CK(c, cudaMemcpyAsync(c->h_out, c->d_out, c->lay.total * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(c, cudaStreamSynchronize(st));
-  if (c->h_out[c->lay.flags + 5] != 0.0) return STATS_ETIMEOUT;
-  return STATS_OK;
+  if (c->copy_stream) CK(c, cudaStreamSynchronize(c->copy_stream));
+  return recorded_status(c->h_out + c->lay.flags);
 }
 
 void free_ctx(stats_ctx* c) {
   if (!c) return;
   cudaFree(c->d_g);
-  cudaFree(c->d_call);
   cudaFree(c->d_fs);
   cudaFree(c->d_fshift);
   cudaFree(c->d_core_slots);
@@ -1141,16 +1154,16 @@ stats_status create(stats_ctx** out, const stats_config* cfg) {
   cudaError_t e = cudaSuccess;
   const size_t T = static_cast<size_t>(c->p) * (c->p + 1) / 2;
   if (c->mode == STATS_EXACT) {
-    e = cudaMalloc(&c->d_g, kDigits * kDigits * sizeof(long long));
-    if (e == cudaSuccess) e = cudaMemset(c->d_g, 0, kDigits * kDigits * sizeof(long long));
-    // scratch: per-call accumulator, ticket, error word, status word
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_call, kDigits * kDigits * sizeof(unsigned long long) + 256);
-    if (e == cudaSuccess) e = cudaMemset(c->d_call, 0, kDigits * kDigits * sizeof(unsigned long long) + 256);
+    // accumulator, status word, then the scratch of a call: its accumulator, ticket and error word
+    const size_t g = kDigits * kDigits * sizeof(long long);
+    e = cudaMalloc(&c->d_g, 2 * g + 512);
+    if (e == cudaSuccess) e = cudaMemset(c->d_g, 0, 2 * g + 512);
     if (e == cudaSuccess) {
+      c->d_status = reinterpret_cast<unsigned int*>(c->d_g + kDigits * kDigits);
+      c->d_call = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(c->d_g) + g + 256);
       unsigned int* words = reinterpret_cast<unsigned int*>(c->d_call + kDigits * kDigits);
       c->d_ticket = words;
       c->d_err = words + 1;
-      c->d_status = words + 2;
       c->xp.call_acc = c->d_call;
       c->xp.ticket = c->d_ticket;
       c->xp.err = c->d_err;
@@ -1506,7 +1519,7 @@ stats_status stats_accumulate_csv(stats_ctx* ctx, const char* path, int64_t skip
     CK(ctx, cudaMemsetAsync(S.status, 0, sizeof(uint32_t), st));
     CK(ctx, cudaMemsetAsync(S.bad, 0xFF, sizeof(unsigned long long), st));
     CK(ctx, launch_csv_lines(d_text[b], nb, S, st));
-    CK(ctx, launch_csv_parse(d_text[b], nb, S, k, row_cap, ctx->sms, st));
+    CK(ctx, launch_csv_parse(d_text[b], nb, S, k, row_cap, INT64_MAX, ctx->sms, st));
     CK(ctx, cudaMemcpyAsync(&out->total, S.total, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     CK(ctx, cudaMemcpyAsync(&out->status, S.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     CK(ctx, cudaMemcpyAsync(&out->bad, S.bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
@@ -1771,21 +1784,21 @@ stats_status stats_reset(stats_ctx* ctx) {
   if (s != STATS_OK) return s;
   // stream-ordered: work already enqueued on the ctx's stream completes first
   cudaStream_t st = ctx->last;
+  // one clear: the status word lies behind the accumulator
   if (ctx->mode == STATS_EXACT) {
-    CK(ctx, cudaMemsetAsync(ctx->d_g, 0, kDigits * kDigits * sizeof(long long), st));
+    CK(ctx, cudaMemsetAsync(ctx->d_g, 0, kDigits * kDigits * sizeof(long long) + sizeof(unsigned int), st));
   } else {
     const size_t T = static_cast<size_t>(ctx->p) * (ctx->p + 1) / 2;
     CK(ctx, cudaMemsetAsync(ctx->d_fs, 0, (2 * ctx->p + 2 * T + ctx->p + 2) * sizeof(double), st));
     ctx->shift_set = false;
   }
-  CK(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(unsigned int), st));
   ctx->rows_enqueued = 0;
   return STATS_OK;
 }
 
 stats_status stats_raw(stats_ctx* ctx, int64_t* n, double* s, double* S_upper, stats_i128* s_exact,
                        stats_i128* S_exact_upper) {
-  stats_status st = stats_sync(ctx);
+  stats_status st = check_sticky(ctx);
   if (st != STATS_OK) return st;
   st = run_finalize(ctx, 0, 0);
   if (st != STATS_OK) return st;
@@ -1809,19 +1822,19 @@ stats_status stats_finalize(stats_ctx* ctx, double* mean, double* cov, double* c
 stats_status stats_finalize_warm(stats_ctx* ctx, double* mean, double* cov, double* corr, double* evals,
                                  double* evecs, int32_t pca_on, const double* evecs_prev, int32_t* sweeps) {
   if (sweeps) *sweeps = -1;
-  stats_status st = stats_sync(ctx);
-  if (st != STATS_OK) return st;
-  if (pca_on != 0 && pca_on != 1) return STATS_EINVAL;
-  // the row count decides whether a covariance exists
-  int64_t n = 0;
-  if (ctx->mode == STATS_EXACT) {
-    CK(ctx, cudaMemcpy(&n, ctx->d_g, sizeof(n), cudaMemcpyDeviceToHost));
-  } else {
-    CK(ctx, cudaMemcpy(&n, ctx->d_fn, sizeof(n), cudaMemcpyDeviceToHost));
+  if (pca_on != 0 && pca_on != 1) {
+    const stats_status st = stats_sync(ctx);
+    return st != STATS_OK ? st : STATS_EINVAL;
   }
-  if (n < 2) return STATS_EINVAL;
+  stats_status st = check_sticky(ctx);
+  if (st != STATS_OK) return st;
   st = run_finalize(ctx, (evals || evecs) ? 1 : 0, pca_on, (evals || evecs) ? evecs_prev : nullptr);
   if (st != STATS_OK) return st;
+  // the row count decides whether a covariance exists
+  int64_t n = 0;
+  memcpy(&n, ctx->h_out + ctx->lay.n, sizeof(n));
+  if (n < 2) return STATS_EINVAL;
+  if (ctx->h_out[ctx->lay.flags + 5] != 0.0) return STATS_ETIMEOUT;
   const FinalLayout& L = ctx->lay;
   const double* h = ctx->h_out;
   const size_t pa = ctx->pa;
@@ -1839,10 +1852,18 @@ stats_status stats_finalize_batched(stats_ctx* const* ctxs, int32_t count, int32
                                     double* const* evecs) {
   if (count < 0 || (count > 0 && !ctxs) || (pca_on != 0 && pca_on != 1)) return STATS_EINVAL;
   if (count == 0) return STATS_OK;
+  // the contexts' streams, each waited for once; their status words and row counts come with the
+  // results (a wait, a status read and a row count read per context took 15 us each)
+  std::vector<cudaStream_t> seen;
   for (int i = 0; i < count; ++i) {
-    if (!ctxs[i]) return STATS_EINVAL;
-    stats_status st = stats_sync(ctxs[i]);
+    const stats_status st = check_sticky(ctxs[i]);
     if (st != STATS_OK) return st;
+    for (int k = 0; k < (ctxs[i]->copy_stream ? 2 : 1); ++k) {
+      const cudaStream_t s = k ? ctxs[i]->copy_stream : ctxs[i]->last;
+      if (std::find(seen.begin(), seen.end(), s) != seen.end()) continue;
+      CK(ctxs[i], cudaStreamSynchronize(s));
+      seen.push_back(s);
+    }
   }
   const bool want_pca = evals || evecs;
   std::vector<FinalParams> params(count);
@@ -1851,52 +1872,59 @@ stats_status stats_finalize_batched(stats_ctx* const* ctxs, int32_t count, int32
   size_t total = 0;
   for (int i = 0; i < count; ++i) {
     off[i] = total;
-    total += static_cast<size_t>(ctxs[i]->lay.total);
+    total += static_cast<size_t>(ctxs[i]->lay.total - ctxs[i]->lay.mean) + 1;
   }
   stats_ctx* c0 = ctxs[0];
   const size_t pbytes = round256(count * sizeof(FinalParams)), jbytes = round256(count * sizeof(EigJob));
+  std::unique_ptr<double[]> h(new (std::nothrow) double[total]);
+  if (!h) return STATS_ENOMEM;
   void* dbuf = nullptr;
   CK(c0, cudaMalloc(&dbuf, pbytes + jbytes + total * sizeof(double)));
   EigJob* djobs = reinterpret_cast<EigJob*>(static_cast<char*>(dbuf) + pbytes);
   double* dout = reinterpret_cast<double*>(static_cast<char*>(dbuf) + pbytes + jbytes);
   for (int i = 0; i < count; ++i) {
+    const FinalLayout& L = ctxs[i]->lay;
     build_final_params(ctxs[i], want_pca ? 1 : 0, pca_on, params[i]);
-    params[i].out = dout + off[i];  // the work scratch stays per context
+    params[i].out = dout + off[i] - L.mean;  // the analysis alone; the work scratch stays per context
+    params[i].analysis_only = 1;
     if (want_pca && batched_eigen_deferred(ctxs[i]->pa)) {
-      const FinalLayout& L = ctxs[i]->lay;
       params[i].defer_m = -1;
       jobs.push_back(EigJob{params[i].out + (pca_on ? L.corr : L.cov), params[i].out + L.evals, params[i].out + L.evecs,
                             params[i].out + L.flags, ctxs[i]->pa, 0});
     }
   }
   std::stable_sort(jobs.begin(), jobs.end(), [](const EigJob& x, const EigJob& y) { return x.n > y.n; });
-  std::vector<double> h(total);
   cudaError_t e = cudaMemcpy(dbuf, params.data(), count * sizeof(FinalParams), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !jobs.empty())
     e = cudaMemcpy(djobs, jobs.data(), jobs.size() * sizeof(EigJob), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = launch_finalize_batched(reinterpret_cast<const FinalParams*>(dbuf), count, djobs, static_cast<int>(jobs.size()),
                                 nullptr);
-  if (e == cudaSuccess) e = cudaMemcpy(h.data(), dout, total * sizeof(double), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(h.get(), dout, total * sizeof(double), cudaMemcpyDeviceToHost);
   cudaFree(dbuf);
   if (e != cudaSuccess) return cuda_fail(c0, e);
+  for (int i = 0; i < count; ++i) {  // an error that some context's device work recorded: no results
+    const FinalLayout& L = ctxs[i]->lay;
+    const stats_status st = recorded_status(h.get() + off[i] + (L.flags - L.mean));
+    if (st != STATS_OK) return st;
+  }
   stats_status ret = STATS_OK;
   for (int i = 0; i < count; ++i) {
     const stats_ctx* c = ctxs[i];
-    const double* r = h.data() + off[i];
     const FinalLayout& L = c->lay;
+    const double* r = h.get() + off[i];
     const size_t pa = c->pa;
     int64_t nrows = 0;
-    memcpy(&nrows, r + L.n, sizeof(nrows));  // the row count is stored as an integer
+    memcpy(&nrows, r + (L.total - L.mean), sizeof(nrows));  // the row count is stored as an integer
     if (nrows < 2) {  // no covariance for fewer than two rows
       ret = STATS_EINVAL;
       continue;
     }
-    if (mean && mean[i]) memcpy(mean[i], r + L.mean, sizeof(double) * pa);
-    if (cov && cov[i]) memcpy(cov[i], r + L.cov, sizeof(double) * pa * pa);
-    if (corr && corr[i]) memcpy(corr[i], r + L.corr, sizeof(double) * pa * pa);
-    if (evals && evals[i]) memcpy(evals[i], r + L.evals, sizeof(double) * pa);
-    if (evecs && evecs[i]) memcpy(evecs[i], r + L.evecs, sizeof(double) * pa * pa);
+    if (mean && mean[i]) memcpy(mean[i], r, sizeof(double) * pa);
+    if (cov && cov[i]) memcpy(cov[i], r + (L.cov - L.mean), sizeof(double) * pa * pa);
+    if (corr && corr[i]) memcpy(corr[i], r + (L.corr - L.mean), sizeof(double) * pa * pa);
+    if (evals && evals[i]) memcpy(evals[i], r + (L.evals - L.mean), sizeof(double) * pa);
+    if (evecs && evecs[i]) memcpy(evecs[i], r + (L.evecs - L.mean), sizeof(double) * pa * pa);
   }
   return ret;
 }

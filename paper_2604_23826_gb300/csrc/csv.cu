@@ -574,7 +574,9 @@ __device__ __forceinline__ int dtype_size(int32_t dt) {
 }
 
 __global__ void __launch_bounds__(256) csv_parse_kernel(const char* __restrict__ t, int64_t nbytes, CsvScratch S, int k,
-                                                       int64_t row_cap, const __grid_constant__ CsvTables TP) {
+                                                       int64_t row_cap, int64_t max_lines,
+                                                       const __grid_constant__ CsvTables TP) {
+  if (*S.total > max_lines) return;
   __shared__ CsvTables T;
   for (int i = threadIdx.x; i < static_cast<int>(sizeof(CsvTables) / 8); i += blockDim.x)
     reinterpret_cast<uint64_t*>(&T)[i] = reinterpret_cast<const uint64_t*>(&TP)[i];
@@ -615,8 +617,7 @@ size_t pad256(size_t b) { return (b + 255) / 256 * 256; }
 
 size_t csv_scratch_bytes(int64_t nbytes, int64_t ends_cap, int k) {
   const int64_t ntiles = (nbytes + kCsvTile - 1) / kCsvTile + 1;
-  return pad256(4 * ntiles) + pad256(8 * ntiles) + pad256(8 * (ends_cap + 1)) + 256 + 256 + 256 + pad256(8 * k) +
-         pad256(4 * k);
+  return pad256(4 * ntiles) + pad256(8 * ntiles) + pad256(8 * (ends_cap + 1)) + pad256(sizeof(CsvHead) + 12 * k);
 }
 
 void csv_scratch_carve(void* base, int64_t nbytes, int64_t ends_cap, int k, CsvScratch& s) {
@@ -629,14 +630,13 @@ void csv_scratch_carve(void* base, int64_t nbytes, int64_t ends_cap, int k, CsvS
   s.ends = reinterpret_cast<int64_t*>(b);
   s.ends_cap = ends_cap;
   b += pad256(8 * (ends_cap + 1));
-  s.total = reinterpret_cast<int64_t*>(b);
-  b += 256;
-  s.status = reinterpret_cast<uint32_t*>(b);
-  b += 256;
-  s.bad = reinterpret_cast<unsigned long long*>(b);
-  b += 256;
+  s.head = reinterpret_cast<CsvHead*>(b);
+  s.total = &s.head->total;
+  s.status = &s.head->status;
+  s.bad = &s.head->bad;
+  b += sizeof(CsvHead);
   s.cols = reinterpret_cast<void**>(b);
-  b += pad256(8 * k);
+  b += 8 * k;
   s.dts = reinterpret_cast<int32_t*>(b);
 }
 
@@ -651,12 +651,12 @@ cudaError_t launch_csv_lines(const char* d_text, int64_t nbytes, const CsvScratc
   return cudaGetLastError();
 }
 
-cudaError_t launch_csv_parse(const char* d_text, int64_t nbytes, const CsvScratch& s, int k, int64_t row_cap, int sms,
-                             cudaStream_t st) {
+cudaError_t launch_csv_parse(const char* d_text, int64_t nbytes, const CsvScratch& s, int k, int64_t row_cap,
+                             int64_t max_lines, int sms, cudaStream_t st) {
   const int64_t want = (s.ends_cap + 255) / 256;
   const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(sms) * 8)));
   static const CsvTables tables = make_csv_tables();
-  csv_parse_kernel<<<grid, 256, 0, st>>>(d_text, nbytes, s, k, row_cap, tables);
+  csv_parse_kernel<<<grid, 256, 0, st>>>(d_text, nbytes, s, k, row_cap, max_lines, tables);
   return cudaGetLastError();
 }
 
@@ -862,27 +862,21 @@ stats_status stats_csv_parse(const char* d_text, int64_t nbytes, int32_t k, cons
   }
   CsvScratch S;
   csv_scratch_carve(scratch, nbytes, ends_cap, k, S);
-  struct Out {
-    int64_t total;
-    uint32_t status;
-    uint32_t pad;
-    unsigned long long bad;
-  } out{};
+  // one copy in (the error words' start, the columns and their types), one out and one wait: a table of
+  // more lines than it may have is left alone by the parse itself
+  char in[sizeof(CsvHead) + 12 * STATS_MAX_P];
+  const CsvHead start{0, ~0ull, 0u, 0u};
+  memcpy(in, &start, sizeof(start));
+  memcpy(in + sizeof(start), d_cols, sizeof(void*) * k);
+  memcpy(in + sizeof(start) + sizeof(void*) * k, dtypes, sizeof(int32_t) * k);
+  CsvHead out{};
   stats_status res = STATS_OK;
-  cudaError_t e = cudaMemcpyAsync(S.cols, d_cols, sizeof(void*) * k, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(S.dts, dtypes, sizeof(int32_t) * k, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(S.status, 0, sizeof(uint32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(S.bad, 0xFF, sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemcpyAsync(S.head, in, sizeof(start) + 12 * k, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = launch_csv_lines(d_text, nbytes, S, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&out.total, S.total, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = launch_csv_parse(d_text, nbytes, S, k, max_rows, max_rows, sms, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&out, S.head, sizeof(out), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e == cudaSuccess && out.total > max_rows) res = STATS_EINVAL;
-  if (e == cudaSuccess && res == STATS_OK) {
-    e = launch_csv_parse(d_text, nbytes, S, k, max_rows, sms, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&out.status, S.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&out.bad, S.bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  }
   cudaFreeAsync(scratch, st);
   if (e != cudaSuccess) {
     cudaGetLastError();

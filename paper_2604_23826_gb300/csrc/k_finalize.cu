@@ -454,6 +454,8 @@ __device__ void finalize_body(const FinalParams& P) {
   double* flags = out + L.flags;
   double* cov = out + L.cov;
   double* corr = out + L.corr;
+  const bool raw = !P.analysis_only;
+  long long rows = 0;
   double n_d = 0.0;
   bool nonpositive = false;  // a variance of zero (EXACT) or not above zero
 
@@ -465,9 +467,10 @@ __device__ void finalize_body(const FinalParams& P) {
     __syncthreads();
     const long long* G = U.exact.G;
     const long long n = G[0];
+    rows = n;
     n_d = static_cast<double>(n);
     if (tid == 0) {
-      reinterpret_cast<long long*>(out)[L.n] = n;
+      if (raw) reinterpret_cast<long long*>(out)[L.n] = n;
       s_den = i256_to_double(i256_mul(i256_from(n), i256_from(n - 1)));
     }
     // exact column sums r_j (scaled by 2^-shift_j)
@@ -477,9 +480,11 @@ __device__ void finalize_body(const FinalParams& P) {
       for (int a = cj.k - 1; a >= 0; --a) r = r * 256 + G[cj.off + a];
       U.exact.r[tid] = r;
       const double s = ldexp(i256_to_double(widen(r)), -cj.shift);
-      out[L.s + tid] = s;
-      reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid] = cj.is_real ? 0 : static_cast<int64_t>(r);
-      reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid + 1] = cj.is_real ? 0 : static_cast<int64_t>(r >> 64);
+      if (raw) {
+        out[L.s + tid] = s;
+        reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid] = cj.is_real ? 0 : static_cast<int64_t>(r);
+        reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid + 1] = cj.is_real ? 0 : static_cast<int64_t>(r >> 64);
+      }
       if (s_idx[tid] >= 0) out[L.mean + s_idx[tid]] = s / n_d;
     }
     __syncthreads();
@@ -489,13 +494,15 @@ __device__ void finalize_body(const FinalParams& P) {
       packed_entry(t, p, j, k);
       const FinalPlanCol cj = P.col[j], ck = P.col[k];
       const i256 R = cross_product(G, cj, ck);
-      out[L.S + t] = ldexp(i256_to_double(R), -(cj.shift + ck.shift));
       int64_t lo = 0, hi = 0;
       if (!cj.is_real && !ck.is_real) {
         if (!i256_fits_i128(R, lo, hi)) atomicOr(&s_over, 1);
       }
-      reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t] = lo;
-      reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t + 1] = hi;
+      if (raw) {
+        out[L.S + t] = ldexp(i256_to_double(R), -(cj.shift + ck.shift));
+        reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t] = lo;
+        reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t + 1] = hi;
+      }
       const int aj = s_idx[j], ak = s_idx[k];
       if (aj >= 0 && ak >= 0 && n >= 2) {
         const i256 C = i256_sub(i256_mul(i256_from(n), R), i256_mul(widen(U.exact.r[j]), widen(U.exact.r[k])));
@@ -510,21 +517,26 @@ __device__ void finalize_body(const FinalParams& P) {
     }
   } else {
     const long long n = *P.fn;
+    rows = n;
     n_d = static_cast<double>(n);
-    if (tid == 0) reinterpret_cast<long long*>(out)[L.n] = n;
+    if (tid == 0 && raw) reinterpret_cast<long long*>(out)[L.n] = n;
     if (tid < p) {
       const double s = raw_sum(P, tid, n_d);
-      out[L.s + tid] = s;
-      reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid] = 0;
-      reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid + 1] = 0;
+      if (raw) {
+        out[L.s + tid] = s;
+        reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid] = 0;
+        reinterpret_cast<int64_t*>(out)[L.s_ex + 2 * tid + 1] = 0;
+      }
       if (s_idx[tid] >= 0) out[L.mean + s_idx[tid]] = s / n_d;
     }
     for (int t = tid; t < T; t += kThreads) {
       int j, k;
       packed_entry(t, p, j, k);
-      out[L.S + t] = raw_S(P, t, j, k, n_d);
-      reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t] = 0;
-      reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t + 1] = 0;
+      if (raw) {
+        out[L.S + t] = raw_S(P, t, j, k, n_d);
+        reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t] = 0;
+        reinterpret_cast<int64_t*>(out)[L.S_ex + 2 * t + 1] = 0;
+      }
       const int aj = s_idx[j], ak = s_idx[k];
       if (aj >= 0 && ak >= 0 && n >= 2) {
         const double v = raw_cov(P, t, j, k, n_d);
@@ -548,7 +560,9 @@ __device__ void finalize_body(const FinalParams& P) {
     flags[3] = 0.0;
     flags[5] = 0.0;
     flags[6] = 0.0;
+    if (P.status) reinterpret_cast<unsigned long long*>(flags)[4] = *P.status;
     if (P.defer_m < 0) flags[7] = pca_ok ? 1.0 : 0.0;
+    if (P.analysis_only) reinterpret_cast<long long*>(flags)[8] = rows;
     if (P.defer_ctl) *P.defer_ctl = pca_ok ? 1 : 0;
   }
   __syncthreads();
@@ -641,6 +655,7 @@ __global__ void __launch_bounds__(kThreads) finalize_wide_kernel(const __grid_co
     flags[3] = 0.0;
     flags[5] = 0.0;
     flags[6] = 0.0;
+    if (P.status) reinterpret_cast<unsigned long long*>(flags)[4] = *P.status;
     if (P.defer_ctl) *P.defer_ctl = pca_ok ? 1 : 0;
   }
   const int gtid = blockIdx.x * kThreads + tid, nthreads = gridDim.x * kThreads, m = P.defer_m;

@@ -352,6 +352,11 @@ struct FinalParams {
   double* defer_A;
   int32_t* defer_ctl;
   int32_t defer_m;
+  // The context's device status word, whose bits go to flags[4] (as an integer), or null.
+  const unsigned int* status;
+  // Batches: only the analysis (mean .. flags) is written, at its offsets from out, and the row count
+  // (int64) after the flags.
+  int32_t analysis_only;
 };
 // Offsets (in doubles) of the finalize result buffer.
 struct FinalLayout {
@@ -375,7 +380,7 @@ __host__ __device__ inline FinalLayout final_layout(int p, int pa) {
   return L;
 }
 // flags: [0] an exact integer entry did not fit 128 bits, [1] zero-variance columns,
-//        [2] Jacobi sweeps, [3] eigenpairs computed (1) or not (0),
+//        [2] Jacobi sweeps, [3] eigenpairs computed (1) or not (0), [4] device status bits,
 //        [5] a grid-wide wait of jacobi_grid_kernel ran out (1), [6] its seed basis was used (1)
 cudaError_t launch_finalize(const FinalParams& P, cudaStream_t stream);
 // An eigen-decomposition of a batch (n of batched_eigen_deferred), after its context's finalize block.
@@ -424,14 +429,21 @@ cudaError_t launch_jacobi_grid(const JacobiParams& J, int grid, cudaStream_t str
 constexpr int kCsvTile = 4096;  // bytes per line-counting tile
 // error bits of CsvScratch::status
 constexpr uint32_t kCsvFormat = 1u, kCsvRange = 2u;
+struct CsvHead {
+  int64_t total;           // number of lines
+  unsigned long long bad;  // (first offending line << 2) | its error bit (all ones: none)
+  uint32_t status;         // kCsvFormat | kCsvRange
+  uint32_t pad;
+};
 struct CsvScratch {
   uint32_t* counts;          // newlines per tile
   int64_t* offs;             // exclusive prefix of counts
   int64_t* ends;             // ends[i]: offset of line i's '\n' (or the text's end), i < ends_cap
   int64_t ends_cap;
-  int64_t* total;            // number of lines
-  uint32_t* status;          // kCsvFormat | kCsvRange
-  unsigned long long* bad;   // (first offending line << 2) | its error bit (all ones: none)
+  CsvHead* head;             // then the next three, and cols and dts right behind it
+  int64_t* total;
+  uint32_t* status;
+  unsigned long long* bad;
   void** cols;               // k device column pointers
   int32_t* dts;              // k stats_dtype values
 };
@@ -442,9 +454,10 @@ void csv_scratch_carve(void* base, int64_t nbytes, int64_t ends_cap, int k, CsvS
 // Counts the lines of d_text[0, nbytes) and writes their ends (no host synchronisation).
 cudaError_t launch_csv_lines(const char* d_text, int64_t nbytes, const CsvScratch& s, cudaStream_t st);
 // Parses the first k fields of lines [0, min(*total, ends_cap)) into s.cols (rows below
-// row_cap are stored; every line is checked); status and bad must be reset before.
-cudaError_t launch_csv_parse(const char* d_text, int64_t nbytes, const CsvScratch& s, int k, int64_t row_cap, int sms,
-                             cudaStream_t st);
+// row_cap are stored; every line is checked), unless there are more than max_lines; status and bad must
+// be reset before.
+cudaError_t launch_csv_parse(const char* d_text, int64_t nbytes, const CsvScratch& s, int k, int64_t row_cap,
+                             int64_t max_lines, int sms, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Table 1 generator and misc.
