@@ -147,37 +147,13 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
 // Exact digits as f16.  A byte b (0..255) placed in the low 8 mantissa bits of
 // the half 0x6400 (= 1024.0) reads 1024 + b exactly (the half has 10 mantissa
 // bits); subtracting 1024 leaves b.  A signed top byte is first XORed with 0x80
-// (so 1024 + (b ^ 0x80) holds b_signed + 1152) and 1152 is subtracted.
+// (so 1024 + (b ^ 0x80) holds b_signed + 1152) and 1152 is subtracted.  Below a zero
+// byte, b is the subnormal half b 2^-24.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t half2_sub(uint32_t a, uint32_t b) {
   uint32_t d;
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
-}
-constexpr uint32_t kMagicLo = 0x6400u;      // 1024.0 in f16
-constexpr uint32_t kMagicHi = 0x6400u << 16;
-constexpr uint32_t kH1024 = 0x64006400u;    // {1024, 1024}
-constexpr uint32_t kH1152lo = 0x64006480u;  // {1152 (low), 1024 (high)}
-constexpr uint32_t kH1152hi = 0x64806400u;  // {1024 (low), 1152 (high)}
-
-// Two unsigned bytes (x low, y high), each already in the low byte of its
-// register's half (x in bits 0..7, y in bits 16..23), to an f16x2 of (x, y).
-__device__ __forceinline__ uint32_t digits2(uint32_t packed_bytes, uint32_t bias = kH1024) {
-  return half2_sub(packed_bytes | kH1024, bias);
-}
-
-__device__ __forceinline__ uint32_t half2_mul(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-// Two small non-negative integers x, y < 256 to an f16x2 of (x, y) on the FMA
-// pipe only: x + 65536 y (one IMAD) holds each value as the bit pattern of the
-// subnormal half v * 2^-24; two exact multiplications by 2^12 rescale it to v.
-__device__ __forceinline__ uint32_t small_pair_f16x2(uint32_t x, uint32_t y) {
-  const uint32_t bits = y * 65536u + x;
-  constexpr uint32_t k2p12 = 0x6C006C00u;  // {4096, 4096}
-  return half2_mul(half2_mul(bits, k2p12), k2p12);
 }
 
 // ---------------------------------------------------------------------------

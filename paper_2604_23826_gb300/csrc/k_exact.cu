@@ -109,65 +109,137 @@ struct SmemT1Src {
 // unit sustains about two per clock per SM, well above what this pass needs.)
 __device__ __forceinline__ uint64_t fixed_f2i(double x, int sh) {
   const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
-  const bool normal = ((hi >> 20) & 0x7FF) != 0;
-  const long long q =
-      __double2ll_rn(__hiloint2double(static_cast<int>(hi + (static_cast<uint32_t>(sh) << 20)), static_cast<int>(lo)));
-  return normal ? static_cast<uint64_t>(q) : 0ull;
+  const uint32_t scaled = (hi & 0x7FF00000u) != 0 ? hi + (static_cast<uint32_t>(sh) << 20) : 0u;
+  return static_cast<uint64_t>(__double2ll_rn(__hiloint2double(static_cast<int>(scaled), static_cast<int>(lo))));
+}
+
+// Two consecutive elements of a column in a stage (the first row is even).
+template <class T>
+__device__ __forceinline__ void two_of(const uint8_t* col, int r, T& x, T& y) {
+  struct alignas(2 * sizeof(T)) Two {
+    T x, y;
+  };
+  const Two v = *reinterpret_cast<const Two*>(col + r * sizeof(T));
+  x = v.x;
+  y = v.y;
 }
 
 // ---- the Table 1 converter: fixed digit plan, column order A B C D E F G H cotC I J K ----
 // slots: 0 ones | 1 B | 2 C | 3 D | 4 E | 5 G | 6 H | 7 K | 8-9 F | 10-11 I | 12-16 A |
 //        17-23 cotC (signed, top byte 23) | 24-30 J | 31 zero
 // The field checks below are exactly the ranges those digit fields can carry.
+// The digits are f16 numbers d 2^-24: a byte below a zero byte is that subnormal as it lies, so a pair
+// of digits is one byte permutation (as 1024 + d, less 1024, it was two or three instructions).  All
+// sums of products are those of the digits times 2^-48, as exact in FP32; kUnit takes them back.
+// A lane takes two rows at once, adjacent ones of a stage: their loads, conversions and checks
+// overlap, and one load brings both values of a column.
+// Bound: HBM for the 60 bytes an L32 row has (1e9 rows: 9.38 ms, 6.4 TB/s; a row at a time with
+// rescaled digits 9.98).  The 44 bytes of L16 wait for the conversions: about 180 instructions per 32
+// rows on four warps a scheduler, half the issue slots and a third of the FP64 unit (1.23e8 rows:
+// 1.17 ms, 1.23 before).
 template <bool L16>
 struct ConvT1 {
-  static constexpr bool kPair = false;
+  static constexpr bool kPair = true, kAdjacent = true;
+  static constexpr float kUnit = 281474976710656.f;  // 2^48
+  struct Row {
+    int64_t A;
+    double cot, J;
+    int32_t B, C, D, E, F, G, H, I, K;
+  };
   template <int TILE>
   __device__ __forceinline__ static SmemT1Src<L16, TILE> smem_src(const uint8_t* st, const ExactParams&, int r) {
     return SmemT1Src<L16, TILE>{st, r};
   }
   template <class Src>
-  __device__ __forceinline__ static void row(const ExactParams& P, const Src& src, uint32_t (&w)[16],
-                                             uint32_t& bad) {
-    int32_t B, C, D, E, F, G, H, I, K;
+  __device__ __forceinline__ static void load(const Src& src, Row& x) {
     if (L16) {
-      B = src.i16(1); C = src.i16(2); D = src.i16(3); E = src.i16(4); G = src.i16(6);
-      H = src.i16(7); I = src.i16(9); K = src.i16(11); F = src.i32(5);
+      x.B = src.i16(1); x.C = src.i16(2); x.D = src.i16(3); x.E = src.i16(4); x.G = src.i16(6);
+      x.H = src.i16(7); x.I = src.i16(9); x.K = src.i16(11); x.F = src.i32(5);
     } else {
-      B = src.i32(1); C = src.i32(2); D = src.i32(3); E = src.i32(4); F = src.i32(5);
-      G = src.i32(6); H = src.i32(7); I = src.i32(9); K = src.i32(11);
+      x.B = src.i32(1); x.C = src.i32(2); x.D = src.i32(3); x.E = src.i32(4); x.F = src.i32(5);
+      x.G = src.i32(6); x.H = src.i32(7); x.I = src.i32(9); x.K = src.i32(11);
     }
-    const int64_t A = src.i64(0);
-    const double cot = src.f64(8), J = src.f64(10);
-    const uint32_t Alo = static_cast<uint32_t>(A), Ahi = static_cast<uint32_t>(static_cast<uint64_t>(A) >> 32);
-    // field checks: one unsigned byte each; two unsigned bytes; five unsigned bytes
-    bad |= static_cast<uint32_t>(B | C | D | E | G | H | K) & 0xFFFFFF00u;
-    bad |= static_cast<uint32_t>(F | I) & 0xFFFF0000u;
-    bad |= Ahi & 0xFFFFFF00u;
-    const int ec = dbl_exp_field(cot), ej = dbl_exp_field(J);
-    const uint64_t uj = static_cast<uint64_t>(__double_as_longlong(J));
-    bad |= (ec > P.real_emax[8]) | (ej > P.real_emax[10]) | ((uj >> 63) & ((uj << 1) != 0));  // J >= 0
-    const uint64_t qc = fixed_f2i(cot, P.real_shift[8]);
-    const uint64_t qj = fixed_f2i(J, P.real_shift[10]);
+    x.A = src.i64(0);
+    x.cot = src.f64(8);
+    x.J = src.f64(10);
+  }
+  // rows r (even) and r + 1 of a stage
+  template <int TILE>
+  __device__ __forceinline__ static void load_two(const uint8_t* st, int r, Row& x, Row& y) {
+    using L = T1Layout<L16, TILE>;
+    auto narrow = [&](int j, int32_t& a, int32_t& b) {
+      if (L16) {
+        int16_t u, v;
+        two_of(st + L::off(j), r, u, v);
+        a = u;
+        b = v;
+      } else {
+        two_of(st + L::off(j), r, a, b);
+      }
+    };
+    two_of(st + L::off(8), r, x.cot, y.cot);
+    two_of(st + L::off(10), r, x.J, y.J);
+    two_of(st + L::off(0), r, x.A, y.A);
+    two_of(st + L::off(5), r, x.F, y.F);
+    narrow(1, x.B, y.B);
+    narrow(2, x.C, y.C);
+    narrow(3, x.D, y.D);
+    narrow(4, x.E, y.E);
+    narrow(6, x.G, y.G);
+    narrow(7, x.H, y.H);
+    narrow(9, x.I, y.I);
+    narrow(11, x.K, y.K);
+  }
+  // not zero: some value of the N rows leaves its digit field
+  template <int N>
+  __device__ __forceinline__ static uint32_t violation(const ExactParams& P, const Row (&x)[N]) {
+    int32_t bytes = 0, halves = 0;
+    uint32_t top = 0, bad = 0;
+    const int limc = static_cast<int>((static_cast<uint32_t>(P.real_emax[8]) << 20) | 0xFFFFFu);
+    const int limj = static_cast<int>((static_cast<uint32_t>(P.real_emax[10]) << 20) | 0xFFFFFu);
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      bytes |= x[u].B | x[u].C | x[u].D | x[u].E | x[u].G | x[u].H | x[u].K;  // one unsigned byte each
+      halves |= x[u].F | x[u].I;                                              // two
+      top |= static_cast<uint32_t>(static_cast<uint64_t>(x[u].A) >> 32);      // five
+      const int mc = __double2hiint(x[u].cot) & 0x7FFFFFFF, mj = __double2hiint(x[u].J) & 0x7FFFFFFF;
+      bad |= (mc > limc) | (mj > limj);                                                            // exponents
+      bad |= (__double2hiint(x[u].J) < 0) & ((mj | __double2loint(x[u].J)) != 0);                  // J >= 0
+    }
+    return bad | (static_cast<uint32_t>(bytes) & 0xFFFFFF00u) | (static_cast<uint32_t>(halves) & 0xFFFF0000u) |
+           (top & 0xFFFFFF00u);
+  }
+  __device__ __forceinline__ static void digits(const ExactParams& P, const Row& x, uint32_t (&w)[16]) {
+    const uint32_t F = x.F, I = x.I;
+    const uint32_t Alo = static_cast<uint32_t>(x.A), Ahi = static_cast<uint32_t>(static_cast<uint64_t>(x.A) >> 32);
+    const uint64_t qc = fixed_f2i(x.cot, P.real_shift[8]);
+    const uint64_t qj = fixed_f2i(x.J, P.real_shift[10]);
     const uint32_t qclo = static_cast<uint32_t>(qc), qchi = static_cast<uint32_t>(qc >> 32) ^ 0x00800000u;
     const uint32_t qjlo = static_cast<uint32_t>(qj), qjhi = static_cast<uint32_t>(qj >> 32);
-    constexpr uint32_t M = 0x64646464u;  // bytes of the f16 exponent 0x64
-    w[0] = small_pair_f16x2(1u, static_cast<uint32_t>(B));
-    w[1] = small_pair_f16x2(static_cast<uint32_t>(C), static_cast<uint32_t>(D));
-    w[2] = small_pair_f16x2(static_cast<uint32_t>(E), static_cast<uint32_t>(G));
-    w[3] = small_pair_f16x2(static_cast<uint32_t>(H), static_cast<uint32_t>(K));
-    w[4] = half2_sub(__byte_perm(static_cast<uint32_t>(F), M, 0x4140), kH1024);
-    w[5] = half2_sub(__byte_perm(static_cast<uint32_t>(I), M, 0x4140), kH1024);
-    w[6] = half2_sub(__byte_perm(Alo, M, 0x4140), kH1024);
-    w[7] = half2_sub(__byte_perm(Alo, M, 0x4342), kH1024);
-    w[8] = digits2(__byte_perm(Ahi, qclo, 0x1410));          // A byte 4 | cotC byte 0
-    w[9] = half2_sub(__byte_perm(qclo, M, 0x4241), kH1024);  // cotC bytes 1, 2
-    w[10] = digits2(__byte_perm(qclo, qchi, 0x0403) & 0x00FF00FFu);  // cotC bytes 3, 4
-    w[11] = half2_sub(__byte_perm(qchi, M, 0x4241), kH1152hi);       // cotC bytes 5, 6 (6 signed)
-    w[12] = half2_sub(__byte_perm(qjlo, M, 0x4140), kH1024);
-    w[13] = half2_sub(__byte_perm(qjlo, M, 0x4342), kH1024);
-    w[14] = half2_sub(__byte_perm(qjhi, M, 0x4140), kH1024);
-    w[15] = half2_sub(__byte_perm(qjhi, M, 0x4342), kH1024);  // J byte 6 | zero (byte 7 of q)
+    w[0] = __byte_perm(1u, static_cast<uint32_t>(x.B), 0x5410);
+    w[1] = __byte_perm(static_cast<uint32_t>(x.C), static_cast<uint32_t>(x.D), 0x5410);
+    w[2] = __byte_perm(static_cast<uint32_t>(x.E), static_cast<uint32_t>(x.G), 0x5410);
+    w[3] = __byte_perm(static_cast<uint32_t>(x.H), static_cast<uint32_t>(x.K), 0x5410);
+    w[4] = __byte_perm(F, 0u, 0x4140);
+    w[5] = __byte_perm(I, 0u, 0x4140);
+    w[6] = __byte_perm(Alo, 0u, 0x4140);
+    w[7] = __byte_perm(Alo, 0u, 0x4342);
+    w[8] = __byte_perm(Ahi, qclo, 0x1410);                 // A byte 4 | cotC byte 0 (A's byte 5 is zero)
+    w[9] = __byte_perm(qclo, 0u, 0x4241);                  // cotC bytes 1, 2
+    w[10] = __byte_perm(qclo, qchi, 0x0403) & 0x00FF00FFu;  // cotC bytes 3, 4
+    w[11] = half2_sub(__byte_perm(qchi, 0u, 0x4241), 0x00800000u);  // cotC bytes 5, 6 (6 signed)
+    w[12] = __byte_perm(qjlo, 0u, 0x4140);
+    w[13] = __byte_perm(qjlo, 0u, 0x4342);
+    w[14] = __byte_perm(qjhi, 0u, 0x4140);
+    w[15] = __byte_perm(qjhi, 0u, 0x4342);  // J byte 6 | zero (byte 7 of q)
+  }
+  template <class Src>
+  __device__ __forceinline__ static void row(const ExactParams& P, const Src& src, uint32_t (&w)[16],
+                                             uint32_t& bad) {
+    Row x[1];
+    load(src, x[0]);
+    bad |= violation(P, x);
+    digits(P, x[0], w);
   }
 };
 
@@ -176,7 +248,7 @@ struct ConvT1 {
 // once, biased to an unsigned field (a signed field's top byte XOR 0x80 is the value plus
 // 2^(8k-1)) and appended to a 64-bit register; every eight bytes that fill it leave as four f16
 // pairs, whose bias takes a signed top byte's 128 off again.  The column loop is uniform across
-// the warp, so its branches cost one instruction each, and two rows of a lane share it.  (Bound: instruction issue, as for Table 1.
+// the warp, so its branches cost one instruction each, and two rows of a lane share it.  (Bound: instruction issue and latency.
 // Eight mixed columns, 36 B a row, 2e7 rows: extracting every digit from its column anew took
 // 2.50 ms, this way 0.56 ms; 0.71 with one row a lane.)
 struct ConvGeneric {
@@ -184,7 +256,8 @@ struct ConvGeneric {
   __device__ __forceinline__ static SmemSrc smem_src(const uint8_t* st, const ExactParams& P, int r) {
     return SmemSrc{st, &P, r};
   }
-  static constexpr bool kPair = true;  // two rows per lane share the walk over the columns
+  static constexpr bool kPair = true, kAdjacent = false;  // two rows per lane share the walk over the columns
+  static constexpr float kUnit = 1.f;                     // digits as f16 integers
   // q = round(x * 2^sh); range violations into bad
   __device__ __forceinline__ static uint64_t real_field(double x, int sh, int emax, bool is_signed, uint32_t& bad) {
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
@@ -334,23 +407,23 @@ __device__ __forceinline__ void warp_mma_32rows(uint32_t tile, int lane, const u
   __syncwarp();
 }
 
-// FP32 accumulators (exact integers below 2^24) into int32 partial sums: registers, or the
+// FP32 accumulators (exact integers below 2^24, over `unit`) into int32 partial sums: registers, or the
 // warp's shared array (each lane its own 24 words, so plain loads and stores suffice).
-__device__ __forceinline__ void flush_f32(WarpAcc& acc, WarpI32& ri) {
+__device__ __forceinline__ void flush_f32(WarpAcc& acc, WarpI32& ri, float unit) {
 #pragma unroll
   for (int e = 0; e < 6; ++e)
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      ri.i[e][r] += __float2int_rn(acc.f[e][r]);
+      ri.i[e][r] += __float2int_rn(acc.f[e][r] * unit);
       acc.f[e][r] = 0.f;
     }
 }
-__device__ __forceinline__ void flush_f32(WarpAcc& acc, int32_t* si, int lane) {
+__device__ __forceinline__ void flush_f32(WarpAcc& acc, int32_t* si, int lane, float unit) {
 #pragma unroll
   for (int e = 0; e < 6; ++e)
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      si[(4 * e + r) * 32 + lane] += __float2int_rn(acc.f[e][r]);
+      si[(4 * e + r) * 32 + lane] += __float2int_rn(acc.f[e][r] * unit);
       acc.f[e][r] = 0.f;
     }
 }
@@ -506,9 +579,9 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) exact_pass_kernel(const __gri
         if ((sub += n) == kFlushRows / 32) {
           sub = 0;
           if (i32_in_smem(W))
-            flush_f32(acc, si, lane);
+            flush_f32(acc, si, lane, Conv::kUnit);
           else
-            flush_f32(acc, ri);
+            flush_f32(acc, ri, Conv::kUnit);
           if (++flushes == kI32Flushes) {
             flushes = 0;
             flush_i32(get_i32, cta_acc, lane);
@@ -517,27 +590,45 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) exact_pass_kernel(const __gri
       };
       if constexpr (Conv::kPair && RPW == 64) {
         // both rows of the lane; one past the end is read as the last row and left out
-        const int r0 = warp * RPW + lane, r1 = r0 + 32, c0 = min(r0, valid - 1), c1 = min(r1, valid - 1);
-        uint32_t w[2][16], b[2] = {0, 0};
-        if (P.direct) {
-          const GlobalSrc src[2] = {{&P, row0 + c0}, {&P, row0 + c1}};
-          Conv::template rows<2>(P, src, w, b);
+        uint32_t w[2][16];
+        bool in0, in1;
+        if (Conv::kAdjacent && !P.direct) {
+          const int r = warp * RPW + 2 * lane;  // a stage's rows are a multiple of eight
+          if constexpr (Conv::kAdjacent) {
+            typename Conv::Row x[2];
+            Conv::template load_two<kTile>(st, min(r, valid - 2), x[0], x[1]);
+            bad |= Conv::violation(P, x);
+            Conv::digits(P, x[0], w[0]);
+            Conv::digits(P, x[1], w[1]);
+          }
+          in0 = in1 = r < valid;
         } else {
-          const auto s0 = Conv::template smem_src<kTile>(st, P, c0), s1 = Conv::template smem_src<kTile>(st, P, c1);
-          const std::remove_const_t<decltype(s0)> src[2] = {s0, s1};
-          Conv::template rows<2>(P, src, w, b);
+          const int r0 = warp * RPW + lane, r1 = r0 + 32, c0 = min(r0, valid - 1), c1 = min(r1, valid - 1);
+          uint32_t b[2] = {0, 0};
+          if (P.direct) {
+            const GlobalSrc src[2] = {{&P, row0 + c0}, {&P, row0 + c1}};
+            if constexpr (Conv::kAdjacent) {
+              Conv::row(P, src[0], w[0], b[0]);
+              Conv::row(P, src[1], w[1], b[1]);
+            } else {
+              Conv::template rows<2>(P, src, w, b);
+            }
+          } else if constexpr (!Conv::kAdjacent) {
+            const auto s0 = Conv::template smem_src<kTile>(st, P, c0), s1 = Conv::template smem_src<kTile>(st, P, c1);
+            const std::remove_const_t<decltype(s0)> src[2] = {s0, s1};
+            Conv::template rows<2>(P, src, w, b);
+          }
+          bad |= (b[0] | b[1]) != 0;  // (a row read twice is checked twice)
+          in0 = r0 < valid;
+          in1 = r1 < valid;
         }
-        if (r0 >= valid) {
+        if (!in0) {
 #pragma unroll
           for (int q = 0; q < 16; ++q) w[0][q] = 0u;
-        } else {
-          bad |= b[0] != 0;
         }
-        if (r1 >= valid) {
+        if (!in1) {
 #pragma unroll
           for (int q = 0; q < 16; ++q) w[1][q] = 0u;
-        } else {
-          bad |= b[1] != 0;
         }
         warp_mma_32rows(tile, lane, w[0], acc);
         warp_mma_32rows(tile, lane, w[1], acc);
@@ -581,9 +672,9 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) exact_pass_kernel(const __gri
       warp_mma_32rows(tile, lane, w, acc);
     }
     if (i32_in_smem(W))
-      flush_f32(acc, si, lane);
+      flush_f32(acc, si, lane, Conv::kUnit);
     else
-      flush_f32(acc, ri);
+      flush_f32(acc, ri, Conv::kUnit);
     flush_i32(get_i32, cta_acc, lane);
   }
   if (bad) atomicOr(&s_bad, DEV_ERANGE);
@@ -810,7 +901,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) exact_tc_kernel(const __grid_co
           ri.i[e][q] = 0;
         }
       warp_mma_32rows(smem_u32(tail_tile), lane, w, acc);
-      flush_f32(acc, ri);
+      flush_f32(acc, ri, Conv::kUnit);
       flush_i32([&](int e, int q) -> int32_t& { return ri.i[e][q]; }, cta_acc, lane);
     }
   } else if (warp == kTcMma) {
@@ -893,8 +984,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) exact_tc_kernel(const __grid_co
       tc05::tmem_hold16(v1);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        part[i] += __float2int_rn(__uint_as_float(v0[i]));
-        part[16 + i] += __float2int_rn(__uint_as_float(v1[i]));
+        part[i] += __float2int_rn(__uint_as_float(v0[i]) * Conv::kUnit);
+        part[16 + i] += __float2int_rn(__uint_as_float(v1[i]) * Conv::kUnit);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
