@@ -201,11 +201,17 @@ __device__ inline int jacobi64(double* A, int lda, double* V, int ldv, int n, Sc
 // 1, 2, .. h - 1, 2h - 1, .. h + 1, h.  After M - 1 rounds every two indices have met and all are back.
 // So with M known at compile time a thread's addresses are a few registers and immediate offsets for
 // the whole solve (rows over the warps, lanes along the pairs: all accesses conflict-free): a rotated
-// row pair costs 28 instructions, a row of V eight.  The rounds are bound by instruction issue:
-// finding pairs and addresses anew in each, order 64 took 3100 cycles a round.
-constexpr int k32Max = 96;  // largest order
+// row pair costs 28 instructions, a row of V eight.  V follows A one round behind, and its rotation
+// fills the time the angles take.  Up to order 32 every warp finds all the angles itself, a pair a
+// lane, and takes those of its row pairs by shuffles: a round has one barrier.  Above, shared memory is
+// the bound (order 64: 512 of a round's 1000 cycles) and that costs more than it saves (324 us against
+// 337 for 64 columns): one warp finds the angles while the others rotate V, then all rotate A.
+// kCross: only the h^2 pairs of an index below h and one above, in h rounds: the lower positions stay,
+// the upper ones move one place around their own ring.
+// Runs on NT threads (numbered tid), the whole block or warps that meet at barrier `bar`.
+constexpr int k32Max = 64;  // largest order
 struct Scratch32 {
-  float2 rot[2][k32Max / 2];  // (c, s) of every pair of a round
+  float2 rot[k32Max / 2];  // (c, s) of every pair of a round
   float red[8];
 };
 // floats of the work area of order m: two copies of the matrix, then two of the vectors
@@ -217,226 +223,209 @@ __device__ __forceinline__ float lds32(uint32_t a) {
   asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(OFF) : "memory");
   return v;
 }
-template <int OFF>
-__device__ __forceinline__ float2 lds64(uint32_t a) {
+__device__ __forceinline__ float2 lds_rot(uint32_t a) {
   float2 v;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "r"(a), "n"(OFF) : "memory");
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
   return v;
+}
+__device__ __forceinline__ void sts_rot(uint32_t a, float2 v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 template <int OFF>
 __device__ __forceinline__ void sts32(uint32_t a, float v) {
   asm volatile("st.shared.f32 [%0+%1], %2;" ::"r"(a), "n"(OFF), "f"(v) : "memory");
 }
 
-template <int M>
+template <int M, int NT = kThreads, bool kCross = false>
 struct Jacobi32 {
   static constexpr int h = M / 2;
   static constexpr int HP = h <= 8 ? 8 : h <= 16 ? 16 : 32;  // lanes along the pairs
-  static constexpr int NSUB = 32 / HP;                       // rows a warp takes at once
-  static constexpr int NG = (h + 31) / 32;                   // pairs of a lane
-  static constexpr int WA = (h + 31) / 32, NW = kThreads / 32 - WA;  // WA warps find the angles, NW rotate V
-  static constexpr int SA = kThreads / 32 * NSUB, SV = NW * NSUB;    // row steps
+  static constexpr int SA = NT / HP;                         // rows the warps take at once
+  static constexpr bool kSelf = h <= 16;                     // every warp finds the angles
+  static constexpr int SV = kSelf ? SA : SA - 1;             // rows of V: all warps, or all but the first
   static constexpr int UA = (h + SA - 1) / SA, UV = (M + SV - 1) / SV;
   static constexpr int kCopy = 4 * M * M;                    // bytes from one copy to the other
-  static_assert(M % 2 == 0 && M <= k32Max, "order");
+  static constexpr int kRounds = kCross ? h : M - 1;
+  // row pair i goes to rows i + kTop and h + i + kBot, but for the ends of the ring
+  static constexpr int kTop = kCross ? 0 : 1, kBot = kCross ? 1 : -1;
+  static_assert(M % 2 == 0 && M <= k32Max && (!kCross || h % 2 == 0) && (kSelf || HP == 32), "order");
 
   static __device__ __forceinline__ int next_place(int t) {
+    if (kCross) return t < h ? t : t == M - 1 ? h : t + 1;
     if (t == 0) return 0;
-    if (t < h) return t == h - 1 ? 2 * h - 1 : t + 1;
+    if (t < h) return t == h - 1 ? M - 1 : t + 1;
     return t == h ? 1 : t - 1;
   }
 
-  uint32_t rot, ang;            // rotations; the angle thread's diagonal block
-  uint32_t rj[NG], ri;          // this lane's and this row pair's rotations
-  uint32_t a;                   // A at this thread's first row pair and pair of columns
-  uint32_t dt[NG], db[NG];      // where row i + 1 of the next copy takes the two columns
-  uint32_t v, vt[NG], vb[NG];   // the same for a row of V
-  uint32_t first_t, first_b, last_t;  // rows' byte offsets from those of i + 1 and h + i - 1 at the ring's ends
-  int i0, j0, r0, tid;
+  uint32_t ang;     // the diagonal block of this lane's pair
+  uint32_t a, v;    // A at this thread's first row pair and pair of columns, V at its first row
+  uint32_t dt, db;  // where row i0 + kTop of the next copy takes the two columns
+  uint32_t vt, vb;  // the same for a row of V
+  uint32_t first_t, first_b, last_t, last_b;  // what the ends of the ring add to the rows' byte offsets
+  uint32_t rot;     // the rotations
+  int i0, r0, j0, bar;
 
-  __device__ __forceinline__ Jacobi32(const float* A, const float* V, Scratch32& S) {
-    tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5, sub = lane / HP;
-    j0 = lane % HP;
-    i0 = warp * NSUB + sub;
-    r0 = (warp - WA) * NSUB + sub;
+  __device__ __forceinline__ Jacobi32(const float* A, const float* V, Scratch32& S, int tid, int barrier) {
+    i0 = tid / HP;
+    r0 = kSelf ? i0 : i0 - 1;
     rot = smem_u32(S.rot);
-    ri = rot + 8 * i0;
-    ang = smem_u32(A) + 4 * (tid * M + tid);
-    a = smem_u32(A) + 4 * (i0 * M + j0);
-    v = smem_u32(V) + 4 * (r0 * M + j0);
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-      const int j = j0 + 32 * g, t = j < h ? next_place(j) : 0, b = j < h ? next_place(h + j) : 0;
-      rj[g] = rot + 8 * j;
-      dt[g] = smem_u32(A) + 4 * ((i0 + 1) * M + t);
-      db[g] = smem_u32(A) + 4 * ((i0 + 1) * M + b);
-      vt[g] = smem_u32(V) + 4 * (r0 * M + t);
-      vb[g] = smem_u32(V) + 4 * (r0 * M + b);
-    }
-    // row pair i goes to rows i + 1 and h + i - 1, pair 0 to 0 and 1, and pair h - 1's first row to 2h - 1
-    first_t = i0 == 0 ? static_cast<uint32_t>(-4 * M) : 0u;
-    first_b = i0 == 0 ? static_cast<uint32_t>(4 * M * (1 - (h - 1))) : 0u;
-    last_t = i0 + (UA - 1) * SA == h - 1 ? static_cast<uint32_t>(4 * M * (h - 1)) : 0u;
+    j0 = tid % HP;
+    bar = barrier;
+    const int j = min(j0, h - 1), t = next_place(j), b = next_place(h + j);
+    ang = smem_u32(A) + 4 * (j * M + j);
+    a = smem_u32(A) + 4 * (i0 * M + j);
+    v = smem_u32(V) + 4 * (r0 * M + j);
+    dt = smem_u32(A) + 4 * ((i0 + kTop) * M + t);
+    db = smem_u32(A) + 4 * ((i0 + kTop) * M + b);
+    vt = smem_u32(V) + 4 * (r0 * M + t);
+    vb = smem_u32(V) + 4 * (r0 * M + b);
+    const int i1 = i0 + (UA - 1) * SA;  // this thread's last row pair
+    first_t = i0 == 0 ? 4 * M * (next_place(0) - kTop) : 0;
+    first_b = i0 == 0 ? 4 * M * (next_place(h) - (h + kBot)) : 0;
+    last_t = i1 == h - 1 ? 4 * M * (next_place(h - 1) - (h - 1 + kTop)) : 0;
+    last_b = i1 == h - 1 ? 4 * M * (next_place(M - 1) - (M - 1 + kBot)) : 0;
   }
 
-  __device__ __forceinline__ bool lane_has(int g) const { return j0 + 32 * g < h; }
-
-  // V's columns by the rotations in rot[1 - B], from copy 1 - B to copy B (warps WA on)
-  template <int B>
-  __device__ __forceinline__ void rotate_V() const {
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-      if (!lane_has(g)) continue;
-      const float2 r = B ? lds64<0>(rj[g]) : lds64<8 * (k32Max / 2)>(rj[g]);
-      rows_of_V<B>(g, r, std::make_integer_sequence<int, UV>{});
-    }
-  }
-  template <int B, int... U>
-  __device__ __forceinline__ void rows_of_V(int g, const float2& r, std::integer_sequence<int, U...>) const {
-    float x[UV], y[UV];
-    (load_V<B, U>(g, x[U], y[U]), ...);
-    (store_V<B, U>(g, r, x[U], y[U]), ...);
-  }
   template <int B, int U>
-  __device__ __forceinline__ void load_V(int g, float& x, float& y) const {
-    if (r0 + U * SV >= M) return;
-    constexpr int o = (1 - B) * kCopy + 4 * U * SV * M;
-    x = g ? lds32<o + 128>(v) : lds32<o>(v);
-    y = g ? lds32<o + 4 * h + 128>(v) : lds32<o + 4 * h>(v);
-  }
-  template <int B, int U>
-  __device__ __forceinline__ void store_V(int g, const float2& r, float x, float y) const {
-    if (r0 + U * SV >= M) return;
-    constexpr int o = B * kCopy + 4 * U * SV * M;
-    sts32<o>(vt[g], fmaf(r.x, x, -(r.y * y)));
-    sts32<o>(vb[g], fmaf(r.y, x, r.x * y));
-  }
-
-  // row pairs of A by the rotations in rot[B] from both sides, from copy B to copy 1 - B
-  template <int B>
-  __device__ __forceinline__ void rotate_A() const {
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-      if (!lane_has(g)) continue;
-      const float2 r = B ? lds64<8 * (k32Max / 2)>(rj[g]) : lds64<0>(rj[g]);
-      pairs_of_A<B>(g, r, std::make_integer_sequence<int, UA>{});
-    }
-  }
-  template <int B, int... U>
-  __device__ __forceinline__ void pairs_of_A(int g, const float2& r, std::integer_sequence<int, U...>) const {
-    float x[UA][4];
-    float2 q[UA];
-    (load_A<B, U>(g, x[U], q[U]), ...);
-    (store_A<B, U>(g, r, x[U], q[U]), ...);
-  }
-  template <int B, int U>
-  __device__ __forceinline__ void load_A(int g, float (&x)[4], float2& q) const {
+  __device__ __forceinline__ void load_A(float (&x)[4]) const {
     if ((U + 1) * SA > h && i0 + U * SA >= h) return;
     constexpr int o = B * kCopy + 4 * U * SA * M;
-    q = lds64<8 * U * SA + B * 8 * (k32Max / 2)>(ri);
-    x[0] = g ? lds32<o + 128>(a) : lds32<o>(a);
-    x[1] = g ? lds32<o + 4 * h + 128>(a) : lds32<o + 4 * h>(a);
-    x[2] = g ? lds32<o + 4 * h * M + 128>(a) : lds32<o + 4 * h * M>(a);
-    x[3] = g ? lds32<o + 4 * h * M + 4 * h + 128>(a) : lds32<o + 4 * h * M + 4 * h>(a);
+    x[0] = lds32<o>(a);
+    x[1] = lds32<o + 4 * h>(a);
+    x[2] = lds32<o + 4 * h * M>(a);
+    x[3] = lds32<o + 4 * h * M + 4 * h>(a);
   }
   template <int B, int U>
-  __device__ __forceinline__ void store_A(int g, const float2& rj_, const float (&x)[4], const float2& q) const {
-    if ((U + 1) * SA > h && i0 + U * SA >= h) return;
-    constexpr int o = (1 - B) * kCopy + 4 * U * SA * M, ob = o + 4 * M * (h - 2);  // rows i + 1 and h + i - 1
-    const float u00 = fmaf(rj_.x, x[0], -(rj_.y * x[1])), u01 = fmaf(rj_.y, x[0], rj_.x * x[1]);
-    const float u10 = fmaf(rj_.x, x[2], -(rj_.y * x[3])), u11 = fmaf(rj_.y, x[2], rj_.x * x[3]);
-    const bool diag = i0 + U * SA == j0 + 32 * g;  // the rotated pair's own entry is zero by construction
-    const float y00 = fmaf(q.x, u00, -(q.y * u10)), y11 = fmaf(q.y, u01, q.x * u11);
-    const float y01 = diag ? 0.f : fmaf(q.x, u01, -(q.y * u11)), y10 = diag ? 0.f : fmaf(q.y, u00, q.x * u10);
-    uint32_t tt = dt[g], tb = db[g], bt = dt[g], bb = db[g];
-    if (U == 0) {
-      tt += first_t;
-      tb += first_t;
-      bt += first_b;
-      bb += first_b;
-    }
-    if (U == UA - 1) {
-      tt += last_t;
-      tb += last_t;
-    }
-    sts32<o>(tt, y00);
-    sts32<o>(tb, y01);
-    sts32<ob>(bt, y10);
-    sts32<ob>(bb, y11);
+  __device__ __forceinline__ void store_A(float c, float s, const float (&x)[4], float ci, float si) const {
+    if (((U + 1) * SA > h && i0 + U * SA >= h) || (HP > h && j0 >= h)) return;
+    constexpr int o = (1 - B) * kCopy + 4 * U * SA * M, ob = o + 4 * M * (h + kBot - kTop);
+    const float u00 = fmaf(c, x[0], -(s * x[1])), u01 = fmaf(s, x[0], c * x[1]);
+    const float u10 = fmaf(c, x[2], -(s * x[3])), u11 = fmaf(s, x[2], c * x[3]);
+    const bool diag = i0 + U * SA == j0;  // the rotated pair's own entry is zero by construction
+    const float y00 = fmaf(ci, u00, -(si * u10)), y11 = fmaf(si, u01, ci * u11);
+    const float y01 = diag ? 0.f : fmaf(ci, u01, -(si * u11)), y10 = diag ? 0.f : fmaf(si, u00, ci * u10);
+    const uint32_t top = (U == 0 ? first_t : 0u) + (U == UA - 1 ? last_t : 0u);
+    const uint32_t bot = (U == 0 ? first_b : 0u) + (U == UA - 1 ? last_b : 0u);
+    sts32<o>(dt + top, y00);
+    sts32<o>(db + top, y01);
+    sts32<ob>(dt + bot, y10);
+    sts32<ob>(db + bot, y11);
+  }
+  template <int B, int U>
+  __device__ __forceinline__ void load_V(float (&x)[2]) const {
+    if ((U + 1) * SV > M && r0 + U * SV >= M) return;
+    constexpr int o = B * kCopy + 4 * U * SV * M;
+    x[0] = lds32<o>(v);
+    x[1] = lds32<o + 4 * h>(v);
+  }
+  template <int B, int U>
+  __device__ __forceinline__ void store_V(float c, float s, const float (&x)[2]) const {
+    if (((U + 1) * SV > M && r0 + U * SV >= M) || (HP > h && j0 >= h)) return;
+    constexpr int o = (1 - B) * kCopy + 4 * U * SV * M;
+    sts32<o>(vt, fmaf(c, x[0], -(s * x[1])));
+    sts32<o>(vb, fmaf(s, x[0], c * x[1]));
   }
 
-  // one round on copy B of A; the last round's rotations of V if there are any
-  template <int B>
-  __device__ __forceinline__ void round(bool pending) const {
-    if (tid < 32 * WA) {
-      if (tid < h) {
-        const float x = lds32<B * kCopy + 4 * h>(ang);
-        const float d = lds32<B * kCopy + 4 * h * M + 4 * h>(ang) - lds32<B * kCopy>(ang);
-        const float t = fabsf(x) > 1e-18f ? tan32(d, x) : 0.f;  // the matrix is scaled to order one
-        const float c = rsqrt32(fmaf(t, t, 1.f));
-        sts32<B * 8 * (k32Max / 2)>(rot + 8 * tid, c);
-        sts32<B * 8 * (k32Max / 2) + 4>(rot + 8 * tid, t * c);
+  // V's rows by the rotations of the round before, from copy B to copy 1 - B
+  template <int B, int... W>
+  __device__ __forceinline__ void rotate_V(float2 rot, std::integer_sequence<int, W...>) const {
+    float y[UV][2];
+    (load_V<B, W>(y[W]), ...);
+    (store_V<B, W>(rot.x, rot.y, y[W]), ...);
+  }
+  __device__ __forceinline__ void meet() const {
+    if (NT == kThreads)
+      __syncthreads();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
+  }
+  // the rotation that annihilates apq
+  __device__ __forceinline__ static float2 angle(float apq, float app, float aqq) {
+    const float t = fabsf(apq) > 1e-18f ? tan32(aqq - app, apq) : 0.f;  // the matrix is scaled to order one
+    const float c = rsqrt32(fmaf(t, t, 1.f));
+    return make_float2(c, t * c);
+  }
+  // one round of A, from copy B to copy 1 - B, and (kV) of V the round before (now: the last round's
+  // rotation of this lane's pair, then this one's)
+  template <int B, bool kV, int... U, class SeqV>
+  __device__ __forceinline__ void round(float2& now, std::integer_sequence<int, U...>, SeqV uv) const {
+    float x[UA][4];
+    float2 q[UA];
+    if (kSelf) {
+      const float apq = lds32<B * kCopy + 4 * h>(ang), app = lds32<B * kCopy>(ang);
+      const float aqq = lds32<B * kCopy + 4 * h * M + 4 * h>(ang);
+      (load_A<B, U>(x[U]), ...);
+      const float2 r = angle(apq, app, aqq);
+      if (kV) rotate_V<1 - B>(now, uv);
+      now = r;
+      ((q[U].x = __shfl_sync(0xffffffffu, r.x, min(i0 + U * SA, h - 1)),
+        q[U].y = __shfl_sync(0xffffffffu, r.y, min(i0 + U * SA, h - 1))),
+       ...);
+    } else {
+      if (i0 == 0) {
+        const float apq = lds32<B * kCopy + 4 * h>(ang), app = lds32<B * kCopy>(ang);
+        const float aqq = lds32<B * kCopy + 4 * h * M + 4 * h>(ang);
+        const float2 r = angle(apq, app, aqq);
+        if (j0 < h) sts_rot(rot + 8 * j0, r);
+      } else if (kV) {
+        rotate_V<1 - B>(now, uv);
       }
-    } else if (pending) {
-      rotate_V<B>();
+      meet();
+      now = lds_rot(rot + 8 * min(j0, h - 1));
+      ((q[U] = lds_rot(rot + 8 * min(i0 + U * SA, h - 1))), ...);
+      (load_A<B, U>(x[U]), ...);
     }
-    __syncthreads();
-    rotate_A<B>();
-    __syncthreads();
+    (store_A<B, U>(now.x, now.y, x[U], q[U].x, q[U].y), ...);
+    meet();
   }
   // (by value: the copy lives in registers)
   template <int B>
-  static __device__ __noinline__ void sweep(Jacobi32 J, bool pending) {
+  static __device__ __noinline__ void sweep(Jacobi32 J) {
+    constexpr auto ua = std::make_integer_sequence<int, UA>{};
+    constexpr auto uv = std::make_integer_sequence<int, UV>{};
+    float2 now = make_float2(1.f, 0.f);
+    J.template round<B, false>(now, ua, uv);
 #pragma unroll 1
-    for (int r = 0; r < h - 1; ++r) {
-      J.template round<B>(pending);
-      J.template round<1 - B>(true);
-      pending = true;
+    for (int r = 0; r < (kRounds - 1) / 2; ++r) {
+      J.template round<1 - B, true>(now, ua, uv);
+      J.template round<B, true>(now, ua, uv);
     }
-    J.template round<B>(pending);
+    if (kRounds % 2 == 0) J.template round<1 - B, true>(now, ua, uv);
+    if (kSelf || J.i0 > 0) J.template rotate_V<kRounds % 2 ? B : 1 - B>(now, uv);
+    J.meet();
   }
 };
 
 // Cyclic Jacobi in FP32 on A (M x M floats, followed by its next copy), its rotations applied to V's
-// columns (the same).  At most max_sweeps; stops once the off-diagonal part is at the level of FP32
-// rounding.  Returns the sweeps taken; `copy`: which copies hold the results.
+// columns (the same), by the whole block.  At most max_sweeps; stops once the off-diagonal part is at
+// the level of FP32 rounding.  Returns the sweeps taken; `copy`: which copies hold the results.
 template <int M>
 __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_sweeps, Scratch32& S, int& copy) {
   const int tid = threadIdx.x;
-  const Jacobi32<M> J(A, V, S);
+  const Jacobi32<M> J(A, V, S, tid, 0);
   float prev = 0.f, fro2 = 0.f;
   int sweep = 0;
   copy = 0;
   for (; sweep < max_sweeps; ++sweep) {
-    if (max_sweeps > 1) {
-      const float* X = A + copy * M * M;
-      float off = 0.f, dia = 0.f;
-      for (int i = tid; i < M * M; i += kThreads) {
-        const float x = X[i];
-        if (i / M != i % M)
-          off = fmaf(x, x, off);
-        else
-          dia = fmaf(x, x, dia);
-      }
-      off = block_total(off, S.red);
-      if (sweep == 0) fro2 = block_total(dia, S.red) + off;
-      if (!(off > 1e-14f * fro2) || (sweep > 0 && off <= 1e-9f * fro2 && off > 0.25f * prev)) break;
-      prev = off;
+    const float* X = A + copy * M * M;
+    float off = 0.f, dia = 0.f;
+    for (int i = tid; i < M * M; i += kThreads) {
+      const float x = X[i];
+      if (i / M != i % M)
+        off = fmaf(x, x, off);
+      else
+        dia = fmaf(x, x, dia);
     }
+    off = block_total(off, S.red);
+    if (sweep == 0) fro2 = block_total(dia, S.red) + off;
+    if (!(off > 1e-14f * fro2) || (sweep > 0 && off <= 1e-9f * fro2 && off > 0.25f * prev)) break;
+    prev = off;
     if (copy == 0)
-      Jacobi32<M>::template sweep<0>(J, sweep > 0);
+      Jacobi32<M>::template sweep<0>(J);
     else
-      Jacobi32<M>::template sweep<1>(J, sweep > 0);
+      Jacobi32<M>::template sweep<1>(J);
     copy ^= 1;
   }
-  if (sweep > 0 && tid >= 32 * Jacobi32<M>::WA) {
-    if (copy == 0)
-      J.template rotate_V<0>();
-    else
-      J.template rotate_V<1>();
-  }
-  __syncthreads();
   return sweep;
 }
 // the order FP32 rotations take n columns at: a multiple of eight up to 32, of sixteen above

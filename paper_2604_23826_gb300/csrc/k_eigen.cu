@@ -3,10 +3,9 @@
 // 256-thread block per SM at most, whose blocks meet at bounded grid-wide barriers.
 //
 //   1. (seed) accepted only if its columns are orthonormal to 1e-9; T = V^T A V.  Cold: T = A, V = I.
-//   2. FP32 Jacobi on T scaled to order one: up to 96 columns in one block's shared memory (a round
-//      is two block barriers), above that block-cyclic over the grid: pairs of 16-column blocks,
-//      a 32 x 32 problem each, swept once in shared memory, then every 32 x 32 block of T and V
-//      multiplied by the pairs' rotations: two grid barriers a block round.
+//   2. FP32 Jacobi on T scaled to order one: up to 64 columns in one block's shared memory, above
+//      that block-cyclic over the grid: pairs of 16-column blocks, a 32 x 32 problem each, and every
+//      32 x 32 block of T and V multiplied by the pairs' rotations: one grid barrier a block round.
 //   3. X = V Q, then the Ogita-Aishima refinement in FP64: W = A X, S = X^T W, G = X^T X, the
 //      correction E from S, G and X <- X + X E, until E is below 5e-9 (its square is left): two or
 //      three steps of four products, each spread over the grid in 16 x 16 tiles.
@@ -31,7 +30,6 @@ constexpr int kJW = 8;         // FP64 block Jacobi: indices per block
 constexpr int kJP = 2 * kJW;   // order of a block pair's diagonal problem
 static_assert(kJP * kJP == kThreads, "one thread per entry of a block-pair tile");
 constexpr int kFW = 16, kFP = 2 * kFW;  // the same for the FP32 block Jacobi
-constexpr int kFLd = kFP + 1;
 constexpr unsigned long long kGridWaitNs = 2000000000ull;  // a grid-wide wait gives up after 2 s
 constexpr unsigned int kDead = 0x80000000u;
 
@@ -95,7 +93,7 @@ struct Shared {
   int ok;
 };
 constexpr size_t kDynFloats32 = jacobi32_floats(k32Max);  // step 2 in one block
-constexpr size_t kDynFloatsF = jacobi32_floats(kFP) + 4 * kFP * kFLd;  // step 2 over the grid
+constexpr size_t kDynFloatsF = 2 * jacobi32_floats(kFP) + 2 * kFP * kFP;  // step 2 over the grid
 constexpr size_t kDynBytes = sizeof(float) * (kDynFloats32 > kDynFloatsF ? kDynFloats32 : kDynFloatsF);
 
 // Z(i, j) = sum_k X(i, k) Y(k, j) for 16 x 16 tiles shared out over the grid; X, Y: element
@@ -177,16 +175,23 @@ __device__ double slots_max(const double* slots, Shared& S) {
 }
 
 // FP32 block-cyclic Jacobi over the grid (m a multiple of 32): A and its next copy B, V = I on entry.
+// A sweep meets every two indices once: those of a block in its first round, with the rest of the
+// pair's 32 x 32 problem, the two blocks' with one another in every round.
+// An item of a round is one 32 x 32 block of A off the pairs' diagonal (and its transpose) or one of V.
+// Its block of threads solves the two pairs' problems itself, half a block each: the same bits
+// everywhere, and a grid barrier and a trip through memory less than solving them once.  (256 columns,
+// all of the solver: 2.44 ms with full sweeps of problems solved once and two barriers a round, 1.72 so.)
 // Returns the sweeps, -1 after a wait that ran out.
-__device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float* dyn, float* A, float* B, float* V,
-                             float* Q) {
+__device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float* dyn, float* A, float* B, float* V) {
   const int m = J.m, nb = m / kFW, np = nb / 2, tid = threadIdx.x;
-  float* sA = dyn + jacobi32_floats(kFP);
-  float* sQ = sA + kFP * kFLd;
-  float* sB = sQ + kFP * kFLd;
-  float* sT = sB + kFP * kFLd;
+  constexpr int kE = kFP * kFP;
+  float* sX = dyn + 2 * jacobi32_floats(kFP);
+  float* sT = sX + kE;
   auto row_of = [](int bi, int bj, int l) { return l < kFW ? bi * kFW + l : bj * kFW + l - kFW; };
   const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
+  const int half = tid / (kThreads / 2), ht = tid % (kThreads / 2);
+  float* pA = dyn + half * jacobi32_floats(kFP);  // this half's problem: two copies, then the rotations' two
+  float* pV = pA + 2 * kE;
   double fro2 = 0.0, prev = 0.0;
   int sweep = 0;
   for (; sweep < 20; ++sweep) {
@@ -209,32 +214,8 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
     if (!(off > 1e-14 * fro2) || (sweep > 0 && off <= 1e-9 * fro2 && off > 0.25 * prev)) break;
     prev = off;
     for (int br = 0; br < nb - 1; ++br) {
-      for (int P = blockIdx.x; P < np; P += gridDim.x) {
-        int bi, bj;
-        pair_of(br, P, nb, bi, bj);
-        float* pA = dyn;
-        float* pV = dyn + 2 * kFP * kFP;
-        for (int e = tid; e < kFP * kFP; e += kThreads) {
-          const int r = e / kFP, c = e % kFP;
-          pA[e] = __ldcg(A + static_cast<size_t>(row_of(bi, bj, r)) * m + row_of(bi, bj, c));
-          pV[e] = r == c ? 1.f : 0.f;
-        }
-        __syncthreads();
-        int copy;
-        jacobi32<kFP>(pA, pV, 1, S.s32, copy);
-        pA += copy * kFP * kFP;
-        pV += copy * kFP * kFP;
-        for (int e = tid; e < kFP * kFP; e += kThreads) {
-          const int r = e / kFP, c = e % kFP;
-          __stcg(B + static_cast<size_t>(row_of(bi, bj, r)) * m + row_of(bi, bj, c), pA[e]);
-          __stcg(Q + static_cast<size_t>(P) * kFP * kFP + e, pV[e]);
-        }
-        __syncthreads();
-      }
-      if (!grid.sync()) return -1;
-      // Q_P^T A[P rows][P' cols] Q_P' for P < P' (and its transpose), and V[strip][P' cols] Q_P'
-      const int nA = np * (np - 1) / 2, nItems = nA + (m / kFP) * np;
-      const int tr = (tid / 16) * 2, tc = (tid % 16) * 2;
+      const int copy = br == 0 ? 1 : 0;  // where the problems' results lie: 31 rounds, then 16 each
+      const int nA = np * (np - 1) / 2, nItems = nA + np * np;
       for (int it = blockIdx.x; it < nItems; it += gridDim.x) {
         const bool isA = it < nA;
         int P1 = 0, P2, bi = 0, bj = 0, ci, cj;
@@ -247,44 +228,90 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
           P2 += P1 + 1;
           pair_of(br, P1, nb, bi, bj);
         } else {
-          P1 = (it - nA) / np;  // strip
+          P1 = (it - nA) / np;  // strip of V
           P2 = (it - nA) % np;
         }
         pair_of(br, P2, nb, ci, cj);
-        for (int e = tid; e < kFP * kFP; e += kThreads) {
-          const int r = e / kFP, c = e % kFP;
-          const int gr = isA ? row_of(bi, bj, r) : P1 * kFP + r;
-          sA[r * kFLd + c] = __ldcg((isA ? A : V) + static_cast<size_t>(gr) * m + row_of(ci, cj, c));
-          sB[r * kFLd + c] = __ldcg(Q + static_cast<size_t>(P2) * kFP * kFP + e);
-          if (isA) sQ[r * kFLd + c] = __ldcg(Q + static_cast<size_t>(P1) * kFP * kFP + e);
+        const bool solves = isA || half == 1;
+        if (solves) {
+          const int di = half ? ci : bi, dj = half ? cj : bj;
+          float x[kE / (kThreads / 2)];
+#pragma unroll
+          for (int u = 0; u < kE / (kThreads / 2); ++u) {
+            const int e = ht + u * (kThreads / 2), r = e / kFP, c = e % kFP;
+            x[u] = __ldcg(A + static_cast<size_t>(row_of(di, dj, r)) * m + row_of(di, dj, c));
+          }
+#pragma unroll
+          for (int u = 0; u < kE / (kThreads / 2); ++u) {
+            const int e = ht + u * (kThreads / 2);
+            pA[e] = x[u];
+            pV[e] = e / kFP == e % kFP ? 1.f : 0.f;
+          }
+        }
+        {
+          float x[kE / kThreads];
+#pragma unroll
+          for (int u = 0; u < kE / kThreads; ++u) {
+            const int e = tid + u * kThreads, r = e / kFP, c = e % kFP;
+            const int gr = isA ? row_of(bi, bj, r) : P1 * kFP + r;
+            x[u] = __ldcg((isA ? A : V) + static_cast<size_t>(gr) * m + row_of(ci, cj, c));
+          }
+#pragma unroll
+          for (int u = 0; u < kE / kThreads; ++u) sX[tid + u * kThreads] = x[u];
         }
         __syncthreads();
-        float* L = sA;
-        if (isA) {
+        if (solves) {  // (the halves are whole warps, and meet at barriers of their own)
+          if (br == 0) {
+            const Jacobi32<kFP, kThreads / 2, false> K(pA, pV, S.s32, ht, 1 + half);
+            K.template sweep<0>(K);
+          } else {
+            const Jacobi32<kFP, kThreads / 2, true> K(pA, pV, S.s32, ht, 1 + half);
+            K.template sweep<0>(K);
+          }
+        }
+        __syncthreads();
+        const float* Q1 = dyn + 2 * kE + copy * kE;
+        const float* Q2 = Q1 + jacobi32_floats(kFP);
+        if (!isA && P1 == 0) {  // the pair's own problem, once
+          const float* D = dyn + jacobi32_floats(kFP) + copy * kE;
+#pragma unroll
+          for (int u = 0; u < kE / kThreads; ++u) {
+            const int e = tid + u * kThreads, r = e / kFP, c = e % kFP;
+            __stcg(B + static_cast<size_t>(row_of(ci, cj, r)) * m + row_of(ci, cj, c), D[e]);
+          }
+        }
+        const int tr = (tid / 16) * 2, tc = (tid % 16) * 2;
+        const float* L = sX;
+        if (isA) {  // T = Q1^T X
           float t00 = 0.f, t01 = 0.f, t10 = 0.f, t11 = 0.f;
 #pragma unroll 8
           for (int k = 0; k < kFP; ++k) {
-            const float a0 = sQ[k * kFLd + tr], a1 = sQ[k * kFLd + tr + 1], b0 = sA[k * kFLd + tc], b1 = sA[k * kFLd + tc + 1];
-            t00 = fmaf(a0, b0, t00);
-            t01 = fmaf(a0, b1, t01);
-            t10 = fmaf(a1, b0, t10);
-            t11 = fmaf(a1, b1, t11);
+            const float2 x = *reinterpret_cast<const float2*>(Q1 + k * kFP + tr);
+            const float2 y = *reinterpret_cast<const float2*>(sX + k * kFP + tc);
+            t00 = fmaf(x.x, y.x, t00);
+            t01 = fmaf(x.x, y.y, t01);
+            t10 = fmaf(x.y, y.x, t10);
+            t11 = fmaf(x.y, y.y, t11);
           }
-          sT[tr * kFLd + tc] = t00;
-          sT[tr * kFLd + tc + 1] = t01;
-          sT[(tr + 1) * kFLd + tc] = t10;
-          sT[(tr + 1) * kFLd + tc + 1] = t11;
+          *reinterpret_cast<float2*>(sT + tr * kFP + tc) = make_float2(t00, t01);
+          *reinterpret_cast<float2*>(sT + (tr + 1) * kFP + tc) = make_float2(t10, t11);
           __syncthreads();
           L = sT;
         }
         float y[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll 8
-        for (int k = 0; k < kFP; ++k) {
-          const float a0 = L[tr * kFLd + k], a1 = L[(tr + 1) * kFLd + k], b0 = sB[k * kFLd + tc], b1 = sB[k * kFLd + tc + 1];
-          y[0][0] = fmaf(a0, b0, y[0][0]);
-          y[0][1] = fmaf(a0, b1, y[0][1]);
-          y[1][0] = fmaf(a1, b0, y[1][0]);
-          y[1][1] = fmaf(a1, b1, y[1][1]);
+#pragma unroll 2
+        for (int k = 0; k < kFP; k += 4) {
+          const float4 a = *reinterpret_cast<const float4*>(L + tr * kFP + k);
+          const float4 b = *reinterpret_cast<const float4*>(L + (tr + 1) * kFP + k);
+          const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float2 q = *reinterpret_cast<const float2*>(Q2 + (k + u) * kFP + tc);
+            y[0][0] = fmaf(av[u], q.x, y[0][0]);
+            y[0][1] = fmaf(av[u], q.y, y[0][1]);
+            y[1][0] = fmaf(bv[u], q.x, y[1][0]);
+            y[1][1] = fmaf(bv[u], q.y, y[1][1]);
+          }
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u)
@@ -551,9 +578,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
           case 16: n = jacobi32<16>(sA, sV, 20, S.s32, copy); break;
           case 32: n = jacobi32<32>(sA, sV, 20, S.s32, copy); break;
           case 48: n = jacobi32<48>(sA, sV, 20, S.s32, copy); break;
-          case 64: n = jacobi32<64>(sA, sV, 20, S.s32, copy); break;
-          case 80: n = jacobi32<80>(sA, sV, 20, S.s32, copy); break;
-          default: n = jacobi32<96>(sA, sV, 20, S.s32, copy); break;
+          default: n = jacobi32<64>(sA, sV, 20, S.s32, copy); break;
         }
         sV += copy * m * m;
         for (int i = tid; i < m * m; i += kThreads) __stcg(Q32 + i, sV[i]);
@@ -568,7 +593,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
       }
       alive = grid.sync();
       if (alive) {
-        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32, reinterpret_cast<float*>(J.q));
+        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32);
         alive = sweeps >= 0;
       }
     }

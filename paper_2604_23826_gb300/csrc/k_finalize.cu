@@ -269,9 +269,21 @@ __device__ void put_eigenpairs(const double* lambda, const double* V, int ld, in
 }
 
 // Z(i, j) = sum_k X(k, i) Y(k, j) for 2 x 2 tiles shared out over the block's threads (FP64-bound: a
-// tile's four multiply-adds take 256 cycles a warp, its loads hide behind them)
+// tile's four multiply-adds take 256 cycles a warp, its loads hide behind them), or, up to kOneByOne
+// columns, whose tiles would not fill the SM's four FP64 units, an entry a thread (11 columns:
+// 2816 cycles in tiles, 704 so).
+constexpr int kOneByOne = 16;
 template <class FX, class FY, class Put>
 __device__ __forceinline__ void block_product(int n, FX&& X, FY&& Y, Put&& put) {
+  if (n <= kOneByOne) {
+    const int t = threadIdx.x, i = t / n, j = t % n;
+    if (i < n) {
+      double z = 0.0;
+      for (int k = 0; k < n; ++k) z = fma(X(k, i), Y(k, j), z);
+      put(i, j, z);
+    }
+    return;
+  }
   const int nt = (n + 1) / 2;
   for (int t = threadIdx.x; t < nt * nt; t += kThreads) {
     const int i0 = 2 * (t / nt), j0 = 2 * (t % nt), i1 = min(i0 + 1, n - 1), j1 = min(j0 + 1, n - 1);
@@ -342,9 +354,24 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
           [&](int i, int j, double v) { W[i * ld + j] = v; });
       __syncthreads();
       // X^T W on and above the diagonal of S, X^T X below it (its diagonal in gd)
-      const int nt = (n + 1) / 2, half = nt * (nt + 1) / 2;
+      const bool single = kGraded && n <= kOneByOne;
+      const int nt = single ? n : (n + 1) / 2, half = nt * (nt + 1) / 2;
       for (int t = tid; t < 2 * half; t += kThreads) {
         const bool gram = t >= half;
+        if (single) {
+          int i, j;
+          packed_entry(gram ? t - half : t, n, i, j);
+          const double* Y = gram ? X : W;
+          double z = 0.0;
+          for (int k = 0; k < n; ++k) z = fma(X[k * ld + i], Y[k * ld + j], z);
+          if (!gram)
+            S[i * ld + j] = z;
+          else if (i == j)
+            M.gd[i] = z;
+          else
+            S[j * ld + i] = z;
+          continue;
+        }
         int I, Jt;
         packed_entry(gram ? t - half : t, nt, I, Jt);
         const double* Y = gram ? X : W;

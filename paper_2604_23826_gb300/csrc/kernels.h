@@ -415,8 +415,8 @@ struct JacobiParams {
   int64_t wait_ns;          // limit of one grid-wide wait (<= 0: 2 s)
   int32_t absent_block;     // testing: this block leaves before its first arrival (-1: none)
 };
-// Order of the padded matrix: a multiple of 16, of 32 above 96 (the FP32 rotations' block pairs).
-__host__ __device__ inline int jacobi_order(int pa) { return pa <= 96 ? (pa + 15) / 16 * 16 : (pa + 31) / 32 * 32; }
+// Order of the padded matrix: a multiple of 16, of 32 above 64 (the FP32 rotations' block pairs).
+__host__ __device__ inline int jacobi_order(int pa) { return pa <= 64 ? (pa + 15) / 16 * 16 : (pa + 31) / 32 * 32; }
 // Doubles of scratch jacobi_grid_kernel needs for pa analysis columns.
 size_t jacobi_scratch_doubles(int pa);
 // Blocks of the cooperative grid for pa columns on a device of `sms` SMs (0: not possible).
