@@ -25,8 +25,7 @@
 //   warp 1      tensor memory (allocated by both CTAs together) and, in the leader, the MMA
 //               issuer: it waits until both CTAs have converted the stage and drained the
 //               accumulator buffer, issues the stage's MMAs, and commits to the stage-free and
-//               (at a chain's end) chain-done barriers of both CTAs (multicast); in the peer,
-//               one thread relays the epilogue's drained chains to the leader;
+//               (at a chain's end) chain-done barriers of both CTAs (multicast);
 //   warps 2-3   in the peer, relays of converted stages (warp 2 the even stages, warp 3 the
 //               odd): the converter warps arrive on local barriers, and a relay thread forwards
 //               each completed phase to the leader with a single cluster-scope arrive (a release
@@ -37,7 +36,15 @@
 //               and (BF16x3) sums of l^2;
 //   warps 8-15  epilogue: two warps per TMEM lane quarter, 128 columns each; every chain is
 //               added into FP32 registers (round to nearest), and every flush into (hi, lo)
-//               pairs in the CTA's slot.
+//               pairs in the CTA's slot.  Its warps tell the leader that a buffer is drained by
+//               relaxed cluster-scope arrivals: only tensor memory changes hands, which the
+//               tcgen05 fences order, so nothing waits for a release.
+// Bound: the two accumulator buffers.  Of a 64-row stage's 2350 cycles the MMAs take 1100 and the
+// issuer waited 900 for a drained buffer: the drain (16 columns a load, the next load in flight while
+// one is added) and the two crossings of the pair are longer than the other buffer's MMAs.  Relayed
+// and unpipelined drains: 1.2e7 rows x 256, BF16x3, 3.04 ms; now 2.89 (4.25 TB/s); 1e7 x 200, BF16x4,
+// 2.81 ms, now 2.63.  Registers 96 / 160: 2.99 and 2.79, 80 / 176: 2.97 and 2.63 (spills on one side
+// or the other).  Eight converter warps (of 56 or 64 registers) were slower: 3.1 to 4.0 ms.
 // A second kernel adds the pairs' slots, in pair order, into the context's double-double
 // accumulators.  Every wait is bounded; on expiry the CTA records STATS_ETIMEOUT and winds
 // down; both CTAs always reach the final cluster barrier (no early exit).
@@ -67,7 +74,7 @@ constexpr int kPStages = 6;                      // 192 KB ring
 constexpr int kPThreads = 512;
 constexpr int kPConv = 4;                        // converter warps 4..7, four 8-column groups each
 constexpr int kPEpi = 8;                         // epilogue warps 8..15
-constexpr int kPRegsLow = 96, kPRegsEpi = 160;   // 2 x 128 x 96 + 2 x 128 x 160 = 65536
+constexpr int kPRegsLow = 88, kPRegsEpi = 168;   // 2 x 128 x 88 + 2 x 128 x 168 = 65536
 constexpr int kPGroupsAtOnce = 2;  // 8-column groups a converter warp loads before converting
 constexpr uint32_t kPLbo = 256, kPSbo = 2048;    // next K group (8 rows), next 8 operand rows
 constexpr int kPTmemCols = 512;                  // two 256-column accumulators
@@ -87,6 +94,11 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* local, uint32_t ran
 }
 __device__ __forceinline__ void arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// the same without ordering the thread's writes: for hand-overs of tensor memory, which the tcgen05
+// fences on both sides order
+__device__ __forceinline__ void arrive_cluster_relaxed(uint32_t cluster_bar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 __device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity, uint32_t ns) {
   uint32_t ok;
@@ -133,7 +145,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     wide2_kernel(const __grid_constant__ Wide2Params P) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t f_full[kPStages], c_full[kPStages], f_empty[kPStages], d_full[2], d_empty[2],
-      fin, r_conv[kPStages], r_epi[2];
+      fin, r_conv[kPStages];
   __shared__ uint32_t s_tmem;
   __shared__ volatile unsigned int s_dead;
   __shared__ int s_rows[kPStages];
@@ -157,8 +169,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&d_full[b], 1);
-      mbar_init(&d_empty[b], kPEpi + 1);  // the leader's: its epilogue warps + the peer's relay
-      mbar_init(&r_epi[b], kPEpi);        // the peer's: its epilogue warps, forwarded by the relay
+      mbar_init(&d_empty[b], 2 * kPEpi);  // the leader's: both CTAs' epilogue warps
     }
     mbar_init(&fin, 1);
     s_dead = 0;
@@ -210,25 +221,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       }
     }
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer (leader) / relay (peer)
-    if (!leader && lane == 0) {
-      // the peer's epilogue warps arrive on local barriers; this thread forwards each drained
-      // chain to the leader (one cluster-scope arrive per chain)
-      const uint32_t remote0 = cluster_addr(&d_empty[0], 0);
-      int b = 0;
-      uint32_t ph = 0;
-      for (int64_t k = 0; k < nchains; ++k) {
-        if (!tc05::wait_live(&r_epi[b], ph, &s_dead)) {
-          record_timeout(&s_dead, P.status);
-          break;
-        }
-        arrive_cluster(remote0 + static_cast<uint32_t>(b * sizeof(uint64_t)));
-        if (++b == 2) {
-          b = 0;
-          ph ^= 1u;
-        }
-      }
-    }
+    // ---------------------------------------------------------------- MMA issuer (leader)
     if (leader) {
       int s = 0, bd = 0;
       uint32_t ph = 0, phd = 0;
@@ -385,7 +378,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
             for (int q = 0; q < 4; ++q) {
               h[q] = pack_bf16x2(r[q].x, r[q].y);
               e[q] = __ffma2_rn(make_float2(bf_lo(h[q]), bf_hi(h[q])), m1, r[q]);  // r - h, exact
-              l[q] = X4 ? pack_bf16x2(e[q].x, e[q].y) : pack_bf16x2(2.f * e[q].x, 2.f * e[q].y);
+              const float2 le = X4 ? e[q] : __fadd2_rn(e[q], e[q]);
+              l[q] = pack_bf16x2(le.x, le.y);
             }
             t = __fadd2_rn(t, __fadd2_rn(__fadd2_rn(r[0], r[1]), __fadd2_rn(r[2], r[3])));
             if (!X4)
@@ -433,7 +427,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     const int quarter = warp & 3;                 // TMEM lanes 32 quarter .. 32 quarter + 31
     const int half = (warp - 8) >> 2;             // accumulator columns 128 half .. 128 half + 127
     const int m = 32 * quarter + lane;            // this thread's row of the CTA's 128 x 256 half
-    uint64_t* ebar = leader ? d_empty : r_epi;  // the leader's own barrier, or the peer's relay
+    const uint32_t ebar = cluster_addr(d_empty, 0);
     float acc[128];
 #pragma unroll
     for (int i = 0; i < 128; ++i) acc[i] = 0.f;
@@ -468,20 +462,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t taddr =
           tmem + (static_cast<uint32_t>(32 * quarter) << 16) + static_cast<uint32_t>(bd * 256 + 128 * half);
-      // one 16-column load per wait (registers: 128 sums + 16); the warp sharing this SMSP
-      // covers the load latency
+      // the next 16 columns in flight while these are added
+      uint32_t v[2][16];
+      tc05::tmem_ld16_issue(taddr, v[0]);
 #pragma unroll
-      for (int c0 = 0; c0 < 128; c0 += 16) {
-        uint32_t v[16];
-        tc05::tmem_ld16_issue(taddr + c0, v);
+      for (int c = 0; c < 8; ++c) {
         tc05::tmem_wait_ld();
-        tc05::tmem_hold16(v);
+        tc05::tmem_hold16(v[c & 1]);
+        if (c < 7) tc05::tmem_ld16_issue(taddr + 16 * (c + 1), v[(c + 1) & 1]);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) acc[c0 + i] += __uint_as_float(v[i]);
+        for (int i = 0; i < 16; ++i) acc[16 * c + i] += __uint_as_float(v[c & 1][i]);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ebar[bd]);
+      if (lane == 0) arrive_cluster_relaxed(ebar + static_cast<uint32_t>(bd * sizeof(uint64_t)));
       if (++bd == 2) {
         bd = 0;
         phd ^= 1u;
