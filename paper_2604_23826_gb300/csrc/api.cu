@@ -476,9 +476,12 @@ stats_status run_gram32(const std::vector<Gram32Job>& jobs, cudaStream_t st) {
         for (size_t i = 0; i < nt; ++i) total += (all[first + i]->nrows + rs - 1) / rs;
         if (total >= (int64_t(1) << 31)) return STATS_EINVAL;  // over 2^31 stages in one call
         // chunks as long as possible while every CTA still gets >= chunks_per_cta of them (long
-        // runs: few per-table partials; many chunks: balanced CTAs), and never below min_chunk
+        // runs: few per-table partials; many chunks: balanced CTAs), and not below min_chunk unless that
+        // leaves SMs without one (the small tables of a batch of 256 ran on one to five SMs, 210 us,
+        // and dealt to all in 33; one table of 3e5 rows x 8: 42 and 6 us)
         const stats_batch_tuning tune = batch_tuning(P, x4 == 1);
-        const int64_t K = std::max<int64_t>(tune.gram32_min_chunk, total / (int64_t(sms) * tune.gram32_chunks_per_cta));
+        const int64_t K = std::max<int64_t>(std::min<int64_t>(tune.gram32_min_chunk, (total + sms - 1) / sms),
+                                            total / (int64_t(sms) * tune.gram32_chunks_per_cta));
         const int grid = static_cast<int>(std::min<int64_t>((total + K - 1) / K, sms));
         const size_t sf = gram32_slot_floats(P);
         size_t slot_floats_total = 0;
