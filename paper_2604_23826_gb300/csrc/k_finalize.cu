@@ -268,13 +268,37 @@ __device__ void put_eigenpairs(const double* lambda, const double* V, int ld, in
   __syncthreads();
 }
 
-// Z(i, j) = sum_k X(k, i) Y(k, j) for 2 x 2 tiles shared out over the block's threads (FP64-bound: a
+// The blocks that work on one decomposition together: a cluster, or one block alone.  Each holds all
+// matrices in its own shared memory; a product's entries are dealt to all of them and put into every
+// copy.
+struct Team {
+  int rank, size;
+  __device__ __forceinline__ void put(double* p, double v) const {
+    *p = v;
+    for (int d = 1; d < size; ++d) {
+      uint32_t a;
+      const int to = rank + d < size ? rank + d : rank + d - size;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(to));
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+    }
+  }
+  // all of the team's threads, with what they have put
+  __device__ __forceinline__ void meet() const {
+    if (size > 1)
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else
+      __syncthreads();
+  }
+};
+constexpr int kTeamMax = 4;
+
+// Z(i, j) = sum_k X(k, i) Y(k, j) for 2 x 2 tiles shared out over the team's threads (FP64-bound: a
 // tile's four multiply-adds take 256 cycles a warp, its loads hide behind them), or, up to kOneByOne
 // columns, whose tiles would not fill the SM's four FP64 units, an entry a thread (11 columns:
 // 2816 cycles in tiles, 704 so).
 constexpr int kOneByOne = 16;
 template <class FX, class FY, class Put>
-__device__ __forceinline__ void block_product(int n, FX&& X, FY&& Y, Put&& put) {
+__device__ __forceinline__ void team_product(const Team& team, int n, FX&& X, FY&& Y, Put&& put) {
   if (n <= kOneByOne) {
     const int t = threadIdx.x, i = t / n, j = t % n;
     if (i < n) {
@@ -285,7 +309,7 @@ __device__ __forceinline__ void block_product(int n, FX&& X, FY&& Y, Put&& put) 
     return;
   }
   const int nt = (n + 1) / 2;
-  for (int t = threadIdx.x; t < nt * nt; t += kThreads) {
+  for (int t = threadIdx.x + team.rank * kThreads; t < nt * nt; t += team.size * kThreads) {
     const int i0 = 2 * (t / nt), j0 = 2 * (t % nt), i1 = min(i0 + 1, n - 1), j1 = min(j0 + 1, n - 1);
     double z00 = 0.0, z01 = 0.0, z10 = 0.0, z11 = 0.0;
     for (int k = 0; k < n; ++k) {
@@ -308,17 +332,22 @@ struct MixedScratch {
     Scratch64 s64;
   };
   double lambda[kEigBlockMax], gd[kEigBlockMax], red[8];
+  double found[kTeamMax][2];  // each block's largest correction and what it found bad
 };
 
 // Eigenpairs of A (n x n, 1 <= n <= 64, anywhere) in one block: FP32 Jacobi, FP64 refinement, and FP64
 // Jacobi from the refined basis where eigenvalues are too close for it (or from A as it is).  X, W, S:
 // shared memory of leading dimension ld (odd, above n), S right behind W.  The eigenvalues are left in M.lambda, the
 // vectors in the columns of X (which may become the buffer S or W was).  Returns the sweeps taken.
+// A team shares the refinement (not kGraded); the rotations, and everything decided, all its blocks do
+// alike.
 // kGraded (at most 23 columns; else at least 24): the refinement goes on until an off-diagonal is small against its own two eigenvalues, not
 // only against the largest, as covariances of columns of very different units want it.
 template <bool kGraded>
-__device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double* S, int ld, MixedScratch& M) {
-  const int tid = threadIdx.x;
+__device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double* S, int ld, MixedScratch& M,
+                           const Team& team) {
+  const int tid = threadIdx.x, first = tid + team.rank * kThreads, step = team.size * kThreads;
+  const Team alone{0, 1};
   double f = 0.0;
   for (int i = tid; i < n * n; i += kThreads) f = fma(A[i], A[i], f);
   const double fro2 = block_total(f, M.red);
@@ -346,17 +375,17 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
                          : jacobi32<64>(fA, fV, 20, M.s32, copy);
     fV += copy * m * m;
     for (int i = tid; i < n * n; i += kThreads) X[(i / n) * ld + i % n] = f32_to_f64(fV[(i / n) * m + i % n]);
-    __syncthreads();
+    team.meet();  // the others may put into W and S now
     const double unit = 16.0 * 1.1102230246251565e-16, noise = unit * sqrt(fro2);
     for (int it = 0; it < 5; ++it) {
-      block_product(
-          n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
-          [&](int i, int j, double v) { W[i * ld + j] = v; });
-      __syncthreads();
+      team_product(
+          team, n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
+          [&](int i, int j, double v) { team.put(W + i * ld + j, v); });
+      team.meet();
       // X^T W on and above the diagonal of S, X^T X below it (its diagonal in gd)
       const bool single = kGraded && n <= kOneByOne;
       const int nt = single ? n : (n + 1) / 2, half = nt * (nt + 1) / 2;
-      for (int t = tid; t < 2 * half; t += kThreads) {
+      for (int t = first; t < 2 * half; t += step) {
         const bool gram = t >= half;
         if (single) {
           int i, j;
@@ -386,12 +415,7 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
         }
         auto put = [&](int i, int j, double v) {
           if (i > j) return;
-          if (!gram)
-            S[i * ld + j] = v;
-          else if (i == j)
-            M.gd[i] = v;
-          else
-            S[j * ld + i] = v;
+          team.put(!gram ? S + i * ld + j : i == j ? M.gd + i : S + j * ld + i, v);
         };
         put(i0, j0, z00);
         put(i0, j1, z01);
@@ -400,26 +424,37 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
           put(i1, j1, z11);
         }
       }
-      __syncthreads();
+      team.meet();
       if (tid < n) M.lambda[tid] = S[tid * ld + tid] / M.gd[tid];
       __syncthreads();
       int bad = 0;
       double mx = 0.0;
-      for (int i = tid; i < n * n; i += kThreads) {
+      for (int i = first; i < n * n; i += step) {
         const int r = i / n, c = i % n, lo = min(r, c), hi = max(r, c);
         const double lr = M.lambda[r], lc = M.lambda[c];
         const double e = correction(r, c, S[lo * ld + hi], r == c ? M.gd[r] : S[hi * ld + lo], lr, lc,
                                     kGraded ? unit * sqrt(fabs(lr * lc)) : noise, bad);
         mx = fmax(mx, fabs(e));
-        W[r * ld + c] = e;
+        team.put(W + r * ld + c, e);
       }
       mx = block_max(mx, M.red);
       bad = block_max(bad, reinterpret_cast<int*>(M.red));
+      if (team.size > 1) {
+        if (tid == 0) {
+          team.put(&M.found[team.rank][0], mx);
+          team.put(&M.found[team.rank][1], bad > 1 ? 2.0 : bad ? 1.0 : 0.0);
+        }
+        team.meet();
+        for (int r = 0; r < team.size; ++r) {
+          mx = fmax(mx, M.found[r][0]);
+          bad = max(bad, M.found[r][1] > 1.5 ? 2 : M.found[r][1] > 0.5 ? 1 : 0);
+        }
+      }
       if (bad > 1 || mx > 0.5) break;  // not a refinement any more
-      block_product(
-          n, [&](int k, int i) { return X[i * ld + k]; }, [&](int k, int j) { return W[k * ld + j]; },
-          [&](int i, int j, double v) { S[i * ld + j] = X[i * ld + j] + v; });
-      __syncthreads();
+      team_product(
+          team, n, [&](int k, int i) { return X[i * ld + k]; }, [&](int k, int j) { return W[k * ld + j]; },
+          [&](int i, int j, double v) { team.put(S + i * ld + j, X[i * ld + j] + v); });
+      team.meet();
       double* t = X;
       X = S;
       S = t;
@@ -432,12 +467,12 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
   }
   if (!refined) {
     if (warm) {  // FP64 Jacobi on X^T A X, from the refined basis
-      block_product(
-          n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
+      team_product(
+          alone, n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
           [&](int i, int j, double v) { W[i * ld + j] = v; });
       __syncthreads();
-      block_product(
-          n, [&](int k, int i) { return X[k * ld + i]; }, [&](int k, int j) { return W[k * ld + j]; },
+      team_product(
+          alone, n, [&](int k, int i) { return X[k * ld + i]; }, [&](int k, int j) { return W[k * ld + j]; },
           [&](int i, int j, double v) {
             if (i <= j) S[i * ld + j] = S[j * ld + i] = v;
           });
@@ -608,7 +643,8 @@ __device__ void finalize_body(const FinalParams& P) {
     // the batched eigen-solver takes over
   } else if (pa <= kSmallMax) {
     double* X = U.small.X;
-    const int sweeps = eigen_mixed<true>(src, pa, X, U.small.W, U.small.S, kSmallLd, U.small.scratch);
+    const int sweeps = eigen_mixed<true>(src, pa, X, U.small.W, U.small.S, kSmallLd, U.small.scratch,
+                                        Team{0, 1});
     put_eigenpairs(U.small.scratch.lambda, X, kSmallLd, pa, s_order, out + L.evals, out + L.evecs);
     if (tid == 0) {
       flags[2] = sweeps;
@@ -726,15 +762,24 @@ static_assert(jacobi32_floats(kBatchMax) <= 2 * 2 * kBatchMax * kBatchLd, "the F
 
 }  // namespace
 
+// A job a cluster of 1, 2 or 4 blocks.  Bound: the refinement's FP64 products, 68 us each for 64 columns
+// on one SM (two steps of three such), next to 200 us of rotations, which every block of a cluster does
+// alike.  126 matrices of 24 to 64 columns: one block each 838 us, two 551; 63 matrices 804 and, four
+// each, 447.  (Past two blocks an SM the repeated rotations would cost more than the shared products
+// save.)
 __global__ void __launch_bounds__(kThreads, 2) eig_batched_kernel(const EigJob* __restrict__ jobs) {
   extern __shared__ __align__(16) double dynd[];
   __shared__ MixedScratch M;
   __shared__ int s_order[256];
-  const EigJob job = jobs[blockIdx.x];
+  Team team;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(team.rank));
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(team.size));
+  const EigJob job = jobs[blockIdx.x / team.size];
   if (job.flags[7] == 0.0) return;  // the finalize kernel found the eigenpairs undefined
   double* X = dynd;
   const int sweeps = eigen_mixed<false>(job.matrix, job.n, X, dynd + kBatchMax * kBatchLd, dynd + 2 * kBatchMax * kBatchLd,
-                                        kBatchLd, M);
+                                        kBatchLd, M, team);
+  if (team.rank != 0) return;
   put_eigenpairs(M.lambda, X, kBatchLd, job.n, s_order, job.evals, job.evecs);
   if (threadIdx.x == 0) {
     job.flags[2] = sweeps;
@@ -752,8 +797,23 @@ cudaError_t launch_finalize_batched(const FinalParams* d_params, int count, cons
   if (e != cudaSuccess || njobs <= 0) return e;
   e = cudaFuncSetAttribute(eig_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBatchBytes));
   if (e != cudaSuccess) return e;
-  eig_batched_kernel<<<njobs, kThreads, kBatchBytes, stream>>>(d_jobs);
-  return cudaGetLastError();
+  // as many blocks a job as still run side by side, two on an SM
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int size = 4 * njobs <= 2 * sms ? 4 : 2 * njobs <= 2 * sms ? 2 : 1;
+  cudaLaunchAttribute cluster{};
+  cluster.id = cudaLaunchAttributeClusterDimension;
+  cluster.val.clusterDim.x = size;
+  cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(njobs * size);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kBatchBytes;
+  cfg.stream = stream;
+  cfg.attrs = &cluster;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, eig_batched_kernel, d_jobs);
 }
 
 cudaError_t launch_finalize(const FinalParams& P, cudaStream_t stream) {
