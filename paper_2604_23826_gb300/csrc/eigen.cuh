@@ -339,11 +339,18 @@ struct Jacobi32 {
     else
       asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
   }
-  // the rotation that annihilates apq
+  // The rotation (c, s) that annihilates apq, |angle| <= pi / 4: cos(2 angle) = |d| / sqrt(d^2 + 4 apq^2),
+  // d = aqq - app, then c and s from the half-angle formulas, and c once more from c^2 + s^2 = 1 (the
+  // roots' last bits would change the vectors' lengths, round after round): a chain of two reciprocal
+  // roots, where the tangent's had four special functions.
   __device__ __forceinline__ static float2 angle(float apq, float app, float aqq) {
-    const float t = fabsf(apq) > 1e-18f ? tan32(aqq - app, apq) : 0.f;  // the matrix is scaled to order one
-    const float c = rsqrt32(fmaf(t, t, 1.f));
-    return make_float2(c, t * c);
+    const float d = aqq - app;
+    const float r = rsqrt32(fmaf(d, d, 4.f * apq * apq));
+    const float c2 = fmaf(0.5f * fabsf(d), r, 0.5f);
+    const float y = rsqrt32(c2), c = c2 * y, s = (d >= 0.f ? apq : -apq) * r * y;
+    const float e = fmaf(c, c, fmaf(s, s, -1.f));
+    const bool turn = fabsf(apq) > 1e-18f;  // the matrix is scaled to order one
+    return make_float2(turn ? fmaf(-0.5f * e, y, c) : 1.f, turn ? s : 0.f);
   }
   // one round of A, from copy B to copy 1 - B, and (kV) of V the round before (now: the last round's
   // rotation of this lane's pair, then this one's)
@@ -418,7 +425,9 @@ __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_
     }
     off = block_total(off, S.red);
     if (sweep == 0) fro2 = block_total(dia, S.red) + off;
-    if (!(off > 1e-14f * fro2) || (sweep > 0 && off <= 1e-9f * fro2 && off > 0.25f * prev)) break;
+    // (mixed units, which only the smaller orders' refinement looks at closely, want more)
+    const float done = M <= 24 ? 1e-14f : 1e-12f;
+    if (!(off > done * fro2) || (sweep > 0 && off <= 1e-9f * fro2 && off > 0.25f * prev)) break;
     prev = off;
     if (copy == 0)
       Jacobi32<M>::template sweep<0>(J);

@@ -180,7 +180,7 @@ __device__ double slots_max(const double* slots, Shared& S) {
 // An item of a round is one 32 x 32 block of A off the pairs' diagonal (and its transpose) or one of V.
 // Its block of threads solves the two pairs' problems itself, half a block each: the same bits
 // everywhere, and a grid barrier and a trip through memory less than solving them once.  (256 columns,
-// all of the solver: 2.44 ms with full sweeps of problems solved once and two barriers a round, 1.72 so.)
+// all of the solver: 2.44 ms with full sweeps of problems solved once and two barriers a round, 1.64 so.)
 // Returns the sweeps, -1 after a wait that ran out.
 __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float* dyn, float* A, float* B, float* V) {
   const int m = J.m, nb = m / kFW, np = nb / 2, tid = threadIdx.x;
@@ -211,7 +211,7 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
     if (!grid.sync()) return -1;
     const double off = slots_total(J.slots, S);
     if (sweep == 0) fro2 = off + slots_total(J.slots + 512, S);
-    if (!(off > 1e-14 * fro2) || (sweep > 0 && off <= 1e-9 * fro2 && off > 0.25 * prev)) break;
+    if (!(off > 1e-12 * fro2) || (sweep > 0 && off <= 1e-9 * fro2 && off > 0.25 * prev)) break;
     prev = off;
     for (int br = 0; br < nb - 1; ++br) {
       const int copy = br == 0 ? 1 : 0;  // where the problems' results lie: 31 rounds, then 16 each
