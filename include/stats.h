@@ -71,8 +71,7 @@ typedef enum { STATS_I16 = 0, STATS_I32 = 1, STATS_I64 = 2, STATS_F32 = 3, STATS
  *                      before it can round (all products and partial sums are exact
  *                      integers below 2^24).  Centering in exact integer arithmetic.
  *   STATS_FP64         the plain FP64 CUDA-core kernel with raw moments, as in the
- *                      paper (covariance = (S - s s^T / n) / (n - 1) in FP64); a
- *                      row-parallel kernel for p <= 12, a tiled one above.
+ *                      paper (covariance = (S - s s^T / n) / (n - 1) in FP64).
  *   STATS_FP64_SHIFTED FP64 CUDA cores on x - c, c = the mean of the first rows accumulated
  *                      (the first 64 rows of the first call, or all of them if fewer; for
  *                      FP32 data in the BF16 and FP32 modes rounded to FP32).  A pivot near the
@@ -233,12 +232,13 @@ stats_status stats_finalize(stats_ctx* ctx, double* mean, double* cov, double* c
  *   evecs_prev: HOST, p_a*p_a doubles, row k = eigenvector k, as written by an earlier
  *     stats_finalize / stats_finalize_warm (any ctx with the same p_a), or NULL (cold
  *     start).  The matrix M (cov, or corr with pca_on = 1) is rotated into that basis,
- *     V^T M V, before the cyclic Jacobi sweeps.  A seed whose columns are not orthonormal
+ *     V^T M V, before the Jacobi sweeps.  A seed whose columns are not orthonormal
  *     (max |V^T V - I| > 1e-9, or NaN) is ignored.  The eigenpairs are those of M
  *     whatever the seed, up to rounding; inside a cluster of equal eigenvalues the
  *     eigenvectors may be another basis of the same subspace.
- *   sweeps: may be NULL; receives the number of Jacobi sweeps taken, -1 when no
- *     eigenpairs were computed.
+ *   sweeps: may be NULL; receives the number of Jacobi sweeps taken (FP32 ones, and FP64
+ *     ones where eigenvalues were too close for the refinement that follows them), -1 when
+ *     no eigenpairs were computed.
  * The other arguments are those of stats_finalize.  With more than 23 analysis columns,
  * or with a seed, the eigen-solver is a cooperative launch over the GPU's SMs.
  * Errors: those of stats_finalize; ETIMEOUT when a grid-wide wait of the eigen-solver

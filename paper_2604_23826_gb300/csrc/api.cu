@@ -1032,8 +1032,8 @@ void build_final_params(const stats_ctx* c, int want_pca, int pca_on, FinalParam
 }
 
 // From this many analysis columns on, the eigen-solver runs over the whole GPU
-// (jacobi_grid_kernel) instead of inside the one-block finalize kernel: GB300 has
-// about 2 FP64 FMAs per SM clock, so one block is far too slow for p_a in the hundreds.
+// (jacobi_grid_kernel) instead of inside the one-block finalize kernel: GB300 has about 2 FP64
+// operations per SM clock, so the refinement's products want many SMs.
 constexpr int kGridJacobiMinColumns = 24;
 
 // Finalize on the ctx's stream.  With want_pca, the eigen-decomposition runs either in the

@@ -134,7 +134,7 @@ __device__ __forceinline__ void two_of(const uint8_t* col, int r, T& x, T& y) {
 // A lane takes two rows at once, adjacent ones of a stage: their loads, conversions and checks
 // overlap, and one load brings both values of a column.
 // Bound: HBM for the 60 bytes an L32 row has (1e9 rows: 9.38 ms, 6.4 TB/s; a row at a time with
-// rescaled digits 9.98).  The 44 bytes of L16 wait for the conversions: about 180 instructions per 32
+// rescaled digits 9.98).  The 44 bytes of L16 wait for the conversions: about 205 instructions per 32
 // rows on four warps a scheduler, half the issue slots and a third of the FP64 unit (1.23e8 rows:
 // 1.17 ms, 1.23 before).
 template <bool L16>

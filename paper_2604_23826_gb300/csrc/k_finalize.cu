@@ -17,7 +17,7 @@
 // block finds all standard deviations for itself, so no block waits for another.
 //
 // Eigenpairs: up to 23 columns in this kernel; a single wider context goes to the grid-wide solver
-// (k_eigen.cu).  In a batch, contexts of 24..64 columns take a block each.  Either way FP32 Jacobi in
+// (k_eigen.cu).  In a batch, contexts of 24..64 columns take a cluster of 1 to 4 blocks each.  Either way FP32 Jacobi in
 // shared memory, then the Ogita-Aishima refinement in FP64, with FP64 Jacobi from the refined basis
 // where eigenvalues are too close for it (a round of FP64 rotations alone takes 2800 cycles: chains of
 // 64-cycle operations); wider ones of a batch FP64 Jacobi.
