@@ -443,27 +443,48 @@ __host__ __device__ constexpr int jacobi32_order(int n) { return n <= 32 ? (n + 
 // ------------------------------- refinement -------------------------------
 // One entry of the correction of approximate eigenvectors X of A (Ogita and Aishima, "Iterative
 // refinement for symmetric eigenvalue decomposition", 2018): with S = X^T A X, G = X^T X and
-// lambda_i = S_ii / G_ii, X (I + E) is better by a square.  A pair whose eigenvalues are too close
-// for the first-order step (unresolved; its off-diagonal above `noise`) is counted in bad, and only
-// made orthogonal.
+// lambda_i = S_ii / G_ii, X (I + E) is better by a square; its largest entry goes into mx.  A pair whose
+// eigenvalues are too close for the first-order step is only made orthogonal, and counted in bad unless
+// its off-diagonal is no more than `noise`, what rounding leaves.  What the two entries of a pair get is
+// decided alike: E_ij + E_ji = -G_ij.
+// coarse (the first step; later 0): off-diagonals this small are still the squares of FP32's errors, and
+// within a cluster of equal eigenvalues hundreds of corrections of a tenth would add up (matrices of rank
+// p / 2 went to the FP64 rotations: 256 columns 26 ms, 2.4 so); above 1e-3 they wait for the next step.
 __device__ __forceinline__ double correction(int i, int j, double S, double G, double li, double lj, double noise,
-                                             int& bad) {
-  const double num = i == j ? 1.0 - G : fma(-lj, G, S), an = fabs(num);
-  if (!(an <= 1e300)) {  // not finite
+                                             double coarse, double& mx, int& bad) {
+  const double num = i == j ? 1.0 - G : fma(-lj, G, S), an = i == j ? fabs(num) : fmax(fabs(num), fabs(fma(-li, G, S)));
+  if (!(fabs(num) <= 1e300) || !(an <= 1e300)) {  // not finite
     bad = 2;
     return 0.0;
   }
-  if (i == j) return 0.5 * num;
-  const double gap = lj - li, ag = fabs(gap);
-  const bool small = an <= noise;
-  if (ag > 0.0 && an <= (small ? 1e-9 : 0.125) * ag) return num / gap;
-  if (!small) bad = max(bad, 1);
-  return -0.5 * G;
+  double e;
+  if (i == j) {
+    e = 0.5 * num;
+  } else {
+    const double gap = lj - li, ag = fabs(gap);
+    const bool small = an <= noise, waits = !small && an <= coarse;
+    if (ag > 0.0 && an <= (small ? 1e-9 : waits ? 1e-3 : 0.125) * ag) {
+      e = num / gap;
+    } else {
+      if (waits)
+        mx = fmax(mx, 1e-3);
+      else if (!small)
+        bad = max(bad, 1);
+      e = -0.5 * G;
+    }
+    if (small) return e;
+  }
+  mx = fmax(mx, fabs(e));
+  return e;
 }
+// what rounding leaves, of the matrix's norm, in an entry of X^T A X that should be zero
+constexpr double kNoise = 16.0 * 1.1102230246251565e-16;
 // E - 1023 for a matrix whose squared Frobenius norm is fro2 (normal): every |entry| < 2^(E - 1023)
 __device__ __forceinline__ int scale_exponent(double fro2) { return 1023 + (exp_field(fro2) - 1023 + 2 + 2048) / 2 - 1024; }
 // corrections below this need no further step: what it leaves behind is their square times sqrt(m)
 constexpr double kRefined = 5e-9;
+// off-diagonals below this of the matrix's norm may, in the first step, be the squares of FP32's errors
+constexpr double kCoarse = 1e-11;
 
 }  // namespace eig
 }  // namespace ss

@@ -11,9 +11,10 @@
 //      three steps of four products, each spread over the grid in 16 x 16 tiles.
 //   4. If eigenvalues are too close for the refinement (or it fails), block-cyclic Jacobi in FP64,
 //      from the refined basis (or from the matrix as it came).
-// Bound: FP64, at 2 operations per clock and SM.  FP64 Jacobi alone spent it on chains of divisions
-// and square roots of one warp (256 columns, 11 sweeps: 14.7 ms); the products of step 3 are four
-// times 256^3 multiplications a step, 30 us each over 152 SMs, and step 2 has no FP64 at all.
+// Bound: latency.  A block round of step 2 takes 18,000 cycles: 17 dependent rounds of its 32 x 32
+// problems 10,400, their loads, the product, and the stores and barrier the rest.  Step 3 is FP64 at 2
+// operations per clock and SM: 256 columns, 0.13 ms a step.  (FP64 rotations alone, chains of divisions
+// and square roots of one warp: 256 columns, 11 sweeps, 14.7 ms; all of this 1.64.)
 #include <math.h>
 
 #include "common.cuh"
@@ -610,7 +611,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     }
     double* W = J.x;  // A X, then the corrections
     X = J.w;
-    const double noise = 16.0 * 1.1102230246251565e-16 * sqrt(fro2);
+    const double noise = kNoise * sqrt(fro2), coarse = kCoarse * sqrt(fro2);
     for (int it = 0; alive && it < 5; ++it) {
       grid_product(
           m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(X + at(k, j)); },
@@ -624,8 +625,8 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
       double mx = 0.0;
       for (int i = gtid; i < m * m; i += nthreads) {
         const int r = i / m, c = i % m;
-        const double e = correction(r, c, __ldcg(J.b + i), __ldcg(J.g + i), S.lambda[r], S.lambda[c], noise, bad);
-        mx = fmax(mx, fabs(e));
+        const double e = correction(r, c, __ldcg(J.b + i), __ldcg(J.g + i), S.lambda[r], S.lambda[c], noise,
+                                    it == 0 ? coarse : 0.0, mx, bad);
         __stcg(W + i, e);
       }
       mx = block_max(mx, S.red);

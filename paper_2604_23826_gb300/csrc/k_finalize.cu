@@ -376,7 +376,7 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
     fV += copy * m * m;
     for (int i = tid; i < n * n; i += kThreads) X[(i / n) * ld + i % n] = f32_to_f64(fV[(i / n) * m + i % n]);
     team.meet();  // the others may put into W and S now
-    const double unit = 16.0 * 1.1102230246251565e-16, noise = unit * sqrt(fro2);
+    const double noise = kNoise * sqrt(fro2), coarse = kCoarse * sqrt(fro2);
     for (int it = 0; it < 5; ++it) {
       team_product(
           team, n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
@@ -433,8 +433,8 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
         const int r = i / n, c = i % n, lo = min(r, c), hi = max(r, c);
         const double lr = M.lambda[r], lc = M.lambda[c];
         const double e = correction(r, c, S[lo * ld + hi], r == c ? M.gd[r] : S[hi * ld + lo], lr, lc,
-                                    kGraded ? unit * sqrt(fabs(lr * lc)) : noise, bad);
-        mx = fmax(mx, fabs(e));
+                                    kGraded ? kNoise * sqrt(fabs(lr * lc)) : noise, !kGraded && it == 0 ? coarse : 0.0, mx,
+                                    bad);
         team.put(W + r * ld + c, e);
       }
       mx = block_max(mx, M.red);

@@ -103,3 +103,12 @@ def test_extreme_scales(p, scale):
 def test_zero_matrix(p):
     for an in both(np.full((p, 100), 2.5)):
         assert np.all(an.evals == 0) and np.array_equal(np.abs(an.evecs), np.eye(p))
+
+
+@pytest.mark.parametrize("p", [24, 40, 64, 65, 100, 256])
+def test_rank_deficient(p):
+    """Fewer rows than columns, and every column twice: half of the eigenvalues are zero."""
+    rng = np.random.default_rng(p)
+    for X in (rng.standard_normal((p, p // 2)), np.repeat(rng.standard_normal((p - p // 2, 4 * p)), 2, axis=0)[:p]):
+        for an in both(X):
+            check(an, an.cov)
