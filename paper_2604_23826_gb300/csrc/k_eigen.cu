@@ -84,6 +84,7 @@ struct Shared {
   double x[16][17], y[16][17], z[16][17], t[16][17];
   double qa[kJP][kJP + 1], qb[kJP][kJP + 1];
   double c[8], s[8];
+  int null[8];
   double lambda[256];
   double red[8];
   unsigned long long key[256];
@@ -339,18 +340,22 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
 }
 
 // FP64 block-cyclic Jacobi over the grid: diagonalises A (B: its next copy), rotating V's columns.
+// Only the first n rows and columns take part, the matrix's own rounded up to a pair of blocks.
 // Returns the sweeps (A then points to the diagonal form), -1 after a wait that ran out.
+// Bound: the chains of the local rounds.  Angles from FP32 (rotation64) instead of an FP64 division and
+// two roots, and 112 rows instead of 128 for 100 columns: a matrix of 100 columns in four clusters of
+// eigenvalues 8.3 ms, 5.4 so; 256 columns 25.3 and 19.5.
 __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V) {
-  const int tid = threadIdx.x, m = J.m, nb = m / kJW, np = nb / 2;
+  const int tid = threadIdx.x, m = J.m, n = (J.pa + kJP - 1) / kJP * kJP, nb = n / kJW, np = nb / 2;
   const int lr_ = tid / kJP, lc_ = tid % kJP;
   const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
   double fro2 = 0.0, prev = 0.0;
   int sweep = 0;
   for (; sweep < 60; ++sweep) {
     double o = 0.0, d = 0.0;
-    for (int i = gtid; i < m * m; i += nthreads) {
-      const double x = __ldcg(A + i);
-      if (i / m != i % m)
+    for (int i = gtid; i < n * n; i += nthreads) {
+      const double x = __ldcg(A + static_cast<size_t>(i / n) * m + i % n);
+      if (i / n != i % n)
         o = fma(x, x, o);
       else
         d = fma(x, x, d);
@@ -382,16 +387,12 @@ __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, doubl
           if (tid < kJP / 2) {
             int p, q;
             pair_of(lr, tid, kJP, p, q);
-            double c = 1.0, sn = 0.0;
-            const double apq = S.x[p][q];
-            if (apq != 0.0) {
-              const double dd = S.x[q][q] - S.x[p][p];
-              const double t = (dd >= 0.0 ? 2.0 * apq : -2.0 * apq) / (fabs(dd) + sqrt(dd * dd + 4.0 * apq * apq));
-              c = rsqrt(t * t + 1.0);
-              sn = t * c;
-            }
+            double c, sn;
+            bool null;
+            rotation64(S.x[p][p], S.x[q][q], S.x[p][q], c, sn, null);
             S.c[tid] = c;
             S.s[tid] = sn;
+            S.null[tid] = null;
           }
           __syncthreads();
           if (tid < (kJP / 2) * kJP) {  // rows p, q
@@ -416,9 +417,10 @@ __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, doubl
             double(*X)[kJP + 1] = onS ? S.x : S.y;
             if (sn != 0.0) {
               const double xkp = X[k][p], xkq = X[k][q];
-              // the rotated pair's off-diagonal entries are zero by construction
-              X[k][p] = (onS && k == q) ? 0.0 : c * xkp - sn * xkq;
-              X[k][q] = (onS && k == p) ? 0.0 : sn * xkp + c * xkq;
+              // what is left of the rotated pair's off-diagonal entries may be zero
+              const bool zero = onS && S.null[i];
+              X[k][p] = (zero && k == q) ? 0.0 : c * xkp - sn * xkq;
+              X[k][q] = (zero && k == p) ? 0.0 : sn * xkp + c * xkq;
             }
           }
           __syncthreads();
@@ -430,7 +432,7 @@ __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, doubl
       if (!grid.sync()) return -1;
       // (2) the other blocks of A, Q_P^T A[P rows][P' cols] Q_P' (into B), and V's columns,
       //     V[rows][P' cols] Q_P' (in place: every entry belongs to one item)
-      const int nA = np * np, nItems = nA + (m / kJP) * np;
+      const int nA = np * np, nItems = nA + (n / kJP) * np;
       for (int it = blockIdx.x; it < nItems; it += gridDim.x) {
         if (it < nA && it / np == it % np) continue;  // diagonal blocks came from step (1)
         const bool isA = it < nA;
