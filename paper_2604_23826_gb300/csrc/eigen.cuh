@@ -38,6 +38,17 @@ __device__ __forceinline__ float scaled32(double x, int E) {
                          : 0.f;
 }
 
+// About a^2 / |p q| of an entry a between the diagonal's p and q, from the exponents alone (a power of
+// two, at most 1; 0 for a = 0): sums of these tell how far a matrix is from diagonal in each pair's own
+// units.  Columns of very different units have eigenvalues far below the rounding of the largest, and an
+// off-diagonal that is nothing beside the norm may be everything to two of those.  floor: the exponent of
+// the smallest variance; what lies below it is rounding, or owes its size to cancellation.
+__device__ __forceinline__ float square_ratio(int ea, int ep, int eq, int floor) {
+  const int d = 2 * ea - max(ep, floor) - max(eq, floor);
+  return ea == 0 || d < -126 ? 0.f : __int_as_float((127 + min(d, 0)) << 23);
+}
+__device__ __forceinline__ int exp_field32(float x) { return (__float_as_int(x) >> 23) & 0xFF; }
+
 __device__ __forceinline__ float rsqrt32(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -116,6 +127,20 @@ __device__ __forceinline__ T block_max(T v, T* s_red) {
   __syncthreads();
   return t;
 }
+__device__ __forceinline__ int block_or(int v, int* s_red) {
+  v = __reduce_or_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  const int t = __reduce_or_sync(0xffffffffu, s_red[threadIdx.x & 7]);
+  __syncthreads();
+  return t;
+}
+
+// exponent field of the smallest of a matrix's diagonal that is not zero, by the block
+__device__ __forceinline__ int smallest_variance(const double* A, int ld, int n, int* s_red) {
+  const int e = static_cast<int>(threadIdx.x) < n ? exp_field(A[static_cast<size_t>(threadIdx.x) * (ld + 1)]) : 0;
+  return -block_max(e ? -e : -0x7FF, s_red);
+}
 
 // ------------------------------- FP64 -------------------------------
 struct Scratch64 {
@@ -123,25 +148,44 @@ struct Scratch64 {
   int p[128], q[128], null[128];
 };
 
+// FP64 rotations are at an end when the off-diagonal is negligible (`norm`, by the caller) and so are the
+// sum of its ratios in the pairs' own units: below 1e-28, or at the level of rounding (2e-15 an entry) and
+// falling no further, or falling no further for four sweeps.  (Rotations from the refined basis of a
+// cluster of close eigenvalues may reduce little in their first sweeps.)
+struct Ratios64 {
+  float prev = 0.f;
+  int stalled = 0;
+  __device__ __forceinline__ bool done(bool norm, float rel, int n) {
+    stalled = norm && prev > 0.f && rel > 0.0625f * prev ? stalled + 1 : 0;
+    prev = rel;
+    return norm && (rel <= 1e-28f || (stalled >= 1 && rel <= 4e-30f * n * n) || stalled >= 4);
+  }
+};
+
 // Cyclic Jacobi on A (order n, at most 256; shared or global memory), its rotations applied to V's
-// columns, which hold the basis on entry.  Returns the sweeps taken.
-__device__ inline int jacobi64(double* A, int lda, double* V, int ldv, int n, Scratch64& S) {
+// columns, which hold the basis on entry; floor: square_ratio's.  Returns the sweeps taken.
+__device__ inline int jacobi64(double* A, int lda, double* V, int ldv, int n, int floor, Scratch64& S) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, m = n + (n & 1), h = m / 2;
   double fro2 = 0.0;
+  Ratios64 ratios;
   int sweep = 0;
   for (; sweep < 60; ++sweep) {
     double off = 0.0, dia = 0.0;
+    float rel = 0.f;
     for (int r = warp; r < n; r += kThreads / 32)
       for (int c = lane; c < n; c += 32) {
         const double x = A[r * lda + c];
-        if (r != c)
+        if (r != c) {
           off = fma(x, x, off);
-        else
+          rel += square_ratio(exp_field(x), exp_field(A[r * lda + r]), exp_field(A[c * lda + c]), floor);
+        } else {
           dia = fma(x, x, dia);
+        }
       }
     off = block_total(off, S.red);
+    rel = block_total(rel, reinterpret_cast<float*>(S.red));
     if (sweep == 0) fro2 = block_total(dia, S.red) + off;
-    if (off == 0.0 || off <= 1e-34 * fro2) break;
+    if (off == 0.0 || ratios.done(off <= 1e-34 * fro2, rel, n)) break;
     for (int round = 0; round < m - 1; ++round) {
       if (tid < h) {
         int p, q;
@@ -349,7 +393,7 @@ struct Jacobi32 {
     const float c2 = fmaf(0.5f * fabsf(d), r, 0.5f);
     const float y = rsqrt32(c2), c = c2 * y, s = (d >= 0.f ? apq : -apq) * r * y;
     const float e = fmaf(c, c, fmaf(s, s, -1.f));
-    const bool turn = fabsf(apq) > 1e-18f;  // the matrix is scaled to order one
+    const bool turn = fabsf(apq) > 1e-18f;  // 30 decades below the matrix's norm (kUp32)
     return make_float2(turn ? fmaf(-0.5f * e, y, c) : 1.f, turn ? s : 0.f);
   }
   // one round of A, from copy B to copy 1 - B, and (kV) of V the round before (now: the last round's
@@ -403,32 +447,45 @@ struct Jacobi32 {
   }
 };
 
+// FP32 rotations are at an end when the off-diagonal is at the level of FP32's rounding (or falls no
+// further near it), and in the pairs' own units too: the small eigenvalues of columns of different units
+// (or of a nearly diagonal seeded matrix) are rotated as far as the large ones.
+template <typename T>
+__device__ __forceinline__ bool rotated32(int sweep, T off, T prev, T fro2, T done, float rel, float prev_rel) {
+  const bool norm = !(off > done * fro2) || (sweep > 0 && off <= T(1e-9) * fro2 && off > T(0.25) * prev);
+  return norm && (rel <= 1e-6f || (sweep > 0 && rel > 0.25f * prev_rel));
+}
+
 // Cyclic Jacobi in FP32 on A (M x M floats, followed by its next copy), its rotations applied to V's
 // columns (the same), by the whole block.  At most max_sweeps; stops once the off-diagonal part is at
-// the level of FP32 rounding.  Returns the sweeps taken; `copy`: which copies hold the results.
+// the level of FP32 rounding.  floor: square_ratio's.  Returns the sweeps taken; `copy`: which copies hold
+// the results.
 template <int M>
-__device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_sweeps, Scratch32& S, int& copy) {
+__device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_sweeps, int floor, Scratch32& S, int& copy) {
   const int tid = threadIdx.x;
   const Jacobi32<M> J(A, V, S, tid, 0);
-  float prev = 0.f, fro2 = 0.f;
+  float prev = 0.f, prev_rel = 0.f, fro2 = 0.f;
   int sweep = 0;
   copy = 0;
   for (; sweep < max_sweeps; ++sweep) {
     const float* X = A + copy * M * M;
-    float off = 0.f, dia = 0.f;
+    float off = 0.f, dia = 0.f, rel = 0.f;
     for (int i = tid; i < M * M; i += kThreads) {
       const float x = X[i];
-      if (i / M != i % M)
+      const int r = i / M, c = i % M;
+      if (r != c) {
         off = fmaf(x, x, off);
-      else
+        rel += square_ratio(exp_field32(x), exp_field32(X[r * M + r]), exp_field32(X[c * M + c]), floor);
+      } else {
         dia = fmaf(x, x, dia);
+      }
     }
     off = block_total(off, S.red);
+    rel = block_total(rel, S.red);
     if (sweep == 0) fro2 = block_total(dia, S.red) + off;
-    // (mixed units, which only the smaller orders' refinement looks at closely, want more)
-    const float done = M <= 24 ? 1e-14f : 1e-12f;
-    if (!(off > done * fro2) || (sweep > 0 && off <= 1e-9f * fro2 && off > 0.25f * prev)) break;
+    if (rotated32(sweep, off, prev, fro2, M <= 24 ? 1e-14f : 1e-12f, rel, prev_rel)) break;
     prev = off;
+    prev_rel = rel;
     if (copy == 0)
       Jacobi32<M>::template sweep<0>(J);
     else
@@ -441,50 +498,100 @@ __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_
 __host__ __device__ constexpr int jacobi32_order(int n) { return n <= 32 ? (n + 7) / 8 * 8 : (n + 15) / 16 * 16; }
 
 // ------------------------------- refinement -------------------------------
+// What rounding leaves in an entry of X^T A X that should be zero depends on its two columns: a
+// covariance's |a_kl| <= sqrt(a_kk a_ll), so products of the columns i and j of X leave about eps b_i b_j,
+// b_j^2 = sum_l a_ll x_lj^2, which is far below the norm's rounding where both columns are combinations of
+// table columns of small units (and near it where a rank-deficient matrix has its zero eigenvalues).
+// A column's share of that, and of the rounding of its eigenvalue, is kept as its noise: an entry's is
+// the product of two.  (A bound from the norm took FP32's leavings among small eigenvalues for rounding:
+// 40 columns of units over four decades, vectors wrong by 3e-7, over eight by 4e-3; now to 1e-14.)
+struct Noise {
+  double unit;  // 2^(exponent / 2)
+  int E;        // scaled32's exponent for the values: an even one, no |entry| larger
+  float root;   // 4 sqrt(columns)
+  // of a column: `weight` = sum_l a_ll x_lj^2, scaled; `f` and `inverse` for the ratios of two columns
+  __device__ __forceinline__ double column(double lambda, float weight, float& f, float& inverse) const {
+    f = 1.0536712e-8f * sqrtf(fmaxf(16.f * fabsf(scaled32(lambda, E)), root * weight));  // sqrt(2^-53) times
+    inverse = f > 0.f ? 1.f / f : 0.f;
+    return f32_to_f64(f) * unit;
+  }
+};
+// an exponent E with every |entry| < 2^(E - 1023), for a matrix whose squared Frobenius norm is fro2 (normal)
+__device__ __forceinline__ int scale_exponent(double fro2) { return 1023 + (exp_field(fro2) - 1023 + 2 + 2048) / 2 - 1024; }
+__device__ __forceinline__ Noise noise_of(int E, int n) {
+  const int h = (E - 1023 + 1 + 2048) / 2 - 1024;
+  return Noise{__hiloint2double((1023 + h) << 20, 0), 1023 + 2 * h, 4.f * sqrtf(static_cast<float>(n))};
+}
+// FP32 rotations take the matrix at 2^40 times its scale, so that what they leave alone (1e-18, whose square
+// FP32 still holds) lies 30 decades below the norm
+constexpr int kUp32 = 40;
+// square_ratio's floor of the matrix those work on
+__device__ __forceinline__ int floor32(int floor, int E) { return max(0, min(254, floor - E + kUp32 + 127)); }
+
+// corrections below this need no further step: what it leaves behind is their square times sqrt(m)
+constexpr float kRefined = 5e-9f;
+// of an entry's noise: off-diagonals below this may, in the first step, be the squares of FP32's errors
+constexpr double kCoarse = 5000.0;
+constexpr int kSteps = 8;
+// what a step found
+constexpr int kMore = 1;    // some correction is too large to be the last
+constexpr int kClose = 2;   // some eigenvalues are too close for the refinement
+constexpr int kFailed = 4;  // not a refinement any more
+
+// the largest correction that a step takes
+__device__ __forceinline__ double reach(int step) {
+  return step < 2 ? 0.125 : step == 2 ? 0.03 : step == 3 ? 2e-3 : kRefined;
+}
+
 // One entry of the correction of approximate eigenvectors X of A (Ogita and Aishima, "Iterative
 // refinement for symmetric eigenvalue decomposition", 2018): with S = X^T A X, G = X^T X and
-// lambda_i = S_ii / G_ii, X (I + E) is better by a square; its largest entry goes into mx.  A pair whose
-// eigenvalues are too close for the first-order step is only made orthogonal, and counted in bad unless
-// its off-diagonal is no more than `noise`, what rounding leaves.  What the two entries of a pair get is
-// decided alike: E_ij + E_ji = -G_ij.
-// coarse (the first step; later 0): off-diagonals this small are still the squares of FP32's errors, and
-// within a cluster of equal eigenvalues hundreds of corrections of a tenth would add up (matrices of rank
-// p / 2 went to the FP64 rotations: 256 columns 26 ms, 2.4 so); above 1e-3 they wait for the next step.
+// lambda_i = S_ii / G_ii, X (I + E) is better by a square.  A pair whose eigenvalues are too close for the
+// first-order step is only made orthogonal, and reported unless its off-diagonal is no more than
+// rounding leaves.  What the two entries of a pair get is decided alike: E_ij + E_ji = -G_ij.
+// Off-diagonals at the level of rounding (`noise`) are corrected like others in the first two steps,
+// but for eigenvalues that rounding cannot tell apart; from then on they are rounding and stay.
+// coarse (the first step): off-diagonals this small are still the squares of FP32's errors, and within a
+// cluster of equal eigenvalues hundreds of corrections of a tenth would add up (matrices of rank p / 2
+// went to the FP64 rotations: 256 columns 26 ms, 2.4 so); above 1e-3 they wait for the next step.
+// Later steps take only what converges at least as fast as squares do, the last two only corrections that
+// need no further step: the rest, clusters of close eigenvalues, ends as an orthonormal basis that FP64
+// rotations start from (they started from the identity: 12 columns in clusters of 1e-6, seeded, 395 us, 285 so;
+// 256 columns, four such clusters, 18.4 ms, 9.8 so).
+// up, down: column i's noise over j's, and j's over i's.  A correction puts X_i's eigenvalue times its
+// square into lambda_j, so it counts that much more where i's eigenvalue is the larger.
 __device__ __forceinline__ double correction(int i, int j, double S, double G, double li, double lj, double noise,
-                                             double coarse, double& mx, int& bad) {
+                                             float up, float down, int step, bool coarse, int& found) {
   const double num = i == j ? 1.0 - G : fma(-lj, G, S), an = i == j ? fabs(num) : fmax(fabs(num), fabs(fma(-li, G, S)));
   if (!(fabs(num) <= 1e300) || !(an <= 1e300)) {  // not finite
-    bad = 2;
+    found |= kFailed;
     return 0.0;
   }
-  double e;
-  if (i == j) {
-    e = 0.5 * num;
-  } else {
+  double e = i == j ? 0.5 * num : -0.5 * G;
+  float weight = 1.f;
+  if (i != j) {
     const double gap = lj - li, ag = fabs(gap);
-    const bool small = an <= noise, waits = !small && an <= coarse;
-    if (ag > 0.0 && an <= (small ? 1e-9 : waits ? 1e-3 : 0.125) * ag) {
-      e = num / gap;
-    } else {
-      if (waits)
-        mx = fmax(mx, 1e-3);
-      else if (!small)
-        bad = max(bad, 1);
-      e = -0.5 * G;
+    bool turn = ag > 0.0;
+    if (an <= noise) {
+      if (turn && an * f32_to_f64(fmaxf(1.f, fmaxf(up, down))) <= 1e-9 * ag) return num / gap;
+      turn = step < 2 && ag > 64.0 * noise;
+    } else if (coarse && an <= kCoarse * noise && an > 1e-3 * ag) {
+      found |= kMore;
+      turn = false;
+    } else if (!turn || !(an <= reach(step) * ag)) {
+      found |= kClose;
+      turn = false;
     }
-    if (small) return e;
+    if (turn) {
+      e = num / gap;
+      weight = fmaxf(1.f, up);
+    }
   }
-  mx = fmax(mx, fabs(e));
+  if (!(fabs(e) <= 0.5))
+    found |= kFailed;
+  else if (weight * fabsf(scaled32(e, 1023)) > kRefined)
+    found |= kMore;
   return e;
 }
-// what rounding leaves, of the matrix's norm, in an entry of X^T A X that should be zero
-constexpr double kNoise = 16.0 * 1.1102230246251565e-16;
-// E - 1023 for a matrix whose squared Frobenius norm is fro2 (normal): every |entry| < 2^(E - 1023)
-__device__ __forceinline__ int scale_exponent(double fro2) { return 1023 + (exp_field(fro2) - 1023 + 2 + 2048) / 2 - 1024; }
-// corrections below this need no further step: what it leaves behind is their square times sqrt(m)
-constexpr double kRefined = 5e-9;
-// off-diagonals below this of the matrix's norm may, in the first step, be the squares of FP32's errors
-constexpr double kCoarse = 1e-11;
 
 }  // namespace eig
 }  // namespace ss

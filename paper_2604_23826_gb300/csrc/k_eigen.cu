@@ -8,7 +8,9 @@
 //      32 x 32 block of T and V multiplied by the pairs' rotations: one grid barrier a block round.
 //   3. X = V Q, then the Ogita-Aishima refinement in FP64: W = A X, S = X^T W, G = X^T X, the
 //      correction E from S, G and X <- X + X E, until E is below 5e-9 (its square is left): two or
-//      three steps of four products, each spread over the grid in 16 x 16 tiles.
+//      three steps of four products, each spread over the grid in 16 x 16 tiles.  What is rounding is
+//      told from each pair's own columns, so the eigenpairs of columns of very different units are
+//      as good as those of like ones.
 //   4. If eigenvalues are too close for the refinement (or it fails), block-cyclic Jacobi in FP64,
 //      from the refined basis (or from the matrix as it came).
 // Bound: latency.  A block round of step 2 takes 18,000 cycles: 17 dependent rounds of its 32 x 32
@@ -85,7 +87,8 @@ struct Shared {
   double qa[kJP][kJP + 1], qb[kJP][kJP + 1];
   double c[8], s[8];
   int null[8];
-  double lambda[256];
+  double lambda[256], noise[256];
+  float nf[256], ni[256];
   double red[8];
   unsigned long long key[256];
   int order[256];
@@ -124,8 +127,9 @@ __device__ void grid_product(int m, Shared& S, FX&& X, FY&& Y, Put&& put) {
 }
 
 // S = X^T W and G = X^T X (both symmetric): the tiles on or above the diagonal of each, shared out
-// over the grid
-__device__ void grid_grams(int m, Shared& S, const double* X, const double* W, double* SO, double* GO) {
+// over the grid; and the columns' weights sum_l a_ll x_lj^2 (FP32, beside G's diagonal tiles)
+__device__ void grid_grams(int m, Shared& S, const double* X, const double* W, double* SO, double* GO, const double* A,
+                           int E, float* weights) {
   const int nt = m / 16, r = threadIdx.x / 16, c = threadIdx.x % 16, half = nt * (nt + 1) / 2;
   for (int t = blockIdx.x; t < 2 * half; t += gridDim.x) {
     int I = 0, J = t % half;
@@ -136,19 +140,36 @@ __device__ void grid_grams(int m, Shared& S, const double* X, const double* W, d
     J += I;
     const double* Y = t < half ? W : X;
     double* O = t < half ? SO : GO;
+    const bool weigh = t >= half && I == J;
     double acc = 0.0;
+    float b = 0.f;
     double nx = __ldcg(X + static_cast<size_t>(r) * m + I * 16 + c), ny = __ldcg(Y + static_cast<size_t>(r) * m + J * 16 + c);
+    double nd = weigh ? __ldcg(A + static_cast<size_t>(r) * (m + 1)) : 0.0;
     for (int k0 = 0; k0 < m; k0 += 16) {
       S.x[r][c] = nx;
       S.y[r][c] = ny;
+      if (weigh) {  // this thread's row of column c
+        const float x = scaled32(nx, 1023);
+        b = fmaf(fabsf(scaled32(nd, E)) * x, x, b);
+      }
       __syncthreads();
       if (k0 + 16 < m) {
         nx = __ldcg(X + static_cast<size_t>(k0 + 16 + r) * m + I * 16 + c);
         ny = __ldcg(Y + static_cast<size_t>(k0 + 16 + r) * m + J * 16 + c);
+        if (weigh) nd = __ldcg(A + static_cast<size_t>(k0 + 16 + r) * (m + 1));
       }
 #pragma unroll
       for (int k = 0; k < 16; ++k) acc = fma(S.x[k][r], S.y[k][c], acc);
       __syncthreads();
+    }
+    if (weigh) {
+      S.t[r][c] = b;
+      __syncthreads();
+      if (threadIdx.x < 16) {
+        float w = 0.f;
+        for (int k = 0; k < 16; ++k) w += static_cast<float>(S.t[k][threadIdx.x]);
+        __stcg(weights + I * 16 + threadIdx.x, w);
+      }
     }
     // both halves hold the same value
     if (I == J) {
@@ -165,15 +186,21 @@ __device__ void grid_grams(int m, Shared& S, const double* X, const double* W, d
 }
 
 // the blocks' slots[0 .. grid) added (or their maximum taken) in a fixed order, in every thread
-__device__ double slots_total(const double* slots, Shared& S) {
-  double v = 0.0;
+template <typename T>
+__device__ T slots_total(const T* slots, Shared& S) {
+  T v = 0;
   for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += kThreads) v += __ldcg(slots + b);
-  return block_total(v, S.red);
+  return block_total(v, reinterpret_cast<T*>(S.red));
 }
 __device__ double slots_max(const double* slots, Shared& S) {
   double v = 0.0;
   for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += kThreads) v = fmax(v, __ldcg(slots + b));
   return block_max(v, S.red);
+}
+__device__ int slots_or(const double* slots, Shared& S) {
+  int v = 0;
+  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += kThreads) v |= __ldcg(reinterpret_cast<const int*>(slots + b));
+  return block_or(v, reinterpret_cast<int*>(S.red));
 }
 
 // FP32 block-cyclic Jacobi over the grid (m a multiple of 32): A and its next copy B, V = I on entry.
@@ -184,7 +211,8 @@ __device__ double slots_max(const double* slots, Shared& S) {
 // everywhere, and a grid barrier and a trip through memory less than solving them once.  (256 columns,
 // all of the solver: 2.44 ms with full sweeps of problems solved once and two barriers a round, 1.64 so.)
 // Returns the sweeps, -1 after a wait that ran out.
-__device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float* dyn, float* A, float* B, float* V) {
+__device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float* dyn, float* A, float* B, float* V,
+                             int floor) {
   const int m = J.m, nb = m / kFW, np = nb / 2, tid = threadIdx.x;
   constexpr int kE = kFP * kFP;
   float* sX = dyn + 2 * jacobi32_floats(kFP);
@@ -195,26 +223,34 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
   float* pA = dyn + half * jacobi32_floats(kFP);  // this half's problem: two copies, then the rotations' two
   float* pV = pA + 2 * kE;
   double fro2 = 0.0, prev = 0.0;
+  float prev_rel = 0.f;
   int sweep = 0;
   for (; sweep < 20; ++sweep) {
-    float o = 0.f, d = 0.f;
+    float o = 0.f, d = 0.f, q = 0.f;
     for (int i = gtid; i < m * m; i += nthreads) {
       const float x = __ldcg(A + i);
-      if (i / m != i % m)
+      const int r = i / m, c = i % m;
+      if (r != c) {
         o = fmaf(x, x, o);
-      else
+        q += square_ratio(exp_field32(x), exp_field32(__ldcg(A + r * (m + 1))), exp_field32(__ldcg(A + c * (m + 1))), floor);
+      } else {
         d = fmaf(x, x, d);
+      }
     }
     const double bo = block_total(static_cast<double>(o), S.red), bd = block_total(static_cast<double>(d), S.red);
+    const float bq = block_total(q, reinterpret_cast<float*>(S.red));
     if (tid == 0) {
       __stcg(J.slots + blockIdx.x, bo);
+      __stcg(reinterpret_cast<float*>(J.slots + 256) + blockIdx.x, bq);
       __stcg(J.slots + 512 + blockIdx.x, bd);
     }
     if (!grid.sync()) return -1;
     const double off = slots_total(J.slots, S);
+    const float rel = slots_total(reinterpret_cast<const float*>(J.slots + 256), S);
     if (sweep == 0) fro2 = off + slots_total(J.slots + 512, S);
-    if (!(off > 1e-12 * fro2) || (sweep > 0 && off <= 1e-9 * fro2 && off > 0.25 * prev)) break;
+    if (rotated32(sweep, off, prev, fro2, 1e-12, rel, prev_rel)) break;
     prev = off;
+    prev_rel = rel;
     for (int br = 0; br < nb - 1; ++br) {
       const int copy = br == 0 ? 1 : 0;  // where the problems' results lie: 31 rounds, then 16 each
       const int nA = np * (np - 1) / 2, nItems = nA + np * np;
@@ -345,32 +381,44 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
 // Bound: the chains of the local rounds.  Angles from FP32 (rotation64) instead of an FP64 division and
 // two roots, and 112 rows instead of 128 for 100 columns: a matrix of 100 columns in four clusters of
 // eigenvalues 8.3 ms, 5.4 so; 256 columns 25.3 and 19.5.
-__device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V) {
+__device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V, int floor) {
   const int tid = threadIdx.x, m = J.m, n = (J.pa + kJP - 1) / kJP * kJP, nb = n / kJW, np = nb / 2;
   const int lr_ = tid / kJP, lc_ = tid % kJP;
   const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
   double fro2 = 0.0, prev = 0.0;
-  int sweep = 0;
+  Ratios64 ratios;
+  int sweep = 0, stalled = 0;
   for (; sweep < 60; ++sweep) {
     double o = 0.0, d = 0.0;
+    float q = 0.f;
+    auto at = [m](int r, int c) { return static_cast<size_t>(r) * m + c; };
     for (int i = gtid; i < n * n; i += nthreads) {
-      const double x = __ldcg(A + static_cast<size_t>(i / n) * m + i % n);
-      if (i / n != i % n)
+      const int r = i / n, c = i % n;
+      const double x = __ldcg(A + at(r, c));
+      if (r != c) {
         o = fma(x, x, o);
-      else
+        q += square_ratio(exp_field(x), exp_field(__ldcg(A + at(r, r))), exp_field(__ldcg(A + at(c, c))), floor);
+      } else {
         d = fma(x, x, d);
+      }
     }
     const double bo = block_total(o, S.red), bd = block_total(d, S.red);
+    const float bq = block_total(q, reinterpret_cast<float*>(S.red));
     if (tid == 0) {
       __stcg(J.slots + blockIdx.x, bo);
+      __stcg(reinterpret_cast<float*>(J.slots + 256) + blockIdx.x, bq);
       __stcg(J.slots + 512 + blockIdx.x, bd);
     }
     if (!grid.sync()) return -1;
     const double off = slots_total(J.slots, S);
+    const float rel = slots_total(reinterpret_cast<const float*>(J.slots + 256), S);
     if (sweep == 0) fro2 = off + slots_total(J.slots + 512, S);
     // converged: off-diagonal mass negligible, or (block updates leave rounding noise in every
-    // off-diagonal entry) no longer falling quadratically once below 1e-26 of ||A||^2
-    if (off == 0.0 || off <= 1e-34 * fro2 || (sweep > 0 && off <= 1e-26 * fro2 && off > 0.0625 * prev)) break;
+    // off-diagonal entry) no longer falling quadratically, at once at the level of rounding (2e-15 an
+    // entry), in four sweeps below 1e-26 of ||A||^2; and the same in the pairs' own units
+    stalled = sweep > 0 && off > 0.0625 * prev ? stalled + 1 : 0;
+    const bool norm = off <= 1e-34 * fro2 || (stalled >= 1 && off <= 4e-30 * n * fro2) || (stalled >= 4 && off <= 1e-26 * fro2);
+    if (off == 0.0 || ratios.done(norm, rel, n)) break;
     prev = off;
     for (int br = 0; br < nb - 1; ++br) {
       // (1) every block pair's kJP x kJP diagonal problem: one cyclic Jacobi sweep in shared
@@ -488,7 +536,7 @@ int jacobi_grid_blocks(int pa, int sms) {
   const int np = jacobi_order(pa) / kJP;
   int g = 2 * np * np;
   if (g > sms) g = sms;
-  if (g > 256) g = 256;  // two partial sums per block, at 0 and 512 of the 1024 slots
+  if (g > 256) g = 256;  // three partial sums per block, at 0, 256 and 512 of the 1024 slots
   return g < 1 ? 1 : g;
 }
 
@@ -526,7 +574,8 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     if (tid == 0) __stcg(J.slots + blockIdx.x, f);
     alive = grid.sync();
   }
-  const double fro2 = alive ? slots_total(J.slots, S) : 0.0;
+  const double fro2 = alive ? slots_total<double>(J.slots, S) : 0.0;
+  const int floor = smallest_variance(A, m, pa, reinterpret_cast<int*>(S.red));
   if (alive && J.basis) {
     // the seed is used only if its columns are orthonormal: max |V^T V - I| <= 1e-9
     double dev = 0.0;
@@ -564,8 +613,8 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     float* F = reinterpret_cast<float*>(J.g);  // two m x m FP32 matrices
     float* Q32 = reinterpret_cast<float*>(J.x);  // V of step 2
     auto t32 = [&](int r, int c) {
-      if (T == J.a) return scaled32(__ldcg(T + at(r, c)), E);
-      return scaled32(0.5 * (__ldcg(T + at(r, c)) + __ldcg(T + at(c, r))), E);
+      if (T == J.a) return scaled32(__ldcg(T + at(r, c)), E - kUp32);
+      return scaled32(0.5 * (__ldcg(T + at(r, c)) + __ldcg(T + at(c, r))), E - kUp32);
     };
     if (m <= k32Max) {
       if (blockIdx.x == 0) {
@@ -578,10 +627,10 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
         __syncthreads();
         int n = 0, copy = 0;
         switch (m) {
-          case 16: n = jacobi32<16>(sA, sV, 20, S.s32, copy); break;
-          case 32: n = jacobi32<32>(sA, sV, 20, S.s32, copy); break;
-          case 48: n = jacobi32<48>(sA, sV, 20, S.s32, copy); break;
-          default: n = jacobi32<64>(sA, sV, 20, S.s32, copy); break;
+          case 16: n = jacobi32<16>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
+          case 32: n = jacobi32<32>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
+          case 48: n = jacobi32<48>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
+          default: n = jacobi32<64>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
         }
         sV += copy * m * m;
         for (int i = tid; i < m * m; i += kThreads) __stcg(Q32 + i, sV[i]);
@@ -596,7 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
       }
       alive = grid.sync();
       if (alive) {
-        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32);
+        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32, floor32(floor, E));
         alive = sweeps >= 0;
       }
     }
@@ -613,34 +662,33 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     }
     double* W = J.x;  // A X, then the corrections
     X = J.w;
-    const double noise = kNoise * sqrt(fro2), coarse = kCoarse * sqrt(fro2);
-    for (int it = 0; alive && it < 5; ++it) {
+    const Noise noise = noise_of(E, pa);
+    float* weights = reinterpret_cast<float*>(J.slots + 256);
+    for (int it = 0; alive && it < kSteps; ++it) {
       grid_product(
           m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(X + at(k, j)); },
           [&](int i, int j, double v) { __stcg(W + at(i, j), v); });
       if (!(alive = grid.sync())) break;
-      grid_grams(m, S, X, W, J.b, J.g);
+      grid_grams(m, S, X, W, J.b, J.g, A, noise.E, weights);
       if (!(alive = grid.sync())) break;
-      if (tid < m) S.lambda[tid] = __ldcg(J.b + at(tid, tid)) / __ldcg(J.g + at(tid, tid));
+      if (tid < m) {
+        const double l = __ldcg(J.b + at(tid, tid)) / __ldcg(J.g + at(tid, tid));
+        S.lambda[tid] = l;
+        S.noise[tid] = noise.column(l, __ldcg(weights + tid), S.nf[tid], S.ni[tid]);
+      }
       __syncthreads();
-      int bad = 0;
-      double mx = 0.0;
+      int found = 0;
       for (int i = gtid; i < m * m; i += nthreads) {
         const int r = i / m, c = i % m;
-        const double e = correction(r, c, __ldcg(J.b + i), __ldcg(J.g + i), S.lambda[r], S.lambda[c], noise,
-                                    it == 0 ? coarse : 0.0, mx, bad);
+        const double e = correction(r, c, __ldcg(J.b + i), __ldcg(J.g + i), S.lambda[r], S.lambda[c],
+                                    S.noise[r] * S.noise[c], S.nf[r] * S.ni[c], S.nf[c] * S.ni[r], it, it == 0, found);
         __stcg(W + i, e);
       }
-      mx = block_max(mx, S.red);
-      const double fb = block_max(static_cast<double>(bad), S.red);
-      if (tid == 0) {
-        __stcg(J.slots + blockIdx.x, mx);
-        __stcg(J.slots + 512 + blockIdx.x, fb);
-      }
+      found = block_or(found, reinterpret_cast<int*>(S.red));
+      if (tid == 0) __stcg(reinterpret_cast<int*>(J.slots + blockIdx.x), found);
       if (!(alive = grid.sync())) break;
-      mx = slots_max(J.slots, S);
-      const double anybad = slots_max(J.slots + 512, S);
-      if (anybad > 1.5 || mx > 0.5) break;  // not a refinement any more
+      found = slots_or(J.slots, S);
+      if (found & kFailed) break;
       grid_product(
           m, S, [&](int i, int k) { return __ldcg(X + at(i, k)); }, [&](int k, int j) { return __ldcg(W + at(k, j)); },
           [&](int i, int j, double v) { __stcg(Xn + at(i, j), __ldcg(X + at(i, j)) + v); });
@@ -648,8 +696,8 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
       double* t = X;
       X = Xn;
       Xn = t;
-      if (mx <= kRefined) {
-        refined = anybad == 0.0;
+      if (!(found & kMore)) {
+        refined = !(found & kClose);
         warm = !refined;
         break;
       }
@@ -677,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     }
     alive = alive && grid.sync();
     if (alive) {
-      const int n = grid_jacobi64(J, grid, S, A, J.b, X);
+      const int n = grid_jacobi64(J, grid, S, A, J.b, X, floor);
       alive = n >= 0;
       sweeps += max(n, 0);
       if (alive && tid < m) S.lambda[tid] = __ldcg(A + at(tid, tid));

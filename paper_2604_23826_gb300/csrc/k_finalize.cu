@@ -331,19 +331,19 @@ struct MixedScratch {
     Scratch32 s32;
     Scratch64 s64;
   };
-  double lambda[kEigBlockMax], gd[kEigBlockMax], red[8];
-  double found[kTeamMax][2];  // each block's largest correction and what it found bad
+  double lambda[kEigBlockMax], noise[kEigBlockMax], gd[kEigBlockMax], red[8];
+  float diag[kEigBlockMax], nf[kEigBlockMax], ni[kEigBlockMax];
+  double found[kTeamMax];  // what each block found
 };
 
 // Eigenpairs of A (n x n, 1 <= n <= 64, anywhere) in one block: FP32 Jacobi, FP64 refinement, and FP64
 // Jacobi from the refined basis where eigenvalues are too close for it (or from A as it is).  X, W, S:
 // shared memory of leading dimension ld (odd, above n), S right behind W.  The eigenvalues are left in M.lambda, the
 // vectors in the columns of X (which may become the buffer S or W was).  Returns the sweeps taken.
-// A team shares the refinement (not kGraded); the rotations, and everything decided, all its blocks do
+// A team shares the refinement (not kSmall); the rotations, and everything decided, all its blocks do
 // alike.
-// kGraded (at most 23 columns; else at least 24): the refinement goes on until an off-diagonal is small against its own two eigenvalues, not
-// only against the largest, as covariances of columns of very different units want it.
-template <bool kGraded>
+// kSmall: at most 23 columns; else at least 24.
+template <bool kSmall>
 __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double* S, int ld, MixedScratch& M,
                            const Team& team) {
   const int tid = threadIdx.x, first = tid + team.rank * kThreads, step = team.size * kThreads;
@@ -351,6 +351,7 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
   double f = 0.0;
   for (int i = tid; i < n * n; i += kThreads) f = fma(A[i], A[i], f);
   const double fro2 = block_total(f, M.red);
+  const int floor = smallest_variance(A, n, n, reinterpret_cast<int*>(M.red));
   bool refined = false, warm = false;
   int sweeps = 0;
   if (fro2 > 1e-280 && fro2 < 1e280) {
@@ -360,30 +361,31 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
     float* fV = fA + 2 * m * m;
     for (int i = tid; i < m * m; i += kThreads) {
       const int r = i / m, c = i % m;
-      fA[i] = r < n && c < n ? scaled32(A[r * n + c], E) : 0.f;
+      fA[i] = r < n && c < n ? scaled32(A[r * n + c], E - kUp32) : 0.f;
       fV[i] = r == c ? 1.f : 0.f;
     }
+    const Noise noise = noise_of(E, n);
+    if (tid < n) M.diag[tid] = fabsf(scaled32(A[tid * n + tid], noise.E));
     __syncthreads();
     int copy = 0;
-    if (kGraded)  // at most 23 columns
-      sweeps = m == 8    ? jacobi32<8>(fA, fV, 20, M.s32, copy)
-               : m == 16 ? jacobi32<16>(fA, fV, 20, M.s32, copy)
-                         : jacobi32<24>(fA, fV, 20, M.s32, copy);
+    if (kSmall)  // at most 23 columns
+      sweeps = m == 8    ? jacobi32<8>(fA, fV, 20, floor32(floor, E), M.s32, copy)
+               : m == 16 ? jacobi32<16>(fA, fV, 20, floor32(floor, E), M.s32, copy)
+                         : jacobi32<24>(fA, fV, 20, floor32(floor, E), M.s32, copy);
     else
-      sweeps = m <= 32   ? jacobi32<32>(fA, fV, 20, M.s32, copy)
-               : m == 48 ? jacobi32<48>(fA, fV, 20, M.s32, copy)
-                         : jacobi32<64>(fA, fV, 20, M.s32, copy);
+      sweeps = m <= 32   ? jacobi32<32>(fA, fV, 20, floor32(floor, E), M.s32, copy)
+               : m == 48 ? jacobi32<48>(fA, fV, 20, floor32(floor, E), M.s32, copy)
+                         : jacobi32<64>(fA, fV, 20, floor32(floor, E), M.s32, copy);
     fV += copy * m * m;
     for (int i = tid; i < n * n; i += kThreads) X[(i / n) * ld + i % n] = f32_to_f64(fV[(i / n) * m + i % n]);
     team.meet();  // the others may put into W and S now
-    const double noise = kNoise * sqrt(fro2), coarse = kCoarse * sqrt(fro2);
-    for (int it = 0; it < 5; ++it) {
+    for (int it = 0; it < kSteps; ++it) {
       team_product(
           team, n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
           [&](int i, int j, double v) { team.put(W + i * ld + j, v); });
       team.meet();
       // X^T W on and above the diagonal of S, X^T X below it (its diagonal in gd)
-      const bool single = kGraded && n <= kOneByOne;
+      const bool single = kSmall && n <= kOneByOne;
       const int nt = single ? n : (n + 1) / 2, half = nt * (nt + 1) / 2;
       for (int t = first; t < 2 * half; t += step) {
         const bool gram = t >= half;
@@ -425,32 +427,32 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
         }
       }
       team.meet();
-      if (tid < n) M.lambda[tid] = S[tid * ld + tid] / M.gd[tid];
+      if (tid < n) {
+        const double l = S[tid * ld + tid] / M.gd[tid];
+        float w = 0.f;
+        for (int k = 0; k < n; ++k) {
+          const float x = scaled32(X[k * ld + tid], 1023);
+          w = fmaf(M.diag[k] * x, x, w);
+        }
+        M.lambda[tid] = l;
+        M.noise[tid] = noise.column(l, w, M.nf[tid], M.ni[tid]);
+      }
       __syncthreads();
-      int bad = 0;
-      double mx = 0.0;
+      int found = 0;
       for (int i = first; i < n * n; i += step) {
         const int r = i / n, c = i % n, lo = min(r, c), hi = max(r, c);
-        const double lr = M.lambda[r], lc = M.lambda[c];
-        const double e = correction(r, c, S[lo * ld + hi], r == c ? M.gd[r] : S[hi * ld + lo], lr, lc,
-                                    kGraded ? kNoise * sqrt(fabs(lr * lc)) : noise, !kGraded && it == 0 ? coarse : 0.0, mx,
-                                    bad);
+        const double e = correction(r, c, S[lo * ld + hi], r == c ? M.gd[r] : S[hi * ld + lo], M.lambda[r], M.lambda[c],
+                                    M.noise[r] * M.noise[c], M.nf[r] * M.ni[c], M.nf[c] * M.ni[r], it, !kSmall && it == 0,
+                                    found);
         team.put(W + r * ld + c, e);
       }
-      mx = block_max(mx, M.red);
-      bad = block_max(bad, reinterpret_cast<int*>(M.red));
+      found = block_or(found, reinterpret_cast<int*>(M.red));
       if (team.size > 1) {
-        if (tid == 0) {
-          team.put(&M.found[team.rank][0], mx);
-          team.put(&M.found[team.rank][1], bad > 1 ? 2.0 : bad ? 1.0 : 0.0);
-        }
+        if (tid == 0) team.put(&M.found[team.rank], __longlong_as_double(found));
         team.meet();
-        for (int r = 0; r < team.size; ++r) {
-          mx = fmax(mx, M.found[r][0]);
-          bad = max(bad, M.found[r][1] > 1.5 ? 2 : M.found[r][1] > 0.5 ? 1 : 0);
-        }
+        for (int r = 0; r < team.size; ++r) found |= static_cast<int>(__double_as_longlong(M.found[r]));
       }
-      if (bad > 1 || mx > 0.5) break;  // not a refinement any more
+      if (found & kFailed) break;
       team_product(
           team, n, [&](int k, int i) { return X[i * ld + k]; }, [&](int k, int j) { return W[k * ld + j]; },
           [&](int i, int j, double v) { team.put(S + i * ld + j, X[i * ld + j] + v); });
@@ -458,8 +460,8 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
       double* t = X;
       X = S;
       S = t;
-      if (mx <= kRefined) {
-        refined = bad == 0;
+      if (!(found & kMore)) {
+        refined = !(found & kClose);
         warm = !refined;
         break;
       }
@@ -483,7 +485,7 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
       }
     }
     __syncthreads();
-    sweeps += jacobi64(S, ld, X, ld, n, M.s64);
+    sweeps += jacobi64(S, ld, X, ld, n, floor, M.s64);
     if (tid < n) M.lambda[tid] = S[tid * ld + tid];
   }
   __syncthreads();
@@ -658,7 +660,8 @@ __device__ void finalize_body(const FinalParams& P) {
       V[i] = i / pa == i % pa ? 1.0 : 0.0;
     }
     __syncthreads();
-    const int sweeps = jacobi64(A, pa, V, pa, pa, U.any);
+    const int floor = smallest_variance(A, pa, pa, reinterpret_cast<int*>(U.any.red));
+    const int sweeps = jacobi64(A, pa, V, pa, pa, floor, U.any);
     if (tid < pa) s_lambda[tid] = A[tid * pa + tid];
     __syncthreads();
     put_eigenpairs(s_lambda, V, pa, pa, s_order, out + L.evals, out + L.evecs);
