@@ -494,9 +494,6 @@ __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_
   }
   return sweep;
 }
-// the order FP32 rotations take n columns at: a multiple of eight up to 32, of sixteen above
-__host__ __device__ constexpr int jacobi32_order(int n) { return n <= 32 ? (n + 7) / 8 * 8 : (n + 15) / 16 * 16; }
-
 // ------------------------------- refinement -------------------------------
 // What rounding leaves in an entry of X^T A X that should be zero depends on its two columns: a
 // covariance's |a_kl| <= sqrt(a_kk a_ll), so products of the columns i and j of X leave about eps b_i b_j,

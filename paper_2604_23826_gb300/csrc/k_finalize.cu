@@ -336,6 +336,22 @@ struct MixedScratch {
   double found[kTeamMax];  // what each block found
 };
 
+// The order eigen_mixed's FP32 rotations take n columns at: the matrices are laid out by it and the
+// rotations compiled for it.
+template <bool kSmall>
+__host__ __device__ constexpr int mixed_order(int n) {
+  return kSmall ? (n + 7) / 8 * 8 : n <= 32 ? 32 : (n + 15) / 16 * 16;
+}
+constexpr bool orders_exist() {
+  for (int n = 1; n <= kEigBlockMax; ++n) {
+    const bool small = n <= kSmallMax;
+    const int m = small ? mixed_order<true>(n) : mixed_order<false>(n);
+    if (m < n || !(small ? m == 8 || m == 16 || m == 24 : m == 32 || m == 48 || m == 64)) return false;
+  }
+  return true;
+}
+static_assert(orders_exist(), "eigen_mixed has the rotations of every order");
+
 // Eigenpairs of A (n x n, 1 <= n <= 64, anywhere) in one block: FP32 Jacobi, FP64 refinement, and FP64
 // Jacobi from the refined basis where eigenvalues are too close for it (or from A as it is).  X, W, S:
 // shared memory of leading dimension ld (odd, above n), S right behind W.  The eigenvalues are left in M.lambda, the
@@ -356,7 +372,7 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
   int sweeps = 0;
   if (fro2 > 1e-280 && fro2 < 1e280) {
     const int E = scale_exponent(fro2);
-    const int m = jacobi32_order(n);
+    const int m = mixed_order<kSmall>(n);
     float* fA = reinterpret_cast<float*>(W);  // W and S, one behind the other
     float* fV = fA + 2 * m * m;
     for (int i = tid; i < m * m; i += kThreads) {
@@ -368,14 +384,19 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
     if (tid < n) M.diag[tid] = fabsf(scaled32(A[tid * n + tid], noise.E));
     __syncthreads();
     int copy = 0;
-    if (kSmall)  // at most 23 columns
-      sweeps = m == 8    ? jacobi32<8>(fA, fV, 20, floor32(floor, E), M.s32, copy)
-               : m == 16 ? jacobi32<16>(fA, fV, 20, floor32(floor, E), M.s32, copy)
-                         : jacobi32<24>(fA, fV, 20, floor32(floor, E), M.s32, copy);
-    else
-      sweeps = m <= 32   ? jacobi32<32>(fA, fV, 20, floor32(floor, E), M.s32, copy)
-               : m == 48 ? jacobi32<48>(fA, fV, 20, floor32(floor, E), M.s32, copy)
-                         : jacobi32<64>(fA, fV, 20, floor32(floor, E), M.s32, copy);
+    if constexpr (kSmall) {
+      switch (m) {
+        case 8: sweeps = jacobi32<8>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+        case 16: sweeps = jacobi32<16>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+        case 24: sweeps = jacobi32<24>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+      }
+    } else {
+      switch (m) {
+        case 32: sweeps = jacobi32<32>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+        case 48: sweeps = jacobi32<48>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+        case 64: sweeps = jacobi32<64>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+      }
+    }
     fV += copy * m * m;
     for (int i = tid; i < n * n; i += kThreads) X[(i / n) * ld + i % n] = f32_to_f64(fV[(i / n) * m + i % n]);
     team.meet();  // the others may put into W and S now

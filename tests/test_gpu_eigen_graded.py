@@ -78,6 +78,19 @@ def test_close_eigenvalues_of_small_units(p, width):
         check(an)
 
 
+@pytest.mark.parametrize("p", [24, 25, 31, 32, 33, 40, 47, 48, 49, 56, 63, 64])
+def test_batched_results_come_from_the_refinement(p):
+    """Well separated eigenvalues: the refinement of a batch adds the same products in the same order as the
+    grid's, after FP32 rotations of the same order, so its results are a single call's bits; FP64 rotations
+    (what a batch falls back to) leave others."""
+    X = separated(p, 0)
+    a, b = context(X, N), context(X, N)
+    single = G.stats_finalize(a)
+    check(single)
+    for an in G.stats_finalize_batched([a, b]):
+        assert np.array_equal(an.evals, single.evals) and np.array_equal(an.evecs, single.evecs)
+
+
 def test_snapshots_agree_with_cold_results():
     """A stream's seeded snapshots against the cold result of the same rows, vector by vector."""
     X = separated(12, 6)
