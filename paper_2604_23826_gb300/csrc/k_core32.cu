@@ -22,7 +22,8 @@
 // per element, 0.427 ms now (its FMAs alone: 0.135 ms).
 // Each block writes one slot of (hi, lo) pairs; a second kernel adds the slots of an entry in row
 // order, in three-term FP32 expansions and then FP64 pairs (a fixed order: a given grid
-// reproduces its bits).
+// reproduces its bits).  Sums that leave FP32's range on the way are added in FP64 instead, so only a
+// thread's own rows have to stay within it.
 #include <algorithm>
 
 #include "core.cuh"
@@ -60,6 +61,11 @@ __device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) {
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   f32x2 d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
@@ -204,8 +210,25 @@ __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ 
     const float2 w = parts(v[e / kMJ / 2][e % kMJ]);
     return (e / kMJ) & 1 ? w.y : w.x;
   };
-  // the slices' pairs, added in a fixed tree through shared memory
+  // the slices' pairs, added in a fixed tree through shared memory; near the end of FP32's range all of the
+  // block's are taken at 2^-10 (at most 512 slices)
   float2* buf = reinterpret_cast<float2*>(smem);
+  float scale = 1.f;
+  if (P.slices > 1) {
+    float top = 0.f;
+#pragma unroll
+    for (int e = 0; e < kE; ++e) top = fmaxf(top, fabsf(at(hi, e)));
+    if (__syncthreads_or(top >= 0x1p117f)) {
+      scale = 0x1p10f;
+#pragma unroll
+      for (int i = 0; i < kMI / 2; ++i)
+#pragma unroll
+        for (int j = 0; j < kMJ; ++j) {
+          hi[i][j] = mul2(hi[i][j], twice(0x1p-10f));
+          lo[i][j] = mul2(lo[i][j], twice(0x1p-10f));
+        }
+    }
+  }
   for (int n = P.slices; n > 1;) {
     const int h = (n + 1) / 2;
     __syncthreads();
@@ -251,12 +274,14 @@ __global__ void __launch_bounds__(kNT, 1) core32_kernel(const __grid_constant__ 
     }
     slot[static_cast<size_t>(kE) * tg + tid] = make_float2(h, l);
   }
+  if (tid == 0) slot[static_cast<size_t>(kE) * tg + W] = make_float2(scale, 0.f);
 }
 
 // Adds the ranges' slots of 32 entries per block (kSeg consecutive runs of ranges at once) into
 // the accumulators.  Within a run a three-term FP32 expansion keeps every rounding of the pairs'
 // additions (72 bits; FP64 adds would cost 64 cycles a warp each); the runs are added in order in
-// FP64 pairs.
+// FP64 pairs.  A run that leaves FP32's range, and all runs when some block scaled its sums, are added
+// in FP64 pairs throughout.
 constexpr int kSeg = 8;
 __device__ __forceinline__ float two_sum32(float& s, float v) {
   const float t = s + v, bp = t - s, e = (s - (t - bp)) + (v - bp);
@@ -264,13 +289,19 @@ __device__ __forceinline__ float two_sum32(float& s, float v) {
   return e;
 }
 
-__global__ void __launch_bounds__(32 * kSeg) core32_merge_kernel(const __grid_constant__ Core32Params P) {
+__global__ void __launch_bounds__(32 * kSeg, 8) core32_merge_kernel(const __grid_constant__ Core32Params P) {
   __shared__ double sh[kSeg][32], sl[kSeg][32];
   const int p = P.p, tg = P.tiles_per_group, lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
   const int nS = P.ntiles * kE;
   const int x = blockIdx.x * 32 + lane;  // entry: tiles' values, then the column sums
   const size_t sp = core32_slot_pairs(p, tg);
-  int j = -1, k = -1;
+  const float2* slots = reinterpret_cast<const float2*>(P.slots);
+  const size_t at_scale = static_cast<size_t>(kE) * tg + width_of(p);
+  bool scaled = false;
+  for (int b = threadIdx.x; P.slices > 1 && b < P.groups * P.ranges; b += blockDim.x)
+    scaled |= __ldcg(slots + b * sp + at_scale).x != 1.f;
+  scaled = __syncthreads_or(scaled);
+  int j = -1, k = -1, group = 0;
   size_t off = 0;
   if (x < nS) {
     const int e = x / P.ntiles, t = x % P.ntiles, g = t / tg;
@@ -279,16 +310,17 @@ __global__ void __launch_bounds__(32 * kSeg) core32_merge_kernel(const __grid_co
     j = kMI * bi + e / kMJ;
     k = kMJ * bj + e % kMJ;
     if (j > k || k >= p) j = -1;
-    off = static_cast<size_t>(g) * sp + static_cast<size_t>(e) * tg + (t - g * tg);
+    group = g;
+    off = static_cast<size_t>(e) * tg + (t - g * tg);
   } else if (x < nS + p) {
     j = k = x - nS;
     off = static_cast<size_t>(kE) * tg + j;
   }
   float h = 0.f, l = 0.f, ll = 0.f;
-  if (j >= 0) {
-    const float2* src = reinterpret_cast<const float2*>(P.slots) + off;
-    const size_t step = static_cast<size_t>(P.groups) * sp;
-    const int r0 = P.ranges * seg / kSeg, r1 = P.ranges * (seg + 1) / kSeg;
+  const float2* src = slots + group * sp + off;
+  const size_t step = static_cast<size_t>(P.groups) * sp;
+  const int r0 = P.ranges * seg / kSeg, r1 = P.ranges * (seg + 1) / kSeg;
+  if (j >= 0 && !scaled) {
 #pragma unroll 8
     for (int r = r0; r < r1; ++r) {
       const float2 v = __ldcg(src + r * step);
@@ -298,8 +330,19 @@ __global__ void __launch_bounds__(32 * kSeg) core32_merge_kernel(const __grid_co
     }
   }
   double dh = h, dl = 0.0;
-  pair_add(dh, dl, static_cast<double>(l));
-  dl += ll;
+  if (j >= 0 && (scaled || !(fabsf(h) <= 0x1.fffffep127f))) {
+    const float2* scales = slots + group * sp + at_scale;
+    dh = 0.0;
+    for (int r = r0; r < r1; ++r) {
+      const float2 v = __ldcg(src + r * step);
+      const double s = x < nS ? __ldcg(scales + r * step).x : 1.0;
+      pair_add(dh, dl, v.x * s);
+      dl += v.y * s;
+    }
+  } else {
+    pair_add(dh, dl, static_cast<double>(l));
+    dl += ll;
+  }
   sh[seg][lane] = dh;
   sl[seg][lane] = dl;
   __syncthreads();
@@ -352,6 +395,13 @@ void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P) {
   P.log_rows = lr;
   const int64_t nst = (nrows + (int64_t(1) << lr) - 1) >> lr;
   P.ranges = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, nst)));
+  // Sums of squares up to FP32's range are promised for a thread's rows as 64 x 64 tiles of four blocks an SM
+  // dealt them, 4096 rows a block at least.  Wide tables of few slices (176..192 columns and from 252 on)
+  // give a thread up to a third more, and take their rows in two launches.
+  const int nb = (p + 63) / 64, tiles = nb * (nb + 1) / 2;
+  const int64_t dealt = std::min<int64_t>(nrows / 4096, (4 * int64_t(sms) + tiles - 1) / tiles);
+  P.launches = blocks <= 0 && int64_t(P.ranges) * P.slices < dealt ? 2 : 1;
+  P.ranges *= P.launches;
 }
 
 size_t core32_slot_bytes(const Core32Params& P) {
@@ -362,9 +412,18 @@ cudaError_t launch_core32(const Core32Params& P, cudaStream_t stream) {
   const size_t smem = smem_bytes(width_of(P.p), 1 << P.log_rows);
   cudaError_t e = cudaFuncSetAttribute(core32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  core32_kernel<<<P.groups * P.ranges, kNT, smem, stream>>>(P);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  const int64_t nst = (P.nrows + (int64_t(1) << P.log_rows) - 1) >> P.log_rows;
+  for (int i = 0; i < P.launches; ++i) {  // whole stages: the columns stay as aligned as they were
+    const int64_t first = nst * i / P.launches << P.log_rows;
+    Core32Params Q = P;
+    Q.ranges = P.ranges / P.launches;
+    Q.nrows = std::min(P.nrows, nst * (i + 1) / P.launches << P.log_rows) - first;
+    Q.slots = P.slots + 2 * core32_slot_pairs(P.p, P.tiles_per_group) * P.groups * Q.ranges * i;
+    for (int c = 0; c < P.p; ++c) Q.cols[c] = static_cast<const char*>(P.cols[c]) + first * dtype_bytes(P.dtype[c]);
+    core32_kernel<<<P.groups * Q.ranges, kNT, smem, stream>>>(Q);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   core32_merge_kernel<<<(P.ntiles * kE + P.p + 31) / 32, 32 * kSeg, 0, stream>>>(P);
   return cudaGetLastError();
 }

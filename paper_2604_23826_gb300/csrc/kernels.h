@@ -280,8 +280,8 @@ struct Core32Params {
   int32_t flush_rows;   // rows of a thread between flushes into (hi, lo) pairs
   int64_t nrows;
   // the cut (core32_plan): micro-tiles, groups of blocks over them, row slices of a block,
-  // 2^log_rows rows a stage, row ranges; groups * ranges blocks
-  int32_t ntiles, groups, tiles_per_group, slices, log_rows, ranges;
+  // 2^log_rows rows a stage, row ranges; groups * ranges blocks, in one or two launches
+  int32_t ntiles, groups, tiles_per_group, slices, log_rows, ranges, launches;
   float* slots;         // scratch: core32_slot_bytes
   double* acc_s;        // ctx accumulators, double-double
   double* acc_s_lo;
@@ -289,9 +289,9 @@ struct Core32Params {
   double* acc_S_lo;
   long long* acc_n;
 };
-// (hi, lo) pairs of a block's slot: its tiles' entries, then the padded columns' sums
+// (hi, lo) pairs of a block's slot: its tiles' entries, the padded columns' sums, and the entries' scale
 __host__ __device__ inline size_t core32_slot_pairs(int p, int tiles_per_group) {
-  return static_cast<size_t>(tiles_per_group) * 32 + (p + 7) / 8 * 8;
+  return static_cast<size_t>(tiles_per_group) * 32 + (p + 7) / 8 * 8 + 1;
 }
 void core32_plan(int p, int64_t nrows, int sms, int blocks, Core32Params& P);
 size_t core32_slot_bytes(const Core32Params& P);
