@@ -15,9 +15,14 @@
 // 250,001 rows x 48 columns: 6.60 ms as 64 x 64 tiles on 61 blocks, 0.67 ms now (FMAs, shift and
 // sums of those rows alone: 0.50 ms), plus 12 us to add the slots.  Up to 12 columns one thread kept a
 // row's 90 sums in registers (2e7 rows of Table 1: 5.08 ms); its eight warps an SM spent half their
-// time on loads and conversions.  This way: 3.85 ms (90 operations a row alone: 2.9 ms).
+// time on loads and conversions.  This way: 3.88 ms (90 operations a row alone: 2.9 ms).
 // Each block writes one slot; a second kernel adds an entry's slots in row order into the ctx's
 // double-double accumulators (a fixed order: a given grid reproduces its bits).
+// Sums are kept in blocks: a 2 x 2 tile's and a column's go to a second sum every kChain of a thread's rows
+// or less (one addition in 128 FMAs or more), so the roundings on the way to a slot are at most kChain, the
+// number of those blocks and the slices' tree: fewer at any row count than the 300 and a 78,000th of the
+// rows that a grid of row-per-thread sums had (unblocked: an 8,000th; 12 columns x 1e7 rows 1.98 ms, 2.00 so).  4 x 4 tiles, from 13 columns on, have no registers
+// for it and more threads to a row than 64 x 64 tiles had.
 #include <algorithm>
 
 #include "core.cuh"
@@ -30,6 +35,7 @@ using namespace core;
 
 constexpr int kMaxThreads = 512;
 constexpr int kBatch = 4;  // loads a lane has in flight
+constexpr int kChain = 256;
 
 __host__ __device__ inline int row_stride(int p, int MI) { return ((p + MI - 1) / MI * MI) | 1; }
 
@@ -54,7 +60,16 @@ __device__ __forceinline__ void convert_rows(const void* col, int64_t r0, int ro
 }
 
 template <int MI>
-__global__ void __launch_bounds__(kMaxThreads) core64_kernel(const __grid_constant__ Core64Params P) {
+constexpr bool kBlocked = MI == 2;
+// shared memory ahead of the second sums: a stage's rows, or the slices' partial sums
+__host__ __device__ inline size_t first_bytes(const Core64Params& P, int MI) {
+  const size_t rows = (size_t(1) << P.log_rows) * row_stride(P.p, MI), tree = static_cast<size_t>(MI) * MI * (P.threads / 2);
+  return (rows > tree ? rows : tree) * sizeof(double);
+}
+
+// (registers: blocks of 384 threads fit three and two times on an SM)
+template <int MI>
+__global__ void __maxnreg__(MI == 2 ? 56 : 80) core64_kernel(const __grid_constant__ Core64Params P) {
   constexpr int kE = MI * MI;
   extern __shared__ __align__(16) uint8_t smem[];
   double* X = reinterpret_cast<double*>(smem);  // [R][S], rows of x - c
@@ -76,6 +91,10 @@ __global__ void __launch_bounds__(kMaxThreads) core64_kernel(const __grid_consta
     for (int j = 0; j < MI; ++j) acc[i][j] = 0.0;
   const int cc = tid % p, cq = tid / p, ncq = NT / p;  // column sums: this thread's column and rows
   double s = 0.0;
+  // second sums of this thread's entries and column, in shared memory (registers would cost a block an SM)
+  double* second = reinterpret_cast<double*>(smem + first_bytes(P, MI)) + tid;
+  if (kBlocked<MI>)
+    for (int e = 0; e <= kE; ++e) second[e * NT] = 0.0;
   // the columns that pad the last micro-tile are zero
   for (int i = tid; i < R * (S - p); i += NT) X[(i / (S - p)) * S + p + i % (S - p)] = 0.0;
 
@@ -116,6 +135,20 @@ __global__ void __launch_bounds__(kMaxThreads) core64_kernel(const __grid_consta
           for (int j = 0; j < MI; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
       }
     }
+    if (kBlocked<MI> && (st & P.chain_mask) == 0) {
+#pragma unroll
+      for (int e = 0; e < kE; ++e) {
+        second[e * NT] += acc[e / MI][e % MI];
+        acc[e / MI][e % MI] = 0.0;
+      }
+      second[kE * NT] += s;
+      s = 0.0;
+    }
+  }
+  if (kBlocked<MI>) {
+#pragma unroll
+    for (int e = 0; e < kE; ++e) acc[e / MI][e % MI] += second[e * NT];
+    s += second[kE * NT];
   }
   // the slices' partial sums, added in a fixed tree through shared memory
   double* buf = X;
@@ -202,8 +235,7 @@ __global__ void __launch_bounds__(32 * kSeg) core64_merge_kernel(const __grid_co
 }
 
 size_t smem_bytes(const Core64Params& P) {
-  return std::max<size_t>((size_t(1) << P.log_rows) * row_stride(P.p, P.micro) * sizeof(double),
-                          static_cast<size_t>(P.micro) * P.micro * (P.threads / 2) * sizeof(double));
+  return first_bytes(P, P.micro) + (P.micro == 2 ? 5 * sizeof(double) * P.threads : 0);
 }
 
 const void* kernel_of(int micro) {
@@ -216,6 +248,7 @@ const void* kernel_of(int micro) {
 cudaError_t core64_plan(int p, int64_t nrows, bool shifted, int sms, int blocks, Core64Params& P) {
   double best = 0;
   for (int micro : {4, 2}) {
+    if (micro == 4 && p <= 12) continue;
     const int M = core::tile_count(p, micro, micro);
     for (int nt = 128; nt <= kMaxThreads; nt += 128) {
       if (nt < p) continue;  // the column sums take a thread per column
@@ -245,6 +278,9 @@ cudaError_t core64_plan(int p, int64_t nrows, bool shifted, int sms, int blocks,
          (nrows >> (lr + 1)) >= 4 * int64_t(std::max(1, sms / P.groups)))
     ++lr;
   P.log_rows = lr;
+  const int per_stage = ((1 << lr) + std::min(P.slices, P.threads / p) - 1) / std::min(P.slices, P.threads / p);
+  P.chain_mask = 0;  // a thread's rows of chain_mask + 1 stages: at most kChain, or one stage's
+  while (2 * (P.chain_mask + 1) * per_stage <= kChain) P.chain_mask = 2 * P.chain_mask + 1;
   const size_t smem = smem_bytes(P);
   cudaError_t e = cudaFuncSetAttribute(kernel_of(P.micro), cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;

@@ -305,6 +305,7 @@ struct Core64Params {
   // the cut (core64_plan): order of the micro-tiles, their number, threads of a block, groups of
   // blocks over the tiles, row slices of a block, 2^log_rows rows a stage, row ranges
   int32_t micro, ntiles, threads, groups, tiles_per_group, slices, log_rows, ranges;
+  int32_t chain_mask;   // sums go to their second level after each stage of a multiple of this plus one
   double* slots;        // scratch: core64_slot_bytes
   double* acc_s;        // ctx accumulators, double-double
   double* acc_s_lo;
