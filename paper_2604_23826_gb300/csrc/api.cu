@@ -986,7 +986,11 @@ stats_status launch_pass(stats_ctx* c, const void* const* dcols, int64_t nrows, 
       C.shift = c->d_shift;
     }
     CK(c, core64_plan(c->p, nrows, C.shift != nullptr, c->sms, c->grid, C));
-    const stats_status s = ensure_core_slots(c, core64_slot_bytes(C));
+    // up to 12 columns the first call's scratch serves calls of any size (half a megabyte): a larger one
+    // neither waits for the device nor allocates, also under stream capture
+    size_t bytes = core64_slot_bytes(C);
+    if (c->p <= 12) bytes = std::max(bytes, bytes / C.ranges * std::max(4 * c->sms, c->grid));
+    const stats_status s = ensure_core_slots(c, bytes);
     if (s != STATS_OK) return s;
     C.nrows = nrows;
     C.slots = static_cast<double*>(c->d_core_slots);
