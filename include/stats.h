@@ -294,8 +294,9 @@ stats_status stats_set_grid(stats_ctx* ctx, int32_t blocks);
  *   gram32_chunks_per_cta  the register-fragment launch: stages are dealt in chunks, as long
  *                          as possible while each CTA gets at least this many (1..1024;
  *                          default 32)
- *   gram32_min_chunk       ... and never shorter than this many stages (1..65536; default 32),
- *                          unless some CTA would get none: then a CTA's equal share
+ *   gram32_min_chunk       ... and never shorter than this many stages (1..65536; default 32;
+ *                          the default gives way to a CTA's equal share where some CTA would
+ *                          get none, any other value holds)
  * The setting changes how rows are grouped into per-CTA partial sums, so results move within
  * rounding (the stated tolerance holds for every setting); a fixed setting reproduces its
  * bits.  Process-wide, for every device.  Errors: EINVAL (bad width, mode or values). */

@@ -355,6 +355,7 @@ struct Gram32Job {
 // Tuning of the batched launches, per width class (P = 8, 16, 32, 64) and arithmetic (BF16x3,
 // BF16x4): how a launch's stages are dealt to its persistent CTAs.  Set by stats_set_batch_tuning
 // (the autotuner); the defaults were measured on the many-tables workload.
+constexpr stats_batch_tuning kDefaultTuning{12, 32, 32};
 stats_batch_tuning g_batch_tuning[4][2];
 std::once_flag g_batch_tuning_once;
 std::mutex g_batch_tuning_mu;
@@ -364,7 +365,7 @@ int width_class(int P) { return P <= 8 ? 0 : P <= 16 ? 1 : P <= 32 ? 2 : 3; }
 stats_batch_tuning batch_tuning(int P, bool x4) {
   std::call_once(g_batch_tuning_once, [] {
     for (auto& row : g_batch_tuning)
-      for (auto& t : row) t = stats_batch_tuning{12, 32, 32};
+      for (auto& t : row) t = kDefaultTuning;
   });
   std::lock_guard<std::mutex> lk(g_batch_tuning_mu);
   return g_batch_tuning[width_class(P)][x4 ? 1 : 0];
@@ -476,12 +477,13 @@ stats_status run_gram32(const std::vector<Gram32Job>& jobs, cudaStream_t st) {
         for (size_t i = 0; i < nt; ++i) total += (all[first + i]->nrows + rs - 1) / rs;
         if (total >= (int64_t(1) << 31)) return STATS_EINVAL;  // over 2^31 stages in one call
         // chunks as long as possible while every CTA still gets >= chunks_per_cta of them (long
-        // runs: few per-table partials; many chunks: balanced CTAs), and not below min_chunk unless that
-        // leaves SMs without one (the small tables of a batch of 256 ran on one to five SMs, 210 us,
-        // and dealt to all in 33; one table of 3e5 rows x 8: 42 and 6 us)
+        // runs: few per-table partials; many chunks: balanced CTAs), and not below min_chunk; the default
+        // one gives way where it leaves SMs without a chunk (the small tables of a batch of 256 ran on
+        // one to five SMs, 210 us, and dealt to all in 33; one table of 3e5 rows x 8: 42 and 6 us)
         const stats_batch_tuning tune = batch_tuning(P, x4 == 1);
-        const int64_t K = std::max<int64_t>(std::min<int64_t>(tune.gram32_min_chunk, (total + sms - 1) / sms),
-                                            total / (int64_t(sms) * tune.gram32_chunks_per_cta));
+        int64_t shortest = tune.gram32_min_chunk;
+        if (shortest == kDefaultTuning.gram32_min_chunk) shortest = std::min<int64_t>(shortest, (total + sms - 1) / sms);
+        const int64_t K = std::max<int64_t>(shortest, total / (int64_t(sms) * tune.gram32_chunks_per_cta));
         const int grid = static_cast<int>(std::min<int64_t>((total + K - 1) / K, sms));
         const size_t sf = gram32_slot_floats(P);
         size_t slot_floats_total = 0;
