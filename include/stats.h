@@ -106,8 +106,9 @@ typedef enum {
  *                 column; may be NULL.  STATS_EXACT only: they fix each column's
  *                 digit field (integers: the bytes needed for [lo, hi]; reals: the
  *                 binary exponent e with max(|lo|,|hi|) < 2^e, fixed point
- *                 q = round(x * 2^(P - e)) with 56 bits).  NULL means the full
- *                 range of the integer dtype; real columns need bounds in STATS_EXACT.
+ *                 q = round(x * 2^(P - e)) with 56 bits, to nearest, ties to even).
+ *                 NULL means the full range of the integer dtype; real columns need
+ *                 bounds in STATS_EXACT.
  *   mode          a stats_mode value                                              */
 typedef struct {
   int32_t p;

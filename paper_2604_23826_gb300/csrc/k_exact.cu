@@ -104,9 +104,9 @@ struct SmemT1Src {
 };
 
 // The Table 1 real columns convert on the FP64 unit: q = round-to-nearest-even(x * 2^sh),
-// the scaling an exponent-field add (exact), zero and subnormal inputs giving 0.  (The
-// integer-only fixed_rn keeps the ALU pipe busier; on sm_103a the FP64 conversion
-// unit sustains about two per clock per SM, well above what this pass needs.)
+// the scaling an exponent-field add (exact), zero and subnormal inputs giving 0.  (In integers alone
+// the ALU pipe is busier; on sm_103a the FP64 conversion unit sustains about two per clock per SM,
+// well above what this pass needs.)
 __device__ __forceinline__ uint64_t fixed_f2i(double x, int sh) {
   const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
   const uint32_t scaled = (hi & 0x7FF00000u) != 0 ? hi + (static_cast<uint32_t>(sh) << 20) : 0u;
@@ -258,15 +258,22 @@ struct ConvGeneric {
   }
   static constexpr bool kPair = true, kAdjacent = false;  // two rows per lane share the walk over the columns
   static constexpr float kUnit = 1.f;                     // digits as f16 integers
-  // q = round(x * 2^sh); range violations into bad
+  // q = round(x * 2^sh) to nearest, ties to even; range violations into bad
   __device__ __forceinline__ static uint64_t real_field(double x, int sh, int emax, bool is_signed, uint32_t& bad) {
-    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
-    const int ef = static_cast<int>((hi >> 20) & 0x7FFu);
+    uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+    int ef = static_cast<int>((hi >> 20) & 0x7FFu);
     bad |= ef > emax;
     if (!is_signed) bad |= (hi >> 31) & (((hi << 1) | lo) != 0);  // negative, not -0
     // the scaling is an exponent-field add, the rounding one conversion on the FP64 unit; a scaled
-    // value below the normal range rounds to 0, a subnormal input is scaled by integers
-    if (ef == 0) return ((hi << 1) | lo) ? fixed_rn<true>(x, sh) : 0;
+    // value below the normal range rounds to 0, a subnormal input is made normal first
+    if (ef == 0) {
+      if (((hi << 1) | lo) == 0) return 0;
+      x *= 18014398509481984.0;  // 2^54
+      sh -= 54;
+      hi = static_cast<uint32_t>(__double2hiint(x));
+      lo = static_cast<uint32_t>(__double2loint(x));
+      ef = static_cast<int>((hi >> 20) & 0x7FFu);
+    }
     return ef + sh > 0 ? static_cast<uint64_t>(__double2ll_rn(__hiloint2double(
                              static_cast<int>(hi + (static_cast<uint32_t>(sh) << 20)), static_cast<int>(lo))))
                        : 0;
