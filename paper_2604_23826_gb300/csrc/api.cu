@@ -117,6 +117,7 @@ struct stats_ctx {
   void* h_stage[2] = {nullptr, nullptr};
   size_t h_stage_bytes = 0;
   cudaStream_t last = nullptr;
+  cudaEvent_t ev_default = nullptr;     // the default stream's work before a finalize on another stream
   int grid = 0;
   int sms = 0;
   // rows enqueued into the accumulator so far (host-side count; reset, merge and import keep it)
@@ -1082,6 +1083,11 @@ stats_status run_finalize(stats_ctx* c, int want_pca, int pca_on, const double* 
     if (seed) CK(c, cudaMemcpyAsync(basis, seed, sizeof(double) * pa * pa, cudaMemcpyHostToDevice, st));
     CK(c, cudaMemsetAsync(J.bar, 0, 8 * sizeof(unsigned int), st));
   }
+  if (st) {  // behind the default stream's work too: a replayed graph's passes may run there
+    if (!c->ev_default) CK(c, cudaEventCreateWithFlags(&c->ev_default, cudaEventDisableTiming));
+    CK(c, cudaEventRecord(c->ev_default, nullptr));
+    CK(c, cudaStreamWaitEvent(st, c->ev_default, 0));
+  }
   CK(c, launch_finalize(F, st));
   if (grid > 0) CK(c, launch_jacobi_grid(J, grid, st));
   CK(c, cudaMemcpyAsync(c->h_out, c->d_out, c->lay.total * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1109,6 +1115,7 @@ void free_ctx(stats_ctx* c) {
     if (c->ev_copied[b]) cudaEventDestroy(c->ev_copied[b]);
     if (c->ev_done[b]) cudaEventDestroy(c->ev_done[b]);
   }
+  if (c->ev_default) cudaEventDestroy(c->ev_default);
   if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
   delete c;
 }
