@@ -604,8 +604,8 @@ def run_ours(args, rank: int, world: int, local_rank: int):
 MODE_NAMES = {"BF16X3": "STATS_BF16X3", "BF16X4": "STATS_BF16X4", "FP32": "STATS_FP32", "FP64S": "STATS_FP64_SHIFTED",
               "FP64": "STATS_FP64"}
 MODE_KERNEL = {"BF16X3": "split_kernel (mma.sync bf16)", "BF16X4": "split_kernel (mma.sync bf16)",
-               "FP32": "core_kernel<float>", "FP64S": "core_kernel<double> (shifted; fp64 kernel for p <= 12)",
-               "FP64": "core_kernel<double> (raw moments, the paper's plain FP64 kernel; fp64 kernel for p <= 12)"}
+               "FP32": "core32_kernel", "FP64S": "core64_kernel (shifted)",
+               "FP64": "core64_kernel (raw moments, the paper's plain FP64 kernel)"}
 
 
 def _base_line(args, world, metric, value, ms_per_step, config, roofline, clocks, launches, extra):

@@ -230,6 +230,9 @@ stats_status stats_finalize(stats_ctx* ctx, double* mean, double* cov, double* c
  * quantity from (n, s, S) alone ("Data Representation and Sufficient Statistics"), so a
  * snapshot can be taken between any two accumulate calls; this call makes a snapshot's
  * PCA ("Principal Component Analysis Results") cheap when the matrix has moved little.
+ *   Rounding: the error that products of FP64 columns of the matrix leave in an eigenpair, in the
+ *     units of its own columns (small eigenvalues of columns of small units are as accurate,
+ *     relative to themselves, as large ones), whichever path computed it.
  *   evecs_prev: HOST, p_a*p_a doubles, row k = eigenvector k, as written by an earlier
  *     stats_finalize / stats_finalize_warm (any ctx with the same p_a), or NULL (cold
  *     start).  The matrix M (cov, or corr with pca_on = 1) is rotated into that basis,
@@ -247,9 +250,10 @@ stats_status stats_finalize(stats_ctx* ctx, double* mean, double* cov, double* c
 stats_status stats_finalize_warm(stats_ctx* ctx, double* mean, double* cov, double* corr, double* evals,
                                  double* evecs, int32_t pca_on, const double* evecs_prev, int32_t* sweeps);
 
-/* stats_finalize for many contexts in one launch (one thread block per context; the
- * FP64 eigen-solver of each block is what a single call costs, so many contexts cost
- * about one call per SM-load instead of one call each).  Synchronises every context.
+/* stats_finalize for many contexts at once: one thread block per context, eigenpairs
+ * included below 24 analysis columns and above 64 (there by FP64 Jacobi rotations in the
+ * one block); the decompositions of 24..64 columns follow in a second launch, 1 to 4
+ * blocks each, as FP32 rotations and an FP64 refinement.  Synchronises every context.
  * mean, cov and corr are those of stats_finalize bit for bit; the eigenpairs too below 24
  * analysis columns, while from 24 columns (where stats_finalize runs its eigen-solver
  * over the whole GPU) they agree with stats_finalize's to rounding.

@@ -482,6 +482,8 @@ __device__ __forceinline__ uint64_t load8(const char* t, int64_t p, int64_t n) {
   return v;
 }
 
+// Eight digits in a word, the well-known way: a byte is no digit if XOR '0' leaves it above 9, and the digits are
+// joined two, four and eight at a time by multiplications with 10 * 2^8 + 1, 100 * 2^16 + 1 and 10000 * 2^32 + 1.
 // how many of the eight characters, from the first on, are digits; d: the bytes XOR '0'
 __device__ __forceinline__ int leading_digits(uint64_t d) {
   const uint64_t other = (((d & 0x7F7F7F7F7F7F7F7Full) + 0x7676767676767676ull) | d) & 0x8080808080808080ull;
@@ -490,9 +492,9 @@ __device__ __forceinline__ int leading_digits(uint64_t d) {
 // value of the first nd (1..8) digits: moved to the high bytes, then digits, pairs and fours joined
 __device__ __forceinline__ uint32_t digits_value(uint64_t d, int nd) {
   uint64_t v = d << (64 - 8 * nd);
-  v = (v * 2561u >> 8) & 0x00FF00FF00FF00FFull;
-  v = (v * 6553601u >> 16) & 0x0000FFFF0000FFFFull;
-  return static_cast<uint32_t>(v * 42949672960001ull >> 32);
+  v = (v * (10u << 8 | 1u) >> 8) & 0x00FF00FF00FF00FFull;
+  v = (v * (100u << 16 | 1u) >> 16) & 0x0000FFFF0000FFFFull;
+  return static_cast<uint32_t>(v * (10000ull << 32 | 1ull) >> 32);
 }
 
 // A run of digits from p on into v (at most 19 of them kept count of; more overflow v, and the

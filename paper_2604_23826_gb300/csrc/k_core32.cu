@@ -8,8 +8,8 @@
 //   - the output's upper triangle is cut into 8 x 4 register micro-tiles, one per thread: three
 //     128-bit shared loads and four register pairs feed 16 packed FMAs of two entries each (which
 //     take two cycles, so the other instructions issue beside them).  Only tiles on or above the
-//     diagonal exist, so 100 columns cost 5408 FMAs a row for 5050 entries.  Tiles of 8 x 8 with
-//     eight warps and 255 registers were slower (779 against 485 us, both with plain FMAs);
+//     diagonal exist, so 100 columns cost 5408 FMAs a row for 5050 entries (8 x 8 tiles would want
+//     192 registers for the sums and their (hi, lo) pairs);
 //   - when there are fewer tiles than threads, the rows of a stage are dealt to several slices of
 //     threads; when there are more, groups of blocks take a part of the tiles each.  core32_plan
 //     picks the number of groups by the instructions a row costs;
@@ -18,8 +18,7 @@
 //     while other warps still multiply the stage before: one barrier a stage.
 // Columns of other types, or not 16-byte aligned, are converted (x - c in FP64) into the same
 // stage by plain loads.
-// 1e6 rows x 100 columns: 8.78 ms as 64 x 64 tiles of scalar shared loads with an FP64 subtraction
-// per element, 0.427 ms now (its FMAs alone: 0.135 ms).
+// 1e6 rows x 100 columns: 0.427 ms (its FMAs alone: 0.135; as 64 x 64 tiles of scalar loads 8.78).
 // Each block writes one slot of (hi, lo) pairs; a second kernel adds the slots of an entry in row
 // order, in three-term FP32 expansions and then FP64 pairs (a fixed order: a given grid
 // reproduces its bits).  Sums that leave FP32's range on the way are added in FP64 instead, so only a

@@ -843,7 +843,7 @@ cudaError_t launch_finalize_batched(const FinalParams* d_params, int count, cons
 cudaError_t launch_finalize(const FinalParams& P, cudaStream_t stream) {
   // one block holds a wider table's entries too, but takes up to a millisecond over them
   if (P.mode != 0 && P.p > kSmallMax && (P.defer_A || !P.want_pca)) {
-    const int blocks = std::min((P.p * (P.p + 1) / 2 + kThreads - 1) / kThreads, 148);
+    const int blocks = (P.p * (P.p + 1) / 2 + kThreads - 1) / kThreads;  // 129 at most
     finalize_wide_kernel<<<blocks, kThreads, 0, stream>>>(P);
   } else {
     finalize_kernel<<<1, kThreads, 0, stream>>>(P);

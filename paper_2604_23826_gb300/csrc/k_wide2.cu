@@ -41,10 +41,8 @@
 //               tcgen05 fences order, so nothing waits for a release.
 // Bound: the two accumulator buffers.  Of a 64-row stage's 2350 cycles the MMAs take 1100 and the
 // issuer waited 900 for a drained buffer: the drain (16 columns a load, the next load in flight while
-// one is added) and the two crossings of the pair are longer than the other buffer's MMAs.  Relayed
-// and unpipelined drains: 1.2e7 rows x 256, BF16x3, 3.04 ms; now 2.89 (4.25 TB/s); 1e7 x 200, BF16x4,
-// 2.81 ms, now 2.63.  Registers 96 / 160: 2.99 and 2.79, 80 / 176: 2.97 and 2.63 (spills on one side
-// or the other).  Eight converter warps (of 56 or 64 registers) were slower: 3.1 to 4.0 ms.
+// one is added) and the two crossings of the pair are longer than the other buffer's MMAs.  With relayed,
+// unpipelined drains 1.2e7 rows x 256, BF16x3, took 3.04 ms; now 2.89 (4.25 TB/s).
 // A second kernel adds the pairs' slots, in pair order, into the context's double-double
 // accumulators.  Every wait is bounded; on expiry the CTA records STATS_ETIMEOUT and winds
 // down; both CTAs always reach the final cluster barrier (no early exit).
