@@ -41,17 +41,17 @@ BYTES_PER_ROW = {0: 60, 1: 44}
 # DRAM traffic per row of the exact pass (dram__bytes_read.sum + dram__bytes_write.sum over
 # the rows of one ncu capture, profiles/exact_pass_table1_L32_n5e7.md), with the hash of the
 # kernel sources it was taken on; reported as null once those sources change.
-NCU_TRAFFIC = {"bytes_per_row": 60.063, "src_hash": "494d4e2285bc479d", "layout": "L32"}
+NCU_TRAFFIC = {"bytes_per_row": 60.069, "src_hash": "d51aecd183f6ceb0", "layout": "L32"}
 
 
 # DRAM traffic of the FP32 split passes (BF16x3) from one ncu capture each on a smaller case:
 # reads per algorithmic byte (they grow with the rows) plus the per-launch slot writes (fixed);
 # profiles/wide2_pairs_p256_bf16x3_n4e6.md and profiles/narrow_tcgen05_p64_bf16x3_n8e6.md.
 NCU_TRAFFIC_SPLIT = {
-    "wide2": {"read_per_byte": 4226468096 / 4096000000, "write_bytes": 129752320,
-              "files": ("k_wide2.cu", "tc05.cuh", "common.cuh"), "src_hash": "8ef0eda9e15ca4b0"},
-    "narrow": {"read_per_byte": 2074064384 / 2048000000, "write_bytes": 30813184,
-               "files": ("k_narrow.cu", "tc05.cuh", "common.cuh"), "src_hash": "5e20ec1b3efe77b0"},
+    "wide2": {"read_per_byte": 4225884160 / 4096000000, "write_bytes": 129276928,
+              "files": ("k_wide2.cu", "tc05.cuh", "common.cuh"), "src_hash": "acbae5e43ac09111"},
+    "narrow": {"read_per_byte": 2074124544 / 2048000000, "write_bytes": 30823168,
+               "files": ("k_narrow.cu", "tc05.cuh", "common.cuh"), "src_hash": "bda23e6f35371f00"},
 }
 
 

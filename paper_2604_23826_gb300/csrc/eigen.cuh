@@ -549,7 +549,7 @@ __device__ __forceinline__ double reach(int step) {
 // but for eigenvalues that rounding cannot tell apart; from then on they are rounding and stay.
 // coarse (the first step): off-diagonals this small are still the squares of FP32's errors, and within a
 // cluster of equal eigenvalues hundreds of corrections of a tenth would add up (matrices of rank p / 2
-// went to the FP64 rotations: 256 columns 26 ms, 2.4 so); above 1e-3 they wait for the next step.
+// went to the FP64 rotations: 256 columns 26 ms, 2.3 so); above 1e-3 they wait for the next step.
 // Later steps take only what converges at least as fast as squares do, the last two only corrections that
 // need no further step: the rest, clusters of close eigenvalues, ends as an orthonormal basis that FP64
 // rotations start from (they started from the identity: 12 columns in clusters of 1e-6, seeded, 395 us, 285 so;

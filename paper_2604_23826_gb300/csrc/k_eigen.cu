@@ -16,7 +16,7 @@
 // Bound: latency.  A block round of step 2 takes 18,000 cycles: 17 dependent rounds of its 32 x 32
 // problems 10,400, their loads, the product, and the stores and barrier the rest.  Step 3 is FP64 at 2
 // operations per clock and SM: 256 columns, 0.13 ms a step.  (FP64 rotations alone, chains of divisions
-// and square roots of one warp: 256 columns, 11 sweeps, 14.7 ms; all of this 1.64.)
+// and square roots of one warp: 256 columns, 11 sweeps, 14.7 ms; all of this 1.61.)
 #include <math.h>
 
 #include "common.cuh"
@@ -380,7 +380,7 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
 // Returns the sweeps (A then points to the diagonal form), -1 after a wait that ran out.
 // Bound: the chains of the local rounds.  Angles from FP32 (rotation64) instead of an FP64 division and
 // two roots, and 112 rows instead of 128 for 100 columns: a matrix of 100 columns in four clusters of
-// eigenvalues 8.3 ms, 5.4 so; 256 columns 25.3 and 19.5.
+// eigenvalues 8.3 ms from the identity, 5.4 so (and 3.1 from the refined basis).
 __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V, int floor) {
   const int tid = threadIdx.x, m = J.m, n = (J.pa + kJP - 1) / kJP * kJP, nb = n / kJW, np = nb / 2;
   const int lr_ = tid / kJP, lc_ = tid % kJP;

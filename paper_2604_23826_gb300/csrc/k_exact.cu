@@ -250,7 +250,7 @@ struct ConvT1 {
 // pairs, whose bias takes a signed top byte's 128 off again.  The column loop is uniform across
 // the warp, so its branches cost one instruction each, and two rows of a lane share it.  (Bound: instruction issue and latency.
 // Eight mixed columns, 36 B a row, 2e7 rows: extracting every digit from its column anew took
-// 2.50 ms, this way 0.56 ms; 0.71 with one row a lane.)
+// 2.50 ms, this way 0.50 ms.)
 struct ConvGeneric {
   template <int TILE>
   __device__ __forceinline__ static SmemSrc smem_src(const uint8_t* st, const ExactParams& P, int r) {
