@@ -41,10 +41,10 @@ __device__ __forceinline__ float scaled32(double x, int E) {
 // About a^2 / |p q| of an entry a between the diagonal's p and q, from the exponents alone (a power of
 // two, at most 1; 0 for a = 0): sums of these tell how far a matrix is from diagonal in each pair's own
 // units.  Columns of very different units have eigenvalues far below the rounding of the largest, and an
-// off-diagonal that is nothing beside the norm may be everything to two of those.  floor: the exponent of
-// the smallest variance; what lies below it is rounding, or owes its size to cancellation.
-__device__ __forceinline__ float square_ratio(int ea, int ep, int eq, int floor) {
-  const int d = 2 * ea - max(ep, floor) - max(eq, floor);
+// off-diagonal that is nothing beside the norm may be everything to two of those.  fp, fq: exponents that
+// the diagonal's count as at least, of what its own rounding comes from.
+__device__ __forceinline__ float square_ratio(int ea, int ep, int eq, int fp, int fq) {
+  const int d = 2 * ea - max(ep, fp) - max(eq, fq);
   return ea == 0 || d < -126 ? 0.f : __int_as_float((127 + min(d, 0)) << 23);
 }
 __device__ __forceinline__ int exp_field32(float x) { return (__float_as_int(x) >> 23) & 0xFF; }
@@ -136,16 +136,29 @@ __device__ __forceinline__ int block_or(int v, int* s_red) {
   return t;
 }
 
-// exponent field of the smallest of a matrix's diagonal that is not zero, by the block
-__device__ __forceinline__ int smallest_variance(const double* A, int ld, int n, int* s_red) {
-  const int e = static_cast<int>(threadIdx.x) < n ? exp_field(A[static_cast<size_t>(threadIdx.x) * (ld + 1)]) : 0;
-  return -block_max(e ? -e : -0x7FF, s_red);
+// A matrix's diagonal (at most 256), by the block: the exponent field of its smallest that is not zero, and the
+// diagonal itself in FP32 over 2^(E - 1023), E - 1023 even and every |entry| below that.
+struct Variances {
+  int least, E;
+};
+__device__ __forceinline__ Variances variances(const double* A, int ld, int n, float* diag, int* s_red) {
+  const int t = threadIdx.x;
+  const double a = t < n ? A[static_cast<size_t>(t) * (ld + 1)] : 0.0;
+  const int e = exp_field(a);
+  Variances v{-block_max(e ? -e : -0x7FF, s_red), block_max(e, s_red) + 1};
+  v.E += (v.E + 1) & 1;
+  if (t < n) diag[t] = fabsf(scaled32(a, v.E));
+  __syncthreads();
+  return v;
 }
+// A column's weight sum_l a_ll x_lj^2, from the scaled diagonal, as an exponent field: products with it round to
+// about eps of that.
+__device__ __forceinline__ int weight_exponent(float w, int E) { return exp_field32(w) ? exp_field32(w) - 127 + E : 0; }
 
 // ------------------------------- FP64 -------------------------------
 struct Scratch64 {
   double c[128], s[128], red[8];
-  int p[128], q[128], null[128];
+  int p[128], q[128], null[128], weight[256];
 };
 
 // FP64 rotations are at an end when the off-diagonal is negligible (`norm`, by the caller) and so are the
@@ -155,16 +168,18 @@ struct Scratch64 {
 struct Ratios64 {
   float prev = 0.f;
   int stalled = 0;
+  bool settled = false;
   __device__ __forceinline__ bool done(bool norm, float rel, int n) {
-    stalled = norm && prev > 0.f && rel > 0.0625f * prev ? stalled + 1 : 0;
+    stalled = settled && rel > 0.0625f * prev ? stalled + 1 : 0;
+    settled |= norm;
     prev = rel;
-    return norm && (rel <= 1e-28f || (stalled >= 1 && rel <= 4e-30f * n * n) || stalled >= 4);
+    return settled && (rel <= 1e-28f || (stalled >= 1 && rel <= 4e-30f * n * n) || stalled >= 4);
   }
 };
 
 // Cyclic Jacobi on A (order n, at most 256; shared or global memory), its rotations applied to V's
-// columns, which hold the basis on entry; floor: square_ratio's.  Returns the sweeps taken.
-__device__ inline int jacobi64(double* A, int lda, double* V, int ldv, int n, int floor, Scratch64& S) {
+// columns, which hold the basis on entry; diag, E: of the matrix in its own basis.  Returns the sweeps taken.
+__device__ inline int jacobi64(double* A, int lda, double* V, int ldv, int n, const float* diag, int E, Scratch64& S) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, m = n + (n & 1), h = m / 2;
   double fro2 = 0.0;
   Ratios64 ratios;
@@ -172,12 +187,22 @@ __device__ inline int jacobi64(double* A, int lda, double* V, int ldv, int n, in
   for (; sweep < 60; ++sweep) {
     double off = 0.0, dia = 0.0;
     float rel = 0.f;
+    if (tid < n) {
+      float w = 0.f;
+      for (int l = 0; l < n; ++l) {
+        const float x = scaled32(V[l * ldv + tid], 1023);
+        w = fmaf(diag[l] * x, x, w);
+      }
+      S.weight[tid] = weight_exponent(w, E);
+    }
+    __syncthreads();
     for (int r = warp; r < n; r += kThreads / 32)
       for (int c = lane; c < n; c += 32) {
         const double x = A[r * lda + c];
         if (r != c) {
           off = fma(x, x, off);
-          rel += square_ratio(exp_field(x), exp_field(A[r * lda + r]), exp_field(A[c * lda + c]), floor);
+          rel += square_ratio(exp_field(x), exp_field(A[r * lda + r]), exp_field(A[c * lda + c]), S.weight[r],
+                              S.weight[c]);
         } else {
           dia = fma(x, x, dia);
         }
@@ -458,7 +483,7 @@ __device__ __forceinline__ bool rotated32(int sweep, T off, T prev, T fro2, T do
 
 // Cyclic Jacobi in FP32 on A (M x M floats, followed by its next copy), its rotations applied to V's
 // columns (the same), by the whole block.  At most max_sweeps; stops once the off-diagonal part is at
-// the level of FP32 rounding.  floor: square_ratio's.  Returns the sweeps taken; `copy`: which copies hold
+// the level of FP32 rounding.  floor: of the smallest variance.  Returns the sweeps taken; `copy`: which copies hold
 // the results.
 template <int M>
 __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_sweeps, int floor, Scratch32& S, int& copy) {
@@ -475,7 +500,7 @@ __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_
       const int r = i / M, c = i % M;
       if (r != c) {
         off = fmaf(x, x, off);
-        rel += square_ratio(exp_field32(x), exp_field32(X[r * M + r]), exp_field32(X[c * M + c]), floor);
+        rel += square_ratio(exp_field32(x), exp_field32(X[r * M + r]), exp_field32(X[c * M + c]), floor, floor);
       } else {
         dia = fmaf(x, x, dia);
       }
@@ -503,8 +528,8 @@ __device__ __forceinline__ int jacobi32(const float* A, const float* V, int max_
 // the product of two.  (A bound from the norm took FP32's leavings among small eigenvalues for rounding:
 // 40 columns of units over four decades, vectors wrong by 3e-7, over eight by 4e-3; now to 1e-14.)
 struct Noise {
-  double unit;  // 2^(exponent / 2)
-  int E;        // scaled32's exponent for the values: an even one, no |entry| larger
+  double unit;  // 2^((E - 1023) / 2)
+  int E;        // of variances()
   float root;   // 4 sqrt(columns)
   // of a column: `weight` = sum_l a_ll x_lj^2, scaled; `f` and `inverse` for the ratios of two columns
   __device__ __forceinline__ double column(double lambda, float weight, float& f, float& inverse) const {
@@ -516,20 +541,20 @@ struct Noise {
 // an exponent E with every |entry| < 2^(E - 1023), for a matrix whose squared Frobenius norm is fro2 (normal)
 __device__ __forceinline__ int scale_exponent(double fro2) { return 1023 + (exp_field(fro2) - 1023 + 2 + 2048) / 2 - 1024; }
 __device__ __forceinline__ Noise noise_of(int E, int n) {
-  const int h = (E - 1023 + 1 + 2048) / 2 - 1024;
-  return Noise{__hiloint2double((1023 + h) << 20, 0), 1023 + 2 * h, 4.f * sqrtf(static_cast<float>(n))};
+  return Noise{__hiloint2double((1023 + (E - 1023) / 2) << 20, 0), E, 4.f * sqrtf(static_cast<float>(n))};
 }
 // FP32 rotations take the matrix at 2^40 times its scale, so that what they leave alone (1e-18, whose square
 // FP32 still holds) lies 30 decades below the norm
 constexpr int kUp32 = 40;
-// square_ratio's floor of the matrix those work on
-__device__ __forceinline__ int floor32(int floor, int E) { return max(0, min(254, floor - E + kUp32 + 127)); }
+// the smallest variance's exponent in the matrix those work on (E: scale_exponent)
+__device__ __forceinline__ int floor32(int least, int E) { return max(0, min(254, least - E + kUp32 + 127)); }
 
 // corrections below this need no further step: what it leaves behind is their square times sqrt(m)
 constexpr float kRefined = 5e-9f;
 // of an entry's noise: off-diagonals below this may, in the first step, be the squares of FP32's errors
 constexpr double kCoarse = 5000.0;
 constexpr int kSteps = 8;
+constexpr int kPolish = 3;  // the step to go on from after FP64 rotations: small corrections, then none but tiny ones
 // what a step found
 constexpr int kMore = 1;    // some correction is too large to be the last
 constexpr int kClose = 2;   // some eigenvalues are too close for the refinement

@@ -12,7 +12,7 @@
 //      told from each pair's own columns, so the eigenpairs of columns of very different units are
 //      as good as those of like ones.
 //   4. If eigenvalues are too close for the refinement (or it fails), block-cyclic Jacobi in FP64,
-//      from the refined basis (or from the matrix as it came).
+//      from the refined basis (or from the matrix as it came), and the refinement's late steps.
 // Bound: latency.  A block round of step 2 takes 18,000 cycles: 17 dependent rounds of its 32 x 32
 // problems 10,400, their loads, the product, and the stores and barrier the rest.  Step 3 is FP64 at 2
 // operations per clock and SM: 256 columns, 0.13 ms a step.  (FP64 rotations alone, chains of divisions
@@ -88,7 +88,8 @@ struct Shared {
   double c[8], s[8];
   int null[8];
   double lambda[256], noise[256];
-  float nf[256], ni[256];
+  float nf[256], ni[256], diag[256];
+  int weight[256];
   double red[8];
   unsigned long long key[256];
   int order[256];
@@ -232,7 +233,8 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
       const int r = i / m, c = i % m;
       if (r != c) {
         o = fmaf(x, x, o);
-        q += square_ratio(exp_field32(x), exp_field32(__ldcg(A + r * (m + 1))), exp_field32(__ldcg(A + c * (m + 1))), floor);
+        q += square_ratio(exp_field32(x), exp_field32(__ldcg(A + r * (m + 1))), exp_field32(__ldcg(A + c * (m + 1))), floor,
+                          floor);
       } else {
         d = fmaf(x, x, d);
       }
@@ -381,23 +383,37 @@ __device__ int grid_jacobi32(const JacobiParams& J, Grid& grid, Shared& S, float
 // Bound: the chains of the local rounds.  Angles from FP32 (rotation64) instead of an FP64 division and
 // two roots, and 112 rows instead of 128 for 100 columns: a matrix of 100 columns in four clusters of
 // eigenvalues 8.3 ms from the identity, 5.4 so (and 3.1 from the refined basis).
-__device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V, int floor) {
+// E: of variances(), whose diagonal is in S.
+__device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, double*& A, double* B, double* V, int E) {
   const int tid = threadIdx.x, m = J.m, n = (J.pa + kJP - 1) / kJP * kJP, nb = n / kJW, np = nb / 2;
   const int lr_ = tid / kJP, lc_ = tid % kJP;
   const int nthreads = gridDim.x * kThreads, gtid = blockIdx.x * kThreads + tid;
   double fro2 = 0.0, prev = 0.0;
   Ratios64 ratios;
   int sweep = 0, stalled = 0;
+  auto at = [m](int r, int c) { return static_cast<size_t>(r) * m + c; };
+  float* weights = reinterpret_cast<float*>(J.slots + 384);
+  auto weigh = [&] {  // V's columns, shared out over the grid
+    for (int j = blockIdx.x; j < n; j += gridDim.x) {
+      const float x = tid < J.pa ? scaled32(__ldcg(V + at(tid, j)), 1023) : 0.f;
+      const float w = block_total(tid < J.pa ? S.diag[tid] * x * x : 0.f, reinterpret_cast<float*>(S.red));
+      if (tid == 0) __stcg(weights + j, w);
+    }
+  };
+  weigh();
+  if (!grid.sync()) return -1;
   for (; sweep < 60; ++sweep) {
+    if (tid < n) S.weight[tid] = weight_exponent(__ldcg(weights + tid), E);
+    __syncthreads();
     double o = 0.0, d = 0.0;
     float q = 0.f;
-    auto at = [m](int r, int c) { return static_cast<size_t>(r) * m + c; };
     for (int i = gtid; i < n * n; i += nthreads) {
       const int r = i / n, c = i % n;
       const double x = __ldcg(A + at(r, c));
       if (r != c) {
         o = fma(x, x, o);
-        q += square_ratio(exp_field(x), exp_field(__ldcg(A + at(r, r))), exp_field(__ldcg(A + at(c, c))), floor);
+        q += square_ratio(exp_field(x), exp_field(__ldcg(A + at(r, r))), exp_field(__ldcg(A + at(c, c))), S.weight[r],
+                          S.weight[c]);
       } else {
         d = fma(x, x, d);
       }
@@ -420,6 +436,7 @@ __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, doubl
     const bool norm = off <= 1e-34 * fro2 || (stalled >= 1 && off <= 4e-30 * n * fro2) || (stalled >= 4 && off <= 1e-26 * fro2);
     if (off == 0.0 || ratios.done(norm, rel, n)) break;
     prev = off;
+    weigh();  // for the next sweep's test, whose barriers are to come
     for (int br = 0; br < nb - 1; ++br) {
       // (1) every block pair's kJP x kJP diagonal problem: one cyclic Jacobi sweep in shared
       //     memory, its rotations accumulated in Q (to J.q), its result written to B
@@ -428,7 +445,8 @@ __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, doubl
         pair_of(br, P, nb, bi, bj);
         const int gr = lr_ < kJW ? bi * kJW + lr_ : bj * kJW + lr_ - kJW;
         const int gc = lc_ < kJW ? bi * kJW + lc_ : bj * kJW + lc_ - kJW;
-        S.x[lr_][lc_] = __ldcg(A + static_cast<size_t>(gr) * m + gc);
+        // both halves alike: what rounding makes of their difference no rotation would take away
+        S.x[lr_][lc_] = 0.5 * (__ldcg(A + at(gr, gc)) + __ldcg(A + at(gc, gr)));
         S.y[lr_][lc_] = lr_ == lc_ ? 1.0 : 0.0;
         __syncthreads();
         for (int lr = 0; lr < kJP - 1; ++lr) {
@@ -526,7 +544,8 @@ __device__ int grid_jacobi64(const JacobiParams& J, Grid& grid, Shared& S, doubl
 
 }  // namespace
 
-// a, b, v, w, g, x: m x m; the FP64 rotations (a quarter of that is the FP32 ones'); the seed; slots
+// a, b, v, w, g, x: m x m (a stays the matrix); the FP64 rotations (a quarter of that is the FP32 ones'); the
+// seed; slots
 size_t jacobi_scratch_doubles(int pa) {
   const size_t m = jacobi_order(pa);
   return 6 * m * m + static_cast<size_t>(pa) * pa + (m / kJP) * kJP * kJP + 1024 + 8;
@@ -575,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     alive = grid.sync();
   }
   const double fro2 = alive ? slots_total<double>(J.slots, S) : 0.0;
-  const int floor = smallest_variance(A, m, pa, reinterpret_cast<int*>(S.red));
+  const Variances var = variances(A, m, pa, S.diag, reinterpret_cast<int*>(S.red));
   if (alive && J.basis) {
     // the seed is used only if its columns are orthonormal: max |V^T V - I| <= 1e-9
     double dev = 0.0;
@@ -603,12 +622,12 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
     }
   }
 
-  bool refined = false;  // lambda and X hold the result
-  bool warm = false;     // X is orthonormal, but some eigenvalues are too close for the refinement
-  double* X = J.x;
+  double* X = J.w;
   double* Xn = V;
+  double* W = J.x;  // A X, then the corrections
   // FP32 has to hold the matrix scaled to order one, FP64 the squares of its entries
-  if (alive && fro2 > 1e-280 && fro2 < 1e280) {
+  const bool in_range = fro2 > 1e-280 && fro2 < 1e280;
+  if (alive && in_range) {
     const int E = scale_exponent(fro2);
     float* F = reinterpret_cast<float*>(J.g);  // two m x m FP32 matrices
     float* Q32 = reinterpret_cast<float*>(J.x);  // V of step 2
@@ -627,10 +646,10 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
         __syncthreads();
         int n = 0, copy = 0;
         switch (m) {
-          case 16: n = jacobi32<16>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
-          case 32: n = jacobi32<32>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
-          case 48: n = jacobi32<48>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
-          default: n = jacobi32<64>(sA, sV, 20, floor32(floor, E), S.s32, copy); break;
+          case 16: n = jacobi32<16>(sA, sV, 20, floor32(var.least, E), S.s32, copy); break;
+          case 32: n = jacobi32<32>(sA, sV, 20, floor32(var.least, E), S.s32, copy); break;
+          case 48: n = jacobi32<48>(sA, sV, 20, floor32(var.least, E), S.s32, copy); break;
+          default: n = jacobi32<64>(sA, sV, 20, floor32(var.least, E), S.s32, copy); break;
         }
         sV += copy * m * m;
         for (int i = tid; i < m * m; i += kThreads) __stcg(Q32 + i, sV[i]);
@@ -645,7 +664,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
       }
       alive = grid.sync();
       if (alive) {
-        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32, floor32(floor, E));
+        sweeps = grid_jacobi32(J, grid, S, dyn, F, F + static_cast<size_t>(m) * m, Q32, floor32(var.least, E));
         alive = sweeps >= 0;
       }
     }
@@ -660,11 +679,15 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
         for (int i = gtid; i < m * m; i += nthreads) __stcg(J.w + i, f32_to_f64(__ldcg(Q32 + i)));
       alive = grid.sync();
     }
-    double* W = J.x;  // A X, then the corrections
-    X = J.w;
-    const Noise noise = noise_of(E, pa);
-    float* weights = reinterpret_cast<float*>(J.slots + 256);
-    for (int it = 0; alive && it < kSteps; ++it) {
+  }
+  // the refinement; if need be FP64 rotations, and its late steps for what they leave
+  const Noise noise = noise_of(var.E, pa);
+  float* weights = reinterpret_cast<float*>(J.slots + 256);
+  int it = 0;
+  for (bool rotated = false; alive; rotated = true) {
+    bool refined = false;  // lambda and X hold the result
+    bool warm = false;     // X is orthonormal, but some eigenvalues are too close for the refinement
+    for (; in_range && it < kSteps; ++it) {
       grid_product(
           m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(X + at(k, j)); },
           [&](int i, int j, double v) { __stcg(W + at(i, j), v); });
@@ -702,35 +725,36 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_grid_kernel(const __grid_c
         break;
       }
     }
-  }
-  if (alive && !refined) {
-    if (warm) {  // A <- X^T A X, symmetrised, and on from there
-      double* W = J.x;
+    if (!alive || refined || rotated) break;
+    double* R = J.g;  // what is rotated: X^T A X, symmetrised, or A
+    if (warm) {
       grid_product(
           m, S, [&](int i, int k) { return __ldcg(A + at(i, k)); }, [&](int k, int j) { return __ldcg(X + at(k, j)); },
           [&](int i, int j, double v) { __stcg(W + at(i, j), v); });
-      alive = grid.sync();
-      if (alive)
-        grid_product(
-            m, S, [&](int i, int k) { return __ldcg(X + at(k, i)); }, [&](int k, int j) { return __ldcg(W + at(k, j)); },
-            [&](int i, int j, double v) { __stcg(J.b + at(i, j), v); });
-      alive = alive && grid.sync();
-      if (alive)
-        for (int i = gtid; i < m * m; i += nthreads)
-          __stcg(A + i, 0.5 * (__ldcg(J.b + i) + __ldcg(J.b + at(i % m, i / m))));
+      if (!(alive = grid.sync())) break;
+      grid_product(
+          m, S, [&](int i, int k) { return __ldcg(X + at(k, i)); }, [&](int k, int j) { return __ldcg(W + at(k, j)); },
+          [&](int i, int j, double v) { __stcg(J.b + at(i, j), v); });
+      if (!(alive = grid.sync())) break;
+      for (int i = gtid; i < m * m; i += nthreads)
+        __stcg(R + i, 0.5 * (__ldcg(J.b + i) + __ldcg(J.b + at(i % m, i / m))));
     } else {
       X = V;
-      for (int i = gtid; alive && i < m * m; i += nthreads) __stcg(X + i, (i / m == i % m) ? 1.0 : 0.0);
+      for (int i = gtid; i < m * m; i += nthreads) {
+        __stcg(X + i, (i / m == i % m) ? 1.0 : 0.0);
+        __stcg(R + i, __ldcg(A + i));
+      }
       seeded = false;
     }
-    alive = alive && grid.sync();
-    if (alive) {
-      const int n = grid_jacobi64(J, grid, S, A, J.b, X, floor);
-      alive = n >= 0;
-      sweeps += max(n, 0);
-      if (alive && tid < m) S.lambda[tid] = __ldcg(A + at(tid, tid));
-      __syncthreads();
-    }
+    if (!(alive = grid.sync())) break;
+    const int n = grid_jacobi64(J, grid, S, R, J.b, X, var.E);
+    if (!(alive = n >= 0)) break;
+    sweeps += n;
+    if (tid < m) S.lambda[tid] = __ldcg(R + at(tid, tid));
+    __syncthreads();
+    Xn = X == V ? J.w : V;
+    it = kPolish;
+    if (!(alive = grid.sync())) break;  // b and g are free again
   }
   if (!alive) {
     if (tid == 0) flags[5] = 1.0;

@@ -353,7 +353,7 @@ constexpr bool orders_exist() {
 static_assert(orders_exist(), "eigen_mixed has the rotations of every order");
 
 // Eigenpairs of A (n x n, 1 <= n <= 64, anywhere) in one block: FP32 Jacobi, FP64 refinement, and FP64
-// Jacobi from the refined basis where eigenvalues are too close for it (or from A as it is).  X, W, S:
+// Jacobi from the refined basis where eigenvalues are too close for it (or from A as it is), refined once more.  X, W, S:
 // shared memory of leading dimension ld (odd, above n), S right behind W.  The eigenvalues are left in M.lambda, the
 // vectors in the columns of X (which may become the buffer S or W was).  Returns the sweeps taken.
 // A team shares the refinement (not kSmall); the rotations, and everything decided, all its blocks do
@@ -367,10 +367,11 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
   double f = 0.0;
   for (int i = tid; i < n * n; i += kThreads) f = fma(A[i], A[i], f);
   const double fro2 = block_total(f, M.red);
-  const int floor = smallest_variance(A, n, n, reinterpret_cast<int*>(M.red));
-  bool refined = false, warm = false;
+  const Variances var = variances(A, n, n, M.diag, reinterpret_cast<int*>(M.red));
+  const Noise noise = noise_of(var.E, n);
   int sweeps = 0;
-  if (fro2 > 1e-280 && fro2 < 1e280) {
+  const bool in_range = fro2 > 1e-280 && fro2 < 1e280;
+  if (in_range) {
     const int E = scale_exponent(fro2);
     const int m = mixed_order<kSmall>(n);
     float* fA = reinterpret_cast<float*>(W);  // W and S, one behind the other
@@ -380,27 +381,30 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
       fA[i] = r < n && c < n ? scaled32(A[r * n + c], E - kUp32) : 0.f;
       fV[i] = r == c ? 1.f : 0.f;
     }
-    const Noise noise = noise_of(E, n);
-    if (tid < n) M.diag[tid] = fabsf(scaled32(A[tid * n + tid], noise.E));
     __syncthreads();
     int copy = 0;
     if constexpr (kSmall) {
       switch (m) {
-        case 8: sweeps = jacobi32<8>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
-        case 16: sweeps = jacobi32<16>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
-        case 24: sweeps = jacobi32<24>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+        case 8: sweeps = jacobi32<8>(fA, fV, 20, floor32(var.least, E), M.s32, copy); break;
+        case 16: sweeps = jacobi32<16>(fA, fV, 20, floor32(var.least, E), M.s32, copy); break;
+        case 24: sweeps = jacobi32<24>(fA, fV, 20, floor32(var.least, E), M.s32, copy); break;
       }
     } else {
       switch (m) {
-        case 32: sweeps = jacobi32<32>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
-        case 48: sweeps = jacobi32<48>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
-        case 64: sweeps = jacobi32<64>(fA, fV, 20, floor32(floor, E), M.s32, copy); break;
+        case 32: sweeps = jacobi32<32>(fA, fV, 20, floor32(var.least, E), M.s32, copy); break;
+        case 48: sweeps = jacobi32<48>(fA, fV, 20, floor32(var.least, E), M.s32, copy); break;
+        case 64: sweeps = jacobi32<64>(fA, fV, 20, floor32(var.least, E), M.s32, copy); break;
       }
     }
     fV += copy * m * m;
     for (int i = tid; i < n * n; i += kThreads) X[(i / n) * ld + i % n] = f32_to_f64(fV[(i / n) * m + i % n]);
+  }
+  // the refinement; if need be FP64 rotations, and its late steps for what they leave
+  int it = 0;
+  for (bool rotated = false;; rotated = true) {
     team.meet();  // the others may put into W and S now
-    for (int it = 0; it < kSteps; ++it) {
+    bool refined = false, warm = false;
+    for (; in_range && it < kSteps; ++it) {
       team_product(
           team, n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
           [&](int i, int j, double v) { team.put(W + i * ld + j, v); });
@@ -487,8 +491,7 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
         break;
       }
     }
-  }
-  if (!refined) {
+    if (refined || rotated) break;
     if (warm) {  // FP64 Jacobi on X^T A X, from the refined basis
       team_product(
           alone, n, [&](int k, int i) { return A[k * n + i]; }, [&](int k, int j) { return X[k * ld + j]; },
@@ -506,8 +509,9 @@ __device__ int eigen_mixed(const double* A, int n, double*& X, double* W, double
       }
     }
     __syncthreads();
-    sweeps += jacobi64(S, ld, X, ld, n, floor, M.s64);
+    sweeps += jacobi64(S, ld, X, ld, n, M.diag, var.E, M.s64);
     if (tid < n) M.lambda[tid] = S[tid * ld + tid];
+    it = kPolish;
   }
   __syncthreads();
   return sweeps;
@@ -528,6 +532,7 @@ __device__ void finalize_body(const FinalParams& P) {
   } U;
   __shared__ short s_idx[256];
   __shared__ double s_sd[256], s_lambda[256];
+  __shared__ float s_diag[256];
   __shared__ int s_order[256];
   __shared__ double s_den;
   __shared__ int s_over;
@@ -681,8 +686,8 @@ __device__ void finalize_body(const FinalParams& P) {
       V[i] = i / pa == i % pa ? 1.0 : 0.0;
     }
     __syncthreads();
-    const int floor = smallest_variance(A, pa, pa, reinterpret_cast<int*>(U.any.red));
-    const int sweeps = jacobi64(A, pa, V, pa, pa, floor, U.any);
+    const Variances var = variances(A, pa, pa, s_diag, reinterpret_cast<int*>(U.any.red));
+    const int sweeps = jacobi64(A, pa, V, pa, pa, s_diag, var.E, U.any);
     if (tid < pa) s_lambda[tid] = A[tid * pa + tid];
     __syncthreads();
     put_eigenpairs(s_lambda, V, pa, pa, s_order, out + L.evals, out + L.evecs);

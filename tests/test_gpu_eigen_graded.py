@@ -117,3 +117,24 @@ def test_clusters_go_on_from_the_refined_basis(p, most):
     assert 0 < an.sweeps <= most
     assert np.abs(an.evecs @ an.evecs.T - np.eye(p)).max() <= 1e-12
     assert np.abs(an.evecs @ an.cov @ an.evecs.T - np.diag(an.evals)).max() <= 1e-13 * scale
+
+
+@pytest.mark.parametrize("p", [6, 12, 23, 24, 40, 64, 100, 256])
+def test_units_and_repeated_columns(p):
+    """Half of the eigenvalues zero, at every unit: their rounding, eps of the repeated columns' variance, hides the
+    eigenvalues of smaller units, so some pairs go through FP64 rotations.  The same bound, by the vectors' own
+    sums: it holds for what ends in the refinement, so for all but batches above 64 columns (FP64 rotations
+    alone, whose intermediate vectors it says nothing about)."""
+    rng = np.random.default_rng(p)
+    L, _ = inputs.wide_factor(p, p)
+    X = inputs.gen_correlated_host(N, L, np.zeros(p), seed=1) * 10.0 ** rng.uniform(-4, 4, p)[:, None]
+    X[p // 2:p // 2 * 2] = X[:p // 2]
+    X = X[rng.permutation(p)]
+    warm = G.stats_finalize_warm(context(X, N))
+    assert 0 < warm.sweeps < 45
+    single, *batch, seeded = all_ways(X)
+    for an in (warm, single, seeded, *(batch if p <= 64 else ())):
+        s = np.abs(an.evecs) @ np.sqrt(np.diag(an.cov))
+        assert np.abs(an.evecs @ an.evecs.T - np.eye(p)).max() <= 1e-12
+        R = an.evecs @ an.cov @ an.evecs.T - np.diag(an.evals)
+        assert np.all(np.abs(R) <= 4 * p * 2.0 ** -53 * np.outer(s, s))
