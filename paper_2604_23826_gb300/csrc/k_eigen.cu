@@ -16,7 +16,7 @@
 // Bound: latency.  A block round of step 2 takes 18,000 cycles: 17 dependent rounds of its 32 x 32
 // problems 10,400, their loads, the product, and the stores and barrier the rest.  Step 3 is FP64 at 2
 // operations per clock and SM: 256 columns, 0.13 ms a step.  (FP64 rotations alone, chains of divisions
-// and square roots of one warp: 256 columns, 11 sweeps, 14.7 ms; all of this 1.61.)
+// and square roots of one warp: 256 columns, 11 sweeps, 14.7 ms; all of this 1.65.)
 #include <math.h>
 
 #include "common.cuh"
